@@ -21,12 +21,10 @@ struct br_ctx {
     int32_t G, H;
     br_params p;              // resolved parameters
     StepArgs base;            // constant part of the kernel arguments
-    int threads;              // threads per instance for large batches
-    int threads_small;        // ... for batches of a few instances (latency path)
-    int inst_per_block;       // single-warp instances per thread block
+    int inst_per_block;       // instances per thread block of br_small_kernel
     bool small_ok;            // the fleet shape fits br_small_kernel
+    double d[BR_MAX_H + 1];   // (1, gamma, ..., gamma^H)
     bool two_probe_ok;        // both sides of the score's peak are strictly monotone up to Delta = 32 s_max
-    size_t smem;
     // latency path
     cudaGraph_t graph;
     cudaGraphExec_t graph_exec;
@@ -70,22 +68,39 @@ inline bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintp
 
 typedef void (*step_kernel_t)(const StepArgs);
 
-// lean: 0 general, 1 constant hazard and no optional outputs, 2 the same on a single warp
-template <int GW>
-step_kernel_t pick_kernel_gw(bool fp, int H, int lean)
+template <bool FP, int HC>
+step_kernel_t pick_kernel_gw(int G)
 {
-    if (!fp) return lean == 2 ? br::br_step_kernel<false, 0, GW, 2> : br::br_step_kernel<false, 0, GW, 0>;
-    if (H == 0) return br::br_step_kernel<true, 0, GW, 0>;
-    if (H <= 4) return lean ? br::br_step_kernel<true, 4, GW, 1> : br::br_step_kernel<true, 4, GW, 0>;
-    if (H <= 8) return lean ? br::br_step_kernel<true, 8, GW, 1> : br::br_step_kernel<true, 8, GW, 0>;
-    if (H <= 16) return lean ? br::br_step_kernel<true, 16, GW, 1> : br::br_step_kernel<true, 16, GW, 0>;
-    // longer horizons (up to BR_MAX_H): projected loads and margins live in shared memory
-    return lean ? br::br_step_kernel<true, BR_MAX_H, GW, 1> : br::br_step_kernel<true, BR_MAX_H, GW, 0>;
+    return G <= 32 ? br::br_step_kernel<FP, 1, HC> : br::br_step_kernel<FP, 2, HC>;
 }
 
-step_kernel_t pick_kernel(bool fp, int H, int G, int lean)
+// Eq. 1 or Eq. 2; one or two workers per router lane; up to 31 or up to 95 horizon offsets
+step_kernel_t pick_kernel(bool fp, int H, int G)
 {
-    return G <= 32 ? pick_kernel_gw<1>(fp, H, lean) : pick_kernel_gw<2>(fp, H, lean);
+    if (!fp) return pick_kernel_gw<false, 1>(G);
+    return H < 32 ? pick_kernel_gw<true, 1>(G) : pick_kernel_gw<true, 3>(G);
+}
+
+constexpr int kSMs = 148;
+
+// Threads per instance of br_step_kernel.  An instance has parallel work for `most` threads (projection:
+// 16 slots a thread, queue: 4 positions a thread); more only lengthen its barriers.  When the batch
+// puts several instances on an SM they share its registers, which hold 28 warps (20 for long
+// horizons): with fewer threads per instance all of them are resident and none waits for a second wave.
+int threads_for(const br_ctx *ctx, int n_instances)
+{
+    if (ctx->p.threads > 0) return ctx->p.threads;
+    const int A = ctx->G * ctx->p.B;
+    int most = ctx->H > 0 ? A / 16 : 64;
+    if (ctx->p.W / 4 > most) most = ctx->p.W / 4;
+    most = (most + 31) / 32;
+    most = most < 1 ? 1 : (most > 8 ? 8 : most);
+    int per_sm = (n_instances + kSMs - 1) / kSMs;
+    const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
+    if (per_sm > fit) per_sm = fit;
+    int w = (ctx->H < 32 ? 28 : 20) / per_sm;
+    w = w < 1 ? 1 : (w > most ? most : w);
+    return 32 * w;
 }
 
 int check_step_args(const br_ctx *ctx, const br_instance_batch *b, const br_worker_state *ws,
@@ -149,10 +164,11 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
     a.term_probs = term_probs;
     a.assign_out = assign_out;
     a.out = *out;
-    // few instances: the launch is latency-bound, so spread each instance over more warps
-    const int tpi = b->n_instances <= 64 ? ctx->threads_small : ctx->threads;
-    if (tpi == 32 && ctx->small_ok && !out->fscore && !out->phase_cycles) {
-        // BR-0 on a small fleet: the one-warp-per-instance kernel
+    // BR-0 on a small fleet runs on one warp per instance; a few instances with more than 1,024 slots are
+    // latency-bound and take the block-per-instance kernel
+    const bool one_warp = ctx->p.threads == 32 ||
+                          (ctx->p.threads <= 0 && (b->n_instances > 64 || ctx->G * ctx->p.B <= 1024));
+    if (one_warp && ctx->small_ok && !out->fscore && !out->phase_cycles) {
         int wpb = ctx->inst_per_block;
         if (wpb > b->n_instances) wpb = b->n_instances;
         const int nt4 = ctx->p.W <= 128 ? 1 : (ctx->p.W <= 256 ? 2 : 4);
@@ -160,34 +176,24 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
         step_kernel_t kern = nt4 == 1 ? (r4 ? br::br_small_kernel<1, 4> : br::br_small_kernel<1, 5>)
                            : nt4 == 2 ? (r4 ? br::br_small_kernel<2, 4> : br::br_small_kernel<2, 5>)
                                       : (r4 ? br::br_small_kernel<4, 4> : br::br_small_kernel<4, 5>);
-        a.tpi = 32;
         const int blocks = (b->n_instances + wpb - 1) / wpb;
         cudaError_t e = launch_overlapped(kern, blocks, 32 * wpb, (size_t)wpb * nt4 * 128 * 2 * sizeof(int), stream, a, overlap);
         if (e == cudaSuccess) e = cudaGetLastError();
         if (e != cudaSuccess) return cuda_fail(e, "br_step launch");
         return BR_OK;
     }
-    const int lean = (ctx->p.term_mode == 1 && !out->fscore && !out->phase_cycles && !ctx->base.big_window)
-                         ? (tpi == 32 ? 2 : 1) : 0;
-    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, lean);
-    // instances are packed several to a block: single-warp ones always, wider ones only in full
-    // blocks (their barriers are block barriers)
-    int per_block = ctx->inst_per_block;
-    if (tpi > 32) { while (per_block > 1 && (per_block * tpi > 256 || b->n_instances % per_block != 0)) --per_block; }
-    if (per_block > b->n_instances) per_block = b->n_instances;
-    while (per_block > 1 && ctx->smem * per_block > 48 * 1024) --per_block;
-    if (tpi > 32 && per_block > 1 && b->n_instances % per_block != 0) per_block = 1;
-    a.tpi = tpi;
-    a.block_sync = (per_block > 1 && b->n_instances % per_block == 0) ? 1 : 0;
-    a.smem_per_inst = (int32_t)ctx->smem;
-    const int blocks = (b->n_instances + per_block - 1) / per_block;
-    if (ctx->smem * per_block > 48 * 1024) {
+    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G);
+    const int threads = threads_for(ctx, b->n_instances);
+    // lanes per worker that turn its buckets into projected loads
+    a.seg_log2 = 0;
+    while (a.seg_log2 < 5 && (ctx->G << (a.seg_log2 + 1)) <= threads && (2 << a.seg_log2) <= ctx->H + 1) ++a.seg_log2;
+    const int smem = a.lay.total;
+    if (smem > 48 * 1024) {
         // beyond the default limit: opt the kernel in (br_create has checked the device maximum)
-        cudaError_t eo = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)(ctx->smem * per_block));
+        cudaError_t eo = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (eo != cudaSuccess) return cuda_fail(eo, "cudaFuncSetAttribute(shared memory)");
     }
-    cudaError_t e = launch_overlapped(kern, blocks, tpi * per_block, ctx->smem * per_block, stream, a, overlap);
+    cudaError_t e = launch_overlapped(kern, b->n_instances, threads, (size_t)smem, stream, a, overlap);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "br_step launch");
     return BR_OK;
@@ -254,30 +260,18 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
             !isfinite(p.alpha) || !isfinite(p.beta))
             return BR_EINVAL;
     }
-    const int A = G * p.B;
-    int threads_small, threads_large;
-    if (p.threads > 0) {
-        if (p.threads % 32 != 0 || p.threads > 256) return BR_EINVAL;
-        threads_small = threads_large = p.threads;
-    } else {
-        const int work = A * (H > 0 ? 2 : 1);
-        int w = (work + 4095) / 4096;
-        threads_large = 32 * (w < 1 ? 1 : (w > 8 ? 8 : w));
-        w = (work + 1023) / 1024;
-        threads_small = 32 * (w < 1 ? 1 : (w > 8 ? 8 : w));
-    }
+    if (p.threads > 0 && (p.threads % 32 != 0 || p.threads > 256)) return BR_EINVAL;
 
     br_ctx *ctx = new (std::nothrow) br_ctx();
     if (!ctx) return BR_ENOMEM;
     memset(ctx, 0, sizeof(*ctx));
     ctx->G = G; ctx->H = H; ctx->p = p;
-    ctx->threads = threads_large; ctx->threads_small = threads_small;
     ctx->inst_per_block = p.inst_per_block > 0 ? (p.inst_per_block > 8 ? 8 : p.inst_per_block) : 4;
     StepArgs &a = ctx->base;
     a.G = G; a.H = H; a.B = p.B; a.W = p.W; a.R_max = p.R_max; a.S_greedy = p.S_greedy;
     a.occ_words = (p.B + 63) / 64;
     a.wl = wl;
-    a.magic_B = (uint32_t)(((1ull << 32) + (unsigned)p.B - 1) / (unsigned)p.B);
+    a.Wp = (p.W + 127) / 128 * 128; a.HS = br::step_row_stride(H);
     a.delta_T = p.delta_T; a.gate = p.gate; a.c_floor = p.c_floor;
     a.term_mode = p.term_mode; a.term_cdf = p.term_cdf;
     a.pred_mode = p.pred_mode; a.out_tab = p.out_tab; a.out_shift = 32 - p.out_tab_log2;
@@ -287,45 +281,49 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
     a.burst_every = p.burst_every; a.burst_size = p.burst_size;
     // d = (1, gamma, ..., gamma^H) by repeated multiplication; D = 1^T d left to right
     volatile double D = 0.0;
-    for (int h = 0; h <= BR_MAX_H; ++h) a.d[h] = 0.0;
+    for (int h = 0; h < BR_MAX_H + 4; ++h) { a.dn[2 * h] = 0.0; a.dn[2 * h + 1] = 0.0; }
+    for (int h = 0; h <= BR_MAX_H; ++h) ctx->d[h] = 0.0;
     if (p.score_mode == 1) {
         for (int h = 0; h <= H; ++h) {
-            volatile double dh = (h == 0) ? 1.0 : a.d[h - 1] * p.gamma;
-            a.d[h] = dh;
+            volatile double dh = (h == 0) ? 1.0 : ctx->d[h - 1] * p.gamma;
+            ctx->d[h] = dh;
+            a.dn[2 * h] = dh; a.dn[2 * h + 1] = -dh * 4503599627370496.0;      // exact: a power of two
             D = D + dh;
         }
         volatile double aD = p.alpha * D;
         a.aD = aD; a.beta = p.beta;
         // The single-request arg-max may use the concavity of Eq. 2 only if no segment slope
-        // alpha D - beta sum_{h in P} d_h (P any set of passed kinks) is within rounding distance of
-        // zero: then fp64 scores of integer lengths are strictly ordered on both sides of the peak.
-        // The 2^(H+1) slopes are enumerated for H <= 16; longer horizons score every request.
-        a.peak_ok = 0;
+        // alpha D - beta sum_{h in P} d_h is within rounding distance of zero: then fp64 scores of integer
+        // lengths are strictly ordered on both sides of the peak.  The kernel checks the slopes of the
+        // kinks at hand (P: the offsets whose kink is passed) against this bound; the slope before the
+        // first kink is alpha D.
+        const double err = 4.0 * (H + 5) * 1.1102230246251565e-16 * (a.aD + p.beta * D) * (double)p.s_max;
+        a.slope_err = err > 1e-9 ? err : 1e-9;
+        if (!(a.aD > a.slope_err)) a.slope_err = INFINITY;                     // never ordered: every request is scored
+        // Subsets of up to 32 requests (Delta <= 32 s_max): the two-probe rule of the large-window solvers
+        // asks the same of all 2^(H+1) sets P, enumerated here for H <= 16.
         if (H <= 16) {
             const int n = H + 1;
             double min_abs = 1e300;
             for (unsigned mask = 0; mask < (1u << n); ++mask) {
                 double w = 0.0;
-                for (int h = 0; h < n; ++h) if (mask >> h & 1u) w += a.d[h];
+                for (int h = 0; h < n; ++h) if (mask >> h & 1u) w += ctx->d[h];
                 const double sl = fabs(a.aD - p.beta * w);
                 if (sl < min_abs) min_abs = sl;
             }
-            const double err = 4.0 * (H + 5) * 1.1102230246251565e-16 * (a.aD + p.beta * D) * (double)p.s_max;
-            a.peak_ok = (min_abs > err && min_abs > 1e-9) ? 1 : 0;
-            // the same for subsets of up to 32 requests (Delta <= 32 s_max): the two-probe rule of the
-            // large-window solvers
             ctx->two_probe_ok = min_abs > 32.0 * err && min_abs > 1e-9;
         }
     } else {
-        a.d[0] = 1.0; a.aD = 1.0; a.beta = (double)G; a.peak_ok = 0;
+        ctx->d[0] = 1.0; a.dn[0] = 1.0; a.aD = 1.0; a.beta = (double)G;
         ctx->two_probe_ok = G >= 2;            // Eq. 1 falls with slope -(G - 1) beyond the margin
+        a.peak_ok = G >= 2;
     }
     // Stage-2 windows beyond five requests are solved by meeting in the middle, which rests on the
     // two-probe rule
     a.big_window = p.R_max > br::kRegWin ? 1 : 0;
     if (a.big_window && !ctx->two_probe_ok) { delete ctx; return BR_EINVAL; }
-    ctx->smem = br::step_smem_bytes(G, H, p.B, p.W, a.occ_words, p.term_mode == 3, a.big_window != 0);
-    if (ctx->smem > 227 * 1024) { delete ctx; return BR_EINVAL; }      // one instance must fit a thread block's shared memory
+    a.lay = br::step_layout(G, H, p.B, p.W, a.occ_words, p.term_mode == 3, a.big_window != 0, H > 0 && p.pred_mode == 0);
+    if (a.lay.total > 227 * 1024) { delete ctx; return BR_EINVAL; }    // one instance must fit a thread block's shared memory
     // br_small_kernel: Eq. 1, one worker per lane, one occupancy word, at most 512 waiting requests,
     // arrivals served by one Philox call, and negative queue keys scoring below every waiting request
     ctx->small_ok = p.score_mode == 0 && G <= 32 && p.B <= 64 && p.W <= 512 && p.term_mode <= 1 && p.R_max <= br::kRegWin &&
@@ -637,7 +635,7 @@ int br_fscore(br_ctx *ctx, const br_instance_batch *batch, const int32_t *s, int
     br::FscoreArgs a;
     a.G = ctx->G; a.H = ctx->H; a.fp = ctx->p.score_mode == 1;
     a.aD = ctx->base.aD; a.beta = ctx->base.beta;
-    for (int h = 0; h <= BR_MAX_H; ++h) a.d[h] = ctx->base.d[h];
+    for (int h = 0; h <= BR_MAX_H; ++h) a.d[h] = ctx->d[h];
     a.n_req = n_requests; a.first_instance = batch->first_instance;
     a.s = s; a.Lh = Lh; a.cap = cap; a.F = F; a.best_g = best_g;
     const int tiles = (n_requests + br::kFsTile - 1) / br::kFsTile;
@@ -664,7 +662,7 @@ int br_best_subset(br_ctx *ctx, const br_instance_batch *batch, const int32_t *w
     memset(&a, 0, sizeof(a));
     a.f.G = ctx->G; a.f.H = ctx->H; a.f.fp = ctx->p.score_mode == 1;
     a.f.aD = ctx->base.aD; a.f.beta = ctx->base.beta;
-    for (int h = 0; h <= BR_MAX_H; ++h) a.f.d[h] = ctx->base.d[h];
+    for (int h = 0; h <= BR_MAX_H; ++h) a.f.d[h] = ctx->d[h];
     a.R = R; a.first_instance = batch->first_instance;
     a.win = win; a.m = margins; a.lim = lim; a.best_mask = best_mask; a.best_F = best_F;
     // windows of 13 requests and more meet in the middle when the two-probe rule holds; without it
@@ -693,7 +691,7 @@ int br_bypass_dispatch(br_ctx *ctx, const br_instance_batch *batch, const int32_
     memset(&a, 0, sizeof(a));
     a.f.G = ctx->G; a.f.H = 0; a.f.fp = ctx->p.score_mode == 1;
     a.f.aD = ctx->base.aD; a.f.beta = ctx->base.beta;
-    for (int h = 0; h <= BR_MAX_H; ++h) a.f.d[h] = ctx->base.d[h];
+    for (int h = 0; h <= BR_MAX_H; ++h) a.f.d[h] = ctx->d[h];
     a.n_req = n_requests; a.first_instance = batch->first_instance;
     a.s = s; a.vload = virtual_load; a.inflight = inflight; a.cap = inflight_cap; a.g_out = worker_out;
     const int blocks = (batch->n_instances + 3) / 4;

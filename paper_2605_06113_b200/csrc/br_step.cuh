@@ -1,21 +1,29 @@
-// The general routing-step kernel: an instance is served by 32 to 256 threads (BR-H, large fleets,
-// optional outputs; BR-0 on small fleets runs on br_small_kernel).
+// The general routing-step kernel: one thread block of 32 to 256 threads per instance (BR-H, large
+// fleets, optional outputs; BR-0 on small fleets runs on br_small_kernel).
 //
 // Phases per decode step k (Section 2.2 model; Algorithms 1 and 2):
 //   ARRIVE -> PREDICT (H > 0) -> ROUTE (Stage 1, Stage 2) -> RECORD -> ADVANCE.
 //
-// Warp 0 is the router.  It keeps the per-worker state (free slots, projected loads
-// L_g(k+h), envelope M_h) in registers, one or two workers per lane, and walks the
-// sequential admission loop with warp reductions only: no block barrier sits on the
-// admission chain.  The waiting queue lives in shared memory as packed 32-bit keys
-// (prompt length in the high bits, inverted position in the low bits) so that "largest
-// s, earliest arrival" is one integer max.
+// Warp 0 is the router and walks the sequential admission loop with warp reductions only; the other
+// warps meanwhile settle the requests that end at this step.  Everything else (projection, queue
+// compaction, write-back) is spread over all threads.
+//
+// The admission loop is bound by instruction latency and instruction fetch: a pop is one chain of
+// dependent warp instructions (measured: warp maximum 22 cycles, warp sum 47, shuffle or ballot 25 to
+// 35, shared-memory load 34, fp64 operation 8), and a loop body of more than a few hundred
+// instructions is fetched again on every pop.  So it is written to be short: one loop for both
+// stages; the projected loads L_g(k+h) in shared memory, with the lanes spread over h for margins,
+// envelope and admission; one lane per worker only for the three selection keys (free slots, L_g(k),
+// min_h m_{g,h}); all requests of a chosen subset admitted at once, one lane each; slots, snapshot
+// edits and rare branches outside the loop.  Against one copy of every part per stage, with the
+// horizon in registers and loops over h unrolled, 1,024 instances of G = 64, W = 1,024, H = 8 went
+// from 112 to 83 us a step, 777 of G = 21, W = 300, H = 6 from 630 to 295 us per three steps, 1,024 of
+// G = 8, W = 512, H = 80 from 503 to 164 us per eight.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
-// one Philox block per worker (the ending slots are walked by geometric gaps), and the few
-// slots whose request ends.  Only the horizon
-// projection of BR-H streams the per-request state.
+// the termination draws and the few slots whose request ends.  Only the horizon projection of BR-H
+// streams the per-request state.
 #pragma once
 #include "br_device.cuh"
 #include "br_mitm.cuh"
@@ -23,10 +31,17 @@
 
 namespace br {
 
+// Shared memory of one instance: byte offsets, filled in by the host.
+struct StepLayout {
+    int32_t q_key, q_id, q_o, Lh, Ch, dn, Ms, md, occ, occ0, fin, endm, L0, cap, sub, scal, bw, due, total;
+};
+
 struct StepArgs {
     int32_t G, H, B, W, R_max, S_greedy, occ_words;
     int32_t wl;                 // log2 of the queue-position field of a packed key
-    uint32_t magic_B;           // ceil(2^32 / B): x / B == umulhi(x, magic_B) for x < 2^16
+    int32_t Wp;                 // W rounded up to whole groups of 128 queue positions
+    int32_t HS;                 // row stride of L_g(k+h) in shared memory (>= H + 1)
+    int32_t seg_log2;           // lanes per worker that turn its prediction buckets into L_g(k+h)
     int32_t delta_T;
     float gate, c_floor;
     int32_t term_mode;
@@ -40,12 +55,12 @@ struct StepArgs {
     int32_t len_shift;
     int32_t burst_every, burst_size;
     double aD, beta;
-    int32_t peak_ok;            // Eq. 2: every slope alpha D - beta sum_{h in P} d_h is clearly off zero (br_create)
+    double slope_err;           // Eq. 2: a segment slope within this of zero makes fp64 scores of integer lengths unordered
+    int32_t peak_ok;            // Eq. 1: scores fall strictly beyond the margin (G >= 2)
     int32_t big_window;         // R_max > 5: Stage 2 solves its window by meeting in the middle
-    double d[BR_MAX_H + 1];
+    double dn[2 * (BR_MAX_H + 4)];   // (d_h, -2^52 d_h), zero beyond H
     int32_t N, first_instance, n_steps;
-    int32_t tpi, smem_per_inst;  // threads and shared-memory bytes per instance
-    int32_t block_sync;          // 1: every barrier is a block barrier (needs full blocks)
+    StepLayout lay;
     br_worker_state ws;
     br_waiting_queue wq;
     const float *term_probs;
@@ -53,64 +68,81 @@ struct StepArgs {
     br_load_out out;
 };
 
-// shared-memory footprint of one instance (bytes), mirrored by the host
-__host__ __device__ inline size_t step_smem_bytes(int G, int H, int B, int W, int occ_words, bool lifetimes = false,
-                                                  bool big_window = false)
+// L_g(k+h) rows are read by lanes that own a worker each (16-byte loads at stride HS) and by lanes
+// that own an offset each (consecutive words): an odd number of 16-byte units keeps both free of
+// bank conflicts.
+__host__ __device__ inline int step_row_stride(int H)
 {
-    size_t n = 0;
-    n += 4 * (size_t)W * 2;                      // q_key, q_id
-    n += 8 * (size_t)G * occ_words * 2;          // occ, end_mask
-    n += 4 * (size_t)G * (H + 1) * 2;            // Lh_s, Ch_s (PREDICT buckets: load sums, counts)
-    n += 4 * (size_t)G;                          // sub_load
-    n += 8 * (size_t)G * occ_words;              // fin_w
-    n += 8 * (size_t)(H + 1) + 4 * (size_t)((H + 2) / 2 * 2);   // md_s (fp64 margins of the selected worker), M_s (envelope)
-    n += 2 * 96 + 2 * 32 + 64;                   // end_list, pre_list, scalars
-    if (H > 0) n += 2 * (size_t)G * B;           // refresh_list
-    n = (n + 15) & ~(size_t)15;
-    if (lifetimes) n += 4 * (size_t)W;           // q_o (output lengths of the waiting requests)
-    n = (n + 15) & ~(size_t)15;
-    if (big_window) n += 8 * (size_t)(1 << 8) + 4 * 16 + 4 * 16;   // sorted half-window subsets, class offsets, window keys
-    return (n + 15) & ~(size_t)15;
+    int u = (H + 1 + 3) / 4;
+    return 4 * (u | 1);
+}
+
+inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool lifetimes, bool big_window, bool classifier)
+{
+    StepLayout l;
+    const int Wp = (W + 127) / 128 * 128, HS = step_row_stride(H), words = 8 * G * occ_words;
+    int n = 0;
+    auto take = [&n](int bytes) { const int at = n; n += (bytes + 15) & ~15; return at; };
+    l.q_key = take(4 * Wp);
+    l.q_id = take(4 * Wp);
+    l.q_o = take(lifetimes ? 4 * Wp : 0);
+    l.Lh = take(4 * G * HS);                    // PREDICT: load sums per (worker, floor(c_hat)); then L_g(k+h)
+    l.Ch = take(H > 0 ? 4 * G * HS : 0);        // PREDICT: request counts
+    l.dn = take(16 * HS);                       // (d_h, -2^52 d_h)
+    l.Ms = take(4 * HS);                        // envelope M_h
+    l.md = take(4 * HS);                        // margins of the selected worker
+    l.occ = take(words);                        // occupied slots
+    l.occ0 = take(words);                       // ... at the start of the step
+    l.fin = take(words);                        // constant hazard: slots whose draw says "ends"
+    l.endm = take(words);                       // slots whose request ends at this step
+    l.L0 = take(4 * G);
+    l.cap = take(4 * G);
+    l.sub = take(4 * G);                        // loads of the requests that end
+    l.scal = take(4 * 32);
+    l.bw = take(big_window ? 8 * (1 << 8) + 4 * 32 : 0);
+    const int most = W < G * B ? W : G * B;     // admissions of a step
+    l.due = take(classifier && G * B > 4 * most ? 2 * G * B : 8 * most);   // requests whose c_hat is refreshed; then the admissions
+    l.total = n;
+    return l;
 }
 
 // Order- and sign-preserving key of a score: Eq. 1 in integers (FP = false) or Eq. 2 in
 // fp64 evaluated term by term in h (FP = true).
-// SL: the horizon is too long for registers; the margins of the selected worker are read from
-// shared memory (mds) and the loops over h are not unrolled.
-template <bool FP, int HM, bool SL = false>
+//
+// A term of Eq. 2 is RN(d_h * over) with over = max(delta - m_h, 0) an integer.  X = 2^52 + over is
+// a double that needs no conversion instruction (its low word is `over`), and one fused operation
+// fma(X, d_h, -2^52 d_h) rounds d_h * over once: the same value as converting and multiplying, at
+// two fp64 instructions per term instead of five.
+template <bool FP>
 struct Scorer {
-    int mi;                 // Eq. 1 margin
-    double md[SL ? 1 : HM + 1];   // Eq. 2 margins
-    span_t<double> mds;     // Eq. 2 margins in shared memory (SL)
-    int mmin;               // min_h m_{g,h}: at or below it the Eq. 2 penalty is exactly zero
+    span_t<int> md;         // Eq. 2: margins m_{g,h} of the selected worker (INT_MAX beyond H)
+    span_t<double> dn;      // (d_h, -2^52 d_h) pairs
+    int mm;                 // min_h m_{g,h} (Eq. 1: the margin); at or below it no term is positive
+    int H, G;
+    double aD, beta;
 
-    __device__ __forceinline__ long long key(const StepArgs &a, int delta) const
+    __device__ __forceinline__ long long key(int delta) const
     {
         if (!FP) {
-            int over = delta - mi;
+            int over = delta - mm;
             over = over > 0 ? over : 0;
-            return (long long)(delta - a.G * over);        // |F| < 2^31 by the create-time proof
+            return (long long)(delta - G * over);          // |F| < 2^31 by the create-time proof
         } else {
-            const double dl = (double)delta;
+            const double two52 = 4503599627370496.0;
             double pen = 0.0;
-            if (SL) {
-#pragma unroll 4
-                for (int h = 0; h <= a.H; ++h) {
-                    double over = __dsub_rn(dl, mds[h]);
-                    over = over > 0.0 ? over : 0.0;
-                    pen = __dadd_rn(pen, __dmul_rn(a.d[h], over));
-                }
-            } else {
+#pragma unroll 1
+            for (int h = 0; h <= H; h += 4) {
+                const int4 m4 = *vec_at<const int4>(md, h);
+                const int m[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-                for (int h = 0; h <= HM; ++h) {
-                    if (h <= a.H) {
-                        double over = __dsub_rn(dl, md[h]);     // exact: integers below 2^53
-                        over = over > 0.0 ? over : 0.0;
-                        pen = __dadd_rn(pen, __dmul_rn(a.d[h], over));
-                    }
+                for (int j = 0; j < 4; ++j) {
+                    const double2 d = *vec_at<const double2>(dn, 2 * (h + j));
+                    const double x = __hiloint2double(0x43300000, max(delta - m[j], 0));
+                    pen = __dadd_rn(pen, __fma_rn(x, d.x, d.y));
                 }
             }
-            return key_of_double(__dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)));
+            const double dl = __dsub_rn(__hiloint2double(0x43300000, delta), two52);
+            return key_of_double(__dsub_rn(__dmul_rn(aD, dl), __dmul_rn(beta, pen)));
         }
     }
     __device__ __forceinline__ static double value(long long k)
@@ -119,30 +151,14 @@ struct Scorer {
     }
 };
 
-// warp arg-max of (64-bit key, then largest 32-bit tie value); returns the winning lane
-__device__ __forceinline__ int warp_argmax_lane(long long key, unsigned tie, long long &wkey)
+// warp maximum of 64-bit keys; returns whether this lane holds it
+__device__ __forceinline__ bool warp_max64(long long key, long long &wkey)
 {
     const int hi = (int)(key >> 32);
-    const unsigned lo = (unsigned)key;
     const int mhi = __reduce_max_sync(kFull, hi);
-    const bool in1 = hi == mhi;
-    const unsigned mlo = __reduce_max_sync(kFull, in1 ? lo : 0u);
-    const bool in2 = in1 && lo == mlo;
-    const unsigned mt = __reduce_max_sync(kFull, in2 ? tie : 0u);
-    const unsigned who = __ballot_sync(kFull, in2 && tie == mt);
+    const unsigned mlo = __reduce_max_sync(kFull, hi == mhi ? (unsigned)key : 0u);
     wkey = (long long)(((unsigned long long)(unsigned)mhi << 32) | mlo);
-    return __ffs(who) - 1;
-}
-
-// same for 32-bit keys (Eq. 1 scores): largest key, then largest tie value
-__device__ __forceinline__ int warp_argmax_lane32(int key, unsigned tie, int &wkey)
-{
-    const int mk = __reduce_max_sync(kFull, key);
-    const bool in1 = key == mk;
-    const unsigned mt = __reduce_max_sync(kFull, in1 ? tie : 0u);
-    const unsigned who = __ballot_sync(kFull, in1 && tie == mt);
-    wkey = mk;
-    return __ffs(who) - 1;
+    return key == wkey;
 }
 
 // Slots of worker g that end at step k under the constant hazard, as bit masks of 64 slots each.
@@ -156,10 +172,10 @@ __device__ __forceinline__ void draw_ending(const CDF cdf, int B, int OW, uint32
 {
     for (int w = 0; w < OW; ++w) out[w] = 0ull;
     int pos = 0;
-    uint4 r = philox4x32_10(k, g, kStreamTerm, 0u, key0, key1);
+    uint4 r = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
     for (unsigned t = 0; t < (unsigned)B; ++t) {          // every draw moves pos forward
-        if (t != 0u && (t & 3u) == 0u) r = philox4x32_10(k, g, kStreamTerm, t >> 2, key0, key1);
+        if ((t & 3u) == 0u) r = philox4x32_10(k, g, kStreamTerm, t >> 2, key0, key1);
         const uint32_t u = word_of(r, t & 3u);
         const int room = B - pos;
         if (u >= cdf[room - 1]) break;                    // the gap reaches past the last slot
@@ -194,115 +210,221 @@ __device__ __forceinline__ void ld_row8(const float *p, float *o)
     for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(r[i]);
 }
 
-// Adds (val, 1) to the prediction bucket `key` (load sum in T, count in C) if key >= 0.  Plain
-// shared-memory atomics: combining the lanes of a warp that share a bucket first (match.any and a
-// masked reduction) measured 70 % slower than letting the atomics collide.
-template <typename TP, typename CP>
-__device__ __forceinline__ void bucket_add(const TP T, const CP C, int key, unsigned val, int lane)
+// Sum and smallest element of the H probabilities of a classifier row.  The order of the fp32 sum is
+// free: it only feeds a bound with slack.
+__device__ __forceinline__ void row_sum(const float *q, int H, bool rows32, float &sum, float &low)
 {
-    (void)lane;
-    if (key >= 0) { atomicAdd(&T[key], val); atomicAdd(&C[key], 1u); }
+    float s = 0.0f, mn = 0.0f;
+    if (rows32) {
+        for (int h = 0; h < H; h += 8) {
+            float v[8];
+            ld_row8(q + h, v);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { s += v[j]; mn = fminf(mn, v[j]); }
+        }
+    } else if ((H & 3) == 0) {
+#pragma unroll 2
+        for (int h = 0; h < H; h += 4) {
+            const float4 v = ld_row4(q + h);
+            s += (v.x + v.y) + (v.z + v.w);
+            mn = fminf(fminf(fminf(mn, v.x), fminf(v.y, v.z)), v.w);
+        }
+    } else {
+#pragma unroll 4
+        for (int h = 0; h < H; ++h) { const float v = __ldg(q + h); s += v; mn = fminf(mn, v); }
+    }
+    sum = s; low = mn;
 }
 
-constexpr int kRegWin = 5;      // Stage-2 windows of up to five requests are scored one subset per lane
-constexpr int kBigWinLow = 8;   // larger windows (up to BR_MAX_RMAX = 16): subsets of the low eight entries are sorted
-constexpr int kPassBUnroll = 2;  // classifier rows in flight per thread (4 and 8 measured the same)
-constexpr int kUnroll = 2;       // slot quads in flight per thread in the BR-H streaming phase (4 measured the same)
-constexpr int kEndList = 96;    // requests ending in one step that are fixed up as one batch
+constexpr int kRegWin = 5;       // Stage-2 windows of up to five requests are scored one subset per lane
+constexpr int kBigWinLow = 8;    // larger windows (up to BR_MAX_RMAX = 16): subsets of the low eight entries are sorted
+constexpr int kQBeyond = (int)0x8000FFFFu;   // key of a position beyond the queue (no slot index reaches 0xFFFF)
 
-// LEAN > 0: constant-hazard terminations and no optional outputs (score matrix, cycle counters);
-// LEAN == 2: in addition the instance is a single warp.  The paths not needed are compiled out,
-// which shortens the code every warp walks.
-template <bool FP, int HM, int GW, int LEAN>
-__global__ void __maxnreg__((FP && HM > 0) ? 128 : 72) br_step_kernel(const StepArgs a)
+// The rarely taken branches of the router live in functions of their own: inlined, they would spread
+// the admission loop over more instructions than the instruction cache of a scheduler holds.
+__device__ __noinline__ uint4 philox_call(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t k0, uint32_t k1)
 {
-    extern __shared__ __align__(16) unsigned char smem_all[];
-    // a.tpi threads serve one instance; a block holds blockDim.x / a.tpi instances (more than one
-    // only when tpi == 32, so that an instance-wide barrier is a warp barrier)
-    constexpr bool SL = HM > 16;          // long horizons: projected loads, envelope and margins in shared memory
-    constexpr int HR = SL ? 0 : HM;       // horizon offsets kept in registers
-    const int NT = a.tpi;
-    const int tid = threadIdx.x % NT, lane = tid & 31, warp = tid >> 5;
-    const int in_block = threadIdx.x / NT, per_block = blockDim.x / NT;
+    return philox4x32_10(c0, c1, c2, 0u, k0, k1);
+}
+
+// the R largest keys of the queue: lane r gets the r-th largest
+__device__ __noinline__ int largest_keys(span_t<int> q_key, int n_w, int R, int lane)
+{
+    int thr = 0x7FFFFFFF, mine = 0;
+#pragma unroll 1
+    for (int r = 0; r < R; ++r) {
+        int x = 0;
+#pragma unroll 1
+        for (int i = lane; i < n_w; i += 32) { const int y = q_key[i]; if (y < thr) x = max(x, y); }
+        thr = __reduce_max_sync(kFull, x);
+        if (lane == r) mine = thr;
+    }
+    return mine;
+}
+
+struct WindowChoice { long long wk; unsigned chosen; int dsum; };
+
+// Best subset of a window of 6 to 16 requests (Appendix "Bit-set subset selection"): lane r holds the
+// r-th largest key in `wkey`.  m0: the margin of offset `lane` (Eq. 2).
+template <bool FP>
+__device__ __noinline__ WindowChoice big_window(const Scorer<FP> sc, span_t<unsigned long long> keys, span_t<int> off,
+                                                span_t<int> win, int wkey, int R, int lim, int WL, int m0, int lane)
+{
+    if (lane < R) win[lane] = wkey >> WL;
+    __syncwarp();
+    const int ra = min(kBigWinLow, (R + 1) / 2), rb = R - ra, n = 1 << ra;
+    // subsets of the low entries, sorted by (size, sum, mask)
+#pragma unroll 1
+    for (int x = lane; x < n; x += 32) {
+        int sum = 0;
+        for (int j = 0; j < ra; ++j) if ((x >> j) & 1) sum += win[j];
+        keys[x] = ((unsigned long long)__popc(x) << 56) | ((unsigned long long)(unsigned)sum << 16) | (unsigned)x;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int k2 = 2; k2 <= n; k2 <<= 1) {
+#pragma unroll 1
+        for (int j = k2 >> 1; j > 0; j >>= 1) {
+#pragma unroll 1
+            for (int i = lane; i < n; i += 32) {
+                const int p = i ^ j;
+                if (p > i) {
+                    const unsigned long long x = keys[i], y = keys[p];
+                    const bool up = (i & k2) == 0;
+                    if ((x > y) == up) { keys[i] = y; keys[p] = x; }
+                }
+            }
+            __syncwarp();
+        }
+    }
+    if (lane == 0) {
+        int at = 0, binom = 1;
+#pragma unroll 1
+        for (int c = 0; c <= ra; ++c) { off[c] = at; at += binom; binom = binom * (ra - c) / (c + 1); }
+        off[ra + 1] = at;
+    }
+    __syncwarp();
+    // the peak of the score in Delta (H <= 16 here, so one offset per lane)
+    int peak = sc.mm;
+    if (FP) {
+        double wsum = 0.0;
+#pragma unroll 1
+        for (int h = 0; h <= sc.H; ++h) if (sc.md[h] <= m0) wsum = __dadd_rn(wsum, sc.dn[2 * h]);
+        const bool past = lane <= sc.H && !(sc.aD > __dmul_rn(sc.beta, wsum));
+        peak = (int)__reduce_min_sync(kFull, past ? (unsigned)m0 : 0x7FFFFFFFu);
+    }
+    MitmBest b; b.lo_sum = -1; b.lo_mask = 0xFFFFFFFFu; b.hi_sum = 0x7FFFFFFF; b.hi_mask = 0xFFFFFFFFu;
+#pragma unroll 1
+    for (unsigned mh = lane; mh < (1u << rb); mh += 32) {
+        const int ph = __popc(mh);
+        if (ph > lim) continue;
+        int sh = 0;
+        for (unsigned t = mh; t; t &= t - 1) sh += win[ra + __ffs(t) - 1];
+        mitm_probe(keys, off, ra, lim, peak, mh, sh, ph, b);
+    }
+    // largest sum at or below the peak, smallest above it, lowest mask among equals
+    const int ls = __reduce_max_sync(kFull, b.lo_sum);
+    const unsigned lm = __reduce_min_sync(kFull, b.lo_sum == ls ? b.lo_mask : 0xFFFFFFFFu);
+    const int hs = __reduce_min_sync(kFull, b.hi_sum);
+    const unsigned hm = __reduce_min_sync(kFull, b.hi_sum == hs ? b.hi_mask : 0xFFFFFFFFu);
+    WindowChoice r; r.wk = kNoKey; r.chosen = 1u; r.dsum = 0;
+    const long long f = sc.key((lane & 1) ? (hs != 0x7FFFFFFF ? hs : 0) : max(ls, 0));
+    const long long fl = __shfl_sync(kFull, f, 0), fh = __shfl_sync(kFull, f, 1);
+    if (ls >= 0) { r.wk = fl; r.chosen = lm; r.dsum = ls; }
+    if (hs != 0x7FFFFFFF && (fh > r.wk || (fh == r.wk && hm < r.chosen))) { r.wk = fh; r.chosen = hm; r.dsum = hs; }
+    __syncwarp();
+    return r;
+}
+
+// argmax_i F_g({i}) by scoring every waiting request, earliest arrival on ties; packed key, 0 if none.
+// Safe requests (s <= min_h m_{g,h}) score alpha D s exactly, which grows with s, so of those only the
+// largest key per lane is scored.
+template <bool FP>
+__device__ __noinline__ int best_of_all(const Scorer<FP> sc, span_t<int> q_key, int n_w, int WL, unsigned posmask, int lane)
+{
+    long long bk = kNoKey; int bkey = 0, best_safe = 0;
+#pragma unroll 1
+    for (int i = lane; i < n_w + 32; i += 32) {
+        int x = i < n_w ? q_key[i] : 0;
+        if (x > 0 && (x >> WL) <= sc.mm) { best_safe = max(best_safe, x); x = 0; }
+        if (i >= n_w) x = best_safe;
+        if (x > 0) {
+            const long long f = sc.key(x >> WL);
+            if (f > bk || (f == bk && ((unsigned)x & posmask) > ((unsigned)bkey & posmask))) { bk = f; bkey = x; }
+        }
+    }
+    long long wk;
+    const bool in = warp_max64(bk, wk);
+    const unsigned mt = __reduce_max_sync(kFull, in ? (unsigned)bkey & posmask : 0u);
+    const int who = (int)__reduce_min_sync(kFull, in && ((unsigned)bkey & posmask) == mt ? (unsigned)lane : 32u);
+    return wk == kNoKey ? 0 : __shfl_sync(kFull, bkey, who);
+}
+
+// row g of the optional F-score matrix: F_g({i}) of every waiting request
+template <bool FP>
+__device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t<int> q_key, int n_w, int W, int G, int WL, int lane)
+{
+#pragma unroll 1
+    for (int i = lane; i < W; i += 32)
+        F[(size_t)i * G] = i < n_w ? Scorer<FP>::value(sc.key(q_key[i] >> WL)) : 0.0;
+}
+
+// FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  HC: horizon offsets per lane (H < 32 HC).
+template <bool FP, int GW, int HC>
+__global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_constant__ StepArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
     stream_order_gate();
-    if (blockIdx.x * per_block + in_block >= a.N) return;            // whole instance groups only
-    unsigned char *smem_raw = smem_all + (size_t)in_block * a.smem_per_inst;
-    // Instance-wide barrier.  Single-warp instances that share a block may also be aligned with a
-    // block barrier (a.block_sync): the warps then walk the same code at about the same time, which
-    // pays off in instruction fetch although no data crosses between them.
-    // (Giving wider instances that share a block a named barrier each, so that one never waits for
-    // its neighbour, measured 3 % slower on the 1024-instance BR-H batch: instances that walk the
-    // phases together share instruction fetch and keep the memory phases aligned.)
-    auto inst_sync = [&]() { if (NT == 32 && !a.block_sync) __syncwarp(); else __syncthreads(); };
-    const int nwarps = LEAN == 2 ? 1 : (NT >> 5);
-    const int term_mode = LEAN ? 1 : a.term_mode;
-    const int G = a.G, H = a.H, B = a.B, W = a.W, H1 = H + 1, A = G * B, OW = a.occ_words;
-    const int A8 = A >> 3;
-    const int WL = a.wl;
+    const int G = a.G, H = FP ? a.H : 0, B = a.B, W = a.W, A = G * B, OW = a.occ_words, WL = a.wl;
+    const int H1 = H + 1, HS = a.HS;
     const unsigned posmask = (1u << WL) - 1u;
-    const int inst = a.first_instance + blockIdx.x * per_block + in_block;
+    const int inst = a.first_instance + blockIdx.x;
+    const bool life = a.term_mode == 3;               // requests carry their output lengths
+    const bool classifier = FP && H > 0 && a.pred_mode == 0;
     const unsigned t_entry = (unsigned)clock64();
 
-    // ---- shared-memory carve-up (sizes match step_smem_bytes) ----
-    // (raw carve-up first; every array is then used through a span that knows its length)
-    int *q_key_p = reinterpret_cast<int *>(smem_raw);                               // [W]
-    unsigned *q_id_p = reinterpret_cast<unsigned *>(q_key_p + W);                   // [W]
-    unsigned long long *occ_p = reinterpret_cast<unsigned long long *>(q_id_p + W); // [G][OW]
-    unsigned long long *end_mask_p = occ_p + (size_t)G * OW;                        // [G][OW]
-    unsigned long long *fin_w_p = end_mask_p + (size_t)G * OW;                      // [G][OW] slots whose draw says "ends"
-    double *md_s_p = reinterpret_cast<double *>(fin_w_p + (size_t)G * OW);          // [H1] margins of the selected worker
-    int *M_s_p = reinterpret_cast<int *>(md_s_p + H1);                              // [H1 rounded up to even] envelope
-    unsigned *Lh_s_p = reinterpret_cast<unsigned *>(M_s_p + (H1 + 1) / 2 * 2);      // [G][H1]
-    unsigned *Ch_s_p = Lh_s_p + (size_t)G * H1;                                     // [G][H1]
-    unsigned *sub_load_p = Ch_s_p + (size_t)G * H1;                                 // [G]
-    unsigned short *end_list_p = reinterpret_cast<unsigned short *>(sub_load_p + G);// [kEndList]
-    unsigned short *pre_list_p = end_list_p + kEndList;                             // [32]
-    int *scal_p = reinterpret_cast<int *>(pre_list_p + 32);                         // [16]
-    unsigned short *refresh_list_p = reinterpret_cast<unsigned short *>(scal_p + 16);   // [A] (H > 0 only)
-    // output lengths of the waiting requests (term_mode 3 only), behind everything else
-    int *q_o_p = reinterpret_cast<int *>(smem_raw + ((step_smem_bytes(G, H, B, W, OW) + 15) & ~(size_t)15));
-    // large Stage-2 windows: sorted subsets of the low half, class offsets, the window's keys
-    unsigned long long *bw_keys_p = reinterpret_cast<unsigned long long *>(
-        smem_raw + step_smem_bytes(G, H, B, W, OW, !LEAN && a.term_mode == 3));
-    int *bw_off_p = reinterpret_cast<int *>(bw_keys_p + (1 << kBigWinLow));
-    const bool life = !LEAN && a.term_mode == 3;          // requests carry their output lengths
-    const bool bigw = !LEAN && a.big_window != 0;
-    const auto q_key = mk_span(q_key_p, W);
-    const auto q_id = mk_span(q_id_p, W);
-    const auto occ = mk_span(occ_p, G * OW);
-    const auto end_mask = mk_span(end_mask_p, G * OW);
-    const auto fin_w = mk_span(fin_w_p, G * OW);
-    const auto md_s = mk_span(md_s_p, H1);
-    const auto M_s = mk_span(M_s_p, H1);
-    const auto Lh_s = mk_span(Lh_s_p, 2 * G * H1);        // Ch_s follows it; the two are cleared as one block
-    const auto Ch_s = mk_span(Ch_s_p, G * H1);
-    const auto sub_load = mk_span(sub_load_p, G);
-    const auto end_list = mk_span(end_list_p, kEndList);
-    const auto pre_list = mk_span(pre_list_p, 32);
-    const auto scal = mk_span(scal_p, 16);
-    const auto refresh_list = mk_span(refresh_list_p, H > 0 ? A : 0);
-    const auto q_o = mk_span(q_o_p, life ? W : 0);
-    const auto bw_keys = mk_span(bw_keys_p, bigw ? (1 << kBigWinLow) : 0);
-    const auto bw_off = mk_span(bw_off_p, bigw ? 16 : 0);
-    const auto bw_win = mk_span(bw_off_p + 16, bigw ? 16 : 0);
-    // scal: [0] queue length after routing, [1] admitted, [2] Stage-1 iterations,
-    //       [3] Stage-2 pops, [4] status bits of the step, [5] status bits of the prologue,
-    //       [6] requests that ended this step and were not prefetched, [7] prefetched ones,
-    //       [8] requests whose c_hat is refreshed at this step,
-    //       [9] set when requests that end were found before routing and did not fit the lists
+    // ---- shared memory ----
+    const auto q_key = mk_span(reinterpret_cast<int *>(smem + a.lay.q_key), a.Wp);
+    const auto q_id = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.q_id), a.Wp);
+    const auto q_o = mk_span(reinterpret_cast<int *>(smem + a.lay.q_o), life ? a.Wp : 0);
+    const auto Lh = mk_span(reinterpret_cast<int *>(smem + a.lay.Lh), G * HS);
+    const auto Ch = mk_span(reinterpret_cast<int *>(smem + a.lay.Ch), H > 0 ? G * HS : 0);
+    const auto dn_s = mk_span(reinterpret_cast<double *>(smem + a.lay.dn), FP ? 2 * HS : 0);
+    const auto Ms = mk_span(reinterpret_cast<int *>(smem + a.lay.Ms), HS);
+    const auto md = mk_span(reinterpret_cast<int *>(smem + a.lay.md), HS);
+    const auto occ = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ), G * OW);
+    const auto occ0 = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ0), G * OW);
+    const auto occ032 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.occ0), 2 * G * OW);
+    const auto fin = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.fin), G * OW);
+    const auto endm = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.endm), G * OW);
+    const auto endm32 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.endm), 2 * G * OW);
+    const auto endm8 = mk_span(smem + a.lay.endm, 8 * G * OW);
+    const auto occ32 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.occ), 2 * G * OW);
+    const auto L0_s = mk_span(reinterpret_cast<int *>(smem + a.lay.L0), G);
+    const auto cap_s = mk_span(reinterpret_cast<int *>(smem + a.lay.cap), G);
+    const auto sub_load = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.sub), G);
+    const auto scal = mk_span(reinterpret_cast<int *>(smem + a.lay.scal), 32);
+    const auto bw_keys = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.bw), a.big_window ? (1 << kBigWinLow) : 0);
+    const auto bw_off = mk_span(reinterpret_cast<int *>(smem + a.lay.bw + (8 << kBigWinLow)), a.big_window ? 16 : 0);
+    const auto bw_win = mk_span(reinterpret_cast<int *>(smem + a.lay.bw + (8 << kBigWinLow) + 64), a.big_window ? 16 : 0);
+    const auto due_list = mk_span(reinterpret_cast<unsigned short *>(smem + a.lay.due), classifier ? A : 0);
+    // admissions of the step in order: (key, worker << 16 | free slots of the worker before it); shares the
+    // memory of the due list, which is not needed once the projection stands
+    const auto adm = mk_span(reinterpret_cast<int2 *>(smem + a.lay.due), min(W, A));
+    // scal: [0] queue length after routing, [1] admitted, [2] Stage-1 iterations, [3] Stage-2 pops,
+    //       [4] status bits of the step, [5] status bits of the prologue, [6] lowest admitted position,
+    //       [8] requests on the due list, [16..31] kept entries per warp (two sets of eight, compaction)
 
     // ---- per-instance global rows ----
-    const auto g_load = mk_span(reinterpret_cast<long long *>(a.ws.load) + (size_t)inst * G, G);
-    const auto g_nact = mk_span(a.ws.nact + (size_t)inst * G, G);
-    const auto g_occ = mk_span(reinterpret_cast<unsigned long long *>(a.ws.occ) + (size_t)inst * G * OW, G * OW);
     const auto g_base = mk_span(a.ws.act_base + (size_t)inst * A, A);
     const auto g_aid = mk_span(a.ws.act_id ? a.ws.act_id + (size_t)inst * A : nullptr, A);
     const auto g_chat0 = mk_span(a.ws.act_chat0 ? a.ws.act_chat0 + (size_t)inst * A : nullptr, A);
     const auto g_kref = mk_span(a.ws.act_kref ? a.ws.act_kref + (size_t)inst * A : nullptr, A);
     const auto g_end = mk_span(life ? a.ws.act_end + (size_t)inst * A : nullptr, A);
-    const auto g_qo = mk_span(life ? a.wq.o + (size_t)inst * W : nullptr, W);
     const auto g_qs = mk_span(a.wq.s + (size_t)inst * W, W);
     const auto g_qid = mk_span(a.wq.id + (size_t)inst * W, W);
+    const auto g_qo = mk_span(life ? a.wq.o + (size_t)inst * W : nullptr, W);
     const auto t_len = mk_span(a.len_tab, a.len_tab ? (1ll << (32 - a.len_shift)) : 0);
     const auto t_out = mk_span(a.out_tab, a.out_tab ? (1ll << (32 - a.out_shift)) : 0);
     const auto t_term = mk_span(a.term_cdf, B);
@@ -312,404 +434,401 @@ __global__ void __maxnreg__((FP && HM > 0) ? 128 : 72) br_step_kernel(const Step
     int k = a.ws.step[inst];
     uint32_t next_id = a.ws.next_id[inst];
     int n_w = a.wq.n[inst];
-    int prologue_status = 0;
-    if (n_w < 0 || n_w > W) { prologue_status |= BR_ST_BAD_STATE; n_w = n_w < 0 ? 0 : W; }
+    int bad = 0;
+    if (n_w < 0 || n_w > W) { bad = BR_ST_BAD_STATE; n_w = n_w < 0 ? 0 : W; }
 
-    if (tid < 16) scal[tid] = 0;
-    // queue -> packed keys and ids in shared memory (16-byte loads).  The first chunks are
-    // requested without waiting for the queue length (rows always hold W entries).
-    auto fetch_queue = [&](int i) {
-        const int4 v = *vec_at<const int4>(g_qs, i);
-        const uint4 u = *vec_at<const uint4>(g_qid, i);
+    // ---- snapshot to shared memory ----
+    if (tid < 32) scal[tid] = 0;
+#pragma unroll 1
+    for (int p0 = 4 * tid; p0 < a.Wp; p0 += 4 * NT) {
+        int4 v = make_int4(0, 0, 0, 0), o = make_int4(0, 0, 0, 0); uint4 u = make_uint4(0u, 0u, 0u, 0u);
+        if (p0 < W) {
+            v = *vec_at<const int4>(g_qs, p0);
+            u = *vec_at<const uint4>(g_qid, p0);
+            if (life) o = *vec_at<const int4>(g_qo, p0);
+        }
         int4 kk;
-        kk.x = (v.x << WL) | (int)(posmask - (unsigned)(i + 0));
-        kk.y = (v.y << WL) | (int)(posmask - (unsigned)(i + 1));
-        kk.z = (v.z << WL) | (int)(posmask - (unsigned)(i + 2));
-        kk.w = (v.w << WL) | (int)(posmask - (unsigned)(i + 3));
-        *vec_at<int4>(q_key, i) = kk;
-        *vec_at<uint4>(q_id, i) = u;
-        if (life) *vec_at<int4>(q_o, i) = *vec_at<const int4>(g_qo, i);
-    };
-    {
-        const int i0 = tid * 4, i1 = (NT + tid) * 4;
-        if (i0 < W) fetch_queue(i0);
-        if (i1 < W) fetch_queue(i1);
+        kk.x = p0 + 0 < n_w ? (v.x << WL) | (int)(posmask - (unsigned)(p0 + 0)) : kQBeyond;
+        kk.y = p0 + 1 < n_w ? (v.y << WL) | (int)(posmask - (unsigned)(p0 + 1)) : kQBeyond;
+        kk.z = p0 + 2 < n_w ? (v.z << WL) | (int)(posmask - (unsigned)(p0 + 2)) : kQBeyond;
+        kk.w = p0 + 3 < n_w ? (v.w << WL) | (int)(posmask - (unsigned)(p0 + 3)) : kQBeyond;
+        *vec_at<int4>(q_key, p0) = kk;
+        *vec_at<uint4>(q_id, p0) = u;
+        if (life) *vec_at<int4>(q_o, p0) = o;
     }
-    for (int i = (2 * NT + tid) * 4; i < n_w; i += NT * 4) fetch_queue(i);
-    for (int i = tid; i < G * OW; i += NT) { occ[i] = g_occ[i]; fin_w[i] = 0ull; }
-    for (int i = tid; i < 2 * G * H1; i += NT) Lh_s[i] = 0u;      // Lh_s and Ch_s are adjacent
-    for (int i = tid; i < G; i += NT) sub_load[i] = 0u;
-
-    // router registers: lane owns workers lane and lane + 32
-    int cap[GW];
-    int L[GW][HR + 1];
-    int Mh[HR + 1];
-    const auto L_s = mk_span(reinterpret_cast<int *>(raw_of(Lh_s)), G * H1);     // SL: the buckets become L_g(k+h) in place
-#pragma unroll
-    for (int h = 0; h <= HR; ++h) Mh[h] = 0;
-#pragma unroll
-    for (int w = 0; w < GW; ++w) {
-        const int g = lane + 32 * w;
-        cap[w] = -1;
-#pragma unroll
-        for (int h = 0; h <= HR; ++h) L[w][h] = 0;
-        if (warp == 0 && g < G) {
-            int na = g_nact[g];
-            if (na < 0 || na > B) { prologue_status |= BR_ST_BAD_STATE; na = na < 0 ? 0 : B; }
-            cap[w] = B - na;
-            L[w][0] = (int)g_load[g];
-        }
+#pragma unroll 1
+    for (int i = tid; i < G * OW; i += NT) {
+        const unsigned long long o = reinterpret_cast<const unsigned long long *>(a.ws.occ)[(size_t)inst * G * OW + i];
+        occ[i] = o; occ0[i] = o; endm[i] = 0ull;
     }
-    inst_sync();
-    if (prologue_status) atomicOr(&scal[5], prologue_status);
-
-    // this step's constant-hazard draws of workers first, first + stride, ...
-    auto draw_fin = [&](int first, int stride) {
 #pragma unroll 1
-        for (int g = first; g < G; g += stride)
-            draw_ending(t_term, B, OW, (uint32_t)k, (uint32_t)g, key0, key1, fin_w + (size_t)g * OW);
-    };
-
-    // Per worker word: which running requests end at this step (occupancy & termination draws).
-    // Writes end_mask and lists the ending slots; with `prefetch` the first 32 go to pre_list so
-    // that their loads can be requested at once by one lane each.
-    auto scan_workers = [&](bool prefetch) {
+    for (int g = tid; g < G; g += NT) {
+        int na = a.ws.nact[(size_t)inst * G + g];
+        if (na < 0 || na > B) { bad = BR_ST_BAD_STATE; na = na < 0 ? 0 : B; }
+        cap_s[g] = B - na;
+        L0_s[g] = (int)a.ws.load[(size_t)inst * G + g];
+        sub_load[g] = 0u;
+    }
+    if (FP) {
 #pragma unroll 1
-        for (int idx = tid; idx < G * OW; idx += NT) {
-            const int g = idx / OW, x = idx - g * OW;
-            const unsigned long long occw = occ[idx];
-            const unsigned long long finw = term_mode != 0 ? fin_w[idx] : 0ull;
-            unsigned long long ended = occw & finw;
-            end_mask[idx] = ended;
-            while (ended) {
-                const int j = __ffsll((long long)ended) - 1;
-                ended &= ended - 1;
-                const int sa = g * B + 64 * x + j;
-                int at = prefetch ? atomicAdd(&scal[7], 1) : 32;
-                if (at < 32) {
-                    pre_list[at] = (unsigned short)sa;
-                } else {
-                    at = atomicAdd(&scal[6], 1);
-                    if (at < kEndList) {
-                        end_list[at] = (unsigned short)sa;
-                    } else {                                         // list full: fix this slot up at once
-                        atomicAdd(&sub_load[g], (unsigned)(g_base[sa] + k));
-                        // before routing the request still runs (the projection of this step counts
-                        // it): its slot is emptied in ADVANCE, found again through end_mask
-                        if (prefetch) scal[9] = 1; else g_base[sa] = kEmpty;
-                    }
-                }
-            }
-        }
-    };
+        for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
+#pragma unroll 1
+        for (int h = tid; h < HS; h += NT) { Ms[h] = h < H1 ? 0 : 0x7FFFFFFF; md[h] = 0x7FFFFFFF; dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1]; }
+    }
+    __syncthreads();
+    if (bad) atomicOr(&scal[5], bad);
 
+#pragma unroll 1
     for (int it = 0; it < a.n_steps; ++it, ++k) {
         const size_t orow = (size_t)it * a.N + inst;
         const auto probs = mk_span(a.term_probs ? a.term_probs + orow * (size_t)A * H : nullptr, (long long)A * H);
         unsigned t_phase[7];
-        const bool timing = !LEAN && a.out.phase_cycles != nullptr && tid == 0;
+        const bool timing = a.out.phase_cycles != nullptr && tid == 0;
         if (timing) t_phase[0] = (unsigned)clock64();
 
         // ================= ARRIVE =================
-        // the arrival-count row is requested first; a single-warp block draws the termination
-        // words while that load is in flight
-        uint32_t row0 = 0xFFFFFFFFu, row1 = 0xFFFFFFFFu;
+        // The arrival-count row and the prompt lengths that the first arrivals would take are asked
+        // for together; they are used after the projection.
+        uint32_t row0 = 0xFFFFFFFFu, row1 = 0xFFFFFFFFu, u_arr = 0u;
         span_t<const uint32_t> row = mk_span((const uint32_t *)nullptr, 0);
+        int s_new = 0;
         if (a.arr_cdf) {
             row = mk_span(a.arr_cdf + ((size_t)inst * a.arr_inst_stride + (size_t)(k % a.arr_period)) * a.arr_len, a.arr_len);
             if (lane < a.arr_len) row0 = row[lane];
             if (lane + 32 < a.arr_len) row1 = row[lane + 32];
+            const uint4 r = philox_call((uint32_t)k, (uint32_t)tid >> 2, kStreamArrLen, key0, key1);
+            s_new = t_len[word_of(r, tid & 3) >> a.len_shift];
+            u_arr = philox_call((uint32_t)k, 0u, kStreamArrCount, key0, key1).x;
         }
-        // A single-warp instance also resolves, right away, which of the requests already
-        // running end at this step, and requests their loads: the values are used only after
-        // routing, so that memory latency is off the step's critical path.
-        const bool have_pre = (nwarps == 1 && term_mode == 1);
-        int pend = 0, n_pre = 0;
-        if (have_pre) {
-            draw_fin(tid, NT);
-            __syncwarp();
-            scan_workers(true);
-            __syncwarp();
-            n_pre = min(scal[7], 32);
-            if (tid < n_pre) pend = g_base[pre_list[tid]];
+        if (timing) t_phase[1] = (unsigned)clock64();
+
+        // ============ PREDICT (H > 0): c_hat maintenance + horizon projection ============
+        // Every running request adds (cur, 1) to the bucket (worker, floor(c_hat)); the buckets become
+        // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  A thread takes eight slots
+        // of one worker at a time and consecutive threads take different workers, so that the
+        // atomics of a warp fall on different rows.
+        if (FP && H > 0) {
+            const unsigned A8 = (unsigned)A >> 3;
+#pragma unroll 1
+            for (unsigned o = tid; o < A8; o += NT) {
+                const int p = (int)(o / (unsigned)G), g = (int)o - p * G, a0 = g * B + 8 * p;
+                const int4 b0 = *vec_at<const int4>(g_base, a0), b1 = *vec_at<const int4>(g_base, a0 + 4);
+                const int bs[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                if (a.pred_mode == 1) {
+                    // perfect lookahead: c_hat = min(r_i(k), H) with r_i(k) = act_end - k + 1 steps still to run.
+                    // A request whose last step this is (act_end == k) is settled right here.
+                    const int4 e0 = *vec_at<const int4>(g_end, a0), e1 = *vec_at<const int4>(g_end, a0 + 4);
+                    const int en[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+                    unsigned fb = 0u;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if (bs[j] != kEmpty) {
+                            const int nh = min(max(en[j] - k + 1, 0), H);
+                            const unsigned cur = (unsigned)(bs[j] + k);
+                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur);
+                            atomicAdd(&Ch[g * HS + nh], 1);
+                            if (en[j] == k) { fb |= 1u << j; atomicAdd(&sub_load[g], cur); g_base[a0 + j] = kEmpty; }
+                        }
+                    }
+                    endm8[g * OW * 8 + p] = (unsigned char)fb;
+                } else {
+                    // requests that are not due only age; the ones due for a refresh take c_hat = H (gate closed:
+                    // the conservative anchor) and go on a list, whose rows are read below
+                    const float4 c0 = *vec_at<const float4>(g_chat0, a0), c1 = *vec_at<const float4>(g_chat0, a0 + 4);
+                    float cs[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+                    unsigned kr[2] = {*vec_at<const unsigned>(g_kref, a0), *vec_at<const unsigned>(g_kref, a0 + 4)};
+                    unsigned due = 0u;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if (bs[j] != kEmpty) {
+                            const unsigned sh = 8 * (j & 3);
+                            const int t = (k - (int)((kr[j >> 2] >> sh) & 0xFFu)) & 255;
+                            const float c = cs[j] - (float)t;
+                            const bool d = t >= a.delta_T || c < a.c_floor;
+                            int nh = H;
+                            if (d) {
+                                due |= 1u << j;
+                                cs[j] = (float)H;
+                                kr[j >> 2] = (kr[j >> 2] & ~(0xFFu << sh)) | ((unsigned)(k & 255) << sh);
+                            } else {
+                                nh = (int)floorf(c);
+                                nh = nh < 0 ? 0 : (nh > H ? H : nh);
+                            }
+                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), (unsigned)(bs[j] + k));
+                            atomicAdd(&Ch[g * HS + nh], 1);
+                        }
+                    }
+                    if (due) {
+                        if (due & 0x0Fu) { *vec_at<float4>(g_chat0, a0) = make_float4(cs[0], cs[1], cs[2], cs[3]); *vec_at<unsigned>(g_kref, a0) = kr[0]; }
+                        if (due & 0xF0u) { *vec_at<float4>(g_chat0, a0 + 4) = make_float4(cs[4], cs[5], cs[6], cs[7]); *vec_at<unsigned>(g_kref, a0 + 4) = kr[1]; }
+                        int at = atomicAdd(&scal[8], __popc(due));
+                        while (due) {
+                            due_list[at++] = (unsigned short)(a0 + __ffs(due) - 1);
+                            due &= due - 1u;
+                        }
+                    }
+                }
+            }
         }
+        // arrivals join the queue
         int n_arr = 0;
         if (a.arr_cdf) {
-            const uint32_t u = philox4x32_10((uint32_t)k, 0u, kStreamArrCount, 0u, key0, key1).x;
-            n_arr = __popc(__ballot_sync(kFull, lane < a.arr_len && u >= row0)) +
-                    __popc(__ballot_sync(kFull, lane + 32 < a.arr_len && u >= row1));
+            n_arr = __popc(__ballot_sync(kFull, lane < a.arr_len && u_arr >= row0)) +
+                    __popc(__ballot_sync(kFull, lane + 32 < a.arr_len && u_arr >= row1));
+#pragma unroll 1
             for (int j0 = 64; j0 < a.arr_len; j0 += 32) {
                 const int j = j0 + lane;
-                const bool ge = (j < a.arr_len) && (u >= row[j]);
-                n_arr += __popc(__ballot_sync(kFull, ge));
+                n_arr += __popc(__ballot_sync(kFull, (j < a.arr_len) && (u_arr >= row[j])));
             }
             if (a.burst_every > 0 && k > 0 && (k % a.burst_every) == 0) n_arr += a.burst_size;
         }
         const int n_w_old = n_w;
-        const uint32_t id0 = next_id;             // id of arrival 0 of this step
+#pragma unroll 1
         for (int j = tid; j < n_arr; j += NT) {
             const int pos = n_w_old + j;
-            if (pos < W) {
-                const uint4 r = philox4x32_10((uint32_t)k, (uint32_t)j >> 2, kStreamArrLen, 0u, key0, key1);
-                const int s = t_len[word_of(r, j & 3) >> a.len_shift];
-                q_key[pos] = (s << WL) | (int)(posmask - (unsigned)pos);
-                q_id[pos] = id0 + (unsigned)j;
-                if (life) {
-                    const uint4 ro = philox4x32_10((uint32_t)k, (uint32_t)j >> 2, kStreamArrOut, 0u, key0, key1);
-                    q_o[pos] = t_out[word_of(ro, j & 3) >> a.out_shift];
-                }
+            if (pos >= W) break;
+            int s = s_new;
+            if (j != tid) {
+                const uint4 r = philox_call((uint32_t)k, (uint32_t)j >> 2, kStreamArrLen, key0, key1);
+                s = t_len[word_of(r, j & 3) >> a.len_shift];
+            }
+            q_key[pos] = (s << WL) | (int)(posmask - (unsigned)pos);
+            q_id[pos] = next_id + (unsigned)j;
+            if (life) {
+                const uint4 ro = philox_call((uint32_t)k, (uint32_t)j >> 2, kStreamArrOut, key0, key1);
+                q_o[pos] = t_out[word_of(ro, j & 3) >> a.out_shift];
             }
         }
-        int n_drop = n_w + n_arr - W;
-        n_drop = n_drop > 0 ? n_drop : 0;
+        const int n_drop = max(n_w + n_arr - W, 0);
         n_w = n_w + n_arr - n_drop;
         next_id += (uint32_t)n_arr;
-        if (timing) t_phase[1] = (unsigned)clock64();
 
-        // ============ PREDICT (H > 0): c_hat maintenance + horizon projection ============
-        // Every running request adds (cur, 1) to the bucket (worker, floor(c_hat)); the router turns
-        // the buckets into L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.
-        // Pass A streams the per-request state and settles the requests that only age; the ones due
-        // for a refresh are listed, and pass B reads their classifier rows with independent loads.
-        if (HM > 0 && H > 0 && !LEAN && a.pred_mode == 1) {
-            // perfect lookahead: c_hat = min(r_i(k), H) with r_i(k) = act_end - k + 1 steps still to run
-            const int A4 = A >> 2;
-#pragma unroll 2
-            for (int q0 = 0; q0 < A4; q0 += NT) {
-                const int q4 = q0 + tid;
-                const bool inr = q4 < A4;
-                const int4 bq = inr ? *vec_at<const int4>(g_base, 4 * q4) : make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
-                const int4 eq = inr ? *vec_at<const int4>(g_end, 4 * q4) : make_int4(0, 0, 0, 0);
-                const int bs4[4] = {bq.x, bq.y, bq.z, bq.w};
-                const int en4[4] = {eq.x, eq.y, eq.z, eq.w};
-                const int g = (int)__umulhi((unsigned)(4 * q4), a.magic_B);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const bool live = bs4[j] != kEmpty;
-                    int nh = en4[j] - k + 1;
-                    nh = nh < 0 ? 0 : (nh > H ? H : nh);
-                    bucket_add(Lh_s, Ch_s, live ? g * H1 + nh : -1, live ? (unsigned)(bs4[j] + k) : 0u, lane);
-                }
-            }
-        } else if (HM > 0 && H > 0) {
-            const int A4 = A >> 2;
+        if (FP) {
+            __syncthreads();                              // buckets and due list complete
+            if (classifier) {
+                // the classifier row of every request on the list, two in flight per thread.
+                // p_fin = 1 - prod (1 - q_h) <= sum q_h for probabilities: when the fp32 sum is clearly below
+                // the gate the fp64 product cannot reach it and is not evaluated.
+                const int n_due = scal[8];
+                const bool rows32 = (H & 7) == 0 && (reinterpret_cast<size_t>(raw_of(probs)) & 31) == 0;
+                const float *rows = reinterpret_cast<const float *>(raw_of(probs));
 #pragma unroll 1
-            for (int q_base = 0; q_base < A4; q_base += NT * kUnroll) {
-                int4 bq[kUnroll]; float4 cq[kUnroll]; unsigned kq[kUnroll];
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int q4 = q_base + u * NT + tid;
-                    const bool inr = q4 < A4;
-                    bq[u] = inr ? *vec_at<const int4>(g_base, 4 * q4) : make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
-                    cq[u] = inr ? *vec_at<const float4>(g_chat0, 4 * q4) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    kq[u] = inr ? *vec_at<const unsigned>(g_kref, 4 * q4) : 0u;
-                }
-#pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    const int q4 = q_base + u * NT + tid;
-                    const int bs4[4] = {bq[u].x, bq[u].y, bq[u].z, bq[u].w};
-                    const float c04[4] = {cq[u].x, cq[u].y, cq[u].z, cq[u].w};
-                    const int g = (int)__umulhi((unsigned)(4 * q4), a.magic_B);      // slot / B
-                    // which of the four requests are due for a refresh; one list append per quad and warp
-                    bool due4[4]; float c4[4]; unsigned dm4[4];
-                    int n_due = 0;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool live = bs4[j] != kEmpty;
-                        const int t = (k - (int)((kq[u] >> (8 * j)) & 0xFFu)) & 255;
-                        c4[j] = c04[j] - (float)t;
-                        due4[j] = live && (t >= a.delta_T || c4[j] < a.c_floor);
-                        dm4[j] = __ballot_sync(kFull, due4[j]);
-                        n_due += __popc(dm4[j]);
-                    }
-                    if (n_due) {                                             // uniform over the warp
-                        int at = 0;
-                        if (lane == 0) at = atomicAdd(&scal[8], n_due);
-                        at = __shfl_sync(kFull, at, 0);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (due4[j]) refresh_list[at + __popc(dm4[j] & ((1u << lane) - 1u))] = (unsigned short)(4 * q4 + j);
-                            at += __popc(dm4[j]);
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool settle = bs4[j] != kEmpty && !due4[j];
-                        int nh = (int)floorf(c4[j]);
-                        nh = nh < 0 ? 0 : (nh > H ? H : nh);
-                        bucket_add(Lh_s, Ch_s, settle ? g * H1 + nh : -1, settle ? (unsigned)(bs4[j] + k) : 0u, lane);
-                    }
-                }
-            }
-            inst_sync();
-            const int n_ref = scal[8];
-            // Pass B: the classifier row of every request on the list.  The loop runs the same number of
-            // rounds on every lane.
-#pragma unroll kPassBUnroll
-            for (int e0 = 0; e0 < n_ref; e0 += NT) {
-                const int e = e0 + tid;
-                int key = -1;
-                unsigned cur = 0u;
-                if (e < n_ref) {
-                    const int s0 = refresh_list[e];
-                    const auto q = probs + (long long)s0 * H;
-                    double v = (double)H;                               // gate closed: the conservative anchor
-                    if (SL) {
-                        // long classifier rows stay in memory: p_fin and c* in one pass
-                        double surv = 1.0, cs = 0.0;
+                for (int e0 = tid; e0 < n_due; e0 += 2 * NT) {
+                    const int e1 = e0 + NT;
+                    const int sa0 = due_list[e0], sa1 = e1 < n_due ? due_list[e1] : sa0;
+                    float sum[2], low[2];
+                    row_sum(rows + (size_t)sa0 * H, H, rows32, sum[0], low[0]);
+                    row_sum(rows + (size_t)sa1 * H, H, rows32, sum[1], low[1]);
+#pragma unroll 1
+                    for (int e = 0; e < 2; ++e) {
+                        const float sm = e ? sum[1] : sum[0], lo = e ? low[1] : low[0];
+                        if ((lo >= 0.0f && sm * 1.0001f < a.gate) || (e && e1 >= n_due)) continue;
+                        const int sa = e ? sa1 : sa0;
+                        // gate open: E[min(r, H)] = sum_h prod_{j<h} (1 - q_j)
+                        double surv = 1.0, c = 0.0;
+#pragma unroll 1
                         for (int h = 0; h < H; ++h) {
-                            cs = __dadd_rn(cs, surv);
-                            surv = __dmul_rn(surv, __dsub_rn(1.0, (double)q[h]));
+                            c = __dadd_rn(c, surv);
+                            surv = __dmul_rn(surv, __dsub_rn(1.0, (double)__ldg(rows + (size_t)sa * H + h)));
                         }
-                        if (__dsub_rn(1.0, surv) >= (double)a.gate) v = cs;
-                    } else {
-                        float qv[HR > 0 ? HR : 1];
-                        if (HR == 8 && H == 8 && (reinterpret_cast<size_t>(raw_of(probs)) & 31) == 0) {
-                            ld_row8(reinterpret_cast<const float *>(vec_at<const double4>(q, 0)), qv);
-                        } else if ((H & 3) == 0) {
-#pragma unroll
-                            for (int h = 0; h < HR; h += 4) {
-                                if (h < H) {
-                                    const float4 qq = ld_row4(reinterpret_cast<const float *>(vec_at<const float4>(q, h)));
-                                    qv[h] = qq.x; qv[h + 1] = qq.y; qv[h + 2] = qq.z; qv[h + 3] = qq.w;
-                                }
-                            }
-                        } else {
-#pragma unroll
-                            for (int h = 0; h < HR; ++h) if (h < H) qv[h] = q[h];
-                        }
-                        // p_fin = 1 - prod (1 - q_h) <= sum q_h for probabilities: when the fp32 sum is
-                        // clearly below the gate the fp64 product cannot reach it and is not evaluated
-                        float qsum = 0.0f, qmin = 0.0f;
-#pragma unroll
-                        for (int h = 0; h < HR; ++h) if (h < H) { qsum += qv[h]; qmin = fminf(qmin, qv[h]); }
-                        double p_fin = 0.0;
-                        if (!(qmin >= 0.0f && qsum * 1.0001f < a.gate)) {
-                            double surv = 1.0;
-#pragma unroll
-                            for (int h = 0; h < HR; ++h)
-                                if (h < H) surv = __dmul_rn(surv, __dsub_rn(1.0, (double)qv[h]));
-                            p_fin = __dsub_rn(1.0, surv);
-                        }
-                        if (p_fin >= (double)a.gate) {
-                            // gate open: E[min(r, H)] = sum_h prod_{j<h} (1 - q_j)
-                            double sv = 1.0, cs = 0.0;
-#pragma unroll
-                            for (int h = 0; h < HR; ++h) {
-                                if (h < H) {
-                                    cs = __dadd_rn(cs, sv);
-                                    sv = __dmul_rn(sv, __dsub_rn(1.0, (double)qv[h]));
-                                }
-                            }
-                            v = cs;
+                        if (!(__dsub_rn(1.0, surv) >= (double)a.gate)) continue;
+                        if (c < (double)a.c_floor) c = (double)a.c_floor;   // clipped to [floor, H]
+                        if (c > (double)H) c = (double)H;
+                        const float cf = (float)c;
+                        g_chat0[sa] = cf;
+                        int nh = (int)floorf(cf);
+                        nh = nh < 0 ? 0 : (nh > H ? H : nh);
+                        if (nh != H) {                                      // from the anchor's bucket to its own
+                            const int g = sa / B;
+                            const unsigned cur = (unsigned)(g_base[sa] + k);
+                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + H]), 0u - cur);
+                            atomicAdd(&Ch[g * HS + H], -1);
+                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur);
+                            atomicAdd(&Ch[g * HS + nh], 1);
                         }
                     }
-                    if (v < (double)a.c_floor) v = (double)a.c_floor;   // clipped to [floor, H]
-                    if (v > (double)H) v = (double)H;
-                    const float c = (float)v;
-                    cur = (unsigned)(g_base[s0] + k);
-                    g_chat0[s0] = c;
-                    g_kref[s0] = (uint8_t)(k & 255);
-                    int nh = (int)floorf(c);
-                    nh = nh < 0 ? 0 : (nh > H ? H : nh);
-                    key = (int)__umulhi((unsigned)s0, a.magic_B) * H1 + nh;
                 }
-                bucket_add(Lh_s, Ch_s, key, cur, lane);
+                __syncthreads();
+            }
+            // buckets -> L_g(k+h): 2^seg_log2 lanes per worker, each with a stretch of offsets
+            if (H > 0) {
+                const int SEG = 1 << a.seg_log2, SL = (H1 + SEG - 1) >> a.seg_log2;
+#pragma unroll 1
+                for (int i0 = warp << 5; i0 < (G << a.seg_log2); i0 += NT) {
+                    const int g = (i0 + lane) >> a.seg_log2, sg = lane & (SEG - 1);
+                    const int h0 = sg * SL, h1 = g < G ? min(h0 + SL, H1) : h0;
+                    int T = 0, C = 0;
+#pragma unroll 2
+                    for (int h = h0; h < h1; ++h) { T += Lh[g * HS + h]; C += Ch[g * HS + h]; }
+                    int Ti = T, Ci = C;
+#pragma unroll 1
+                    for (int o = 1; o < SEG; o <<= 1) {
+                        const int t = __shfl_down_sync(kFull, Ti, o), c = __shfl_down_sync(kFull, Ci, o);
+                        if (sg + o < SEG) { Ti += t; Ci += c; }
+                    }
+                    Ti -= T; Ci -= C;                                       // the stretches above this one
+#pragma unroll 2
+                    for (int h = h1 - 1; h >= h0; --h) {
+                        Ti += Lh[g * HS + h]; Ci += Ch[g * HS + h];
+                        Lh[g * HS + h] = Ti + h * Ci;
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (int g = tid; g < G; g += NT) Lh[g * HS] = L0_s[g];
+            }
+            __syncthreads();
+#pragma unroll 1
+            for (int h = lane; h < H1; h += 32) {                           // envelope M_h
+                int v = 0;
+#pragma unroll 4
+                for (int g = warp; g < G; g += nwarps) v = max(v, Lh[g * HS + h]);
+                atomicMax(&Ms[h], v);
             }
         }
-        inst_sync();                                              // B1
+        __syncthreads();
         if (timing) t_phase[2] = (unsigned)clock64();
+
+        // ---- requests running before this step that end at it: by warps 1.. while warp 0 routes ----
+        if ((warp > 0 || nwarps == 1) && a.pred_mode != 1) {
+            const int t0 = nwarps == 1 ? tid : tid - 32, nt = nwarps == 1 ? NT : NT - 32;
+            if (a.term_mode == 1) {
+#pragma unroll 1
+                for (int g = t0; g < G; g += nt) {
+                    draw_ending(t_term, B, OW, (uint32_t)k, (uint32_t)g, key0, key1, fin + (size_t)g * OW);
+                    unsigned sub = 0u;
+#pragma unroll 1
+                    for (int x = 0; x < OW; ++x) {
+                        unsigned long long e = occ0[g * OW + x] & fin[g * OW + x];
+                        endm[g * OW + x] = e;
+#pragma unroll 1
+                        for (; e; e &= e - 1ull) {
+                            const int sa = g * B + 64 * x + __ffsll((long long)e) - 1;
+                            sub += (unsigned)(g_base[sa] + k);
+                            g_base[sa] = kEmpty;
+                        }
+                    }
+                    sub_load[g] = sub;
+                }
+            } else if (a.term_mode >= 2) {
+                const unsigned A8 = (unsigned)A >> 3;
+#pragma unroll 1
+                for (unsigned o = t0; o < A8; o += nt) {
+                    const int p = (int)(o / (unsigned)G), g = (int)o - p * G, a0 = g * B + 8 * p;
+                    const unsigned ob = (unsigned)(occ0[g * OW + (p >> 3)] >> (8 * (p & 7))) & 0xFFu;
+                    unsigned fb = 0u;
+                    if (life) {
+                        // a request ends with its o_i-th step: act_end == k
+                        const int4 e0 = *vec_at<const int4>(g_end, a0), e1 = *vec_at<const int4>(g_end, a0 + 4);
+                        const int en[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) if (en[j] == k) fb |= 1u << j;
+                    } else {
+                        // Bernoulli(term_probs[slot][0]): 24-bit uniform below the probability
+#pragma unroll 1
+                        for (int half = 0; half < 2; ++half) {
+                            if (!((ob >> (4 * half)) & 0xFu)) continue;
+                            const uint4 r = philox_call((uint32_t)k, (uint32_t)((a0 >> 2) + half), kStreamTerm, key0, key1);
+                            const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                if ((ob >> (4 * half + j)) & 1u) {
+                                    const float q = probs[(size_t)(a0 + 4 * half + j) * H];
+                                    if (__fmul_rn((float)(rr[j] >> 8), 5.9604644775390625e-8f) < q) fb |= 1u << (4 * half + j);
+                                }
+                        }
+                    }
+                    fb &= ob;
+                    endm8[g * OW * 8 + p] = (unsigned char)fb;
+#pragma unroll 1
+                    for (; fb; fb &= fb - 1u) {
+                        const int sa = a0 + __ffs(fb) - 1;
+                        atomicAdd(&sub_load[g], (unsigned)(g_base[sa] + k));
+                        g_base[sa] = kEmpty;
+                    }
+                }
+            }
+        }
 
         if (warp == 0) {
             // ================= ROUTE (warp 0 only, warp-synchronous) =================
-            if (SL) {
-                // buckets -> L_g(k+h) in place (each lane owns the rows of its workers), then the envelope
-                // with the lanes spread over h
+            // lane owns workers lane and lane + 32 (selection keys) and offsets lane, lane + 32, ... (envelope)
+            int cap[GW], L0[GW], mm[GW], M[HC];
 #pragma unroll
-                for (int w = 0; w < GW; ++w) {
-                    const int g = lane + 32 * w;
-                    if (g < G) {
-                        int accT = 0, accC = 0;
-                        for (int h = H; h >= 0; --h) {
-                            accT += (int)Lh_s[g * H1 + h]; accC += (int)Ch_s[g * H1 + h];
-                            L_s[g * H1 + h] = accT + h * accC;
-                        }
-                        L[w][0] = accT;
+            for (int w = 0; w < GW; ++w) {
+                const int g = lane + 32 * w;
+                cap[w] = g < G ? cap_s[g] : -1;
+                L0[w] = g < G ? (FP ? Lh[g * HS] : L0_s[g]) : 0;
+                mm[w] = 0;
+            }
+#pragma unroll
+            for (int c = 0; c < HC; ++c) M[c] = FP ? (lane + 32 * c < HS ? Ms[lane + 32 * c] : 0x7FFFFFFF) : 0;
+            int M0 = 0;                                                     // Eq. 1: envelope
+            if (!FP) {
+                int v = L0[0];
+#pragma unroll
+                for (int w = 1; w < GW; ++w) v = max(v, L0[w]);
+                M0 = __reduce_max_sync(kFull, v);
+#pragma unroll
+                for (int w = 0; w < GW; ++w) mm[w] = M0 - L0[w];
+            }
+            // horizon-min margins min_h (M_h - L_g(k+h)) of all workers, from shared memory
+            auto margins_min = [&]() {
+                if (HC > 1 && G <= 16) {
+#pragma unroll 1
+                    for (int g = 0; g < G; ++g) {
+                        int v = 0x7FFFFFFF;
+#pragma unroll
+                        for (int c = 0; c < HC; ++c)
+                            if (lane + 32 * c < H1) v = min(v, M[c] - Lh[g * HS + lane + 32 * c]);
+                        v = __reduce_min_sync(kFull, v);
+                        if (lane == g) mm[0] = v;
                     }
-                }
-                __syncwarp();
-                for (int h = lane; h <= H; h += 32) {
-                    int v = L_s[h];
-                    for (int g = 1; g < G; ++g) v = max(v, L_s[g * H1 + h]);
-                    M_s[h] = v;
-                }
-                __syncwarp();
-                Mh[0] = M_s[0];
-            } else {
-                if (H > 0) {
+                } else {
 #pragma unroll
                     for (int w = 0; w < GW; ++w) {
                         const int g = lane + 32 * w;
-                        int accT = 0, accC = 0;
-#pragma unroll
-                        for (int h = HR; h >= 0; --h) {
-                            if (g < G && h <= H) { accT += (int)Lh_s[g * H1 + h]; accC += (int)Ch_s[g * H1 + h]; }
-                            L[w][h] = (g < G && h <= H) ? accT + h * accC : 0;
+                        if (g < G) {
+                            int v = 0x7FFFFFFF;
+#pragma unroll 1
+                            for (int h = 0; h < H1; h += 4) {
+                                const int4 x = *vec_at<const int4>(Ms, h), y = *vec_at<const int4>(Lh, g * HS + h);
+                                v = min(min(min(v, x.x - y.x), min(x.y - y.y, x.z - y.z)), x.w - y.w);
+                            }
+                            mm[w] = v;
                         }
                     }
                 }
-#pragma unroll
-                for (int h = 0; h <= HR; ++h) {
-                    int v = L[0][h];
-#pragma unroll
-                    for (int w = 1; w < GW; ++w) v = max(v, L[w][h]);
-                    Mh[h] = (h <= H) ? __reduce_max_sync(kFull, v) : 0;
-                }
-            }
+            };
+            bool stale = FP;                                                // mm has to be rebuilt (the envelope grew)
 
-            Scorer<FP, HM, SL> sc;
-            sc.mds = md_s;
-            // margins of worker g -> every lane's scorer
+            Scorer<FP> sc;
+            sc.md = md; sc.dn = dn_s; sc.H = H; sc.G = G; sc.aD = a.aD; sc.beta = a.beta;
+            int m[HC], v[HC];                                               // margins and loads of the selected worker, by offset
             auto load_margins = [&](int g) {
-                const int src = g & 31;
-                const int set = g >> 5;
-                if (!FP) {
-                    int mine = Mh[0] - L[0][0];
+                if (FP) {
 #pragma unroll
-                    for (int w = 1; w < GW; ++w) if (set == w) mine = Mh[0] - L[w][0];
-                    sc.mi = __shfl_sync(kFull, mine, src);
-                } else if (SL) {
-                    int mmin = 0x7FFFFFFF;
-                    __syncwarp();                          // earlier readers of md_s are done
-                    for (int h = lane; h <= H; h += 32) {
-                        const int mh = M_s[h] - L_s[g * H1 + h];
-                        md_s[h] = (double)mh;
-                        mmin = min(mmin, mh);
+                    for (int c = 0; c < HC; ++c) {
+                        const int h = lane + 32 * c;
+                        v[c] = h < H1 ? Lh[g * HS + h] : 0;
+                        m[c] = M[c] - v[c];
+                        if (h < HS) md[h] = m[c];
                     }
-                    sc.mmin = __reduce_min_sync(kFull, mmin);
                     __syncwarp();
-                } else {
-                    int mmin = 0x7FFFFFFF;
-#pragma unroll
-                    for (int h = 0; h <= HR; ++h) {
-                        int mine = Mh[h] - L[0][h];
-#pragma unroll
-                        for (int w = 1; w < GW; ++w) if (set == w) mine = Mh[h] - L[w][h];
-                        const int mh = __shfl_sync(kFull, mine, src);
-                        sc.md[h] = (double)mh;
-                        if (h <= H) mmin = min(mmin, mh);
-                    }
-                    sc.mmin = mmin;
                 }
             };
 
             // optional F-score matrix before the first admission
-            if (!LEAN && a.out.fscore) {
+            if (a.out.fscore) {
+                if (FP) { margins_min(); stale = false; }
                 double *F = a.out.fscore + orow * (size_t)W * G;
+#pragma unroll 1
                 for (int g = 0; g < G; ++g) {
+                    const int own = (GW > 1 && g >= 32) ? mm[GW - 1] : mm[0];
+                    sc.mm = __shfl_sync(kFull, own, g & 31);
                     load_margins(g);
-                    for (int i = lane; i < W; i += 32)
-                        F[(size_t)i * G + g] = (i < n_w) ? sc.value(sc.key(a, q_key[i] >> WL)) : 0.0;
+                    score_column<FP>(sc, F + g, q_key, n_w, W, G, WL, lane);
+                    __syncwarp();
                 }
             }
 
@@ -717,663 +836,464 @@ __global__ void __maxnreg__((FP && HM > 0) ? 128 : 72) br_step_kernel(const Step
 #pragma unroll
             for (int w = 0; w < GW; ++w) S_tot += cap[w] > 0 ? cap[w] : 0;
             S_tot = (int)__reduce_add_sync(kFull, (unsigned)S_tot);
-            int n_left = n_w;
-            int admitted = 0, s1_iters = 0, s2_pops = 0, status = 0;
-            const int n_tiles = (n_w + 31) >> 5;
+            int n_left = n_w, s1_iters = 0, s2_pops = 0, status = 0, first_rm = W;   // first_rm: per lane, reduced at the end
+            const int n_groups = (n_w + 127) >> 7;
+            // Stage-2 window: each lane keeps its four largest waiting keys, sorted, across the pops of the
+            // step; a lane whose list runs dry although it may hold more keys forces a rebuild
+            int t0 = 0, t1 = 0, t2 = 0, t3 = 0;
+            bool listed = false, full = false, merged = false;
+            int wkey = 0, wdelta = 0, nwin = 0;          // lane r: r-th largest key; lane mask: sum of its subset
+            bool to_stage2 = true;
 
-            // Stage-2 window state: each lane's five largest waiting keys, sorted, built by the first
-            // pop of the step and kept up to date as requests are admitted
-            int wt0 = 0, wt1 = 0, wt2 = 0, wt3 = 0, wt4 = 0;
-            bool w_built = false, w_trunc = false;
-            constexpr bool w_keep = FP;
-            int gw[kRegWin] = {0, 0, 0, 0, 0};
-            bool gw_valid = false;
-
-            // argmax_i F_g({i}) over all waiting requests, earliest arrival on ties.
-            // Returns the packed key of the winner (0 if none).
-            auto best_single = [&]() -> int {
-                if (!FP) {
-                    int bk = kEmpty; int bkey = 0;
-#pragma unroll 4
-                    for (int t = 0; t < n_tiles; ++t) {
-                        const int idx = (t << 5) + lane;
-                        const int qk = idx < n_w ? q_key[idx] : 0;
-                        if (qk > 0) {
-                            const int f = (int)sc.key(a, qk >> WL);
-                            // within a lane positions ascend, so strict > keeps the earliest
-                            if (f > bk) { bk = f; bkey = qk; }
-                        }
-                    }
-                    int wk;
-                    const int src = warp_argmax_lane32(bk, (unsigned)bkey & posmask, wk);
-                    const int res = __shfl_sync(kFull, bkey, src);
-                    return res > 0 ? res : 0;
-                } else if (!SL && a.peak_ok) {
-                    // Eq. 2 is concave and piecewise linear in s with kinks at the m_{g,h}: it rises up
-                    // to s* = the smallest kink at which the slope alpha D - beta sum_{m_h <= kink} d_h
-                    // is no longer positive, and falls after it.  br_create has checked that no such
-                    // slope is within rounding distance of zero, so the fp64 scores of integer lengths
-                    // are strictly ordered on either side, and the arg-max is the largest s <= s* or the
-                    // smallest s > s* (earliest arrival among equal lengths): two integer scans and two
-                    // evaluations of Eq. 2.
-                    double mine = 0.0;
-#pragma unroll
-                    for (int h = 0; h <= HR; ++h) if (lane == h) mine = sc.md[h];
-                    double wsum = 0.0;
-#pragma unroll
-                    for (int h = 0; h <= HR; ++h) if (h <= H && sc.md[h] <= mine) wsum = __dadd_rn(wsum, a.d[h]);
-                    const bool past = lane <= H && !(a.aD > __dmul_rn(a.beta, wsum));
-                    const int sstar = (int)__reduce_min_sync(kFull, past ? (unsigned)(int)mine : 0x7FFFFFFFu);
-                    const int thr = sstar >= (1 << (31 - WL)) ? 0x7FFFFFFF : ((sstar << WL) | (int)posmask);
-                    int below = 0; unsigned above = 0x7FFFFFFFu;
-#pragma unroll 4
-                    for (int t = 0; t < n_tiles; ++t) {
-                        const int idx = (t << 5) + lane;
-                        const int qk = idx < n_w ? q_key[idx] : 0;
-                        if (qk > 0) {
-                            if (qk <= thr) below = max(below, qk);
-                            else above = min(above, (unsigned)qk ^ posmask);
-                        }
-                    }
-                    const int ka = __reduce_max_sync(kFull, below);
-                    const unsigned ab = __reduce_min_sync(kFull, above);
-                    const int kb = ab == 0x7FFFFFFFu ? 0 : (int)(ab ^ posmask);
-                    const long long fa = ka > 0 ? sc.key(a, ka >> WL) : kNoKey;
-                    const long long fb = kb > 0 ? sc.key(a, kb >> WL) : kNoKey;
-                    if (fa > fb) return ka;
-                    if (fb > fa) return kb;
-                    if (ka <= 0) return 0;
-                    return ((unsigned)ka & posmask) > ((unsigned)kb & posmask) ? ka : kb;
-                } else {
-                    // Horizon-safe requests (s <= min_h m_{g,h}) score alpha D s exactly, which grows
-                    // with s: of those only the largest key per lane is scored; the others in full.
-                    long long bk = kNoKey; int bkey = 0, best_safe = 0;
-#pragma unroll 2
-                    for (int t = 0; t < n_tiles; ++t) {
-                        const int idx = (t << 5) + lane;
-                        const int qk = idx < n_w ? q_key[idx] : 0;
-                        if (qk > 0) {
-                            if ((qk >> WL) <= sc.mmin) {
-                                best_safe = max(best_safe, qk);
-                            } else {
-                                const long long f = sc.key(a, qk >> WL);
-                                if (f > bk) { bk = f; bkey = qk; }
-                            }
-                        }
-                    }
-                    if (best_safe > 0) {
-                        const long long f = sc.key(a, best_safe >> WL);
-                        if (f > bk || (f == bk && ((unsigned)best_safe & posmask) > ((unsigned)bkey & posmask))) {
-                            bk = f; bkey = best_safe;
-                        }
-                    }
-                    long long wk;
-                    const int src = warp_argmax_lane(bk, (unsigned)bkey & posmask, wk);
-                    const int res = __shfl_sync(kFull, bkey, src);
-                    return wk == kNoKey ? 0 : res;
-                }
-            };
-
-            // sticky admission of the request with packed key qk to worker g
-            auto commit = [&](int qk, int g) {
-                const int s = qk >> WL;
-                const int pos = (int)(posmask - ((unsigned)qk & posmask));
-                const int src = g & 31, set = g >> 5;
-                if (lane == src) {
-                    int slot = -1;
-                    for (int w = 0; w < OW && slot < 0; ++w) {
-                        const unsigned long long fr = ~occ[g * OW + w];
-                        if (fr) slot = w * 64 + __ffsll((long long)fr) - 1;
-                    }
-                    if (slot >= 0 && slot < B) {
-                        occ[g * OW + (slot >> 6)] |= 1ull << (slot & 63);
-                        const int sa = g * B + slot;
-                        g_base[sa] = s - k;
-                        if (H > 0 && g_chat0) {
-                            g_chat0[sa] = (float)(H + a.delta_T - 1);
-                            g_kref[sa] = (uint8_t)((k + 1 - a.delta_T) & 255);
-                        }
-                        if (life) g_end[sa] = k + q_o[pos] - 1;          // runs at steps k .. k + o_i - 1
-                        if (g_aid) g_aid[sa] = q_id[pos];
-                        q_key[pos] = (int)(0x80000000u | (unsigned)sa);
-                    } else {
-                        status |= BR_ST_BAD_STATE;
-                        q_key[pos] = -1;                  // gone, no slot
-                    }
-#pragma unroll
-                    for (int w = 0; w < GW; ++w) {
-                        if (set == w) {
-                            cap[w] -= 1;
-#pragma unroll
-                            for (int h = 0; h <= HR; ++h) if (h <= H) L[w][h] += s;
-                        }
-                    }
-                }
-                // envelope: only worker g grew, so M_h = max(M_h, L_g(k+h))
-                if (SL) {
-                    for (int h = lane; h <= H; h += 32) {
-                        const int v = L_s[g * H1 + h] + s;
-                        L_s[g * H1 + h] = v;
-                        M_s[h] = max(M_s[h], v);
-                    }
-                    __syncwarp();
-                    Mh[0] = M_s[0];
-                }
-#pragma unroll
-                for (int h = 0; h <= HR; ++h) {
-                    if (!SL && h <= H) {
-                        int mine = L[0][h];
-#pragma unroll
-                        for (int w = 1; w < GW; ++w) if (set == w) mine = L[w][h];
-                        Mh[h] = max(Mh[h], __shfl_sync(kFull, mine, src));
-                    }
-                }
-                if (!w_keep && qk >= gw[kRegWin - 1]) gw_valid = false;   // one of the cached largest keys leaves
-                if (w_keep && w_built && lane == (pos & 31)) {
-                    if (wt0 == qk) { wt0 = wt1; wt1 = wt2; wt2 = wt3; wt3 = wt4; wt4 = 0; }
-                    else if (wt1 == qk) { wt1 = wt2; wt2 = wt3; wt3 = wt4; wt4 = 0; }
-                    else if (wt2 == qk) { wt2 = wt3; wt3 = wt4; wt4 = 0; }
-                    else if (wt3 == qk) { wt3 = wt4; wt4 = 0; }
-                    else if (wt4 == qk) { wt4 = 0; }
-                }
-                __syncwarp();
-                S_tot -= 1; n_left -= 1; admitted += 1;
-            };
-
-            if (S_tot > 0 && n_w > 0) {
-                // ---------- Stage 1: greedy fill ----------
 #pragma unroll 1
-                while (S_tot > a.S_greedy && n_left > 0) {
-                    if (s1_iters >= W) { status |= BR_ST_ITER_CAP; break; }
+            while (n_left > 0 && S_tot > 0) {
+                const bool st1 = S_tot > a.S_greedy;
+                if (FP && stale) { margins_min(); stale = false; }
+                if (!st1 && to_stage2) { to_stage2 = false; if (timing) t_phase[3] = (unsigned)clock64(); }
+                if (st1 ? s1_iters >= W : s2_pops >= W + G) { status |= BR_ST_ITER_CAP; break; }
+                // most free slots; then Stage 1: smallest L_g(k), Stage 2: largest horizon-min margin; lowest g
+                int bc = cap[0];
+#pragma unroll
+                for (int w = 1; w < GW; ++w) bc = max(bc, cap[w]);
+                const int mc = __reduce_max_sync(kFull, bc);
+                if (mc <= 0) break;
+                int bv = kEmpty;
+#pragma unroll
+                for (int w = 0; w < GW; ++w) if (cap[w] == mc) bv = max(bv, st1 ? ~L0[w] : mm[w]);
+                const int mv = __reduce_max_sync(kFull, bv);
+                int gi = 0xFF;
+#pragma unroll
+                for (int w = GW - 1; w >= 0; --w) if (cap[w] == mc && (st1 ? ~L0[w] : mm[w]) == mv) gi = lane + 32 * w;
+                const int g = (int)__reduce_min_sync(kFull, (unsigned)gi);
+                const int src = g & 31;
+                sc.mm = st1 ? __shfl_sync(kFull, (GW > 1 && g >= 32) ? mm[GW - 1] : mm[0], src) : mv;
+                load_margins(g);
+
+                unsigned chosen = 1u;                    // window entries to admit (bit r: lane r holds the key)
+                int dsum = 0;
+                bool single = st1;
+                if (st1) {
                     ++s1_iters;
-                    // most free slots; ties: smallest L_g(k), then lowest g
-                    int bc = cap[0], bl = L[0][0], bg = lane;
-#pragma unroll
-                    for (int w = 1; w < GW; ++w)
-                        if (cap[w] > bc || (cap[w] == bc && L[w][0] < bl)) { bc = cap[w]; bl = L[w][0]; bg = lane + 32 * w; }
-                    const int mc = __reduce_max_sync(kFull, bc);
-                    const unsigned ml = __reduce_min_sync(kFull, bc == mc ? (unsigned)bl : 0xFFFFFFFFu);
-                    const unsigned mg = __reduce_min_sync(kFull, (bc == mc && (unsigned)bl == ml) ? (unsigned)bg : 0xFFFFFFFFu);
-                    const int g = (int)mg;
-                    load_margins(g);
-                    const int qk = best_single();
-                    if (qk <= 0) break;
-                    commit(qk, g);
-                }
-            }
-            if (timing) t_phase[3] = (unsigned)clock64();
-            if (S_tot > 0 && n_left > 0) {
-                // ---------- Stage 2: refined allocation ----------
-#pragma unroll 1
-                while (n_left > 0 && S_tot > 0) {
-                    if (s2_pops >= W + G) { status |= BR_ST_ITER_CAP; break; }
+                } else {
                     ++s2_pops;
-                    // (largest cap, largest horizon-min margin, lowest g) among cap > 0
-                    int bc = -1, bm = -1, bg = 0x7FFFFFFF;
-#pragma unroll
-                    for (int w = 0; w < GW; ++w) {
-                        int mm = Mh[0] - L[w][0];
-                        if (SL) {
-                            const int g = lane + 32 * w;
-                            if (g < G)
-                                for (int h = 1; h <= H; ++h) mm = min(mm, M_s[h] - L_s[g * H1 + h]);
-                        }
-#pragma unroll
-                        for (int h = 1; h <= HR; ++h) if (h <= H) mm = min(mm, Mh[h] - L[w][h]);
-                        if (cap[w] > 0 && (cap[w] > bc || (cap[w] == bc && mm > bm))) { bc = cap[w]; bm = mm; bg = lane + 32 * w; }
-                    }
-                    const int mc = __reduce_max_sync(kFull, bc);
-                    if (mc <= 0) break;
-                    const int mm2 = __reduce_max_sync(kFull, bc == mc ? bm : -1);
-                    const unsigned mg = __reduce_min_sync(kFull, (bc == mc && bm == mm2) ? (unsigned)bg : 0xFFFFFFFFu);
-                    const int g = (int)mg;
-                    load_margins(g);
-
-                    if (!LEAN && a.big_window) {
-                        // ---- windows of 6 to 16 requests (Appendix "Bit-set subset selection") ----
-                        // the R_max largest keys, one warp maximum per entry (keys are distinct)
-                        const int R = min(a.R_max, n_left);
-                        int thr = 0x7FFFFFFF;
-                        for (int r = 0; r < R; ++r) {
-                            int best = 0;
-#pragma unroll 4
-                            for (int t = 0; t < n_tiles; ++t) {
-                                const int idx = (t << 5) + lane;
-                                const int x = idx < n_w ? q_key[idx] : 0;
-                                if (x < thr) best = max(best, x);
-                            }
-                            thr = __reduce_max_sync(kFull, best);
-                            if (lane == 0) bw_win[r] = thr;
-                        }
-                        __syncwarp();
-                        // prompt lengths of the window in shared memory (reusing the key slots' upper half is
-                        // not needed: lengths are recomputed from the keys)
-                        const int lim = min(mc, R);
-                        const int ra = min(kBigWinLow, (R + 1) / 2), rb = R - ra;
-                        // sorted subsets of the low entries (as prompt lengths)
-                        {
-                            const int n = 1 << ra;
-                            for (int m = lane; m < n; m += 32) {
-                                int sum = 0;
-                                for (int j = 0; j < ra; ++j) if ((m >> j) & 1) sum += bw_win[j] >> WL;
-                                bw_keys[m] = ((unsigned long long)__popc(m) << 56) | ((unsigned long long)(unsigned)sum << 16) | (unsigned)m;
-                            }
-                            __syncwarp();
-                            for (int k2 = 2; k2 <= n; k2 <<= 1) {
-                                for (int j = k2 >> 1; j > 0; j >>= 1) {
-                                    for (int i = lane; i < n; i += 32) {
-                                        const int p = i ^ j;
-                                        if (p > i) {
-                                            const unsigned long long x = bw_keys[i], y = bw_keys[p];
-                                            const bool up = (i & k2) == 0;
-                                            if ((x > y) == up) { bw_keys[i] = y; bw_keys[p] = x; }
-                                        }
-                                    }
-                                    __syncwarp();
-                                }
-                            }
-                            if (lane == 0) {
-                                int off = 0, binom = 1;
-                                for (int c = 0; c <= ra; ++c) { bw_off[c] = off; off += binom; binom = binom * (ra - c) / (c + 1); }
-                                bw_off[ra + 1] = off;
-                            }
-                            __syncwarp();
-                        }
-                        // the peak of the score in Delta
-                        int peak;
-                        if (!FP) {
-                            peak = sc.mi;
-                        } else {
-                            double mine = 0.0;
-#pragma unroll
-                            for (int h = 0; h <= HR; ++h) if (lane == h) mine = sc.md[h];
-                            double wsum = 0.0;
-#pragma unroll
-                            for (int h = 0; h <= HR; ++h) if (h <= H && sc.md[h] <= mine) wsum = __dadd_rn(wsum, a.d[h]);
-                            const bool past = lane <= H && !(a.aD > __dmul_rn(a.beta, wsum));
-                            peak = (int)__reduce_min_sync(kFull, past ? (unsigned)(int)mine : 0x7FFFFFFFu);
-                        }
-                        MitmBest b; b.lo_sum = -1; b.lo_mask = 0xFFFFFFFFu; b.hi_sum = 0x7FFFFFFF; b.hi_mask = 0xFFFFFFFFu;
-                        for (unsigned mh = lane; mh < (1u << rb); mh += 32) {
-                            const int ph = __popc(mh);
-                            if (ph > lim) continue;
-                            int sh = 0;
-                            for (unsigned t = mh; t; t &= t - 1) sh += bw_win[ra + __ffs(t) - 1] >> WL;
-                            mitm_probe(bw_keys, bw_off, ra, lim, peak, mh, sh, ph, b);
-                        }
-                        // warp reduction: largest sum at or below the peak, smallest above it, lowest mask among equals
-                        {
-                            const int ls = __reduce_max_sync(kFull, b.lo_sum);
-                            const unsigned lm = __reduce_min_sync(kFull, b.lo_sum == ls ? b.lo_mask : 0xFFFFFFFFu);
-                            const int hs = __reduce_min_sync(kFull, b.hi_sum);
-                            const unsigned hm = __reduce_min_sync(kFull, b.hi_sum == hs ? b.hi_mask : 0xFFFFFFFFu);
-                            b.lo_sum = ls; b.lo_mask = lm; b.hi_sum = hs; b.hi_mask = hm;
-                        }
-                        long long bk = kNoKey; unsigned bmask = 0u;
-                        if (b.lo_sum >= 0) { bk = sc.key(a, b.lo_sum); bmask = b.lo_mask; }
-                        if (b.hi_sum != 0x7FFFFFFF) {
-                            const long long k2 = sc.key(a, b.hi_sum);
-                            if (k2 > bk || (k2 == bk && b.hi_mask < bmask)) { bk = k2; bmask = b.hi_mask; }
-                        }
-                        if (bk == kNoKey) { status |= BR_ST_ITER_CAP; break; }
-                        if (bk <= 0) {
-                            const int qk = best_single();                   // starvation guard
-                            if (qk <= 0) break;
-                            commit(qk, g);
-                        } else {
-                            for (int r = 0; r < R; ++r)
-                                if ((bmask >> r) & 1u) commit(bw_win[r], g);
-                        }
-                        continue;
-                    }
-
+                    long long wk = kNoKey;
                     // window: the R_max largest waiting requests, earliest first on ties
-                    int win[kRegWin];
-                    int nwin = 0;
-                    if (!w_keep) {
-                        // Eq. 1 kernels cache the five largest keys of the queue; the cache stays valid
-                        // until one of them is admitted (the guard mostly admits small requests)
-                        if (!gw_valid) {
-                            int t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0;
-#pragma unroll 4
-                            for (int t = 0; t < n_tiles; ++t) {
-                                const int idx = (t << 5) + lane;
-                                int x = idx < n_w ? q_key[idx] : 0;
-                                int y;
-                                y = max(t0, x); x = min(t0, x); t0 = y;
-                                y = max(t1, x); x = min(t1, x); t1 = y;
-                                y = max(t2, x); x = min(t2, x); t2 = y;
-                                y = max(t3, x); x = min(t3, x); t3 = y;
-                                t4 = max(t4, x);
-                            }
-#pragma unroll
-                            for (int r = 0; r < kRegWin; ++r) {
-                                const int m = __reduce_max_sync(kFull, t0);
-                                gw[r] = m;
-                                if (t0 == m) { t0 = t1; t1 = t2; t2 = t3; t3 = t4; t4 = 0; }
-                            }
-                            gw_valid = true;
-                        }
-#pragma unroll
-                        for (int r = 0; r < kRegWin; ++r) {
-                            win[r] = (r < a.R_max && r < n_left) ? gw[r] : 0;
-                            if (win[r] > 0) nwin = r + 1;
-                        }
+                    const int R = min(a.R_max, n_left);
+                    if (a.big_window) {
+                        wkey = largest_keys(q_key, n_w, R, lane);
+                        const WindowChoice c = big_window<FP>(sc, bw_keys, bw_off, bw_win, wkey, R, min(mc, R), WL, FP ? m[0] : 0, lane);
+                        wk = c.wk; chosen = c.chosen; dsum = c.dsum;
                     } else {
-                        // Eq. 2 kernels keep every lane's sorted candidates across pops and merge the
-                        // heads.  A list that runs dry although its lane holds more keys (possible only
-                        // after several admissions from one lane) forces a rebuild.
+                        while (!merged) {
+                            const bool fresh = !listed;
+                            if (fresh) {
+                                t0 = t1 = t2 = t3 = 0;
 #pragma unroll 1
-                        for (int attempt = 0; attempt < 2; ++attempt) {
-                            if (!w_built) {
-                                int t0 = 0, t1 = 0, t2 = 0, t3 = 0, t4 = 0, cnt = 0;
-#pragma unroll 4
-                                for (int t = 0; t < n_tiles; ++t) {
-                                    const int idx = (t << 5) + lane;
-                                    int x = idx < n_w ? q_key[idx] : 0;
-                                    cnt += x > 0;
-                                    int y;
-                                    y = max(t0, x); x = min(t0, x); t0 = y;
-                                    y = max(t1, x); x = min(t1, x); t1 = y;
-                                    y = max(t2, x); x = min(t2, x); t2 = y;
-                                    y = max(t3, x); x = min(t3, x); t3 = y;
-                                    t4 = max(t4, x);
+                                for (int t = 0; t < n_groups; ++t) {
+                                    const int4 kk = *vec_at<const int4>(q_key, (t * 32 + lane) * 4);
+                                    const int ke[4] = {kk.x, kk.y, kk.z, kk.w};
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j) {
+                                        int x = ke[j], y;
+                                        y = max(t0, x); x = min(t0, x); t0 = y;
+                                        y = max(t1, x); x = min(t1, x); t1 = y;
+                                        y = max(t2, x); x = min(t2, x); t2 = y;
+                                        t3 = max(t3, x);
+                                    }
                                 }
-                                wt0 = t0; wt1 = t1; wt2 = t2; wt3 = t3; wt4 = t4;
-                                w_trunc = cnt > 5;
-                                w_built = true;
+                                full = t3 > 0 && n_groups > 1;             // one group: four keys per lane
                             }
-                            int h0 = wt0, h1 = wt1, h2 = wt2, h3 = wt3, h4 = wt4;
+                            int h0 = t0, h1 = t1, h2 = t2, h3 = t3;
                             bool dry = false;
-                            nwin = 0;
-#pragma unroll
-                            for (int r = 0; r < kRegWin; ++r) {
-                                win[r] = 0;
-                                if (r < a.R_max && r < n_left) {
-                                    dry = dry || (h0 == 0 && w_trunc);
-                                    const int m = __reduce_max_sync(kFull, h0);
-                                    win[r] = m;
-                                    if (m > 0) nwin = r + 1;
-                                    if (h0 == m) { h0 = h1; h1 = h2; h2 = h3; h3 = h4; h4 = 0; }
-                                }
+                            wkey = 0; wdelta = 0;
+#pragma unroll 1
+                            for (int r = 0; r < R; ++r) {
+                                dry = dry || (h0 == 0 && full);
+                                const int x = __reduce_max_sync(kFull, h0);
+                                if (lane == r) wkey = x;
+                                if ((lane >> r) & 1) wdelta += x >> WL;
+                                if (h0 == x) { h0 = h1; h1 = h2; h2 = h3; h3 = 0; }
                             }
-                            if (!__any_sync(kFull, dry)) break;
-                            w_built = false;
+                            nwin = R;
+                            merged = listed = !__any_sync(kFull, dry);
+                            if (!merged && fresh) {
+                                // one lane holds more of the window than its list
+                                wkey = largest_keys(q_key, n_w, R, lane);
+                                wdelta = 0;
+                                for (int r = 0; r < R; ++r) {
+                                    const int x = __shfl_sync(kFull, wkey, r);
+                                    if ((lane >> r) & 1) wdelta += x >> WL;
+                                }
+                                merged = true;
+                            }
                         }
-                    }
-                    // subsets of the window: lane = mask, lowest mask on ties
-                    const int lim = min(mc, a.R_max);
-                    long long fk = kNoKey;
-                    if (lane >= 1 && lane < (1 << nwin) && __popc(lane) <= lim) {
-                        int delta = 0;
-#pragma unroll
-                        for (int r = 0; r < kRegWin; ++r)
-                            if ((lane >> r) & 1) delta += win[r] >> WL;
-                        fk = sc.key(a, delta);
-                    }
-                    long long wk;
-                    int best_mask;
-                    if (!FP) {                          // Eq. 1 scores fit 32 bits
-                        int wk32;
-                        best_mask = warp_argmax_lane32(fk == kNoKey ? kEmpty : (int)fk, 31u - (unsigned)lane, wk32);
-                        wk = wk32 == kEmpty ? kNoKey : (long long)wk32;
-                    } else {
-                        best_mask = warp_argmax_lane(fk, 31u - (unsigned)lane, wk);
+                        // subsets of the window: lane = mask, lowest mask on ties
+                        const bool cand = lane >= 1 && lane < (1 << nwin) && __popc(lane) <= min(mc, a.R_max);
+                        const int dmax = __reduce_max_sync(kFull, cand ? wdelta : 0);
+                        bool best;
+                        if (!FP) {                          // Eq. 1 scores fit 32 bits
+                            const int f = cand ? (int)sc.key(wdelta) : kEmpty;
+                            const int mf = __reduce_max_sync(kFull, f);
+                            wk = mf;
+                            best = f == mf;
+                        } else if (dmax <= sc.mm) {
+                            // every subset is safe at every offset: the score alpha D Delta grows with Delta
+                            wk = dmax;
+                            best = wdelta == dmax;
+                        } else {
+                            best = warp_max64(cand ? sc.key(wdelta) : kNoKey, wk);
+                        }
+                        chosen = __reduce_min_sync(kFull, cand && best ? (unsigned)lane : 32u);
+                        if (dmax == 0) wk = kNoKey;
+                        dsum = __shfl_sync(kFull, wdelta, chosen & 31u);
                     }
                     if (wk == kNoKey) { status |= BR_ST_ITER_CAP; break; }
-                    if (wk <= 0) {
-                        // starvation guard: least-bad single request of all of R_wait
-                        const int qk = best_single();
-                        if (qk <= 0) break;
-                        commit(qk, g);
-                    } else {
+                    single = wk <= 0;                           // starvation guard
+                }
+
+                int mykey = wkey;                               // lane r: the key behind bit r of `chosen`
+                if (single) {
+                    // argmax_i F_g({i}) over all waiting requests, earliest arrival on ties.
+                    // The score is concave and piecewise linear in s (Eq. 2: kinks at the m_{g,h}): it rises up to
+                    // s* = the smallest kink at which the slope alpha D - beta sum_{m_h <= kink} d_h is no longer
+                    // positive (Eq. 1: the margin) and falls after it.  If no slope is within rounding distance of zero,
+                    // the scores of integer lengths are strictly ordered on either side, and the arg-max is the
+                    // largest s <= s* or the smallest s > s*: one pass of two integer minima over the queue.
+                    int peak = sc.mm;
+                    bool ordered = a.peak_ok != 0;
+                    if (FP) {
+                        double ws[HC];
 #pragma unroll
-                        for (int r = 0; r < kRegWin; ++r)
-                            if ((best_mask >> r) & 1) commit(win[r], g);
+                        for (int c = 0; c < HC; ++c) ws[c] = 0.0;
+#pragma unroll 1
+                        for (int h = 0; h < H1; h += 4) {
+                            const int4 m4 = *vec_at<const int4>(md, h);
+                            const int mj[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const double d = dn_s[2 * (h + j)];
+#pragma unroll
+                                for (int c = 0; c < HC; ++c) if (mj[j] <= m[c]) ws[c] = __dadd_rn(ws[c], d);
+                            }
+                        }
+                        peak = 0x7FFFFFFF;
+                        bool flat = false;
+#pragma unroll
+                        for (int c = 0; c < HC; ++c) {
+                            const double sl = __dsub_rn(a.aD, __dmul_rn(a.beta, ws[c]));
+                            if (lane + 32 * c < H1) {
+                                flat = flat || fabs(sl) <= a.slope_err;
+                                if (!(sl > 0.0)) peak = min(peak, m[c]);
+                            }
+                        }
+                        peak = __reduce_min_sync(kFull, peak);
+                        ordered = !__any_sync(kFull, flat);
+                    }
+                    int qk = 0;
+                    if (ordered) {
+                        const int thr = peak >= (1 << (31 - WL)) ? 0x7FFFFFFF : ((peak << WL) | (int)posmask);
+                        // entries that are gone or beyond the queue have negative keys: as unsigned distances they
+                        // lie beyond every waiting one
+                        unsigned below = 0xFFFFFFFFu, above = 0xFFFFFFFFu;
+#pragma unroll 2
+                        for (int t = 0; t < n_groups; ++t) {
+                            const int4 kk = *vec_at<const int4>(q_key, (t * 32 + lane) * 4);
+                            const unsigned ke[4] = {(unsigned)kk.x, (unsigned)kk.y, (unsigned)kk.z, (unsigned)kk.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                below = min(below, (unsigned)thr - ke[j]);
+                                above = min(above, (ke[j] ^ posmask) - ((unsigned)thr + 1u));
+                            }
+                        }
+                        below = __reduce_min_sync(kFull, below);
+                        above = __reduce_min_sync(kFull, above);
+                        const int ka = max((int)((unsigned)thr - below), 0);
+                        const int kx = (int)(above + (unsigned)thr + 1u);
+                        const int kb = kx > thr ? (int)((unsigned)kx ^ posmask) : 0;
+                        if (ka == 0 || kb == 0) {
+                            qk = ka | kb;
+                        } else {
+                            const long long f = sc.key(((lane & 1) ? kb : ka) >> WL);
+                            const long long fa = __shfl_sync(kFull, f, 0), fb = __shfl_sync(kFull, f, 1);
+                            const bool first_a = ((unsigned)ka & posmask) > ((unsigned)kb & posmask);
+                            qk = fa > fb || (fa == fb && first_a) ? ka : kb;
+                        }
+                    } else {
+                        qk = best_of_all<FP>(sc, q_key, n_w, WL, posmask, lane);      // a flat segment
+                    }
+                    if (qk <= 0) break;
+                    mykey = qk;
+                    chosen = 1u;
+                    dsum = qk >> WL;
+                }
+
+                // ---- admission to worker g: lane r takes the request of bit r; slots are given out after routing ----
+                const int n_adm = __popc(chosen);
+                if ((chosen >> lane) & 1u) {
+                    const int at = __popc(chosen & ((1u << lane) - 1u)), pos = (int)(posmask - ((unsigned)mykey & posmask));
+                    adm[n_w - n_left + at] = make_int2(mykey, (g << 16) | (mc - at));
+                    q_key[pos] = kQBeyond;
+                    first_rm = min(first_rm, pos);
+                }
+                // worker g grew by dsum at every offset; only it can lift the envelope
+                if (!FP) {
+                    const int Ln = M0 - sc.mm + dsum, up = max(Ln - M0, 0);
+                    M0 += up;
+#pragma unroll
+                    for (int w = 0; w < GW; ++w) mm[w] += up;
+                } else {
+                    bool grew = false;
+#pragma unroll
+                    for (int c = 0; c < HC; ++c) {
+                        const int h = lane + 32 * c;
+                        if (h < H1) {
+                            const int x = v[c] + dsum;
+                            Lh[g * HS + h] = x;
+                            if (x > M[c]) { M[c] = x; Ms[h] = x; grew = true; }
+                        }
+                    }
+                    stale = __any_sync(kFull, grew);
+                }
+                if (lane == src) {
+#pragma unroll
+                    for (int w = 0; w < GW; ++w)
+                        if ((g >> 5) == w) { cap[w] -= n_adm; L0[w] += dsum; mm[w] -= dsum; }
+                }
+                // the admitted keys leave the lanes' lists; the merged window stays valid while none of it leaves
+                if (listed) {
+#pragma unroll 1
+                    for (unsigned cb = chosen; cb; cb &= cb - 1u) {
+                        const int x = __shfl_sync(kFull, mykey, __ffs(cb) - 1);
+                        if (t0 == x) { t0 = t1; t1 = t2; t2 = t3; t3 = 0; }
+                        else if (t1 == x) { t1 = t2; t2 = t3; t3 = 0; }
+                        else if (t2 == x) { t2 = t3; t3 = 0; }
+                        else if (t3 == x) { t3 = 0; }
                     }
                 }
+                if (merged) {
+                    const int last = __shfl_sync(kFull, wkey, nwin - 1);
+                    merged = single && mykey < last && n_left - 1 >= a.R_max;
+                }
+                __syncwarp();
+                S_tot -= n_adm; n_left -= n_adm;
             }
-            if (timing) t_phase[4] = (unsigned)clock64();
+            if (timing) { t_phase[4] = (unsigned)clock64(); if (to_stage2) t_phase[3] = t_phase[4]; }
 
             // ================= RECORD =================
             {
-                int mx = L[0][0], mn = cap[0] >= 0 ? L[0][0] : 0x7FFFFFFF;
-                long long sum = cap[0] >= 0 ? (long long)L[0][0] : 0;
+                int mx = kEmpty, mn = 0x7FFFFFFF;
+                long long sum = 0;
                 const auto o_load = mk_span(reinterpret_cast<long long *>(a.out.load) + orow * G, G);
-                if (cap[0] >= 0) o_load[lane] = L[0][0];
 #pragma unroll
-                for (int w = 1; w < GW; ++w) {
-                    if (cap[w] >= 0) {
-                        mx = max(mx, L[w][0]); mn = min(mn, L[w][0]); sum += L[w][0];
-                        o_load[lane + 32 * w] = L[w][0];
+                for (int w = 0; w < GW; ++w) {
+                    const int g = lane + 32 * w;
+                    if (g < G) {
+                        mx = max(mx, L0[w]); mn = min(mn, L0[w]); sum += L0[w];
+                        o_load[g] = L0[w];
+                        L0_s[g] = L0[w];
                     }
                 }
                 mx = __reduce_max_sync(kFull, mx);
                 mn = __reduce_min_sync(kFull, mn);
                 for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
                 status = (int)__reduce_or_sync(kFull, (unsigned)status);
+                const int fr = __reduce_min_sync(kFull, first_rm);
                 if (lane == 0) {
                     const auto tr = mk_span(reinterpret_cast<long long *>(a.out.trace) + orow * 3, 3);
                     tr[0] = mx; tr[1] = mn; tr[2] = sum;
-                    scal[0] = n_left; scal[1] = admitted; scal[2] = s1_iters; scal[3] = s2_pops;
+                    scal[0] = n_left; scal[1] = n_w - n_left; scal[2] = s1_iters; scal[3] = s2_pops;
                     scal[4] = status | (n_drop ? BR_ST_QUEUE_OVERFLOW : 0);
+                    scal[6] = fr;
                 }
             }
-        } else if (term_mode == 1) {
-            // warps 1.. draw this step's termination words while warp 0 routes
-            draw_fin(tid - 32, NT - 32);
         }
-        inst_sync();                                              // B2: admissions visible
+        __syncthreads();                                          // admissions visible
 
-        // ============ queue compaction and assignments (warp 0) ============
-        // A lane owns four consecutive positions of every group of 128 (16-byte accesses to the keys,
-        // the ids and the assignment row); an entry's new position is the count of kept entries before it.
-        if (warp == 0) {
-            const auto assign = mk_span(a.assign_out + orow * W, W);
-            int run = 0;
-            const int n_before = n_w;          // queue length after ARRIVE
-            const unsigned lt = (1u << lane) - 1u;
+        // ============ sticky admissions, one thread each ============
+        // a worker's requests take its free slots in ascending order, in the order of their admission
+        const int n_new = scal[0], n_adm = n_w - n_new;
 #pragma unroll 1
-            for (int i0 = 0; i0 < W; i0 += 128) {
-                const int p0 = i0 + lane * 4;
-                if (i0 >= n_before) {
-                    // the rest of the row is beyond the queue: only assignments remain
+        for (int e = tid; e < n_adm; e += NT) {
+            const int2 r = adm[e];
+            const int g = r.y >> 16, s = r.x >> WL, pos = (int)(posmask - ((unsigned)r.x & posmask));
+            int rank = cap_s[g] - (r.y & 0xFFFF), slot = B;
+#pragma unroll 1
+            for (int x = 0; x < 2 * OW; ++x) {
+                unsigned fr = ~occ032[2 * g * OW + x];
+                const int c = __popc(fr);
+                if (rank < c) {
+#pragma unroll 1
+                    for (; rank > 0; --rank) fr &= fr - 1u;
+                    slot = 32 * x + __ffs(fr) - 1;
+                    break;
+                }
+                rank -= c;
+            }
+            if (slot >= B) {                                      // free-slot count and occupancy word disagree: gone, no slot
+                atomicOr(&scal[4], BR_ST_BAD_STATE);
+                continue;
+            }
+            const int sa = g * B + slot;
+            q_key[pos] = (int)(0x80000000u | (unsigned)sa);
+            atomicOr(&occ32[2 * g * OW + (slot >> 5)], 1u << (slot & 31));
+            const int o = life ? q_o[pos] : 0;
+            if (H > 0 && g_chat0) {
+                g_chat0[sa] = (float)(H + a.delta_T - 1);
+                g_kref[sa] = (uint8_t)((k + 1 - a.delta_T) & 255);
+            }
+            if (life) g_end[sa] = k + o - 1;                      // runs at steps k .. k + o_i - 1
+            if (g_aid) g_aid[sa] = q_id[pos];
+            // it may also end at this very step
+            bool ends = false;
+            if (a.term_mode == 1) {
+                ends = (fin[g * OW + (slot >> 6)] >> (slot & 63)) & 1ull;
+            } else if (a.term_mode == 2) {
+                const uint4 w = philox_call((uint32_t)k, (uint32_t)sa >> 2, kStreamTerm, key0, key1);
+                ends = __fmul_rn((float)(word_of(w, sa & 3) >> 8), 5.9604644775390625e-8f) < probs[(size_t)sa * H];
+            } else if (life) {
+                ends = o == 1;
+            }
+            g_base[sa] = ends ? kEmpty : s - k;
+            if (ends) {
+                atomicOr(&endm32[2 * g * OW + (slot >> 5)], 1u << (slot & 31));
+                atomicAdd(&sub_load[g], (unsigned)s);
+            }
+        }
+        __syncthreads();
+
+        // ============ queue compaction and assignments ============
+        // A thread owns four consecutive positions of every stretch of 4 NT; an entry's new position is
+        // the count of kept entries before it.  A moved entry gains the distance in its key's position field.
+        const int first_rm = scal[6];
+        {
+            const auto assign = mk_span(a.assign_out + orow * W, W);
+            int run = 0, par = 0;
+#pragma unroll 1
+            for (int i0 = 0; i0 < W; i0 += 4 * NT) {
+                const int p0 = i0 + 4 * tid;
+                if (i0 >= n_w || i0 + 4 * NT <= first_rm) {
                     if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(-1, -1, -1, -1);
+                    run += 4 * NT;                                // (beyond the queue the count is not used)
                     continue;
                 }
-                int4 kk = make_int4(0, 0, 0, 0); uint4 ii = make_uint4(0u, 0u, 0u, 0u); int4 oo = make_int4(0, 0, 0, 0);
+                int4 kk = make_int4(kQBeyond, kQBeyond, kQBeyond, kQBeyond), oo = make_int4(0, 0, 0, 0);
+                uint4 ii = make_uint4(0u, 0u, 0u, 0u);
                 if (p0 < W) {
                     kk = *vec_at<const int4>(q_key, p0);
                     ii = *vec_at<const uint4>(q_id, p0);
                     if (life) oo = *vec_at<const int4>(q_o, p0);
                 }
-                int ke[4] = {kk.x, kk.y, kk.z, kk.w};
+                const int ke[4] = {kk.x, kk.y, kk.z, kk.w};
                 const unsigned idv[4] = {ii.x, ii.y, ii.z, ii.w};
                 const int ov[4] = {oo.x, oo.y, oo.z, oo.w};
+                const int cnt = (ke[0] > 0) + (ke[1] > 0) + (ke[2] > 0) + (ke[3] > 0);
+                int inc = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(kFull, inc, o); if (lane >= o) inc += x; }
+                if (lane == 31) scal[16 + par + warp] = inc;
                 int as[4];
-                int below = run, total = 0;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if (p0 + j >= n_before) ke[j] = 0;                  // beyond the queue
-                    const unsigned bal = __ballot_sync(kFull, ke[j] > 0);
-                    below += __popc(bal & lt);
-                    total += __popc(bal);
                     const int sa = ke[j] & 0x7FFFFFFF;
-                    const bool gone = ke[j] < 0 && sa < A;
-                    as[j] = gone ? sa : -1;
-                    if (have_pre && gone) {
-                        // a request admitted at this step may also end at it
-                        const int g = (int)__umulhi((unsigned)sa, a.magic_B), slot = sa - g * B;
-                        if ((fin_w[g * OW + (slot >> 6)] >> (slot & 63)) & 1ull) {
-                            atomicOr(&end_mask[g * OW + (slot >> 6)], 1ull << (slot & 63));
-                            const int at = atomicAdd(&scal[6], 1);
-                            if (at < kEndList) {
-                                end_list[at] = (unsigned short)sa;
-                            } else {
-                                atomicAdd(&sub_load[g], (unsigned)(g_base[sa] + k));
-                                g_base[sa] = kEmpty;
-                            }
-                        }
-                    }
+                    as[j] = ke[j] < 0 && sa < A ? sa : -1;
                 }
                 if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(as[0], as[1], as[2], as[3]);
-                __syncwarp();                                           // the group is read before any of it is overwritten
+                __syncthreads();                                  // the stretch is read before any of it is overwritten
+                int below = run + inc - cnt, total = 0;
+#pragma unroll 1
+                for (int x = 0; x < nwarps; ++x) {
+                    const int t = scal[16 + par + x];
+                    if (x < warp) below += t;
+                    total += t;
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     if (ke[j] > 0) {
-                        const int i = p0 + j, dst = below;
-                        const int sv = ke[j] >> WL;
-                        if (dst != i) { q_key[dst] = (sv << WL) | (int)(posmask - (unsigned)dst); q_id[dst] = idv[j]; }
-                        if (dst != i || i >= n_w_old) { g_qs[dst] = sv; g_qid[dst] = idv[j]; }
-                        if (life) {
-                            if (dst != i) q_o[dst] = ov[j];
-                            if (dst != i || i >= n_w_old) g_qo[dst] = ov[j];
+                        const int from = p0 + j;
+                        if (below != from) {
+                            q_key[below] = ke[j] + (from - below);
+                            q_id[below] = idv[j];
+                            if (life) q_o[below] = ov[j];
                         }
                         ++below;
                     }
                 }
-                __syncwarp();
                 run += total;
+                par ^= 8;
             }
         }
-        n_w = scal[0];
+        __syncthreads();
+        // entries that moved or are new go back to the caller's rows
+#pragma unroll 1
+        for (int p0 = (min(first_rm, n_w_old) & ~3) + 4 * tid; p0 < n_new; p0 += 4 * NT) {
+            const int4 kk = *vec_at<const int4>(q_key, p0);
+            const uint4 ii = *vec_at<const uint4>(q_id, p0);
+            const int4 sv = make_int4(kk.x >> WL, kk.y >> WL, kk.z >> WL, kk.w >> WL);
+            if (p0 + 4 <= n_new) {
+                *vec_at<int4>(g_qs, p0) = sv;
+                *vec_at<uint4>(g_qid, p0) = ii;
+                if (life) *vec_at<int4>(g_qo, p0) = *vec_at<const int4>(q_o, p0);
+            } else {
+                const int s4[4] = {sv.x, sv.y, sv.z, sv.w};
+                const unsigned i4[4] = {ii.x, ii.y, ii.z, ii.w};
+#pragma unroll
+                for (int j = 0; j < 3; ++j)
+                    if (p0 + j < n_new) {
+                        g_qs[p0 + j] = s4[j]; g_qid[p0 + j] = i4[j];
+                        if (life) g_qo[p0 + j] = q_o[p0 + j];
+                    }
+            }
+        }
+#pragma unroll 1
+        for (int i = n_new + tid; i < n_w; i += NT) q_key[i] = kQBeyond;        // vacated tail
+        n_w = n_new;
         if (timing) t_phase[5] = (unsigned)clock64();
 
         // ================= ADVANCE =================
-        // Only the occupancy masks, the termination draws and the few ending slots are touched.
-        if (!have_pre) {
-            if (term_mode == 2) {
-                // Bernoulli(term_probs[slot][0]) per running request: 24-bit uniform below the probability
-                const float sc24 = 5.9604644775390625e-8f;
+        // L_g(k+1) = L_g(k) - (loads of the requests that ended) + (number of survivors)
 #pragma unroll 1
-                for (int q8 = tid; q8 < A8; q8 += NT) {
-                    const int a0 = q8 << 3;
-                    const int g = a0 / B, slot0 = a0 - g * B;
-                    const unsigned ob = (unsigned)(occ[g * OW + (slot0 >> 6)] >> (slot0 & 63)) & 0xFFu;
-                    unsigned fb = 0;
-#pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        if (!((ob >> (4 * half)) & 0xFu)) continue;
-                        const uint4 r = philox4x32_10((uint32_t)k, (uint32_t)(q8 * 2 + half), kStreamTerm, 0u, key0, key1);
-                        const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int jj = 4 * half + j;
-                            if ((ob >> jj) & 1u) {
-                                const float q = probs[(size_t)(a0 + jj) * H];
-                                if (__fmul_rn((float)(rr[j] >> 8), sc24) < q) fb |= 1u << jj;
-                            }
-                        }
-                    }
-                    *vec_at<unsigned char>(mk_span(reinterpret_cast<unsigned char *>(raw_of(fin_w)), (long long)G * OW * 8), (long long)g * OW * 8 + (slot0 >> 3)) = (unsigned char)fb;
-                }
-                inst_sync();
-            } else if (term_mode == 3) {
-                // a request ends with its o_i-th step: act_end == k
+        for (int g = tid; g < G; g += NT) {
+            int na = 0;
+            for (int x = 0; x < OW; ++x) {
+                const unsigned long long o = occ[g * OW + x] & ~endm[g * OW + x];
+                occ[g * OW + x] = o; occ0[g * OW + x] = o;
+                na += __popcll(o);
+            }
+            cap_s[g] = B - na;
+            L0_s[g] = L0_s[g] - (int)sub_load[g] + na;
+            sub_load[g] = 0u;
+        }
+        if (FP && it + 1 < a.n_steps) {
 #pragma unroll 1
-                for (int q8 = tid; q8 < A8; q8 += NT) {
-                    const int a0 = q8 << 3;
-                    const int g = a0 / B, slot0 = a0 - g * B;
-                    const unsigned ob = (unsigned)(occ[g * OW + (slot0 >> 6)] >> (slot0 & 63)) & 0xFFu;
-                    unsigned fb = 0;
-                    if (ob) {
-                        const int4 e0 = *vec_at<const int4>(g_end, a0);
-                        const int4 e1 = *vec_at<const int4>(g_end, a0 + 4);
-                        const int en[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) if (((ob >> j) & 1u) && en[j] == k) fb |= 1u << j;
-                    }
-                    *vec_at<unsigned char>(mk_span(reinterpret_cast<unsigned char *>(raw_of(fin_w)), (long long)G * OW * 8), (long long)g * OW * 8 + (slot0 >> 3)) = (unsigned char)fb;
-                }
-                inst_sync();
-            }
-            scan_workers(false);
-        }
-        inst_sync();
-        {
-            // the requests that ended: subtract their load from the worker, free the slot
-            if (tid < n_pre) {
-                const int sa = pre_list[tid];
-                g_base[sa] = kEmpty;
-                atomicAdd(&sub_load[sa / B], (unsigned)(pend + k));
-            }
-            const int n_end = min(scal[6], kEndList);
-            for (int e = tid; e < n_end; e += NT) {
-                const int sa = end_list[e];
-                const int cur = g_base[sa] + k;
-                g_base[sa] = kEmpty;
-                atomicAdd(&sub_load[sa / B], (unsigned)cur);
-            }
-            if (have_pre && scal[9]) {
-                // more requests ended than the lists hold: the rest were subtracted when they were
-                // found, their slots are emptied here (the instance is one warp; the listed slots
-                // have been read by now)
-                __syncwarp();
+            for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
 #pragma unroll 1
-                for (int idx = tid; idx < G * OW; idx += NT) {
-                    const int g = idx / OW, x = idx - g * OW;
-                    unsigned long long ended = end_mask[idx];
-                    while (ended) {
-                        const int j = __ffsll((long long)ended) - 1;
-                        ended &= ended - 1;
-                        g_base[g * B + 64 * x + j] = kEmpty;
-                    }
-                }
-            }
+            for (int h = tid; h < H1; h += NT) Ms[h] = 0;
         }
-        inst_sync();                                              // B3
-
-        if (warp == 0) {
-            // L_g(k+1) = L_g(k) - (loads of the requests that ended) + (number of survivors)
+        if (tid == 0) {
+            if (a.out.counters) {
+                uint32_t *c = a.out.counters + orow * 4;
+                c[0] = (uint32_t)n_drop; c[1] = (uint32_t)scal[1]; c[2] = (uint32_t)scal[2]; c[3] = (uint32_t)scal[3];
+            }
+            if (a.out.status) a.out.status[orow] = scal[4] | scal[5];
+            scal[8] = 0;
+            if (timing) {
+                t_phase[6] = (unsigned)clock64();
+                uint32_t *pc = a.out.phase_cycles + orow * 8;
 #pragma unroll
-            for (int w = 0; w < GW; ++w) {
-                const int g = lane + 32 * w;
-                if (g < G) {
-                    int na = 0;
-                    for (int x = 0; x < OW; ++x) {
-                        const unsigned long long o = occ[g * OW + x] & ~end_mask[g * OW + x];
-                        occ[g * OW + x] = o;
-                        na += __popcll(o);
-                    }
-                    cap[w] = B - na;
-                    L[w][0] = L[w][0] - (int)sub_load[g] + na;
-                    sub_load[g] = 0u;
-                }
-            }
-            if (lane == 0) {
-                if (a.out.counters) {
-                    uint32_t *c = a.out.counters + orow * 4;
-                    c[0] = (uint32_t)n_drop; c[1] = (uint32_t)scal[1]; c[2] = (uint32_t)scal[2]; c[3] = (uint32_t)scal[3];
-                }
-                if (a.out.status) a.out.status[orow] = scal[4] | scal[5];
-                scal[6] = 0; scal[7] = 0; scal[8] = 0; scal[9] = 0;
-                if (timing) {
-                    t_phase[6] = (unsigned)clock64();
-                    uint32_t *pc = a.out.phase_cycles + orow * 8;
-#pragma unroll
-                    for (int p = 0; p < 6; ++p) pc[p] = (uint32_t)(t_phase[p + 1] - t_phase[p]);
-                    pc[6] = it == 0 ? (uint32_t)(t_phase[0] - t_entry) : 0u;
-                    pc[7] = 0u;
-                }
+                for (int p = 0; p < 6; ++p) pc[p] = (uint32_t)(t_phase[p + 1] - t_phase[p]);
+                pc[6] = it == 0 ? (uint32_t)(t_phase[0] - t_entry) : 0u;
+                pc[7] = 0u;
             }
         }
-        if (it + 1 < a.n_steps) {
-            for (int i = tid; i < 2 * G * H1; i += NT) Lh_s[i] = 0u;
-            inst_sync();
-        }
+        __syncthreads();
     }
 
     // ---- write the snapshot back ----
-    if (warp == 0) {
-#pragma unroll
-        for (int w = 0; w < GW; ++w) {
-            const int g = lane + 32 * w;
-            if (g < G) {
-                g_load[g] = (long long)L[w][0];
-                g_nact[g] = B - cap[w];
-                for (int x = 0; x < OW; ++x) g_occ[g * OW + x] = occ[g * OW + x];   // updated by this lane
-            }
-        }
+#pragma unroll 1
+    for (int g = tid; g < G; g += NT) {
+        a.ws.load[(size_t)inst * G + g] = (long long)L0_s[g];
+        a.ws.nact[(size_t)inst * G + g] = B - cap_s[g];
+        for (int x = 0; x < OW; ++x) a.ws.occ[((size_t)inst * G + g) * OW + x] = occ[g * OW + x];
     }
     if (tid == 0) {
         a.ws.step[inst] = k;

@@ -1,0 +1,50 @@
+"""The block-per-instance step kernel at the edges of its tiles: 128-position groups of the queue, 32
+horizon offsets and 32 workers per lane set, the lanes' lists of four largest keys, thread counts.
+Whole numbers against the checker: the tolerance is equality."""
+import numpy as np
+import pytest
+
+from paper_2605_06113_b200 import workload as wlm
+from helpers import run_parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("G,B,W,H,kw", [
+    (32, 8, 124, 15, dict()), (33, 8, 128, 31, dict()), (32, 16, 132, 32, dict(R_max=5)), (64, 8, 512, 63, dict()),
+    (1, 8, 4, 80, dict()), (5, 72, 516, 3, dict(R_max=5)), (64, 64, 260, 8, dict(R_max=1)), (2, 256, 1024, 5, dict()),
+    (33, 8, 640, 0, dict(R_max=5)), (1, 8, 132, 0, dict(threads=64)),
+])
+def test_tile_edges(G, B, W, H, kw):
+    kw = dict(kw)
+    threads = kw.pop("threads", 0)
+    for term_mode, pred_mode, gate in ((1, 0, 0.5), (2, 0, 0.1), (3, 1, 0.5)):
+        if H == 0 and term_mode != 1:
+            continue
+        cfg = wlm.get_config("c2", G=G, B=B, W=W, H=H, init_active=B - B // 8, init_queue=W - 1, hazard=0.05,
+                             term_mode=term_mode, pred_mode=pred_mode, gate=gate, out_mu=2.0, score_mode=-1,
+                             S_greedy=-1, delta_T=-1, arrival=("const", 6.0), **kw)
+        run_parity(cfg, 2, 12, threads=threads, launch_steps=3, check_every=1)
+
+
+@pytest.mark.parametrize("threads", [32, 96, 256])
+@pytest.mark.parametrize("H,R_max", [(0, 5), (4, 5), (40, 4)])
+def test_one_lane_holds_the_whole_window(H, R_max, threads, monkeypatch):
+    # the largest requests sit at positions of one router lane (4 consecutive of each 128): its list of four
+    # keys runs dry inside a window of five, and again after admissions
+    make = wlm.make_workload
+
+    def patched(*args, **kwargs):
+        wl = make(*args, **kwargs)
+        q = wl.state["wq_s"]
+        for i, pos in enumerate([0, 1, 2, 3, 128, 129, 130, 131, 256, 257]):
+            q[:, pos] = 90000 - 7 * i
+        return wl
+
+    monkeypatch.setattr(wlm, "make_workload", patched)
+    cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
+                         term_mode=1, S_greedy=0, score_mode=-1, delta_T=-1)
+    run_parity(cfg, 2, 8, threads=threads, check_every=1)
+    cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
+                         term_mode=1, S_greedy=1 << 20, score_mode=-1, delta_T=-1)
+    run_parity(cfg, 2, 8, threads=threads, check_every=1)
