@@ -694,8 +694,9 @@ int br_bypass_dispatch(br_ctx *ctx, const br_instance_batch *batch, const int32_
     for (int h = 0; h <= BR_MAX_H; ++h) a.f.d[h] = ctx->d[h];
     a.n_req = n_requests; a.first_instance = batch->first_instance;
     a.s = s; a.vload = virtual_load; a.inflight = inflight; a.cap = inflight_cap; a.g_out = worker_out;
-    const int blocks = (batch->n_instances + 3) / 4;
-    br::br_bypass_kernel<<<blocks, 128, 0, (cudaStream_t)batch->stream>>>(a, batch->n_instances);
+    void (*kern)(const br::BypassArgs) = a.f.fp ? (ctx->G <= 32 ? br::br_bypass_kernel<true, 1> : br::br_bypass_kernel<true, 2>)
+                                                : (ctx->G <= 32 ? br::br_bypass_kernel<false, 1> : br::br_bypass_kernel<false, 2>);
+    kern<<<batch->n_instances, 32, 0, (cudaStream_t)batch->stream>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "br_bypass_dispatch launch");
     return BR_OK;

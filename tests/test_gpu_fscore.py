@@ -79,6 +79,31 @@ def test_pool_bypass_dispatch(G, score_mode):
     r.close()
 
 
+@pytest.mark.parametrize("G,n_req,lo,hi", [(1, 31, 1, 9), (2, 32, 1, 4), (33, 33, 1, 40000), (32, 1, 1, 9), (64, 97, 1 << 24, 1 << 26),
+                                           (31, 64, (1 << 25) - 2, (1 << 25) + 2)])
+def test_pool_bypass_edges(G, n_req, lo, hi):
+    # whole and ragged groups of 32 requests, one and two workers per lane, lengths on either side of 2^25 (the packed
+    # key's range), loads beyond 32 bits; whole numbers: equality
+    cfg = wlm.get_config("c3", G=G, init_active=8, init_queue=0)
+    r = Router(wlm.make_workload(cfg, n_instances=1), device="cuda:0")
+    rng = np.random.default_rng(G + n_req)
+    N = 5
+    s = rng.integers(lo, hi, (N, n_req)).astype(np.int32)
+    L = rng.integers(0, 3 * hi, (N, G)).astype(np.int64)
+    L[0] = np.int64(1) << 40
+    L[1, 0] = np.int64(1) << 40
+    infl = rng.integers(0, 3, (N, G)).astype(np.int32)
+    cap = rng.integers(0, 2 + 2 * n_req // G, (N, G)).astype(np.int32)
+    st, Lt, it, ct = (torch.from_numpy(x.copy()).cuda() for x in (s, L, infl, cap))
+    out = torch.full((N, n_req), -7, dtype=torch.int32, device="cuda")
+    r.bypass_dispatch(st, Lt, it, ct, out)
+    for n in range(N):
+        want, Lw, nw = oracle.bypass(G, s[n], L[n], infl[n], cap[n], score_mode=0, alpha=1.0, beta=float(G))
+        assert np.array_equal(out[n].cpu().numpy(), want), n
+        assert np.array_equal(Lt[n].cpu().numpy(), Lw) and np.array_equal(it[n].cpu().numpy(), nw), n
+    r.close()
+
+
 def test_empirical_survival_estimator():
     """br_survival_chat against the checker's counting definition (same fp64 operations: equality)."""
     cfg = wlm.get_config("c4")                              # H = 8
