@@ -1,13 +1,14 @@
-// Batched F-score matrix: F_g({i}) for every (request, worker) pair of an instance
-// (Eq. 1 in int64, Eq. 2 in fp64).  Margins are staged in shared memory, prompt
-// lengths are read with 16-byte loads, the matrix is written with unit stride.
+// Batched F-score matrix: F_g({i}) for every (request, worker) pair of an instance (Eq. 1 exactly,
+// Eq. 2 in fp64 term by term), and the best worker of every request.
 #pragma once
 #include "br_device.cuh"
 #include "../../include/br.h"
 
 namespace br {
 
-constexpr int kFsTile = 1024;   // requests per thread block
+constexpr int kFsWarps = 4;        // warps per thread block
+constexpr int kFsReq = 64;         // requests per warp, two per lane
+constexpr int kFsCols = 8;         // workers staged between two writes of the matrix
 
 struct FscoreArgs {
     int32_t G, H;
@@ -15,6 +16,8 @@ struct FscoreArgs {
     double aD, beta;
     double d[BR_MAX_H + 1];
     int32_t n_req, first_instance;
+    int32_t split_log2;    // log2 of the warps that share 64 requests, each with a stretch of workers
+    int32_t row;           // row stride of the margins in shared memory
     const int32_t *s;      // [N][n_req]
     const int64_t *Lh;     // [N][G][H+1]
     const int32_t *cap;    // [N][G] or NULL
@@ -39,98 +42,140 @@ __device__ __forceinline__ long long fscore_key(const FscoreArgs &a, int delta, 
     return key_of_double(__dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)));
 }
 
-// Thread t of a block owns worker g = t % G for the whole tile (its margins and discounts stay in
-// registers) and walks the requests slice, slice + n_slices, ...: thread t writes elements
-// t, t + n_slices * G, ... of the tile's [request][worker] rows, so every store instruction of a
-// warp covers consecutive addresses.  HM bounds H at compile time (loops over h unrolled); HM > 16
-// stands for any longer horizon: the margins are then read from shared memory in a plain loop.
-template <int HM>
-__global__ void __launch_bounds__(256) br_fscore_kernel(const FscoreArgs a)
+// Warps that share 64 requests: one where there are warps enough, up to four where short calls would
+// leave the schedulers with fewer than four each.
+inline int fscore_split_log2(int n_req, int n_instances, int G)
 {
-    __shared__ long long m_s[BR_MAX_G * (BR_MAX_H + 1)];
-    __shared__ long long Mh[BR_MAX_H + 1];
-    __shared__ __align__(16) int s_tile[kFsTile];
+    int l = 0;
+    while (l < 2 && (kFsCols << l) < G && ((long long)n_instances * ((n_req + kFsReq - 1) / kFsReq) << l) < 4ll * 4 * 148) ++l;
+    return l;
+}
+// margin rows [g][h], (d_h, -2^52 d_h) pairs, one staging area per warp
+inline int fscore_smem(int G, int row) { return 4 * G * row + 16 * row + kFsWarps * kFsReq * (kFsCols + 1) * 8; }
+
+// A lane owns two requests and walks the workers: margins and discounts are read by broadcast, the best
+// worker so far stays in registers, and eight scores of each request at a time go through shared memory so that
+// they are written in runs.  A term of Eq. 2 is RN(d_h * over), over = max(s - m_h, 0) an integer:
+// X = 2^52 + over needs no conversion, and fma(X, d_h, -2^52 d_h) rounds d_h * over once, so a term is two
+// fp64 instructions and one integer one.  Eq. 2 is bound by instruction issue (and, next, by the
+// fp64 pipe, which takes two cycles for an instruction), Eq. 1 by the writes.  200 x 1,024 x 64 scores at
+// H = 8 with best workers: 224 us with five fp64 operations a term, blocks of 1,024 requests and the best
+// worker found by scoring everything again; 57 us this way.
+template <bool FP>
+__global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreArgs a)
+{
+    extern __shared__ __align__(16) unsigned char fs_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, G = a.G, H = FP ? a.H : 0, H1 = H + 1, HS = a.row;
+    int *m_s = reinterpret_cast<int *>(fs_smem);                                 // [g][HS] -m_{g,h}, clipped to the range of s
+    double2 *d_s = reinterpret_cast<double2 *>(fs_smem + 4 * G * HS);            // (d_h, -2^52 d_h)
+    double *stage = reinterpret_cast<double *>(fs_smem + 4 * G * HS + 16 * HS) + warp * kFsReq * (kFsCols + 1);
     __shared__ int cap_s[BR_MAX_G];
-    const int tid = threadIdx.x, G = a.G, H = a.H, H1 = a.H + 1;
     const size_t inst = (size_t)a.first_instance + blockIdx.y;
-    const int tile0 = blockIdx.x * kFsTile;
-    const int n = min(kFsTile, a.n_req - tile0);
 
-    for (int i = tid; i < G * H1; i += blockDim.x) m_s[i] = a.Lh[inst * G * H1 + i];
-    for (int g = tid; g < G; g += blockDim.x) cap_s[g] = a.cap ? a.cap[inst * G + g] : 1;
-    for (int i = tid * 4; i < n; i += blockDim.x * 4)
-        *reinterpret_cast<int4 *>(s_tile + i) =
-            *reinterpret_cast<const int4 *>(a.s + inst * a.n_req + tile0 + i);
-    __syncthreads();
-    if (tid < H1) {
-        long long M = m_s[tid];
-        for (int g = 1; g < G; ++g) M = max(M, m_s[g * H1 + tid]);
-        Mh[tid] = M;
-    }
-    __syncthreads();
-    for (int i = tid; i < G * H1; i += blockDim.x) m_s[i] = Mh[i % H1] - m_s[i];
-    __syncthreads();
-
-    double *F = a.F + (inst * a.n_req + tile0) * G;
-    const int n_slices = blockDim.x / G;
-    const int slice = tid / G, g = tid - slice * G;
-    if (slice < n_slices) {
-        constexpr bool LONG = HM > 16;
-        constexpr int HR = LONG ? 0 : HM;
-        double md[HR + 1], dd[HR + 1];
-        long long m0 = m_s[g * H1], mmin = m0;
-#pragma unroll
-        for (int h = 0; h <= HR; ++h) {
-            md[h] = h <= H ? (double)m_s[g * H1 + h] : 0.0;
-            dd[h] = h <= H ? a.d[h] : 0.0;
-            if (h <= H) mmin = min(mmin, m_s[g * H1 + h]);
+    // margins: one warp per offset, lanes over workers
+    for (int h = warp; h < H1; h += kFsWarps) {
+        const int64_t *row = a.Lh + inst * G * (a.H + 1) + h;
+        const long long none = (long long)0x8000000000000000ull;
+        const long long L0 = lane < G ? row[(size_t)lane * (a.H + 1)] : none;
+        const long long L1 = lane + 32 < G ? row[(size_t)(lane + 32) * (a.H + 1)] : none;
+        long long M = L0 > L1 ? L0 : L1;
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long v = __shfl_xor_sync(kFull, M, o);
+            M = v > M ? v : M;
         }
-        if (LONG) for (int h = 1; h <= H; ++h) mmin = min(mmin, m_s[g * H1 + h]);
-        const long long Gl = (long long)G;
-#pragma unroll 4
-        for (int i = slice; i < n; i += n_slices) {
-            const int si = s_tile[i];
-            double f;
-            if (!a.fp) {
-                long long over = (long long)si - m0;
-                over = over > 0 ? over : 0;
-                f = (double)((long long)si - Gl * over);                    // Eq. 1, exact
+        if (lane < G) m_s[lane * HS + h] = -(int)min(M - L0, 0x7FFFFFFFll);
+        if (lane + 32 < G) m_s[(lane + 32) * HS + h] = -(int)min(M - L1, 0x7FFFFFFFll);
+        if (lane == 0) d_s[h] = make_double2(a.d[h], __dmul_rn(a.d[h], -4503599627370496.0));
+    }
+    for (int g = tid; g < G; g += 32 * kFsWarps) cap_s[g] = a.cap ? a.cap[inst * G + g] : 1;
+    __syncthreads();
+
+    const int split = 1 << a.split_log2, sub = warp & (split - 1);
+    const int r0 = (blockIdx.x * (kFsWarps >> a.split_log2) + (warp >> a.split_log2)) * kFsReq;
+    const int cnt = min(kFsReq, a.n_req - r0);                        // not positive: nothing to do but the barrier
+    const int span = ((G + kFsCols * split - 1) / (kFsCols * split)) * kFsCols;
+    const int g_end = min(G, (sub + 1) * span);
+    const int32_t *s = a.s + inst * a.n_req + r0;
+    const int s0 = lane < cnt ? __ldg(s + lane) : 1, s1 = lane + 32 < cnt ? __ldg(s + lane + 32) : 1;
+    const int o0 = max(s0, 0), o1 = max(s1, 0);                       // (lengths are positive; margins are never negative)
+    const double aDs0 = FP ? __dmul_rn(a.aD, (double)s0) : (double)s0, aDs1 = FP ? __dmul_rn(a.aD, (double)s1) : (double)s1;
+    const double mGl = -(double)G;
+    long long k0 = kNoKey, k1 = kNoKey;
+    int b0 = kNoIdx, b1 = kNoIdx;
+#pragma unroll 1
+    for (int gc = sub * span; gc < g_end && cnt > 0; gc += kFsCols) {
+        const int cols = min(kFsCols, g_end - gc);
+#pragma unroll 1
+        for (int x = 0; x < cols; ++x) {
+            const int g = gc + x;
+            const int *mg = m_s + g * HS;
+            double f0, f1;
+            if (!FP) {
+                const int m = mg[0];
+                f0 = __fma_rn(mGl, (double)__viaddmax_s32(o0, m, 0), aDs0);       // Eq. 1: integers below 2^53, exact
+                f1 = __fma_rn(mGl, (double)__viaddmax_s32(o1, m, 0), aDs1);
             } else {
-                const double dl = (double)si;
-                double pen = 0.0;
-                if (LONG) {
-                    if ((long long)si > mmin) {
-                        for (int h = 0; h <= H; ++h) {
-                            double over = __dsub_rn(dl, (double)m_s[g * H1 + h]);
-                            over = over > 0.0 ? over : 0.0;
-                            pen = __dadd_rn(pen, __dmul_rn(a.d[h], over));
-                        }
-                    }
-                } else if ((long long)si > mmin) {                          // else every (s - m_h)_+ is zero
+                double p0 = 0.0, p1 = 0.0;
+                int h = 0;
+#pragma unroll 2
+                for (; h + 4 <= H1; h += 4) {
+                    const int4 m4 = *reinterpret_cast<const int4 *>(mg + h);
+                    const int mj[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-                    for (int h = 0; h <= HR; ++h) {
-                        if (h <= H) {
-                            double over = __dsub_rn(dl, md[h]);
-                            over = over > 0.0 ? over : 0.0;
-                            pen = __dadd_rn(pen, __dmul_rn(dd[h], over));
-                        }
+                    for (int j = 0; j < 4; ++j) {
+                        const double2 d = d_s[h + j];
+                        p0 = __dadd_rn(p0, __fma_rn(__hiloint2double(0x43300000, __viaddmax_s32(o0, mj[j], 0)), d.x, d.y));
+                        p1 = __dadd_rn(p1, __fma_rn(__hiloint2double(0x43300000, __viaddmax_s32(o1, mj[j], 0)), d.x, d.y));
                     }
                 }
-                f = __dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)) + 0.0;   // Eq. 2 (-0.0 -> +0.0)
+#pragma unroll 1
+                for (; h < H1; ++h) {
+                    const int m = mg[h];
+                    const double2 d = d_s[h];
+                    p0 = __dadd_rn(p0, __fma_rn(__hiloint2double(0x43300000, __viaddmax_s32(o0, m, 0)), d.x, d.y));
+                    p1 = __dadd_rn(p1, __fma_rn(__hiloint2double(0x43300000, __viaddmax_s32(o1, m, 0)), d.x, d.y));
+                }
+                f0 = __dsub_rn(aDs0, __dmul_rn(a.beta, p0)) + 0.0;                // Eq. 2 (-0.0 -> +0.0)
+                f1 = __dsub_rn(aDs1, __dmul_rn(a.beta, p1)) + 0.0;
             }
-            F[(size_t)i * G + g] = f;
+            stage[lane * (kFsCols + 1) + x] = f0;
+            stage[(lane + 32) * (kFsCols + 1) + x] = f1;
+            if (a.best_g && cap_s[g] > 0) {                                       // g ascends: the lower worker is kept on ties
+                const long long c0 = key_of_double(f0), c1 = key_of_double(f1);
+                if (c0 > k0) { k0 = c0; b0 = g; }
+                if (c1 > k1) { k1 = c1; b1 = g; }
+            }
         }
+        __syncwarp();
+        const int x = lane & (kFsCols - 1);
+        double *F = a.F + (inst * a.n_req + r0 + (lane >> 3)) * G + gc + x;
+        const double *from = stage + (lane >> 3) * (kFsCols + 1) + x;
+        if (x < cols) {
+#pragma unroll 4
+            for (int r = lane >> 3; r < cnt; r += 4) {
+                *F = *from;
+                F += 4 * G; from += 4 * (kFsCols + 1);
+            }
+        }
+        __syncwarp();
     }
     if (a.best_g) {
-        for (int i = tid; i < n; i += blockDim.x) {
-            long long bk = kNoKey; int bg = -1;
-            for (int g = 0; g < G; ++g) {
-                if (cap_s[g] <= 0) continue;
-                const long long key = fscore_key(a, s_tile[i], m_s + g * H1);
-                if (bg < 0 || key > bk) { bk = key; bg = g; }
+        if (split > 1) {
+            long long *ks = reinterpret_cast<long long *>(stage);
+            int *is = reinterpret_cast<int *>(stage + kFsReq);
+            ks[lane] = k0; ks[lane + 32] = k1; is[lane] = b0; is[lane + 32] = b1;
+            __syncthreads();
+            if (sub != 0) return;
+            for (int w = 1; w < split; ++w) {
+                const long long *kw = ks + w * kFsReq * (kFsCols + 1);
+                const int *iw = is + 2 * w * kFsReq * (kFsCols + 1);
+                if (kw[lane] > k0) { k0 = kw[lane]; b0 = iw[lane]; }
+                if (kw[lane + 32] > k1) { k1 = kw[lane + 32]; b1 = iw[lane + 32]; }
             }
-            a.best_g[inst * a.n_req + tile0 + i] = bg;
         }
+        int32_t *best = a.best_g + inst * a.n_req + r0;
+        if (lane < cnt) best[lane] = b0 == kNoIdx ? -1 : b0;
+        if (lane + 32 < cnt) best[lane + 32] = b1 == kNoIdx ? -1 : b1;
     }
 }
 
