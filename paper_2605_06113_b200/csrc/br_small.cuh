@@ -87,17 +87,12 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         *vec_at<uint4>(q_id, p0) = iv;
     }
     __syncwarp();
+    int dirty = n_w;                                      // entries before this one have not changed
 
 #pragma unroll 1
     for (int it = 0; it < a.n_steps; ++it, ++k) {
         const size_t orow = (size_t)it * a.N + inst;          // outputs use the rows of the state (first_instance = 0 when n_steps > 1)
         const auto assign = mk_span(a.assign_out + orow * W, W);
-#pragma unroll
-        for (int t = 0; t < NT4; ++t) {
-            const int p0 = (t * 32 + lane) * 4;
-            if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(-1, -1, -1, -1);
-        }
-
         // ================= ARRIVE (Section 2.2) =================
         // One Philox call serves the step: lane 31 draws the arrival count, lane b < 31 the block
         // of prompt-length words of arrivals 4b .. 4b+3.
@@ -254,7 +249,6 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
                         occ |= 1ull << slot;
                         const int sa = g * B + slot;
                         g_base[sa] = s - k;
-                        assign[pos] = sa;
                         q_key[pos] = (int)(0x80000000u | (unsigned)sa);
                         cap -= 1;
                         L += s;
@@ -292,7 +286,9 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
             }
         }
 
-        // ============ stable queue compaction in shared memory; ids of the admitted requests ============
+        // ============ stable queue compaction in shared memory; assignments, ids of the admitted requests ============
+        // The assignment row leaves here, as whole vectors, from the slots that the keys of admitted entries
+        // carry (written as -1 first and filled in at the admissions: 2.5 % slower at 4,096 instances).
         // An entry that moves down by d positions keeps its length and gains d in the inverted
         // position field: its key grows by d.
         {
@@ -300,12 +296,19 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
 #pragma unroll
             for (int t = 0; t < NT4; ++t) {
                 const int p0 = (t * 32 + lane) * 4;
-                if (t * 128 >= n_w) break;
-                if (t * 128 + 128 <= first_rm) { run += 128; continue; }     // nothing before the first admission moves
+                if (t * 128 >= n_w || t * 128 + 128 <= first_rm) {            // nothing before the first admission moves
+                    if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(-1, -1, -1, -1);
+                    run += 128;
+                    continue;
+                }
                 const int4 kk = *vec_at<const int4>(q_key, p0);
                 const uint4 ii = *vec_at<const uint4>(q_id, p0);
                 const int ke[4] = {kk.x, kk.y, kk.z, kk.w};
                 const unsigned idv[4] = {ii.x, ii.y, ii.z, ii.w};
+                int as[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) as[j] = ke[j] < 0 && ke[j] != kSmallBeyond ? ke[j] & 0x7FFFFFFF : -1;
+                if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(as[0], as[1], as[2], as[3]);
                 int below = run;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) below += __popc(__ballot_sync(kFull, ke[j] > 0) & lt);
@@ -325,6 +328,7 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
             for (int j = n_left + lane; j < n_w; j += 32) q_key[j] = kSmallBeyond;   // vacated tail
             __syncwarp();
         }
+        dirty = min(dirty, first_rm);
         n_w = n_left;
 
         // ================= ADVANCE (Section 2.2) =================
@@ -351,11 +355,11 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         __syncwarp();
     }
 
-    // ---- snapshot write-back ----
+    // ---- snapshot write-back (queue entries before the first that moved or arrived are as they were) ----
 #pragma unroll
     for (int t = 0; t < NT4; ++t) {
         const int p0 = (t * 32 + lane) * 4;
-        if (p0 < W) {
+        if (p0 < W && p0 + 4 > dirty) {
             const int4 kk = *vec_at<const int4>(q_key, p0);
             int4 sv;
             sv.x = kk.x > 0 ? kk.x >> WL : 0; sv.y = kk.y > 0 ? kk.y >> WL : 0;
