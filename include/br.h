@@ -187,12 +187,14 @@ int br_graph_step(br_ctx *ctx);
 
 /*
  * Host-buffer variant: every array pointer in worker_state, waiting_queue, term_probs,
- * assign_out and load_out is a HOST pointer (pinned memory gives asynchronous copies).
- * Copies the snapshot to device staging owned by ctx (grown on demand with cudaMalloc),
- * runs the step, copies state and results back and synchronises the stream.  Batches of 512
- * instances or more go through in chunks of instances on three internal streams (created on
- * first use), so that uploads, kernels and downloads of different chunks overlap.
- * h2d_bytes / d2h_bytes, if not NULL, receive the bytes moved in each direction.
+ * assign_out and load_out is a HOST pointer.  Runs the step on the snapshot in host memory and
+ * synchronises the stream.  Arrays in page-locked memory (aligned to 16 bytes) are read and written by the
+ * kernel in place where that is the faster way; the others go through device staging owned by ctx
+ * (grown on demand with cudaMalloc), in batches of 512 instances or more in chunks of instances on three
+ * internal streams (created on first use), so that uploads, kernels and downloads of different chunks
+ * overlap.  Until the call returns the host arrays must not be touched.
+ * h2d_bytes / d2h_bytes, if not NULL, receive the bytes of the arrays moved in each direction; arrays
+ * used in place of which only the slots that change are touched (act_id, act_base with H = 0) do not count.
  * batch.n_steps must be 1 and batch.first_instance 0.
  */
 int br_step_host(br_ctx *ctx, const br_instance_batch *batch, br_worker_state *worker_state,

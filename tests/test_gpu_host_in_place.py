@@ -1,0 +1,45 @@
+"""br_step_host on page-locked buffers, which the kernels use in place, on pageable ones, which are copied, and on a
+mixture: state and outputs equal those of br_step on device buffers."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_06113_b200 import workload as wlm
+from paper_2605_06113_b200.binding import Router
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,n_inst,kw", [("c3", 1, {}), ("c3", 63, {}), ("c3", 700, {}), ("c3", 540, dict(G=40, W=520)), ("c2", 3, {}),
+                                            ("c2", 520, {}), ("c3", 70, dict(term_mode=3)), ("h80", 63, {}), ("h80", 64, {})])
+@pytest.mark.parametrize("pinned", ["all", "some", "misaligned"])
+def test_in_place_matches_device_step(name, n_inst, kw, pinned):
+    cfg = wlm.get_config(name, **kw)
+    wl = wlm.make_workload(cfg, n_instances=n_inst)
+    r = Router(wl, device="cuda:0")
+
+    def host(key, v):
+        v = v.cpu()
+        if pinned == "some" and key in ("wq_s", "trace", "act_base"):
+            return v
+        if pinned == "misaligned" and key in ("wq_id", "load", "act_id"):
+            buf = torch.empty(v.numel() * v.element_size() + 8, dtype=torch.uint8).pin_memory()
+            w = buf[8:].view(v.dtype).view(v.shape)
+            w.copy_(v)
+            return w
+        return v.pin_memory()
+
+    st_d, out_d = r.device_state(), r.outputs(n_inst)
+    st_h = {k: host(k, v) for k, v in st_d.items()}
+    out_h = {k: host(k, v) for k, v in out_d.items()}
+    for k in range(3):
+        probs = torch.from_numpy(np.ascontiguousarray(wlm.term_probs_np(wl, k))) if cfg.H > 0 and cfg.pred_mode == 0 else None
+        r.step_host(st_h, out_h, None if probs is None else host("probs", probs))
+        r.step(st_d, out_d, None if probs is None else probs.cuda())
+        torch.cuda.synchronize()
+        for a, b in ((out_h, out_d), (st_h, st_d)):
+            for key in a:
+                if cfg.pred_mode == 1 and key in ("act_chat0", "act_kref"):
+                    continue                      # not part of a snapshot with known lifetimes: the host step leaves them alone
+                assert torch.equal(a[key], b[key].cpu()), (k, key)
+    r.close()
