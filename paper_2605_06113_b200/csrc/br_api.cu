@@ -68,17 +68,22 @@ inline bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintp
 
 typedef void (*step_kernel_t)(const StepArgs);
 
-template <bool FP, int HC>
+template <bool FP, int NC>
 step_kernel_t pick_kernel_gw(int G)
 {
-    return G <= 32 ? br::br_step_kernel<FP, 1, HC> : br::br_step_kernel<FP, 2, HC>;
+    return G <= 32 ? br::br_step_kernel<FP, 1, NC> : br::br_step_kernel<FP, 2, NC>;
 }
 
-// Eq. 1 or Eq. 2; one or two workers per router lane; up to 31 or up to 95 horizon offsets
+// Eq. 1 or Eq. 2; one or two workers per router lane; horizon offsets unrolled in groups of four or not at all
 step_kernel_t pick_kernel(bool fp, int H, int G)
 {
-    if (!fp) return pick_kernel_gw<false, 1>(G);
-    return H < 32 ? pick_kernel_gw<true, 1>(G) : pick_kernel_gw<true, 3>(G);
+    if (!fp) return pick_kernel_gw<false, 2>(G);
+    switch (br::step_groups(H)) {
+    case 2: return pick_kernel_gw<true, 2>(G);
+    case 3: return pick_kernel_gw<true, 3>(G);
+    case 5: return pick_kernel_gw<true, 5>(G);
+    default: return pick_kernel_gw<true, 0>(G);
+    }
 }
 
 constexpr int kSMs = 148;
@@ -99,7 +104,7 @@ int threads_for(const br_ctx *ctx, int n_instances)
     int per_sm = (n_instances + kSMs - 1) / kSMs;
     const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
     if (per_sm > fit) per_sm = fit;
-    int w = (ctx->H < 32 ? 28 : 20) / per_sm;
+    int w = (br::step_groups(ctx->H) ? 28 : 20) / per_sm;
     w = w < 1 ? 1 : (w > most ? most : w);
     return 32 * w;
 }
@@ -291,7 +296,9 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
     a.burst_every = p.burst_every; a.burst_size = p.burst_size;
     // d = (1, gamma, ..., gamma^H) by repeated multiplication; D = 1^T d left to right
     volatile double D = 0.0;
-    for (int h = 0; h < BR_MAX_H + 4; ++h) { a.dn[2 * h] = 0.0; a.dn[2 * h + 1] = 0.0; }
+    for (int h = 0; h < BR_MAX_H + 8; ++h) { a.dn[2 * h] = 0.0; a.dn[2 * h + 1] = 0.0; a.iw[h] = 0; }
+    a.lpw_log2 = 0;
+    while (G << (a.lpw_log2 + 1) <= 32) ++a.lpw_log2;
     for (int h = 0; h <= BR_MAX_H; ++h) ctx->d[h] = 0.0;
     if (p.score_mode == 1) {
         for (int h = 0; h <= H; ++h) {
@@ -307,9 +314,23 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
         // lengths are strictly ordered on both sides of the peak.  The kernel checks the slopes of the
         // kinks at hand (P: the offsets whose kink is passed) against this bound; the slope before the
         // first kink is alpha D.
-        const double err = 4.0 * (H + 5) * 1.1102230246251565e-16 * (a.aD + p.beta * D) * (double)p.s_max;
-        a.slope_err = err > 1e-9 ? err : 1e-9;
-        if (!(a.aD > a.slope_err)) a.slope_err = INFINITY;                     // never ordered: every request is scored
+        a.rel_err = 4.0 * (H + 5) * 1.1102230246251565e-16 * (a.aD + p.beta * D);
+        const double err = a.rel_err * (double)p.s_max;
+        const double slope_err = err > 1e-9 ? err : 1e-9;
+        // The weights in fixed point: iw_h = floor(scale d_h), so that a sum of up to H + 1 of them is below
+        // scale * sum d_h by less than H + 1.  A segment rises clearly while alpha D - beta sum d_h > slope_err.
+        const double scale = 2147483000.0 / D, most = 2147483640.0;
+        for (int h = 0; h <= H; ++h) a.iw[h] = (int32_t)floor(scale * ctx->d[h]);
+        a.w_below = -1; a.w_above = 2147483647;                        // never ordered: every request is scored
+        if (a.aD > slope_err) {
+            double lo = most, hi = most;                               // beta = 0: rises throughout
+            if (p.beta > 0.0) {
+                lo = floor(scale * ((a.aD - slope_err) / p.beta)) - (H + 4);
+                hi = ceil(scale * ((a.aD + slope_err) / p.beta)) + 2.0;
+            }
+            a.w_below = (int32_t)(lo < -1.0 ? -1.0 : (lo > most ? most : lo));
+            a.w_above = (int32_t)(hi > most ? most : hi);
+        }
         // Subsets of up to 32 requests (Delta <= 32 s_max): the two-probe rule of the large-window solvers
         // asks the same of all 2^(H+1) sets P, enumerated here for H <= 16.
         if (H <= 16) {

@@ -11,14 +11,15 @@
 // The admission loop is bound by instruction latency and instruction fetch: a pop is one chain of
 // dependent warp instructions (measured: warp maximum 22 cycles, warp sum 47, shuffle or ballot 25 to
 // 35, shared-memory load 34, fp64 operation 8), and a loop body of more than a few hundred
-// instructions is fetched again on every pop.  So it is written to be short: one loop for both
-// stages; the projected loads L_g(k+h) in shared memory, with the lanes spread over h for margins,
-// envelope and admission; one lane per worker only for the three selection keys (free slots, L_g(k),
-// min_h m_{g,h}); all requests of a chosen subset admitted at once, one lane each; slots, snapshot
-// edits and rare branches outside the loop.  Against one copy of every part per stage, with the
-// horizon in registers and loops over h unrolled, 1,024 instances of G = 64, W = 1,024, H = 8 went
-// from 112 to 83 us a step, 777 of G = 21, W = 300, H = 6 from 630 to 295 us per three steps, 1,024 of
-// G = 8, W = 512, H = 80 from 503 to 164 us per eight.
+// instructions is fetched again on every pop.  So it is written to be short and straight: one loop for
+// both stages; the margins m_{g,h} in shared memory, a row per worker, with the lanes spread over h;
+// one lane per worker for the three selection keys (free slots, L_g(k), min_h m_{g,h}); the Stage-2
+// window in registers of every lane, refilled by one warp maximum per admission; loops over h unrolled
+// for H < 20; slots, snapshot edits and rare branches outside the loop.  us per call at G = 64,
+// W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
+// 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
+// unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
+// the lanes' lists at every pop, 74 / 273 / 161 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -33,7 +34,7 @@ namespace br {
 
 // Shared memory of one instance: byte offsets, filled in by the host.
 struct StepLayout {
-    int32_t q_key, q_id, q_o, Lh, Ch, dn, Ms, md, occ, occ0, fin, endm, L0, cap, sub, scal, bw, due, total;
+    int32_t q_key, q_id, q_o, Lh, Ch, dn, iw, Ms, occ, occ0, fin, endm, L0, cap, sub, scal, bw, due, total;
 };
 
 struct StepArgs {
@@ -41,6 +42,7 @@ struct StepArgs {
     int32_t wl;                 // log2 of the queue-position field of a packed key
     int32_t Wp;                 // W rounded up to whole groups of 128 queue positions
     int32_t HS;                 // row stride of L_g(k+h) in shared memory (>= H + 1)
+    int32_t lpw_log2;           // log2 of the lanes that share a worker's row (fleets of up to 16 workers, long horizons)
     int32_t seg_log2;           // lanes per worker that turn its prediction buckets into L_g(k+h)
     int32_t delta_T;
     float gate, c_floor;
@@ -55,10 +57,12 @@ struct StepArgs {
     int32_t len_shift;
     int32_t burst_every, burst_size;
     double aD, beta;
-    double slope_err;           // Eq. 2: a segment slope within this of zero makes fp64 scores of integer lengths unordered
+    double rel_err;             // Eq. 2: bound on the rounding error of a score, per unit of Delta
+    int32_t w_below, w_above;   // Eq. 2: fixed-point weight sums up to / from which a segment clearly rises / falls
     int32_t peak_ok;            // Eq. 1: scores fall strictly beyond the margin (G >= 2)
     int32_t big_window;         // R_max > 5: Stage 2 solves its window by meeting in the middle
-    double dn[2 * (BR_MAX_H + 4)];   // (d_h, -2^52 d_h), zero beyond H
+    double dn[2 * (BR_MAX_H + 8)];   // (d_h, -2^52 d_h), zero beyond H
+    int32_t iw[BR_MAX_H + 8];        // d_h in fixed point (their sum stays below 2^31)
     int32_t N, first_instance, n_steps;
     StepLayout lay;
     br_worker_state ws;
@@ -68,13 +72,16 @@ struct StepArgs {
     br_load_out out;
 };
 
-// L_g(k+h) rows are read by lanes that own a worker each (16-byte loads at stride HS) and by lanes
-// that own an offset each (consecutive words): an odd number of 16-byte units keeps both free of
+// Groups of four horizon offsets (h = 0 .. H) that a kernel unrolls: 2, 3 or 5, so that the loops over h
+// of the admission loop are straight code; 0: a longer horizon, three offsets per lane, plain loops.
+__host__ __device__ constexpr int step_groups(int H) { return H < 8 ? 2 : (H < 12 ? 3 : (H < 20 ? 5 : 0)); }
+
+// Rows of L_g(k+h) are read by lanes that own a worker each (16-byte loads at the row stride) and by
+// lanes that own an offset each (consecutive words): an odd number of 16-byte units keeps both free of
 // bank conflicts.
-__host__ __device__ inline int step_row_stride(int H)
+__host__ __device__ constexpr int step_row_stride(int H)
 {
-    int u = (H + 1 + 3) / 4;
-    return 4 * (u | 1);
+    return 4 * ((step_groups(H) ? step_groups(H) : (H + 4) / 4) | 1);
 }
 
 inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool lifetimes, bool big_window, bool classifier)
@@ -86,11 +93,11 @@ inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool li
     l.q_key = take(4 * Wp);
     l.q_id = take(4 * Wp);
     l.q_o = take(lifetimes ? 4 * Wp : 0);
-    l.Lh = take(4 * G * HS);                    // PREDICT: load sums per (worker, floor(c_hat)); then L_g(k+h)
+    l.Lh = take(4 * (G * HS + 4));              // PREDICT: load sums per (worker, floor(c_hat)); L_g(k+h); margins m_{g,h}
     l.Ch = take(H > 0 ? 4 * G * HS : 0);        // PREDICT: request counts
-    l.dn = take(16 * HS);                       // (d_h, -2^52 d_h)
-    l.Ms = take(4 * HS);                        // envelope M_h
-    l.md = take(4 * HS);                        // margins of the selected worker
+    l.dn = take(16 * (HS + 4));                 // (d_h, -2^52 d_h)
+    l.iw = take(4 * (HS + 4));                  // d_h in fixed point
+    l.Ms = take(4 * HS);                        // envelope M_h; then its growth by an admission
     l.occ = take(words);                        // occupied slots
     l.occ0 = take(words);                       // ... at the start of the step
     l.fin = take(words);                        // constant hazard: slots whose draw says "ends"
@@ -115,7 +122,7 @@ inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool li
 // two fp64 instructions per term instead of five.
 template <bool FP>
 struct Scorer {
-    span_t<int> md;         // Eq. 2: margins m_{g,h} of the selected worker (INT_MAX beyond H)
+    span_t<int> md;         // Eq. 2: row of margins m_{g,h} of the selected worker (INT_MAX beyond H)
     span_t<double> dn;      // (d_h, -2^52 d_h) pairs
     int mm;                 // min_h m_{g,h} (Eq. 1: the margin); at or below it no term is positive
     int H, G;
@@ -238,6 +245,13 @@ __device__ __forceinline__ void row_sum(const float *q, int H, bool rows32, floa
 
 constexpr int kRegWin = 5;       // Stage-2 windows of up to five requests are scored one subset per lane
 constexpr int kBigWinLow = 8;    // larger windows (up to BR_MAX_RMAX = 16): subsets of the low eight entries are sorted
+// marks a condition as the exception, so that its block leaves the straight path of the admission loop
+__device__ __forceinline__ bool rare(bool x) { return __builtin_expect(x, 0); }
+
+// descending order of two keys
+__device__ __forceinline__ void order2(int &a, int &b) { const int hi = max(a, b); b = min(a, b); a = hi; }
+
+constexpr int kListEnd = 0x7FFFFFFF;         // head of a lane's list that ran dry although the lane may hold more keys
 constexpr int kQBeyond = (int)0x8000FFFFu;   // key of a position beyond the queue (no slot index reaches 0xFFFF)
 
 // The rarely taken branches of the router live in functions of their own: inlined, they would spread
@@ -369,15 +383,17 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
         F[(size_t)i * G] = i < n_w ? Scorer<FP>::value(sc.key(q_key[i] >> WL)) : 0.0;
 }
 
-// FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  HC: horizon offsets per lane (H < 32 HC).
-template <bool FP, int GW, int HC>
-__global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_constant__ StepArgs a)
+// FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  NC: step_groups(H).
+template <bool FP, int GW, int NC>
+__global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_constant__ StepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
     stream_order_gate();
     const int G = a.G, H = FP ? a.H : 0, B = a.B, W = a.W, A = G * B, OW = a.occ_words, WL = a.wl;
-    const int H1 = H + 1, HS = a.HS;
+    const int H1 = H + 1, HS = NC > 0 ? 4 * (NC | 1) : a.HS;
+    constexpr int HC = NC > 0 ? 1 : 3;                // horizon offsets per lane
+    constexpr int HT = 4 * NC;                        // offsets of the unrolled loops
     const unsigned posmask = (1u << WL) - 1u;
     const int inst = a.first_instance + blockIdx.x;
     const bool life = a.term_mode == 3;               // requests carry their output lengths
@@ -388,11 +404,11 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
     const auto q_key = mk_span(reinterpret_cast<int *>(smem + a.lay.q_key), a.Wp);
     const auto q_id = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.q_id), a.Wp);
     const auto q_o = mk_span(reinterpret_cast<int *>(smem + a.lay.q_o), life ? a.Wp : 0);
-    const auto Lh = mk_span(reinterpret_cast<int *>(smem + a.lay.Lh), G * HS);
+    const auto Lh = mk_span(reinterpret_cast<int *>(smem + a.lay.Lh), G * HS + 4);
     const auto Ch = mk_span(reinterpret_cast<int *>(smem + a.lay.Ch), H > 0 ? G * HS : 0);
-    const auto dn_s = mk_span(reinterpret_cast<double *>(smem + a.lay.dn), FP ? 2 * HS : 0);
+    const auto dn_s = mk_span(reinterpret_cast<double *>(smem + a.lay.dn), FP ? 2 * (HS + 4) : 0);
+    const auto iw_s = mk_span(reinterpret_cast<int *>(smem + a.lay.iw), FP ? HS + 4 : 0);
     const auto Ms = mk_span(reinterpret_cast<int *>(smem + a.lay.Ms), HS);
-    const auto md = mk_span(reinterpret_cast<int *>(smem + a.lay.md), HS);
     const auto occ = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ), G * OW);
     const auto occ0 = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ0), G * OW);
     const auto occ032 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.occ0), 2 * G * OW);
@@ -473,7 +489,11 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
 #pragma unroll 1
         for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
 #pragma unroll 1
-        for (int h = tid; h < HS; h += NT) { Ms[h] = h < H1 ? 0 : 0x7FFFFFFF; md[h] = 0x7FFFFFFF; dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1]; }
+        for (int h = tid; h < HS + 4; h += NT) {
+            dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1];
+            iw_s[h] = a.iw[h];
+            if (h < HS) Ms[h] = h < H1 ? 0 : 0x7FFFFFFF;
+        }
     }
     __syncthreads();
     if (bad) atomicOr(&scal[5], bad);
@@ -504,67 +524,87 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
 
         // ============ PREDICT (H > 0): c_hat maintenance + horizon projection ============
         // Every running request adds (cur, 1) to the bucket (worker, floor(c_hat)); the buckets become
-        // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  A thread takes eight slots
-        // of one worker at a time and consecutive threads take different workers, so that the
-        // atomics of a warp fall on different rows.
+        // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  Consecutive threads take
+        // consecutive slot quads: the loads have to be coalesced.  (Eight slots of one worker per thread and
+        // consecutive workers in consecutive threads keep the atomics of a warp on different rows but touch
+        // 32 lines with every load: 82 us a step against 77 at G = 64, H = 8, 1,024 instances.)  The next quad is
+        // requested before this one is worked on.
         if (FP && H > 0) {
-            const unsigned A8 = (unsigned)A >> 3;
+            const int A4 = A >> 2, B4 = B >> 2;
+            const bool look = a.pred_mode == 1;
+            int4 b4, x4 = make_int4(0, 0, 0, 0);                              // act_base; act_end or chat0
+            unsigned kr = 0u;                                                 // refresh stamps
+            auto fetch = [&](int q) {
+                b4 = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
+                if (q < A4) {
+                    b4 = *vec_at<const int4>(g_base, 4 * q);
+                    if (look) {
+                        x4 = *vec_at<const int4>(g_end, 4 * q);
+                    } else {
+                        x4 = *vec_at<const int4>(g_chat0, 4 * q);
+                        kr = *vec_at<const unsigned>(g_kref, 4 * q);
+                    }
+                }
+            };
+            fetch(tid);
 #pragma unroll 1
-            for (unsigned o = tid; o < A8; o += NT) {
-                const int p = (int)(o / (unsigned)G), g = (int)o - p * G, a0 = g * B + 8 * p;
-                const int4 b0 = *vec_at<const int4>(g_base, a0), b1 = *vec_at<const int4>(g_base, a0 + 4);
-                const int bs[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-                if (a.pred_mode == 1) {
+            for (int q0 = 0; q0 < A4; q0 += NT) {
+                const int q = q0 + tid, g = (int)((unsigned)q / (unsigned)B4);
+                const int bs[4] = {b4.x, b4.y, b4.z, b4.w}, xs[4] = {x4.x, x4.y, x4.z, x4.w};
+                const unsigned k4 = kr;
+                fetch(q + NT);
+                if (look) {
                     // perfect lookahead: c_hat = min(r_i(k), H) with r_i(k) = act_end - k + 1 steps still to run.
                     // A request whose last step this is (act_end == k) is settled right here.
-                    const int4 e0 = *vec_at<const int4>(g_end, a0), e1 = *vec_at<const int4>(g_end, a0 + 4);
-                    const int en[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
                     unsigned fb = 0u;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
+                    for (int j = 0; j < 4; ++j) {
                         if (bs[j] != kEmpty) {
-                            const int nh = min(max(en[j] - k + 1, 0), H);
+                            const int nh = min(max(xs[j] - k + 1, 0), H);
                             const unsigned cur = (unsigned)(bs[j] + k);
                             atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur);
                             atomicAdd(&Ch[g * HS + nh], 1);
-                            if (en[j] == k) { fb |= 1u << j; atomicAdd(&sub_load[g], cur); g_base[a0 + j] = kEmpty; }
+                            if (xs[j] == k) { fb |= 1u << j; atomicAdd(&sub_load[g], cur); g_base[4 * q + j] = kEmpty; }
                         }
                     }
-                    endm8[g * OW * 8 + p] = (unsigned char)fb;
+                    const int slot = 4 * (q - g * B4);
+                    if (fb) atomicOr(&endm32[2 * g * OW + (slot >> 5)], fb << (slot & 31));
                 } else {
                     // requests that are not due only age; the ones due for a refresh take c_hat = H (gate closed:
                     // the conservative anchor) and go on a list, whose rows are read below
-                    const float4 c0 = *vec_at<const float4>(g_chat0, a0), c1 = *vec_at<const float4>(g_chat0, a0 + 4);
-                    float cs[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-                    unsigned kr[2] = {*vec_at<const unsigned>(g_kref, a0), *vec_at<const unsigned>(g_kref, a0 + 4)};
-                    unsigned due = 0u;
+                    unsigned dm[4], kn = k4;
+                    int cs[4], n_due = 0;
+                    bool due[4];
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (bs[j] != kEmpty) {
-                            const unsigned sh = 8 * (j & 3);
-                            const int t = (k - (int)((kr[j >> 2] >> sh) & 0xFFu)) & 255;
-                            const float c = cs[j] - (float)t;
-                            const bool d = t >= a.delta_T || c < a.c_floor;
-                            int nh = H;
-                            if (d) {
-                                due |= 1u << j;
-                                cs[j] = (float)H;
-                                kr[j >> 2] = (kr[j >> 2] & ~(0xFFu << sh)) | ((unsigned)(k & 255) << sh);
-                            } else {
-                                nh = (int)floorf(c);
-                                nh = nh < 0 ? 0 : (nh > H ? H : nh);
-                            }
+                    for (int j = 0; j < 4; ++j) {
+                        const int t = (k - (int)((k4 >> (8 * j)) & 0xFFu)) & 255;
+                        const float c = __int_as_float(xs[j]) - (float)t;
+                        const bool live = bs[j] != kEmpty;
+                        due[j] = live && (t >= a.delta_T || c < a.c_floor);
+                        dm[j] = __ballot_sync(kFull, due[j]);
+                        n_due += __popc(dm[j]);
+                        cs[j] = due[j] ? __float_as_int((float)H) : xs[j];
+                        int nh = H;
+                        if (due[j]) kn = (kn & ~(0xFFu << (8 * j))) | ((unsigned)(k & 255) << (8 * j));
+                        else nh = min(max((int)floorf(c), 0), H);
+                        if (live) {
                             atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), (unsigned)(bs[j] + k));
                             atomicAdd(&Ch[g * HS + nh], 1);
                         }
                     }
-                    if (due) {
-                        if (due & 0x0Fu) { *vec_at<float4>(g_chat0, a0) = make_float4(cs[0], cs[1], cs[2], cs[3]); *vec_at<unsigned>(g_kref, a0) = kr[0]; }
-                        if (due & 0xF0u) { *vec_at<float4>(g_chat0, a0 + 4) = make_float4(cs[4], cs[5], cs[6], cs[7]); *vec_at<unsigned>(g_kref, a0 + 4) = kr[1]; }
-                        int at = atomicAdd(&scal[8], __popc(due));
-                        while (due) {
-                            due_list[at++] = (unsigned short)(a0 + __ffs(due) - 1);
-                            due &= due - 1u;
+                    if (n_due) {                                              // uniform over the warp
+                        int at = 0;
+                        if (lane == 0) at = atomicAdd(&scal[8], n_due);
+                        at = __shfl_sync(kFull, at, 0);
+                        const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            if (due[j]) due_list[at + __popc(dm[j] & lt)] = (unsigned short)(4 * q + j);
+                            at += __popc(dm[j]);
+                        }
+                        if (due[0] || due[1] || due[2] || due[3]) {
+                            *vec_at<int4>(g_chat0, 4 * q) = make_int4(cs[0], cs[1], cs[2], cs[3]);
+                            *vec_at<unsigned>(g_kref, 4 * q) = kn;
                         }
                     }
                 }
@@ -752,8 +792,11 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
 
         if (warp == 0) {
             // ================= ROUTE (warp 0 only, warp-synchronous) =================
-            // lane owns workers lane and lane + 32 (selection keys) and offsets lane, lane + 32, ... (envelope)
-            int cap[GW], L0[GW], mm[GW], M[HC];
+            // lane owns workers lane and lane + 32: the selection keys free slots, L_g(k) and min_h m_{g,h}.
+            // Eq. 2 keeps the margins m_{g,h} = M_h - L_g(k+h) themselves in shared memory, a row per worker: an
+            // admission takes Delta from one row, and only one beyond the worker's smallest margin lifts the
+            // envelope, and with it every row.
+            int cap[GW], L0[GW], mm[GW];
 #pragma unroll
             for (int w = 0; w < GW; ++w) {
                 const int g = lane + 32 * w;
@@ -761,74 +804,122 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
                 L0[w] = g < G ? (FP ? Lh[g * HS] : L0_s[g]) : 0;
                 mm[w] = 0;
             }
-#pragma unroll
-            for (int c = 0; c < HC; ++c) M[c] = FP ? (lane + 32 * c < HS ? Ms[lane + 32 * c] : 0x7FFFFFFF) : 0;
-            int M0 = 0;                                                     // Eq. 1: envelope
-            if (!FP) {
-                int v = L0[0];
-#pragma unroll
-                for (int w = 1; w < GW; ++w) v = max(v, L0[w]);
-                M0 = __reduce_max_sync(kFull, v);
-#pragma unroll
-                for (int w = 0; w < GW; ++w) mm[w] = M0 - L0[w];
-            }
-            // horizon-min margins min_h (M_h - L_g(k+h)) of all workers, from shared memory
-            auto margins_min = [&]() {
-                if (HC > 1 && G <= 16) {
-#pragma unroll 1
-                    for (int g = 0; g < G; ++g) {
-                        int v = 0x7FFFFFFF;
-#pragma unroll
-                        for (int c = 0; c < HC; ++c)
-                            if (lane + 32 * c < H1) v = min(v, M[c] - Lh[g * HS + lane + 32 * c]);
-                        v = __reduce_min_sync(kFull, v);
-                        if (lane == g) mm[0] = v;
+            // rows of all workers: Ms - row (FIRST: loads become margins) or Ms + row (the envelope grew by Ms), and
+            // their minima
+            auto rows = [&](const bool first) {
+                if (NC == 0 && G <= 16) {
+                    // long rows, few workers: 32 / G lanes share a row
+                    const int q = a.lpw_log2, g = lane >> q;
+                    int x = 0x7FFFFFFF;
+                    if (g < G) {
+#pragma unroll 2
+                        for (int h = 4 * (lane & ((1 << q) - 1)); h < H1; h += 4 << q) {
+                            const int4 e = *vec_at<const int4>(Ms, h);
+                            int4 l = *vec_at<const int4>(Lh, g * HS + h);
+                            if (first) { l.x = -l.x; l.y = -l.y; l.z = -l.z; l.w = -l.w; }
+                            l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
+                            *vec_at<int4>(Lh, g * HS + h) = l;
+                            x = min(min(x, l.x), min(min(l.y, l.z), l.w));
+                        }
                     }
+#pragma unroll 1
+                    for (int o = 1; o < (1 << q); o <<= 1) x = min(x, __shfl_xor_sync(kFull, x, o));
+                    mm[0] = __shfl_sync(kFull, x, (lane << q) & 31);
                 } else {
 #pragma unroll
                     for (int w = 0; w < GW; ++w) {
                         const int g = lane + 32 * w;
+                        int x = 0x7FFFFFFF;
                         if (g < G) {
-                            int v = 0x7FFFFFFF;
-#pragma unroll 1
-                            for (int h = 0; h < H1; h += 4) {
-                                const int4 x = *vec_at<const int4>(Ms, h), y = *vec_at<const int4>(Lh, g * HS + h);
-                                v = min(min(min(v, x.x - y.x), min(x.y - y.y, x.z - y.z)), x.w - y.w);
+#pragma unroll
+                            for (int h = 0; h < (NC > 0 ? HT : H1); h += 4) {
+                                const int4 e = *vec_at<const int4>(Ms, h);
+                                int4 l = *vec_at<const int4>(Lh, g * HS + h);
+                                if (first) { l.x = -l.x; l.y = -l.y; l.z = -l.z; l.w = -l.w; }
+                                l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
+                                *vec_at<int4>(Lh, g * HS + h) = l;
+                                x = min(min(x, l.x), min(min(l.y, l.z), l.w));
                             }
-                            mm[w] = v;
                         }
+                        mm[w] = x;
                     }
                 }
+                __syncwarp();
             };
-            bool stale = FP;                                                // mm has to be rebuilt (the envelope grew)
+            if (FP) {
+                rows(true);
+#pragma unroll
+                for (int c = 0; c < HC; ++c) if (lane + 32 * c < HS) Ms[lane + 32 * c] = 0;
+            } else {
+                int v = L0[0];
+#pragma unroll
+                for (int w = 1; w < GW; ++w) v = max(v, L0[w]);
+                const int M0 = __reduce_max_sync(kFull, v);
+#pragma unroll
+                for (int w = 0; w < GW; ++w) mm[w] = M0 - L0[w];
+            }
 
             Scorer<FP> sc;
-            sc.md = md; sc.dn = dn_s; sc.H = H; sc.G = G; sc.aD = a.aD; sc.beta = a.beta;
-            int m[HC], v[HC];                                               // margins and loads of the selected worker, by offset
-            auto load_margins = [&](int g) {
-                if (FP) {
+            sc.md = Lh; sc.dn = dn_s; sc.H = H; sc.G = G; sc.aD = a.aD; sc.beta = a.beta; sc.mm = 0;
+            // the score at the sites of the loop: unrolled for short horizons, else the next four offsets are read while
+            // these are added
+            auto hot_key = [&](int delta) -> long long {
+                if (!FP) return sc.key(delta);
+                double pen = 0.0;
+                if (NC > 0) {
+                    int4 q[NC > 0 ? NC : 1];
 #pragma unroll
-                    for (int c = 0; c < HC; ++c) {
-                        const int h = lane + 32 * c;
-                        v[c] = h < H1 ? Lh[g * HS + h] : 0;
-                        m[c] = M[c] - v[c];
-                        if (h < HS) md[h] = m[c];
+                    for (int c = 0; c < NC; ++c) q[c] = *vec_at<const int4>(sc.md, 4 * c);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const int mj[4] = {q[c].x, q[c].y, q[c].z, q[c].w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            pen = __dadd_rn(pen, __fma_rn(__hiloint2double(0x43300000, max(delta - mj[j], 0)), a.dn[2 * (4 * c + j)], a.dn[2 * (4 * c + j) + 1]));
                     }
-                    __syncwarp();
+                } else {
+                    int4 q = *vec_at<const int4>(sc.md, 0);
+                    double2 d[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) d[j] = *vec_at<const double2>(dn_s, 2 * j);
+#pragma unroll 2
+                    for (int h = 0; h <= H; h += 4) {
+                        const int mj[4] = {q.x, q.y, q.z, q.w};
+                        const double2 e[4] = {d[0], d[1], d[2], d[3]};
+                        q = *vec_at<const int4>(sc.md, h + 4);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) d[j] = *vec_at<const double2>(dn_s, 2 * (h + 4 + j));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            pen = __dadd_rn(pen, __fma_rn(__hiloint2double(0x43300000, max(delta - mj[j], 0)), e[j].x, e[j].y));
+                    }
                 }
+                const double dl = __dsub_rn(__hiloint2double(0x43300000, delta), 4503599627370496.0);
+                return key_of_double(__dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)));
+            };
+            // Eq. 2 with the terms summed across the lanes: off the exact score by at most rel_err * delta
+            int m[HC];                                                      // margins of the selected worker, by offset
+            auto near_score = [&](int delta) -> double {
+                double p = 0.0;
+#pragma unroll
+                for (int c = 0; c < HC; ++c) {
+                    const double x = __dsub_rn(__hiloint2double(0x43300000, max(delta - m[c], 0)), 4503599627370496.0);
+                    p = __fma_rn(x, lane + 32 * c < H1 ? dn_s[2 * (lane + 32 * c)] : 0.0, p);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) p = __dadd_rn(p, __shfl_xor_sync(kFull, p, o));
+                return __fma_rn(a.aD, (double)delta, -__dmul_rn(a.beta, p));
             };
 
             // optional F-score matrix before the first admission
-            if (a.out.fscore) {
-                if (FP) { margins_min(); stale = false; }
+            if (rare(a.out.fscore != nullptr)) {
                 double *F = a.out.fscore + orow * (size_t)W * G;
 #pragma unroll 1
                 for (int g = 0; g < G; ++g) {
                     const int own = (GW > 1 && g >= 32) ? mm[GW - 1] : mm[0];
                     sc.mm = __shfl_sync(kFull, own, g & 31);
-                    load_margins(g);
+                    if (FP) sc.md = Lh + g * HS;
                     score_column<FP>(sc, F + g, q_key, n_w, W, G, WL, lane);
-                    __syncwarp();
                 }
             }
 
@@ -836,41 +927,44 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
 #pragma unroll
             for (int w = 0; w < GW; ++w) S_tot += cap[w] > 0 ? cap[w] : 0;
             S_tot = (int)__reduce_add_sync(kFull, (unsigned)S_tot);
-            int n_left = n_w, s1_iters = 0, s2_pops = 0, status = 0, first_rm = W;   // first_rm: per lane, reduced at the end
+            int n_left = n_w, s1_iters = 0, s2_pops = 0, status = 0, first_rm = W;
             const int n_groups = (n_w + 127) >> 7;
-            // Stage-2 window: each lane keeps its four largest waiting keys, sorted, across the pops of the
-            // step; a lane whose list runs dry although it may hold more keys forces a rebuild
-            int t0 = 0, t1 = 0, t2 = 0, t3 = 0;
-            bool listed = false, full = false, merged = false;
-            int wkey = 0, wdelta = 0, nwin = 0;          // lane r: r-th largest key; lane mask: sum of its subset
+            // Stage-2 window: the R_max largest waiting keys, in registers of every lane, kept across the pops of
+            // the step.  The largest of the rest are in lists of four per lane, sorted; an admitted entry is
+            // replaced by the largest head.  A lane whose list runs dry although it may hold more keys shows kListEnd,
+            // and when that is the largest head everything is built anew.
+            int win[kRegWin], t0 = 0, t1 = 0, t2 = 0, t3 = 0, t_end = 0;
+#pragma unroll
+            for (int r = 0; r < kRegWin; ++r) win[r] = 0;
+            bool valid = false;
             bool to_stage2 = true;
 
 #pragma unroll 1
             while (n_left > 0 && S_tot > 0) {
                 const bool st1 = S_tot > a.S_greedy;
-                if (FP && stale) { margins_min(); stale = false; }
-                if (!st1 && to_stage2) { to_stage2 = false; if (timing) t_phase[3] = (unsigned)clock64(); }
-                if (st1 ? s1_iters >= W : s2_pops >= W + G) { status |= BR_ST_ITER_CAP; break; }
+                if (rare(!st1 && timing && to_stage2)) { to_stage2 = false; t_phase[3] = (unsigned)clock64(); }
+                if (rare(st1 ? s1_iters >= W : s2_pops >= W + G)) { status |= BR_ST_ITER_CAP; break; }
                 // most free slots; then Stage 1: smallest L_g(k), Stage 2: largest horizon-min margin; lowest g
                 int bc = cap[0];
 #pragma unroll
                 for (int w = 1; w < GW; ++w) bc = max(bc, cap[w]);
                 const int mc = __reduce_max_sync(kFull, bc);
-                if (mc <= 0) break;
+                if (rare(mc <= 0)) break;
                 int bv = kEmpty;
 #pragma unroll
-                for (int w = 0; w < GW; ++w) if (cap[w] == mc) bv = max(bv, st1 ? ~L0[w] : mm[w]);
+                for (int w = 0; w < GW; ++w) bv = max(bv, cap[w] == mc ? (st1 ? ~L0[w] : mm[w]) : kEmpty);
                 const int mv = __reduce_max_sync(kFull, bv);
                 int gi = 0xFF;
 #pragma unroll
-                for (int w = GW - 1; w >= 0; --w) if (cap[w] == mc && (st1 ? ~L0[w] : mm[w]) == mv) gi = lane + 32 * w;
+                for (int w = GW - 1; w >= 0; --w) gi = cap[w] == mc && (st1 ? ~L0[w] : mm[w]) == mv ? lane + 32 * w : gi;
                 const int g = (int)__reduce_min_sync(kFull, (unsigned)gi);
-                const int src = g & 31;
-                sc.mm = st1 ? __shfl_sync(kFull, (GW > 1 && g >= 32) ? mm[GW - 1] : mm[0], src) : mv;
-                load_margins(g);
+                sc.mm = st1 ? __shfl_sync(kFull, (GW > 1 && g >= 32) ? mm[GW - 1] : mm[0], g & 31) : mv;
+                if (FP) sc.md = Lh + g * HS;
+#pragma unroll
+                for (int c = 0; c < HC; ++c) m[c] = FP ? (lane + 32 * c < HS ? Lh[g * HS + lane + 32 * c] : 0x7FFFFFFF) : sc.mm;
 
-                unsigned chosen = 1u;                    // window entries to admit (bit r: lane r holds the key)
-                int dsum = 0;
+                unsigned chosen = 1u;                    // window entries to admit
+                int dsum = 0, wkey = 0;
                 bool single = st1;
                 if (st1) {
                     ++s1_iters;
@@ -878,80 +972,82 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
                     ++s2_pops;
                     long long wk = kNoKey;
                     // window: the R_max largest waiting requests, earliest first on ties
-                    const int R = min(a.R_max, n_left);
-                    if (a.big_window) {
+                    const int R = min(a.R_max, n_left), lim = min(mc, R);
+                    if (rare(a.big_window != 0)) {
                         wkey = largest_keys(q_key, n_w, R, lane);
-                        const WindowChoice c = big_window<FP>(sc, bw_keys, bw_off, bw_win, wkey, R, min(mc, R), WL, FP ? m[0] : 0, lane);
+                        const WindowChoice c = big_window<FP>(sc, bw_keys, bw_off, bw_win, wkey, R, lim, WL, FP ? m[0] : 0, lane);
                         wk = c.wk; chosen = c.chosen; dsum = c.dsum;
                     } else {
-                        while (!merged) {
-                            const bool fresh = !listed;
-                            if (fresh) {
-                                t0 = t1 = t2 = t3 = 0;
-#pragma unroll 1
-                                for (int t = 0; t < n_groups; ++t) {
-                                    const int4 kk = *vec_at<const int4>(q_key, (t * 32 + lane) * 4);
-                                    const int ke[4] = {kk.x, kk.y, kk.z, kk.w};
+                        if (!valid) {
+                            t0 = t1 = t2 = t3 = 0;
+#pragma unroll 2
+                            for (int t = 0; t < n_groups; ++t) {
+                                // a lane reads every 32nd position (long-waiting requests gather at the front of the
+                                // queue), sorts its four keys and merges them into its list
+                                int x0 = q_key[t * 128 + lane], x1 = q_key[t * 128 + 32 + lane];
+                                int x2 = q_key[t * 128 + 64 + lane], x3 = q_key[t * 128 + 96 + lane];
+                                order2(x0, x1); order2(x2, x3); order2(x0, x2); order2(x1, x3); order2(x1, x2);
+                                t0 = max(t0, x3); t1 = max(t1, x2); t2 = max(t2, x1); t3 = max(t3, x0);
+                                order2(t0, t2); order2(t1, t3); order2(t0, t1); order2(t2, t3);
+                            }
+                            t_end = t3 > 0 && n_groups > 1 ? kListEnd : 0;    // one group: four keys per lane
+                            valid = true;
 #pragma unroll
-                                    for (int j = 0; j < 4; ++j) {
-                                        int x = ke[j], y;
-                                        y = max(t0, x); x = min(t0, x); t0 = y;
-                                        y = max(t1, x); x = min(t1, x); t1 = y;
-                                        y = max(t2, x); x = min(t2, x); t2 = y;
-                                        t3 = max(t3, x);
-                                    }
+                            for (int r = 0; r < kRegWin; ++r) {
+                                win[r] = 0;
+                                if (r < a.R_max) {
+                                    const int x = __reduce_max_sync(kFull, t0);
+                                    win[r] = x;
+                                    if (t0 == x) { t0 = t1; t1 = t2; t2 = t3; t3 = t_end; }
+                                    valid = valid && x != kListEnd;
                                 }
-                                full = t3 > 0 && n_groups > 1;             // one group: four keys per lane
                             }
-                            int h0 = t0, h1 = t1, h2 = t2, h3 = t3;
-                            bool dry = false;
-                            wkey = 0; wdelta = 0;
-#pragma unroll 1
-                            for (int r = 0; r < R; ++r) {
-                                dry = dry || (h0 == 0 && full);
-                                const int x = __reduce_max_sync(kFull, h0);
-                                if (lane == r) wkey = x;
-                                if ((lane >> r) & 1) wdelta += x >> WL;
-                                if (h0 == x) { h0 = h1; h1 = h2; h2 = h3; h3 = 0; }
-                            }
-                            nwin = R;
-                            merged = listed = !__any_sync(kFull, dry);
-                            if (!merged && fresh) {
+                            if (rare(!valid)) {
                                 // one lane holds more of the window than its list
                                 wkey = largest_keys(q_key, n_w, R, lane);
-                                wdelta = 0;
-                                for (int r = 0; r < R; ++r) {
-                                    const int x = __shfl_sync(kFull, wkey, r);
-                                    if ((lane >> r) & 1) wdelta += x >> WL;
-                                }
-                                merged = true;
+#pragma unroll
+                                for (int r = 0; r < kRegWin; ++r) win[r] = __shfl_sync(kFull, wkey, r);
                             }
                         }
                         // subsets of the window: lane = mask, lowest mask on ties
-                        const bool cand = lane >= 1 && lane < (1 << nwin) && __popc(lane) <= min(mc, a.R_max);
-                        const int dmax = __reduce_max_sync(kFull, cand ? wdelta : 0);
-                        bool best;
-                        if (!FP) {                          // Eq. 1 scores fit 32 bits
-                            const int f = cand ? (int)sc.key(wdelta) : kEmpty;
-                            const int mf = __reduce_max_sync(kFull, f);
-                            wk = mf;
-                            best = f == mf;
-                        } else if (dmax <= sc.mm) {
-                            // every subset is safe at every offset: the score alpha D Delta grows with Delta
-                            wk = dmax;
-                            best = wdelta == dmax;
-                        } else {
-                            best = warp_max64(cand ? sc.key(wdelta) : kNoKey, wk);
+                        int delta = 0;
+#pragma unroll
+                        for (int r = 0; r < kRegWin; ++r) delta += (lane >> r) & 1 ? win[r] >> WL : 0;
+                        const bool cand = lane >= 1 && lane < (1 << R) && __popc(lane) <= lim;
+                        const int dmax = __reduce_max_sync(kFull, cand ? delta : 0);
+                        bool best = delta == dmax;
+                        wk = dmax > 0 ? (long long)dmax : kNoKey;   // safe at every offset: the score alpha D Delta grows with Delta
+                        if (dmax > sc.mm) {
+                            if (!FP) {                          // Eq. 1 scores fit 32 bits
+                                const int f = cand ? (int)sc.key(delta) : kEmpty;
+                                const int mf = __reduce_max_sync(kFull, f);
+                                wk = mf;
+                                best = f == mf;
+                            } else {
+                                // Long horizons first look at the smallest request of the window alone.  The score is
+                                // concave and zero at zero, so F(Delta) <= Delta / s F(s) for Delta >= s: if F(s) is
+                                // negative beyond rounding, so is every subset's score, and the starvation guard is next.
+                                bool none = false;
+                                if (NC == 0) {
+                                    int s = 0;
+#pragma unroll
+                                    for (int r = 0; r < kRegWin; ++r) if (r < R) s = win[r] >> WL;
+                                    none = near_score(s) < -__dmul_rn(a.rel_err, (double)s);
+                                }
+                                wk = -1;
+                                if (!none) best = warp_max64(cand ? hot_key(delta) : kNoKey, wk);
+                            }
                         }
                         chosen = __reduce_min_sync(kFull, cand && best ? (unsigned)lane : 32u);
-                        if (dmax == 0) wk = kNoKey;
-                        dsum = __shfl_sync(kFull, wdelta, chosen & 31u);
+                        dsum = 0;
+#pragma unroll
+                        for (int r = 0; r < kRegWin; ++r) dsum += (chosen >> r) & 1u ? win[r] >> WL : 0;
                     }
-                    if (wk == kNoKey) { status |= BR_ST_ITER_CAP; break; }
+                    if (rare(wk == kNoKey)) { status |= BR_ST_ITER_CAP; break; }
                     single = wk <= 0;                           // starvation guard
                 }
 
-                int mykey = wkey;                               // lane r: the key behind bit r of `chosen`
+                int qk = 0;
                 if (single) {
                     // argmax_i F_g({i}) over all waiting requests, earliest arrival on ties.
                     // The score is concave and piecewise linear in s (Eq. 2: kinks at the m_{g,h}): it rises up to
@@ -962,34 +1058,42 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
                     int peak = sc.mm;
                     bool ordered = a.peak_ok != 0;
                     if (FP) {
-                        double ws[HC];
+                        int ws[HC];
 #pragma unroll
-                        for (int c = 0; c < HC; ++c) ws[c] = 0.0;
-#pragma unroll 1
-                        for (int h = 0; h < H1; h += 4) {
-                            const int4 m4 = *vec_at<const int4>(md, h);
-                            const int mj[4] = {m4.x, m4.y, m4.z, m4.w};
+                        for (int c = 0; c < HC; ++c) ws[c] = 0;
+                        if (NC > 0) {
+                            int4 q[NC > 0 ? NC : 1];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const double d = dn_s[2 * (h + j)];
+                            for (int c = 0; c < NC; ++c) q[c] = *vec_at<const int4>(sc.md, 4 * c);
 #pragma unroll
-                                for (int c = 0; c < HC; ++c) if (mj[j] <= m[c]) ws[c] = __dadd_rn(ws[c], d);
+                            for (int c = 0; c < NC; ++c) {
+                                const int mj[4] = {q[c].x, q[c].y, q[c].z, q[c].w};
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) ws[0] += mj[j] <= m[0] ? a.iw[4 * c + j] : 0;
+                            }
+                        } else {
+                            int4 q = *vec_at<const int4>(sc.md, 0), w4 = *vec_at<const int4>(iw_s, 0);
+#pragma unroll 2
+                            for (int h = 0; h < H1; h += 4) {
+                                const int mj[4] = {q.x, q.y, q.z, q.w}, wj[4] = {w4.x, w4.y, w4.z, w4.w};
+                                q = *vec_at<const int4>(sc.md, h + 4); w4 = *vec_at<const int4>(iw_s, h + 4);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                                    for (int c = 0; c < HC; ++c) ws[c] += mj[j] <= m[c] ? wj[j] : 0;
                             }
                         }
                         peak = 0x7FFFFFFF;
                         bool flat = false;
 #pragma unroll
-                        for (int c = 0; c < HC; ++c) {
-                            const double sl = __dsub_rn(a.aD, __dmul_rn(a.beta, ws[c]));
+                        for (int c = 0; c < HC; ++c)
                             if (lane + 32 * c < H1) {
-                                flat = flat || fabs(sl) <= a.slope_err;
-                                if (!(sl > 0.0)) peak = min(peak, m[c]);
+                                flat = flat || (ws[c] > a.w_below && ws[c] < a.w_above);
+                                if (ws[c] > a.w_below) peak = min(peak, m[c]);
                             }
-                        }
-                        peak = __reduce_min_sync(kFull, peak);
-                        ordered = !__any_sync(kFull, flat);
+                        peak = __reduce_min_sync(kFull, flat ? -1 : peak);
+                        ordered = peak >= 0;
                     }
-                    int qk = 0;
                     if (ordered) {
                         const int thr = peak >= (1 << (31 - WL)) ? 0x7FFFFFFF : ((peak << WL) | (int)posmask);
                         // entries that are gone or beyond the queue have negative keys: as unsigned distances they
@@ -1010,69 +1114,91 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
                         const int ka = max((int)((unsigned)thr - below), 0);
                         const int kx = (int)(above + (unsigned)thr + 1u);
                         const int kb = kx > thr ? (int)((unsigned)kx ^ posmask) : 0;
-                        if (ka == 0 || kb == 0) {
-                            qk = ka | kb;
-                        } else {
-                            const long long f = sc.key(((lane & 1) ? kb : ka) >> WL);
-                            const long long fa = __shfl_sync(kFull, f, 0), fb = __shfl_sync(kFull, f, 1);
-                            const bool first_a = ((unsigned)ka & posmask) > ((unsigned)kb & posmask);
-                            qk = fa > fb || (fa == fb && first_a) ? ka : kb;
+                        qk = ka | kb;
+                        if (ka != 0 && kb != 0) {
+                            bool take_a = false, clear = false;
+                            if (FP && NC == 0) {
+                                const double df = __dsub_rn(near_score(ka >> WL), near_score(kb >> WL));
+                                clear = fabs(df) > __dmul_rn(a.rel_err, (double)(ka >> WL) + (double)(kb >> WL));
+                                take_a = df > 0.0;
+                            }
+                            if (!clear) {
+                                const long long f = hot_key(((lane & 1) ? kb : ka) >> WL);
+                                const long long fa = __shfl_sync(kFull, f, 0), fb = __shfl_sync(kFull, f, 1);
+                                take_a = fa > fb || (fa == fb && ((unsigned)ka & posmask) > ((unsigned)kb & posmask));
+                            }
+                            qk = take_a ? ka : kb;
                         }
                     } else {
                         qk = best_of_all<FP>(sc, q_key, n_w, WL, posmask, lane);      // a flat segment
                     }
-                    if (qk <= 0) break;
-                    mykey = qk;
+                    if (rare(qk <= 0)) break;
                     chosen = 1u;
                     dsum = qk >> WL;
                 }
 
-                // ---- admission to worker g: lane r takes the request of bit r; slots are given out after routing ----
+                // ---- admissions to worker g; slots are given out after routing ----
                 const int n_adm = __popc(chosen);
-                if ((chosen >> lane) & 1u) {
-                    const int at = __popc(chosen & ((1u << lane) - 1u)), pos = (int)(posmask - ((unsigned)mykey & posmask));
-                    adm[n_w - n_left + at] = make_int2(mykey, (g << 16) | (mc - at));
-                    q_key[pos] = kQBeyond;
-                    first_rm = min(first_rm, pos);
-                }
-                // worker g grew by dsum at every offset; only it can lift the envelope
-                if (!FP) {
-                    const int Ln = M0 - sc.mm + dsum, up = max(Ln - M0, 0);
-                    M0 += up;
-#pragma unroll
-                    for (int w = 0; w < GW; ++w) mm[w] += up;
-                } else {
-                    bool grew = false;
-#pragma unroll
-                    for (int c = 0; c < HC; ++c) {
-                        const int h = lane + 32 * c;
-                        if (h < H1) {
-                            const int x = v[c] + dsum;
-                            Lh[g * HS + h] = x;
-                            if (x > M[c]) { M[c] = x; Ms[h] = x; grew = true; }
-                        }
-                    }
-                    stale = __any_sync(kFull, grew);
-                }
-                if (lane == src) {
-#pragma unroll
-                    for (int w = 0; w < GW; ++w)
-                        if ((g >> 5) == w) { cap[w] -= n_adm; L0[w] += dsum; mm[w] -= dsum; }
-                }
-                // the admitted keys leave the lanes' lists; the merged window stays valid while none of it leaves
-                if (listed) {
 #pragma unroll 1
-                    for (unsigned cb = chosen; cb; cb &= cb - 1u) {
-                        const int x = __shfl_sync(kFull, mykey, __ffs(cb) - 1);
-                        if (t0 == x) { t0 = t1; t1 = t2; t2 = t3; t3 = 0; }
-                        else if (t1 == x) { t1 = t2; t2 = t3; t3 = 0; }
-                        else if (t2 == x) { t2 = t3; t3 = 0; }
-                        else if (t3 == x) { t3 = 0; }
+                for (int e = 0; e < n_adm; ++e) {
+                    const int r = __ffs(chosen) - 1;
+                    chosen &= chosen - 1u;
+                    int key = qk;
+                    if (!single) {
+                        key = win[0];
+#pragma unroll
+                        for (int x = 1; x < kRegWin; ++x) key = r - e == x ? win[x] : key;   // e entries have left before it
+                        if (rare(a.big_window != 0)) key = __shfl_sync(kFull, wkey, r);
+                    }
+                    const int pos = (int)(posmask - ((unsigned)key & posmask));
+                    if (lane == 0) {
+                        adm[n_w - n_left + e] = make_int2(key, (g << 16) | (mc - e));
+                        q_key[pos] = kQBeyond;
+                    }
+                    first_rm = min(first_rm, pos);
+                    // it leaves the window, where the largest head moves up, or a lane's list
+                    bool gone = false;
+#pragma unroll
+                    for (int x = 0; x < kRegWin; ++x) {
+                        gone = gone || win[x] == key;
+                        win[x] = gone ? (x + 1 < kRegWin ? win[x + 1] : 0) : win[x];
+                    }
+                    if (gone) {
+                        const int x = __reduce_max_sync(kFull, t0);
+#pragma unroll
+                        for (int y = 0; y < kRegWin; ++y) win[y] = y == a.R_max - 1 ? x : win[y];
+                        if (t0 == x) { t0 = t1; t1 = t2; t2 = t3; t3 = t_end; }
+                        valid = valid && x != kListEnd;
+                    } else {
+                        const bool h0 = t0 == key, h1 = h0 || t1 == key, h2 = h1 || t2 == key, h3 = h2 || t3 == key;
+                        t0 = h0 ? t1 : t0; t1 = h1 ? t2 : t1; t2 = h2 ? t3 : t2; t3 = h3 ? t_end : t3;
                     }
                 }
-                if (merged) {
-                    const int last = __shfl_sync(kFull, wkey, nwin - 1);
-                    merged = single && mykey < last && n_left - 1 >= a.R_max;
+                // worker g grew by dsum at every offset; beyond its smallest margin it lifts the envelope
+                const int up0 = dsum - sc.mm;
+                if (FP) {
+#pragma unroll
+                    for (int c = 0; c < HC; ++c)
+                        if (lane + 32 * c < H1) Lh[g * HS + lane + 32 * c] = m[c] - dsum;
+                }
+#pragma unroll
+                for (int w = 0; w < GW; ++w) {
+                    const bool it_is = g == lane + 32 * w;
+                    cap[w] -= it_is ? n_adm : 0;
+                    L0[w] += it_is ? dsum : 0;
+                    mm[w] -= it_is ? dsum : 0;
+                }
+                if (up0 > 0) {
+                    if (FP) {
+#pragma unroll
+                        for (int c = 0; c < HC; ++c)
+                            if (lane + 32 * c < H1) Ms[lane + 32 * c] = max(dsum - m[c], 0);
+                        __syncwarp();
+                        rows(false);
+                    } else {
+#pragma unroll
+                        for (int w = 0; w < GW; ++w) mm[w] += up0;
+                    }
                 }
                 __syncwarp();
                 S_tot -= n_adm; n_left -= n_adm;
@@ -1256,7 +1382,7 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
             int na = 0;
             for (int x = 0; x < OW; ++x) {
                 const unsigned long long o = occ[g * OW + x] & ~endm[g * OW + x];
-                occ[g * OW + x] = o; occ0[g * OW + x] = o;
+                occ[g * OW + x] = o; occ0[g * OW + x] = o; endm[g * OW + x] = 0ull;
                 na += __popcll(o);
             }
             cap_s[g] = B - na;
@@ -1267,7 +1393,7 @@ __global__ void __maxnreg__(HC == 1 ? 72 : 96) br_step_kernel(const __grid_const
 #pragma unroll 1
             for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
 #pragma unroll 1
-            for (int h = tid; h < H1; h += NT) Ms[h] = 0;
+            for (int h = tid; h < HS; h += NT) Ms[h] = h < H1 ? 0 : 0x7FFFFFFF;
         }
         if (tid == 0) {
             if (a.out.counters) {
