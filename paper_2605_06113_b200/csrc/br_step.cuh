@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 74 / 273 / 161 now.
+// the lanes' lists at every pop, 68 / 241 / 145 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -513,12 +513,15 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
         span_t<const uint32_t> row = mk_span((const uint32_t *)nullptr, 0);
         int s_new = 0;
         if (a.arr_cdf) {
-            row = mk_span(a.arr_cdf + ((size_t)inst * a.arr_inst_stride + (size_t)(k % a.arr_period)) * a.arr_len, a.arr_len);
+            row = mk_span(a.arr_cdf + ((size_t)inst * a.arr_inst_stride + (size_t)(a.arr_period == 1 ? 0 : k % a.arr_period)) * a.arr_len, a.arr_len);
             if (lane < a.arr_len) row0 = row[lane];
             if (lane + 32 < a.arr_len) row1 = row[lane + 32];
-            const uint4 r = philox_call((uint32_t)k, (uint32_t)tid >> 2, kStreamArrLen, key0, key1);
-            s_new = t_len[word_of(r, tid & 3) >> a.len_shift];
-            u_arr = philox_call((uint32_t)k, 0u, kStreamArrCount, key0, key1).x;
+            // one call serves both: lane 31 draws the count, its length word is in lane 30's block
+            const bool cnt = lane == 31;
+            const uint4 r = philox_call((uint32_t)k, cnt ? 0u : (uint32_t)tid >> 2, cnt ? kStreamArrCount : kStreamArrLen, key0, key1);
+            u_arr = __shfl_sync(kFull, r.x, 31);
+            const uint32_t last = __shfl_sync(kFull, r.w, 30);
+            s_new = t_len[(cnt ? last : word_of(r, tid & 3)) >> a.len_shift];
         }
         if (timing) t_phase[1] = (unsigned)clock64();
 
@@ -1138,40 +1141,43 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                 }
 
                 // ---- admissions to worker g; slots are given out after routing ----
-                const int n_adm = __popc(chosen);
-#pragma unroll 1
-                for (int e = 0; e < n_adm; ++e) {
-                    const int r = __ffs(chosen) - 1;
-                    chosen &= chosen - 1u;
-                    int key = qk;
-                    if (!single) {
+                const int n_adm = single ? 1 : __popc(chosen);
+                {
+                    int key = single ? qk : wkey;                // lane r: the request of bit r
+                    if (!single && a.big_window == 0) {
                         key = win[0];
 #pragma unroll
-                        for (int x = 1; x < kRegWin; ++x) key = r - e == x ? win[x] : key;   // e entries have left before it
-                        if (rare(a.big_window != 0)) key = __shfl_sync(kFull, wkey, r);
+                        for (int x = 1; x < kRegWin; ++x) key = lane == x ? win[x] : key;
                     }
-                    const int pos = (int)(posmask - ((unsigned)key & posmask));
-                    if (lane == 0) {
-                        adm[n_w - n_left + e] = make_int2(key, (g << 16) | (mc - e));
+                    const int at = __popc(chosen & ((1u << lane) - 1u)), pos = (int)(posmask - ((unsigned)key & posmask));
+                    if ((chosen >> lane) & 1u) {
+                        adm[n_w - n_left + at] = make_int2(key, (g << 16) | (mc - at));
                         q_key[pos] = kQBeyond;
+                        first_rm = min(first_rm, pos);
                     }
-                    first_rm = min(first_rm, pos);
-                    // it leaves the window, where the largest head moves up, or a lane's list
-                    bool gone = false;
+                }
+                // the admitted requests leave the window, where the largest head moves up, or a lane's list
+                unsigned out = chosen;
+                if (single) {
+                    out = 0u;
 #pragma unroll
-                    for (int x = 0; x < kRegWin; ++x) {
-                        gone = gone || win[x] == key;
-                        win[x] = gone ? (x + 1 < kRegWin ? win[x + 1] : 0) : win[x];
-                    }
-                    if (gone) {
+                    for (int x = 0; x < kRegWin; ++x) out |= win[x] == qk ? 1u << x : 0u;
+                    const bool h0 = t0 == qk, h1 = h0 || t1 == qk, h2 = h1 || t2 == qk, h3 = h2 || t3 == qk;
+                    t0 = h0 ? t1 : t0; t1 = h1 ? t2 : t1; t2 = h2 ? t3 : t2; t3 = h3 ? t_end : t3;
+                }
+                if (a.big_window == 0) {
+#pragma unroll 1
+                    while (out) {
+                        const unsigned low = out & (0u - out);
                         const int x = __reduce_max_sync(kFull, t0);
 #pragma unroll
-                        for (int y = 0; y < kRegWin; ++y) win[y] = y == a.R_max - 1 ? x : win[y];
+                        for (int y = 0; y < kRegWin; ++y) {
+                            win[y] = (1u << y) >= low && y + 1 < kRegWin ? win[y + 1 < kRegWin ? y + 1 : y] : win[y];
+                            win[y] = y == a.R_max - 1 ? x : win[y];
+                        }
                         if (t0 == x) { t0 = t1; t1 = t2; t2 = t3; t3 = t_end; }
                         valid = valid && x != kListEnd;
-                    } else {
-                        const bool h0 = t0 == key, h1 = h0 || t1 == key, h2 = h1 || t2 == key, h3 = h2 || t3 == key;
-                        t0 = h0 ? t1 : t0; t1 = h1 ? t2 : t1; t2 = h2 ? t3 : t2; t3 = h3 ? t_end : t3;
+                        out = (out ^ low) >> 1;
                     }
                 }
                 // worker g grew by dsum at every offset; beyond its smallest margin it lifts the envelope
