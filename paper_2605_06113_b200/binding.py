@@ -6,6 +6,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Dict, Optional
 
 import numpy as np
@@ -76,8 +77,7 @@ def lib():
             raise RuntimeError(f"{LIB_PATH} not found: build the CUDA library first "
                                "(python paper_2605_06113_b200/build.py)")
         L = C.CDLL(LIB_PATH)
-        step_args = [C.c_void_p, C.POINTER(BrInstanceBatch), C.POINTER(BrWorkerState),
-                     C.POINTER(BrWaitingQueue), C.c_void_p, C.c_void_p, C.POINTER(BrLoadOut)]
+        step_args = [C.c_void_p] * 7       # structures go by address: byref() of one, or its packed bytes
         L.br_create.argtypes = [C.c_int32, C.c_int32, C.POINTER(BrParams), C.POINTER(C.c_void_p)]
         L.br_step.argtypes = step_args
         L.br_graph_capture.argtypes = step_args
@@ -111,6 +111,18 @@ def use_library(path: Optional[str] = None) -> None:
     global _lib, LIB_PATH
     _lib = None
     LIB_PATH = os.path.join(_HERE, "libbr.so") if path is None else path
+
+
+# The same structures as packed bytes, which the library only reads: filling ctypes fields by name takes
+# longer than the rest of an eager one-instance step.
+_pack_batch = struct.Struct("@iiiP").pack
+_pack_state = struct.Struct("@11P").pack
+_pack_queue = struct.Struct("@4P").pack
+_pack_out = struct.Struct("@6P").pack
+
+
+def _addr(t) -> int:
+    return 0 if t is None else t.data_ptr() if not isinstance(t, np.ndarray) else t.ctypes.data
 
 
 def _ptr(t) -> Optional[int]:
@@ -147,6 +159,8 @@ class Router:
         cfg = wl.cfg
         self.cfg = cfg
         self.device = torch.device(device)
+        self._data_ptr, self._null = torch.Tensor.data_ptr, torch.empty(0)      # the empty tensor's address is NULL
+        self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
         self.len_tab = _to_torch(wl.len_tab, self.device)
         self.arr_cdf = _to_torch(wl.arr_cdf, self.device)
         self.term_cdf = _to_torch(wl.term_cdf, self.device)
@@ -216,15 +230,29 @@ class Router:
 
     def _stream(self, stream):
         if stream is None:
+            if self._raw_stream is not None and self.device.index is not None:
+                return self._raw_stream(self.device.index)        # without building a stream object
             return self.torch.cuda.current_stream(self.device).cuda_stream
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
     # ---- the calls of include/br.h -------------------------------------------
     def step(self, st, out, term_probs=None, N=None, first=0, n_steps=1, stream=None):
-        N = st["step"].shape[0] - first if N is None else N
-        b, ws, wq, lo = self._structs(st, out, N, first, n_steps, self._stream(stream))
-        rc = lib().br_step(self._h, C.byref(b), C.byref(ws), C.byref(wq), _ptr(term_probs),
-                           _ptr(out["assign"]), C.byref(lo))
+        if N is None:
+            N = st["step"].shape[0] - first
+        sget, oget, null = st.get, out.get, self._null
+        arrays = (sget("load", null), sget("nact", null), sget("occ", null), sget("act_base", null),
+                  sget("act_id", null), sget("act_chat0", null), sget("act_kref", null), sget("act_end", null),
+                  sget("step", null), sget("seed", null), sget("next_id", null),
+                  st["wq_s"], st["wq_id"], st["wq_n"], sget("wq_o", null),
+                  null if term_probs is None else term_probs, out["assign"],
+                  out["load"], out["trace"], oget("status", null), oget("counters", null),
+                  oget("fscore", null), oget("phase_cycles", null))
+        try:
+            a = list(map(self._data_ptr, arrays))
+        except TypeError:                      # a None or a numpy array among them
+            a = list(map(_addr, arrays))
+        rc = lib().br_step(self._h, _pack_batch(N, first, n_steps, self._stream(stream) or 0), _pack_state(*a[:11]),
+                           _pack_queue(*a[11:15]), a[15], a[16], _pack_out(*a[17:]))
         if rc != BR_OK:
             raise BrError(rc, "br_step")
 
