@@ -90,9 +90,12 @@ constexpr int kSMs = 148;
 constexpr int kHostWarps = 4;          // instances resident per SM when their rows are in host memory
 
 // Threads per instance of br_step_kernel.  An instance has parallel work for `most` threads (projection:
-// 16 slots a thread, queue: 4 positions a thread); more only lengthen its barriers.  When the batch
-// puts several instances on an SM they share its registers, which hold 28 warps (20 for long
-// horizons): with fewer threads per instance all of them are resident and none waits for a second wave.
+// 16 slots a thread, queue: 4 positions a thread); more only lengthen its barriers.  Four warps pay off even
+// for small ones, because the requests that end are drawn while warp 0 routes (777 instances of G = 21,
+// W = 300, H = 6: 239 us per three steps with three warps, 213 with four; 84 of G = 4, W = 56: 19.9 with one,
+// 15.2 with four).  When the batch puts several instances on an SM they share its registers, which hold 28
+// warps (20 for long horizons): with fewer threads per instance all of them are resident and none waits
+// for a second wave.
 int threads_for(const br_ctx *ctx, int n_instances)
 {
     if (ctx->p.threads > 0) return ctx->p.threads;
@@ -100,7 +103,7 @@ int threads_for(const br_ctx *ctx, int n_instances)
     int most = ctx->H > 0 ? A / 16 : 64;
     if (ctx->p.W / 4 > most) most = ctx->p.W / 4;
     most = (most + 31) / 32;
-    most = most < 1 ? 1 : (most > 8 ? 8 : most);
+    most = most < 4 ? 4 : (most > 8 ? 8 : most);
     int per_sm = (n_instances + kSMs - 1) / kSMs;
     const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
     if (per_sm > fit) per_sm = fit;
