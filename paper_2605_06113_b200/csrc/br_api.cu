@@ -319,6 +319,8 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
         // first kink is alpha D.
         a.rel_err = 4.0 * (H + 5) * 1.1102230246251565e-16 * (a.aD + p.beta * D);
         const double err = a.rel_err * (double)p.s_max;
+        a.fix = 4.0e9 / (D * (double)p.s_max + 1.0);                   // a single request's penalty sum stays below 2^32
+        a.beta_fix = p.beta / a.fix; a.fix_err = 40.0 * a.beta_fix;
         const double slope_err = err > 1e-9 ? err : 1e-9;
         // The weights in fixed point: iw_h = floor(scale d_h), so that a sum of up to H + 1 of them is below
         // scale * sum d_h by less than H + 1.  A segment rises clearly while alpha D - beta sum d_h > slope_err.

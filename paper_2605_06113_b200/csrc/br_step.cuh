@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 68 / 241 / 145 now.
+// the lanes' lists at every pop, 67 / 205 / 128 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -70,6 +70,7 @@ struct StepArgs {
     const float *term_probs;
     int32_t *assign_out;
     br_load_out out;
+    double fix, beta_fix, fix_err;   // scale of penalty sums in fixed point, beta / fix, and what the rounding to it adds
 };
 
 // Groups of four horizon offsets (h = 0 .. H) that a kernel unrolls: 2, 3 or 5, so that the loops over h
@@ -900,18 +901,25 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                 const double dl = __dsub_rn(__hiloint2double(0x43300000, delta), 4503599627370496.0);
                 return key_of_double(__dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)));
             };
-            // Eq. 2 with the terms summed across the lanes: off the exact score by at most rel_err * delta
+            // Eq. 2 with the terms summed across the lanes: off the exact score by at most rel_err * delta + fix_err
+            double w[HC];                                                   // discounts d_h of the lane's offsets
+            int iw[HC];                                                     // ... in fixed point
+#pragma unroll
+            for (int c = 0; c < HC; ++c) {
+                w[c] = FP && lane + 32 * c < H1 ? dn_s[2 * (lane + 32 * c)] : 0.0;
+                iw[c] = FP && lane + 32 * c < H1 ? iw_s[lane + 32 * c] : 0;
+            }
             int m[HC];                                                      // margins of the selected worker, by offset
             auto near_score = [&](int delta) -> double {
                 double p = 0.0;
 #pragma unroll
                 for (int c = 0; c < HC; ++c) {
                     const double x = __dsub_rn(__hiloint2double(0x43300000, max(delta - m[c], 0)), 4503599627370496.0);
-                    p = __fma_rn(x, lane + 32 * c < H1 ? dn_s[2 * (lane + 32 * c)] : 0.0, p);
+                    p = __fma_rn(x, w[c], p);
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) p = __dadd_rn(p, __shfl_xor_sync(kFull, p, o));
-                return __fma_rn(a.aD, (double)delta, -__dmul_rn(a.beta, p));
+                // 32 lanes, each rounded to 1 / fix: the sum fits 32 bits and is off by less than 32 / fix
+                const unsigned q = __reduce_add_sync(kFull, __double2uint_rn(__dmul_rn(p, a.fix)));
+                return __fma_rn(a.aD, (double)delta, -__dmul_rn(a.beta_fix, (double)q));
             };
 
             // optional F-score matrix before the first admission
@@ -981,7 +989,29 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                         const WindowChoice c = big_window<FP>(sc, bw_keys, bw_off, bw_win, wkey, R, lim, WL, FP ? m[0] : 0, lane);
                         wk = c.wk; chosen = c.chosen; dsum = c.dsum;
                     } else {
-                        if (!valid) {
+                        bool none = false;
+                        if (NC == 0) {
+                            // The score is concave and zero at zero, so F(Delta) <= Delta / s F(s) for Delta >= s: if F(s) is
+                            // negative beyond rounding for an s that no window entry is below, every subset's score is, and
+                            // the starvation guard is next.  Before the window is built, the R-th largest of the lanes'
+                            // maxima is such an s, and much cheaper than the window.
+                            int x = 0;
+                            if (valid) {
+#pragma unroll
+                                for (int r = 0; r < kRegWin; ++r) x = r < R ? win[r] : x;
+                            } else {
+                                int x0 = 0;
+#pragma unroll 2
+                                for (int t = 0; t < n_groups; ++t) {
+                                    const int4 kk = *vec_at<const int4>(q_key, (t * 32 + lane) * 4);
+                                    x0 = max(max(x0, max(kk.x, kk.y)), max(kk.z, kk.w));
+                                }
+#pragma unroll 1
+                                for (int r = 0; r < R; ++r) { x = __reduce_max_sync(kFull, x0); x0 = x0 == x ? 0 : x0; }
+                            }
+                            none = near_score(x >> WL) < -__fma_rn(a.rel_err, (double)(x >> WL), a.fix_err);
+                        }
+                        if ((NC > 0 || !none) && !valid) {
                             t0 = t1 = t2 = t3 = 0;
 #pragma unroll 2
                             for (int t = 0; t < n_groups; ++t) {
@@ -1012,39 +1042,32 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                                 for (int r = 0; r < kRegWin; ++r) win[r] = __shfl_sync(kFull, wkey, r);
                             }
                         }
-                        // subsets of the window: lane = mask, lowest mask on ties
-                        int delta = 0;
+                        if (NC == 0 && none) {
+                            wk = -1;
+                        } else {
+                            // subsets of the window: lane = mask, lowest mask on ties
+                            int delta = 0;
 #pragma unroll
-                        for (int r = 0; r < kRegWin; ++r) delta += (lane >> r) & 1 ? win[r] >> WL : 0;
-                        const bool cand = lane >= 1 && lane < (1 << R) && __popc(lane) <= lim;
-                        const int dmax = __reduce_max_sync(kFull, cand ? delta : 0);
-                        bool best = delta == dmax;
-                        wk = dmax > 0 ? (long long)dmax : kNoKey;   // safe at every offset: the score alpha D Delta grows with Delta
-                        if (dmax > sc.mm) {
-                            if (!FP) {                          // Eq. 1 scores fit 32 bits
-                                const int f = cand ? (int)sc.key(delta) : kEmpty;
-                                const int mf = __reduce_max_sync(kFull, f);
-                                wk = mf;
-                                best = f == mf;
-                            } else {
-                                // Long horizons first look at the smallest request of the window alone.  The score is
-                                // concave and zero at zero, so F(Delta) <= Delta / s F(s) for Delta >= s: if F(s) is
-                                // negative beyond rounding, so is every subset's score, and the starvation guard is next.
-                                bool none = false;
-                                if (NC == 0) {
-                                    int s = 0;
-#pragma unroll
-                                    for (int r = 0; r < kRegWin; ++r) if (r < R) s = win[r] >> WL;
-                                    none = near_score(s) < -__dmul_rn(a.rel_err, (double)s);
+                            for (int r = 0; r < kRegWin; ++r) delta += (lane >> r) & 1 ? win[r] >> WL : 0;
+                            const bool cand = lane >= 1 && lane < (1 << R) && __popc(lane) <= lim;
+                            const int dmax = __reduce_max_sync(kFull, cand ? delta : 0);
+                            bool best = delta == dmax;
+                            wk = dmax > 0 ? (long long)dmax : kNoKey;   // safe at every offset: the score alpha D Delta grows with Delta
+                            if (dmax > sc.mm) {
+                                if (!FP) {                          // Eq. 1 scores fit 32 bits
+                                    const int fs = cand ? (int)sc.key(delta) : kEmpty;
+                                    const int mf = __reduce_max_sync(kFull, fs);
+                                    wk = mf;
+                                    best = fs == mf;
+                                } else {
+                                    best = warp_max64(cand ? hot_key(delta) : kNoKey, wk);
                                 }
-                                wk = -1;
-                                if (!none) best = warp_max64(cand ? hot_key(delta) : kNoKey, wk);
                             }
-                        }
-                        chosen = __reduce_min_sync(kFull, cand && best ? (unsigned)lane : 32u);
-                        dsum = 0;
+                            chosen = __reduce_min_sync(kFull, cand && best ? (unsigned)lane : 32u);
+                            dsum = 0;
 #pragma unroll
-                        for (int r = 0; r < kRegWin; ++r) dsum += (chosen >> r) & 1u ? win[r] >> WL : 0;
+                            for (int r = 0; r < kRegWin; ++r) dsum += (chosen >> r) & 1u ? win[r] >> WL : 0;
+                        }
                     }
                     if (rare(wk == kNoKey)) { status |= BR_ST_ITER_CAP; break; }
                     single = wk <= 0;                           // starvation guard
@@ -1061,11 +1084,11 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                     int peak = sc.mm;
                     bool ordered = a.peak_ok != 0;
                     if (FP) {
-                        int ws[HC];
-#pragma unroll
-                        for (int c = 0; c < HC; ++c) ws[c] = 0;
                         if (NC > 0) {
                             int4 q[NC > 0 ? NC : 1];
+                            int ws[HC];
+#pragma unroll
+                            for (int c = 0; c < HC; ++c) ws[c] = 0;
 #pragma unroll
                             for (int c = 0; c < NC; ++c) q[c] = *vec_at<const int4>(sc.md, 4 * c);
 #pragma unroll
@@ -1074,27 +1097,50 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
 #pragma unroll
                                 for (int j = 0; j < 4; ++j) ws[0] += mj[j] <= m[0] ? a.iw[4 * c + j] : 0;
                             }
+                            peak = 0x7FFFFFFF;
+                            bool flat = false;
+                            if (lane < H1) {
+                                flat = flat || (ws[0] > a.w_below && ws[0] < a.w_above);
+                                if (ws[0] > a.w_below) peak = min(peak, m[0]);
+                            }
+                            peak = __reduce_min_sync(kFull, flat ? -1 : peak);
                         } else {
-                            int4 q = *vec_at<const int4>(sc.md, 0), w4 = *vec_at<const int4>(iw_s, 0);
-#pragma unroll 2
-                            for (int h = 0; h < H1; h += 4) {
-                                const int mj[4] = {q.x, q.y, q.z, q.w}, wj[4] = {w4.x, w4.y, w4.z, w4.w};
-                                q = *vec_at<const int4>(sc.md, h + 4); w4 = *vec_at<const int4>(iw_s, h + 4);
+                            // Bisection over the kinks: the score still rises at lo, no more at hi.  The next kink to look
+                            // at is the last one in the lower half of the lengths between them, or the first after.
+                            int lo = -1, hi = -1;
 #pragma unroll
-                                for (int j = 0; j < 4; ++j)
+                            for (int c = 0; c < HC; ++c) hi = max(hi, lane + 32 * c < H1 ? m[c] : -1);
+                            hi = __reduce_max_sync(kFull, hi);
+                            int pv = hi;                         // the last kink first: the score may rise throughout
+                            peak = 0x7FFFFFFF;
+#pragma unroll 1
+                            while (true) {
+                                unsigned ws = 0;
 #pragma unroll
-                                    for (int c = 0; c < HC; ++c) ws[c] += mj[j] <= m[c] ? wj[j] : 0;
+                                for (int c = 0; c < HC; ++c) ws += m[c] <= pv ? (unsigned)iw[c] : 0u;
+                                ws = __reduce_add_sync(kFull, ws);
+                                if ((int)ws > a.w_below) {
+                                    peak = (int)ws < a.w_above ? -1 : pv;
+                                    if (peak < 0) break;
+                                    hi = pv;
+                                } else {
+                                    lo = pv;
+                                    if (lo == hi) break;                         // rises throughout
+                                }
+                                const int mid = lo + ((hi - lo) >> 1);
+                                int b = -1;
+#pragma unroll
+                                for (int c = 0; c < HC; ++c) b = max(b, lane + 32 * c < H1 && m[c] <= mid ? m[c] : -1);
+                                pv = __reduce_max_sync(kFull, b);
+                                if (pv <= lo) {
+                                    b = 0x7FFFFFFF;
+#pragma unroll
+                                    for (int c = 0; c < HC; ++c) b = min(b, lane + 32 * c < H1 && m[c] > mid ? m[c] : 0x7FFFFFFF);
+                                    pv = __reduce_min_sync(kFull, b);
+                                    if (pv >= hi) break;                         // no kink between them
+                                }
                             }
                         }
-                        peak = 0x7FFFFFFF;
-                        bool flat = false;
-#pragma unroll
-                        for (int c = 0; c < HC; ++c)
-                            if (lane + 32 * c < H1) {
-                                flat = flat || (ws[c] > a.w_below && ws[c] < a.w_above);
-                                if (ws[c] > a.w_below) peak = min(peak, m[c]);
-                            }
-                        peak = __reduce_min_sync(kFull, flat ? -1 : peak);
                         ordered = peak >= 0;
                     }
                     if (ordered) {
@@ -1122,7 +1168,7 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                             bool take_a = false, clear = false;
                             if (FP && NC == 0) {
                                 const double df = __dsub_rn(near_score(ka >> WL), near_score(kb >> WL));
-                                clear = fabs(df) > __dmul_rn(a.rel_err, (double)(ka >> WL) + (double)(kb >> WL));
+                                clear = fabs(df) > __fma_rn(a.rel_err, (double)(ka >> WL) + (double)(kb >> WL), __dadd_rn(a.fix_err, a.fix_err));
                                 take_a = df > 0.0;
                             }
                             if (!clear) {
