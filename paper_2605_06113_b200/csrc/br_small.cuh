@@ -23,6 +23,39 @@
 
 namespace br {
 
+__device__ __noinline__ uint4 philox_block(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1)
+{
+    return philox4x32_10(c0, c1, c2, c3, k0, k1);
+}
+
+// draw_ending for one occupancy word.  A binary search over the table is a chain of six dependent loads per
+// draw; the gap is guessed from its logarithm and put right against the table, whatever that holds, and the
+// first draw of a worker, which mostly ends nothing, is compared with a threshold in a register (4,096
+// instances, 16 steps: 184.6 us with the search, 176.5 this way).
+template <typename CDF>
+__device__ __forceinline__ unsigned long long ending_slots(const CDF cdf, int B, uint32_t last, float inv_log, uint32_t k, uint32_t g,
+                                                           uint32_t key0, uint32_t key1)
+{
+    unsigned long long fin = 0ull;
+    uint4 r = philox4x32_10(k, g, kStreamTerm, 0u, key0, key1);
+    uint32_t u = r.x;
+    int pos = 0;
+#pragma unroll 1
+    for (unsigned t = 1u; pos < B && u < (pos == 0 ? last : cdf[B - pos - 1]); ++t) {   // else the gap reaches past the last slot
+        const int room = B - pos;
+        int gap = (int)(__log2f((float)~u * 2.3283064e-10f) * inv_log);
+        gap = min(max(gap, 0), room - 1);
+        while (gap > 0 && u < cdf[gap - 1]) --gap;
+        while (gap < room - 1 && u >= cdf[gap]) ++gap;
+        pos += gap;
+        fin |= 1ull << pos;
+        ++pos;
+        if ((t & 3u) == 0u) r = philox_block(k, g, kStreamTerm, t >> 2, key0, key1);
+        u = word_of(r, t & 3u);
+    }
+    return fin;
+}
+
 constexpr int kSmallBeyond = (int)0x8000FFFFu;   // key of a position beyond the queue (no slot index reaches 0xFFFF)
 
 template <int NT4 /* 128-position groups: W <= 128 * NT4 */, int RM /* window entries kept */>
@@ -49,42 +82,51 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
     const auto t_len = mk_span(a.len_tab, a.len_tab ? (1ll << (32 - a.len_shift)) : 0);
     const auto t_term = mk_span(a.term_cdf, B);
 
-    const unsigned long long seed = a.ws.seed[inst];
-    const uint32_t key0 = (uint32_t)seed, key1 = (uint32_t)(seed >> 32);
-    int k = a.ws.step[inst];
-    uint32_t next_id = a.ws.next_id[inst];
-    int n_w = a.wq.n[inst];
-    int status0 = 0;
-    if (n_w < 0 || n_w > W) { status0 = BR_ST_BAD_STATE; n_w = n_w < 0 ? 0 : W; }
-
-    // worker state of lane g; lanes beyond G hold cap = -1, L = 0 and a full occupancy word
     const unsigned long long slots = B >= 64 ? ~0ull : ((1ull << B) - 1ull);
+    const unsigned long long seed = (unsigned long long)ld_now8(a.ws.seed + inst);
+    int k = ld_now(a.ws.step + inst);
+    uint32_t next_id = (uint32_t)ld_now(a.ws.next_id + inst);
+    int n_w = ld_now(a.wq.n + inst);
+    // worker state of lane g; lanes beyond G hold cap = -1, L = 0 and a full occupancy word
     int cap = -1, L = 0;
     unsigned long long occ = ~0ull;
     if (lane < G) {
-        int na = a.ws.nact[(size_t)inst * G + lane];
-        if (na < 0 || na > B) { status0 = BR_ST_BAD_STATE; na = na < 0 ? 0 : B; }
-        cap = B - na;
-        L = (int)a.ws.load[(size_t)inst * G + lane];
-        occ = a.ws.occ[(size_t)inst * G + lane] | ~slots;
+        cap = ld_now(a.ws.nact + (size_t)inst * G + lane);
+        L = (int)ld_now8(a.ws.load + (size_t)inst * G + lane);
+        occ = (unsigned long long)ld_now8(a.ws.occ + (size_t)inst * G + lane) | ~slots;
     }
+    int4 qv[NT4], qi[NT4];
+#pragma unroll
+    for (int t = 0; t < NT4; ++t) {
+        const int p0 = (t * 32 + lane) * 4;
+        qv[t] = qi[t] = make_int4(0, 0, 0, 0);
+        if (p0 < W) {
+            qv[t] = ld_now4(vec_at<const int4>(g_qs, p0));
+            qi[t] = ld_now4(vec_at<const int4>(g_qid, p0));
+        }
+    }
+    // constant hazard: a draw of `last` and more ends none of the worker's slots; geometric gaps as logarithms
+    const uint32_t last = a.term_mode == 1 ? (uint32_t)ld_now(&t_term[B - 1]) : 0u;
+    const float inv_log = a.term_mode == 1 ? __fdividef(1.0f, __log2f(1.0f - (float)(uint32_t)ld_now(&t_term[0]) * 2.3283064e-10f)) : 0.0f;
 
+    const uint32_t key0 = (uint32_t)seed, key1 = (uint32_t)(seed >> 32);
+    int status0 = 0;
+    if (n_w < 0 || n_w > W) { status0 = BR_ST_BAD_STATE; n_w = n_w < 0 ? 0 : W; }
+    if (lane < G) {
+        if (cap < 0 || cap > B) { status0 = BR_ST_BAD_STATE; cap = cap < 0 ? 0 : B; }
+        cap = B - cap;
+    }
     // ---- the queue moves to shared memory once per launch: packed keys and ids ----
 #pragma unroll
     for (int t = 0; t < NT4; ++t) {
         const int p0 = (t * 32 + lane) * 4;
-        int4 sv = make_int4(0, 0, 0, 0); uint4 iv = make_uint4(0u, 0u, 0u, 0u);
-        if (p0 < W) {
-            sv = *vec_at<const int4>(g_qs, p0);
-            iv = *vec_at<const uint4>(g_qid, p0);
-        }
         int4 kk;
-        kk.x = p0 + 0 < n_w ? (sv.x << WL) | (int)(posmask - (unsigned)(p0 + 0)) : kSmallBeyond;
-        kk.y = p0 + 1 < n_w ? (sv.y << WL) | (int)(posmask - (unsigned)(p0 + 1)) : kSmallBeyond;
-        kk.z = p0 + 2 < n_w ? (sv.z << WL) | (int)(posmask - (unsigned)(p0 + 2)) : kSmallBeyond;
-        kk.w = p0 + 3 < n_w ? (sv.w << WL) | (int)(posmask - (unsigned)(p0 + 3)) : kSmallBeyond;
+        kk.x = p0 + 0 < n_w ? (qv[t].x << WL) | (int)(posmask - (unsigned)(p0 + 0)) : kSmallBeyond;
+        kk.y = p0 + 1 < n_w ? (qv[t].y << WL) | (int)(posmask - (unsigned)(p0 + 1)) : kSmallBeyond;
+        kk.z = p0 + 2 < n_w ? (qv[t].z << WL) | (int)(posmask - (unsigned)(p0 + 2)) : kSmallBeyond;
+        kk.w = p0 + 3 < n_w ? (qv[t].w << WL) | (int)(posmask - (unsigned)(p0 + 3)) : kSmallBeyond;
         *vec_at<int4>(q_key, p0) = kk;
-        *vec_at<uint4>(q_id, p0) = iv;
+        *vec_at<int4>(q_id, p0) = qi[t];
     }
     __syncwarp();
     int dirty = n_w;                                      // entries before this one have not changed
@@ -109,10 +151,19 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
             n_arr = __popc(__ballot_sync(kFull, lane < a.arr_len && u >= r0)) +
                     __popc(__ballot_sync(kFull, lane + 32 < a.arr_len && u >= r1));
         }
+        // prompt length of arrival `lane`, asked for now: word lane % 4 of block lane / 4
+        auto length_word = [&](int j) {
+            const int src = (j >> 2) & 31;
+            const uint32_t w0 = __shfl_sync(kFull, rb.x, src), w1 = __shfl_sync(kFull, rb.y, src);
+            const uint32_t w2 = __shfl_sync(kFull, rb.z, src), w3 = __shfl_sync(kFull, rb.w, src);
+            return (j & 2) ? ((j & 1) ? w3 : w2) : ((j & 1) ? w1 : w0);
+        };
+        int s_new = 0;
+        if (a.arr_cdf) s_new = ld_now(&t_len[length_word(lane) >> a.len_shift]);
         // constant-hazard draws of this step for worker `lane` (used after routing)
         unsigned long long fin = 0ull;
         if (a.term_mode == 1 && lane < G)
-            draw_ending(t_term, B, 1, (uint32_t)k, (uint32_t)lane, key0, key1, &fin);
+            fin = ending_slots(t_term, B, last, inv_log, (uint32_t)k, (uint32_t)lane, key0, key1);
         // a request that was running before this step and ends at it: its load is asked for now
         const unsigned long long pre = occ & fin & slots;
         const int pj = __ffsll((long long)pre) - 1;
@@ -126,14 +177,13 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         const int n_drop = n_arr - n_take;
 #pragma unroll 1
         for (int j0 = 0; j0 < n_take; j0 += 32) {
-            const int j = j0 + lane;                                   // arrival j: word j % 4 of block j / 4
-            const int src = (j >> 2) & 31;
-            const uint32_t w0 = __shfl_sync(kFull, rb.x, src), w1 = __shfl_sync(kFull, rb.y, src);
-            const uint32_t w2 = __shfl_sync(kFull, rb.z, src), w3 = __shfl_sync(kFull, rb.w, src);
+            const int j = j0 + lane;
+            if (rare(j0 > 0)) {
+                const uint32_t w = length_word(j);
+                if (j < n_take) s_new = t_len[w >> a.len_shift];
+            }
             if (j < n_take) {
-                const uint32_t w = (j & 2) ? ((j & 1) ? w3 : w2) : ((j & 1) ? w1 : w0);
-                const int s = t_len[w >> a.len_shift];
-                const int pos = n_w_old + j;
+                const int s = s_new, pos = n_w_old + j;
                 q_key[pos] = (s << WL) | (int)(posmask - (unsigned)pos);
                 q_id[pos] = id0 + (unsigned)j;
             }
@@ -160,7 +210,8 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
             const int mc = __reduce_max_sync(kFull, cap);
             if (mc <= 0) break;
             const unsigned ml = __reduce_min_sync(kFull, cap == mc ? (unsigned)L : 0xFFFFFFFFu);
-            const int g = __ffs(__ballot_sync(kFull, cap == mc && (unsigned)L == ml)) - 1;
+            const int g = (int)__reduce_min_sync(kFull, cap == mc && (unsigned)L == ml ? (unsigned)lane : 32u);
+            int Lg = (int)ml;
             const int m = M - (int)ml;                                  // safe margin m_g (Section 3.1)
             int todo = 0;                                               // window entries to admit (bit r)
             bool single = stage1;
@@ -258,7 +309,8 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
                         cap = 0;
                     }
                 }
-                M = max(M, __shfl_sync(kFull, L, g));
+                Lg += s;
+                M = max(M, Lg);
                 if (qk >= gw[RM - 1]) gw_valid = false;                 // a cached window entry leaves
                 first_rm = min(first_rm, pos);
                 --S_tot; --n_left; ++admitted;

@@ -199,6 +199,26 @@ __device__ __forceinline__ void draw_ending(const CDF cdf, int B, int OW, uint32
     }
 }
 
+// Loads that stay where they are written: a launch opens with one trip to memory for all it needs.
+__device__ __forceinline__ int4 ld_now4(const void *p)
+{
+    int4 v;
+    asm volatile("ld.global.v4.s32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_now(const void *p)
+{
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ long long ld_now8(const void *p)
+{
+    long long v;
+    asm volatile("ld.global.s64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
+
 // Loads of classifier output.  A row is read once, by one thread, at a scattered address; left to
 // itself the L2 fetches 128 bytes around a missing sector, of which a refresh uses 32 on average,
 // so the loads ask for the smallest fetch the instruction set offers (64 bytes).
