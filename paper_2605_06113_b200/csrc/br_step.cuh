@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 67 / 205 / 128 now.
+// the lanes' lists at every pop, 67 / 194 / 127 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -734,20 +734,14 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
 #pragma unroll 2
                     for (int h = h1 - 1; h >= h0; --h) {
                         Ti += Lh[g * HS + h]; Ci += Ch[g * HS + h];
-                        Lh[g * HS + h] = Ti + h * Ci;
+                        const int x = Ti + h * Ci;
+                        Lh[g * HS + h] = x;
+                        atomicMax(&Ms[h], x);                               // envelope M_h
                     }
                 }
             } else {
 #pragma unroll 1
-                for (int g = tid; g < G; g += NT) Lh[g * HS] = L0_s[g];
-            }
-            __syncthreads();
-#pragma unroll 1
-            for (int h = lane; h < H1; h += 32) {                           // envelope M_h
-                int v = 0;
-#pragma unroll 4
-                for (int g = warp; g < G; g += nwarps) v = max(v, Lh[g * HS + h]);
-                atomicMax(&Ms[h], v);
+                for (int g = tid; g < G; g += NT) { Lh[g * HS] = L0_s[g]; atomicMax(&Ms[0], L0_s[g]); }
             }
         }
         __syncthreads();
@@ -1357,7 +1351,7 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                 atomicAdd(&sub_load[g], (unsigned)s);
             }
         }
-        __syncthreads();
+        if (n_adm > 0) __syncthreads();
 
         // ============ queue compaction and assignments ============
         // A thread owns four consecutive positions of every stretch of 4 NT; an entry's new position is
@@ -1369,7 +1363,7 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
 #pragma unroll 1
             for (int i0 = 0; i0 < W; i0 += 4 * NT) {
                 const int p0 = i0 + 4 * tid;
-                if (i0 >= n_w || i0 + 4 * NT <= first_rm) {
+                if (first_rm >= min(i0 + 4 * NT, n_w)) {                       // (or beyond the queue)
                     if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(-1, -1, -1, -1);
                     run += 4 * NT;                                // (beyond the queue the count is not used)
                     continue;
@@ -1384,11 +1378,15 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                 const int ke[4] = {kk.x, kk.y, kk.z, kk.w};
                 const unsigned idv[4] = {ii.x, ii.y, ii.z, ii.w};
                 const int ov[4] = {oo.x, oo.y, oo.z, oo.w};
-                const int cnt = (ke[0] > 0) + (ke[1] > 0) + (ke[2] > 0) + (ke[3] > 0);
-                int inc = cnt;
+                int before = 0, kept = 0;                         // within the warp's 128 positions
+                const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(kFull, inc, o); if (lane >= o) inc += x; }
-                if (lane == 31) scal[16 + par + warp] = inc;
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned b = __ballot_sync(kFull, ke[j] > 0);
+                    before += __popc(b & lt);
+                    kept += __popc(b);
+                }
+                if (lane == 0) scal[16 + par + warp] = kept;
                 int as[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -1397,7 +1395,7 @@ __global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_consta
                 }
                 if (p0 < W) *vec_at<int4>(assign, p0) = make_int4(as[0], as[1], as[2], as[3]);
                 __syncthreads();                                  // the stretch is read before any of it is overwritten
-                int below = run + inc - cnt, total = 0;
+                int below = run + before, total = 0;
 #pragma unroll 1
                 for (int x = 0; x < nwarps; ++x) {
                     const int t = scal[16 + par + x];
