@@ -90,24 +90,28 @@ constexpr int kSMs = 148;
 constexpr int kHostWarps = 4;          // instances resident per SM when their rows are in host memory
 
 // Threads per instance of br_step_kernel.  An instance has parallel work for `most` threads (projection:
-// 16 slots a thread, queue: 4 positions a thread); more only lengthen its barriers.  Four warps pay off even
-// for small ones, because the requests that end are drawn while warp 0 routes (777 instances of G = 21,
-// W = 300, H = 6: 239 us per three steps with three warps, 213 with four; 84 of G = 4, W = 56: 19.9 with one,
-// 15.2 with four).  When the batch puts several instances on an SM they share its registers, which hold 28
-// warps (20 for long horizons): with fewer threads per instance all of them are resident and none waits
-// for a second wave.
+// 16 slots a thread, queue: 4 positions, buckets: 8 offsets); more only lengthen its barriers, but four
+// warps pay off even for small ones, because the requests that end are drawn while warp 0 routes (84 of
+// G = 4, W = 56: 19.9 us with one warp, 15.2 with four).  When the batch puts several instances on an SM they
+// share its registers, which hold 21 warps (16 for long horizons): each takes its share, so that all are
+// resident (777 of G = 21, W = 300, three steps: 234 / 169 / 201 us with two / three / four warps).  Instances
+// that stream 2,048 slots and more of classifier state are bound by memory while they do; fewer of them at a time
+// with more warps each, so that some stream while others route (1,024 of G = 64, H = 8: 77 us with three warps,
+// 64.5 with four, 63.0 with five, 85 with eight).
 int threads_for(const br_ctx *ctx, int n_instances)
 {
     if (ctx->p.threads > 0) return ctx->p.threads;
     const int A = ctx->G * ctx->p.B;
     int most = ctx->H > 0 ? A / 16 : 64;
     if (ctx->p.W / 4 > most) most = ctx->p.W / 4;
+    if (ctx->G * (ctx->H + 1) / 8 > most) most = ctx->G * (ctx->H + 1) / 8;
     most = (most + 31) / 32;
     most = most < 4 ? 4 : (most > 8 ? 8 : most);
     int per_sm = (n_instances + kSMs - 1) / kSMs;
     const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
     if (per_sm > fit) per_sm = fit;
-    int w = (br::step_groups(ctx->H) ? 28 : 20) / per_sm;
+    int w = (4 * (br::step_groups(ctx->H) ? 21 : 16) / per_sm + 1) / 4;
+    if (ctx->H > 0 && ctx->p.pred_mode == 0 && A >= 2048 && w < 5) w = 5;
     w = w < 1 ? 1 : (w > most ? most : w);
     return 32 * w;
 }

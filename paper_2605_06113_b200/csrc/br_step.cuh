@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 67 / 194 / 127 now.
+// the lanes' lists at every pop, 67 / 181 / 119 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -405,8 +405,11 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
 }
 
 // FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  NC: step_groups(H).
+// Registers: the router's chain is the longest path, and it is shorter with more of them than with more
+// warps resident (G = 64, H = 8, one instance: 22.0 us at 72 registers, 19.4 at 96; 777 instances of G = 21,
+// H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128).
 template <bool FP, int GW, int NC>
-__global__ void __maxnreg__(NC > 0 ? 72 : 96) br_step_kernel(const __grid_constant__ StepArgs a)
+__global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_constant__ StepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
