@@ -60,7 +60,8 @@ inline int fscore_smem(int G, int row) { return 4 * G * row + 16 * row + kFsWarp
 // fp64 instructions and one integer one.  Eq. 2 is bound by instruction issue (and, next, by the
 // fp64 pipe, which takes two cycles for an instruction), Eq. 1 by the writes.  200 x 1,024 x 64 scores at
 // H = 8 with best workers: 224 us with five fp64 operations a term, blocks of 1,024 requests and the best
-// worker found by scoring everything again; 57 us this way.
+// worker found by scoring everything again; 57 with the terms above for every pair, 31 with the workers whose
+// smallest margin no request of the warp exceeds left at alpha D s.
 template <bool FP>
 __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreArgs a)
 {
@@ -69,9 +70,13 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
     int *m_s = reinterpret_cast<int *>(fs_smem);                                 // [g][HS] -m_{g,h}, clipped to the range of s
     double2 *d_s = reinterpret_cast<double2 *>(fs_smem + 4 * G * HS);            // (d_h, -2^52 d_h)
     double *stage = reinterpret_cast<double *>(fs_smem + 4 * G * HS + 16 * HS) + warp * kFsReq * (kFsCols + 1);
-    __shared__ int cap_s[BR_MAX_G];
+    __shared__ int cap_s[BR_MAX_G], low_s[BR_MAX_G];                             // low_s: -min_h m_{g,h}
     const size_t inst = (size_t)a.first_instance + blockIdx.y;
 
+    if (FP) {
+        for (int g = tid; g < G; g += 32 * kFsWarps) low_s[g] = (int)0x80000000;
+        __syncthreads();
+    }
     // margins: one warp per offset, lanes over workers
     for (int h = warp; h < H1; h += kFsWarps) {
         const int64_t *row = a.Lh + inst * G * (a.H + 1) + h;
@@ -83,8 +88,14 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
             const long long v = __shfl_xor_sync(kFull, M, o);
             M = v > M ? v : M;
         }
-        if (lane < G) m_s[lane * HS + h] = -(int)min(M - L0, 0x7FFFFFFFll);
-        if (lane + 32 < G) m_s[(lane + 32) * HS + h] = -(int)min(M - L1, 0x7FFFFFFFll);
+#pragma unroll
+        for (int w = 0; w < 2; ++w) {
+            const int g = lane + 32 * w;
+            if (g >= G) continue;
+            const int v = -(int)min(M - (w ? L1 : L0), 0x7FFFFFFFll);
+            m_s[g * HS + h] = v;
+            if (FP) atomicMax(&low_s[g], v);
+        }
         if (lane == 0) d_s[h] = make_double2(a.d[h], __dmul_rn(a.d[h], -4503599627370496.0));
     }
     for (int g = tid; g < G; g += 32 * kFsWarps) cap_s[g] = a.cap ? a.cap[inst * G + g] : 1;
@@ -99,9 +110,12 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
     const int s0 = lane < cnt ? __ldg(s + lane) : 1, s1 = lane + 32 < cnt ? __ldg(s + lane + 32) : 1;
     const int o0 = max(s0, 0), o1 = max(s1, 0);                       // (lengths are positive; margins are never negative)
     const double aDs0 = FP ? __dmul_rn(a.aD, (double)s0) : (double)s0, aDs1 = FP ? __dmul_rn(a.aD, (double)s1) : (double)s1;
+    // a worker whose smallest margin is not below the warp's longest request scores alpha D s: no term is positive
+    const int longest = FP ? __reduce_max_sync(kFull, max(o0, o1)) : 0;
     const double mGl = -(double)G;
     long long k0 = kNoKey, k1 = kNoKey;
     int b0 = kNoIdx, b1 = kNoIdx;
+    double q0 = 0.0, q1 = 0.0;
 #pragma unroll 1
     for (int gc = sub * span; gc < g_end && cnt > 0; gc += kFsCols) {
         const int cols = min(kFsCols, g_end - gc);
@@ -116,7 +130,7 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
                 f1 = __fma_rn(mGl, (double)__viaddmax_s32(o1, m, 0), aDs1);
             } else {
                 double p0 = 0.0, p1 = 0.0;
-                int h = 0;
+                int h = longest + low_s[g] > 0 ? 0 : H1;
 #pragma unroll 2
                 for (; h + 4 <= H1; h += 4) {
                     const int4 m4 = *reinterpret_cast<const int4 *>(mg + h);
@@ -141,9 +155,8 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
             stage[lane * (kFsCols + 1) + x] = f0;
             stage[(lane + 32) * (kFsCols + 1) + x] = f1;
             if (a.best_g && cap_s[g] > 0) {                                       // g ascends: the lower worker is kept on ties
-                const long long c0 = key_of_double(f0), c1 = key_of_double(f1);
-                if (c0 > k0) { k0 = c0; b0 = g; }
-                if (c1 > k1) { k1 = c1; b1 = g; }
+                if (f0 > q0 || b0 == kNoIdx) { q0 = f0; b0 = g; }
+                if (f1 > q1 || b1 == kNoIdx) { q1 = f1; b1 = g; }
             }
         }
         __syncwarp();
@@ -160,6 +173,8 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
         __syncwarp();
     }
     if (a.best_g) {
+        if (b0 != kNoIdx) k0 = key_of_double(q0);
+        if (b1 != kNoIdx) k1 = key_of_double(q1);
         if (split > 1) {
             long long *ks = reinterpret_cast<long long *>(stage);
             int *is = reinterpret_cast<int *>(stage + kFsReq);

@@ -48,6 +48,36 @@ def test_fscore_matrix_and_best_worker(name, H):
     r.close()
 
 
+@pytest.mark.parametrize("G", [1, 2, 7, 9, 33, 64])
+@pytest.mark.parametrize("H", [0, 3, 4, 18])
+@pytest.mark.parametrize("n_req", [4, 60, 64, 260])
+def test_fscore_edges(G, H, n_req):
+    # requests at a worker's smallest margin and one token on either side of it, loads beyond 32 bits (the order of
+    # the terms and every rounding is the checker's: equality)
+    cfg = wlm.get_config("c2", G=G, H=H, init_active=2, init_queue=0, term_mode=1, score_mode=1)
+    r = Router(wlm.make_workload(cfg, n_instances=1), device="cuda:0")
+    rng = np.random.default_rng(G + 100 * H + n_req)
+    N = 3
+    Lh = rng.integers(1000, 9000, (N, G, H + 1)).astype(np.int64)
+    Lh[1] += np.int64(1) << 40
+    Lh[2, G - 1] += np.int64(1) << 34
+    mm = (Lh.max(axis=1, keepdims=True) - Lh).min(axis=2)
+    s = np.clip(mm[:, rng.integers(0, G, n_req)] + rng.integers(-1, 2, (N, n_req)), 1, 200000).astype(np.int32)
+    s[:, 0] = 1
+    st, Lt = torch.from_numpy(s).cuda(), torch.from_numpy(Lh).cuda()
+    F = torch.zeros((N, n_req, G), dtype=torch.float64, device="cuda")
+    best = torch.full((N, n_req), -7, dtype=torch.int32, device="cuda")
+    r.fscore(st, Lt, F, best_g=best)
+    Fh, bh = F.cpu().numpy(), best.cpu().numpy()
+    for n in range(N):
+        M = Lh[n].max(axis=0)
+        for i in list(range(0, n_req, 7)) + [n_req - 1]:
+            ref = np.array([oracle.f_brh(H, cfg.alpha, cfg.beta, cfg.gamma, int(s[n, i]), M - Lh[n, g]) for g in range(G)])
+            assert np.array_equal(Fh[n, i], ref), (n, i)
+            assert bh[n, i] == int(np.argmax(ref)), (n, i)
+    r.close()
+
+
 @pytest.mark.parametrize("G,score_mode", [(32, 0), (64, 0), (5, 0), (16, 1)])
 def test_pool_bypass_dispatch(G, score_mode):
     """br_bypass_dispatch against the checker: workers, virtual loads and inflight counts."""
