@@ -84,11 +84,11 @@ def lib():
         L.br_graph_step.argtypes = [C.c_void_p]
         L.br_step_host.argtypes = step_args + [C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
         L.br_step_host_static.argtypes = step_args + [C.POINTER(C.c_int64), C.POINTER(C.c_int64)]
-        L.br_fscore.argtypes = [C.c_void_p, C.POINTER(BrInstanceBatch), C.c_void_p, C.c_int32,
+        L.br_fscore.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32,
                                 C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         L.br_best_subset.argtypes = [C.c_void_p, C.POINTER(BrInstanceBatch), C.c_void_p, C.c_int32,
                                      C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
-        L.br_bypass_dispatch.argtypes = [C.c_void_p, C.POINTER(BrInstanceBatch), C.c_void_p, C.c_int32,
+        L.br_bypass_dispatch.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32,
                                          C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]
         L.br_survival_chat.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_void_p,
                                        C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p]
@@ -308,19 +308,18 @@ class Router:
         return up.value, down.value
 
     def fscore(self, s, Lh, F, cap=None, best_g=None, N=None, first=0, stream=None):
-        N = s.shape[0] - first if N is None else N
-        b = BrInstanceBatch(n_instances=N, first_instance=first, n_steps=1, stream=self._stream(stream))
-        rc = lib().br_fscore(self._h, C.byref(b), _ptr(s), int(s.shape[1]), _ptr(Lh), _ptr(cap),
-                             _ptr(F), _ptr(best_g))
+        n, n_req = s.shape
+        b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
+        rc = lib().br_fscore(self._h, b, _addr(s), n_req, _addr(Lh), _addr(cap), _addr(F), _addr(best_g))
         if rc != BR_OK:
             raise BrError(rc, "br_fscore")
 
 
     def bypass_dispatch(self, s, virtual_load, inflight, inflight_cap, worker_out, N=None, first=0, stream=None):
-        N = s.shape[0] - first if N is None else N
-        b = BrInstanceBatch(n_instances=N, first_instance=first, n_steps=1, stream=self._stream(stream))
-        rc = lib().br_bypass_dispatch(self._h, C.byref(b), _ptr(s), int(s.shape[1]), _ptr(virtual_load),
-                                      _ptr(inflight), _ptr(inflight_cap), _ptr(worker_out))
+        n, n_req = s.shape
+        b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
+        rc = lib().br_bypass_dispatch(self._h, b, _addr(s), n_req, _addr(virtual_load), _addr(inflight),
+                                      _addr(inflight_cap), _addr(worker_out))
         if rc != BR_OK:
             raise BrError(rc, "br_bypass_dispatch")
 

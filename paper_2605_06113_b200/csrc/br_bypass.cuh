@@ -27,10 +27,11 @@ struct BypassArgs {
 // definition allows.  Eq. 1 falls strictly beyond the margin (G >= 2; one worker needs no order), so
 // argmax_g F_g(s) is the first worker with the largest min(m_g, s): one warp maximum over
 // (min(m_g, s), 63 - g) gives the worker, and its upper part the growth of the envelope,
-// s - min(m_g, s).  Eq. 2 scores, whose rounding may tie, and lengths outside [0, 2^25), which do not
-// fit that key, are scored in full.  Prompt lengths are read and answers written 32 at a time.
+// s - min(m_g, s).  Eq. 2 scores, whose rounding may tie, lengths outside [0, 2^25), which do not fit that
+// key, and margins of 2^30 and more are handled in full.  Prompt lengths are read and answers written 32 at
+// a time, and the next length is fetched while the warp maximum is on its way.
 // 256 instances x 200 requests at G = 32: 74 us with the envelope and a 64-bit score reduced over the warp
-// for every request, 19 us this way.
+// for every request, 19 us with 64-bit margins, 12 this way.
 // FP: Eq. 2 scores; GW: workers per lane.
 template <bool FP, int GW>
 __global__ void __launch_bounds__(32) br_bypass_kernel(const BypassArgs a)
@@ -66,28 +67,39 @@ __global__ void __launch_bounds__(32) br_bypass_kernel(const BypassArgs a)
         const int mine = next, cnt = min(32, a.n_req - i0);
         if (i0 + 32 + lane < a.n_req) next = __ldg(s + i0 + 32 + lane);
         int answer = -1;
-        if (!FP && __all_sync(kFull, (unsigned)mine < (1u << 25))) {
-#pragma unroll 1
+        bool packed = !FP && (unsigned)mine < (1u << 25);
+#pragma unroll
+        for (int w = 0; w < GW; ++w) packed = packed && (m[w] < (1ll << 30) || lane + 32 * w >= G);
+        if (__all_sync(kFull, packed)) {
+            // margins stay below 2^31 for 32 requests
+            int mi[GW], added[GW];
+#pragma unroll
+            for (int w = 0; w < GW; ++w) { mi[w] = (int)m[w]; added[w] = 0; }
+            int si = __shfl_sync(kFull, mine, 0);
+#pragma unroll 2
             for (int i = 0; i < cnt; ++i) {
-                const int si = __shfl_sync(kFull, mine, i);
-                unsigned key = 0u;                                       // every worker at its cap
+                const int after = __shfl_sync(kFull, mine, (i + 1) & 31);
+                unsigned kw[GW], key = 0u;                                // 0: every worker at its cap
 #pragma unroll
                 for (int w = 0; w < GW; ++w) {
-                    const unsigned c = m[w] < (long long)si ? (unsigned)m[w] : (unsigned)si;
-                    if (nfl[w] < cap[w]) key = max(key, (c << 6) + (unsigned)(64 - lane - 32 * w));
+                    kw[w] = nfl[w] < cap[w] ? ((unsigned)min(mi[w], si) << 6) + (unsigned)(64 - lane - 32 * w) : 0u;
+                    key = max(key, kw[w]);
                 }
                 key = __reduce_max_sync(kFull, key);
                 if (key == 0u) break;                                    // ... and none opens again
-                const int g = 63 - (int)((key - 1u) & 63u), grow = si - (int)((key - 1u) >> 6);
+                const int grow = si - (int)((key - 1u) >> 6);
 #pragma unroll
                 for (int w = 0; w < GW; ++w) {
-                    const int it_is = g == lane + 32 * w ? 1 : 0;
-                    m[w] += grow - (it_is ? si : 0);
-                    L[w] += it_is ? si : 0;
-                    nfl[w] += it_is;
+                    const bool it_is = kw[w] == key;                     // (the worker is part of the key)
+                    mi[w] += it_is ? grow - si : grow;
+                    added[w] += it_is ? si : 0;
+                    nfl[w] += it_is ? 1 : 0;
                 }
-                if (lane == i) answer = g;
+                if (lane == i) answer = 63 - (int)((key - 1u) & 63u);
+                si = after;
             }
+#pragma unroll
+            for (int w = 0; w < GW; ++w) { m[w] = mi[w]; L[w] += added[w]; }
         } else {
 #pragma unroll 1
             for (int i = 0; i < cnt; ++i) {
