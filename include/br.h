@@ -88,7 +88,7 @@ typedef struct {
     int32_t burst_every, burst_size; /* burst_size extra arrivals when k > 0 and k % burst_every == 0 */
     int32_t s_max;          /* largest prompt length the caller will ever enqueue (range proof) */
     int32_t threads;        /* threads per instance (multiple of 32, <= 256); <= 0 -> chosen from G*B, H and the batch size */
-    int32_t inst_per_block; /* instances per thread block when an instance runs on one warp (1..8); <= 0 -> 4 */
+    int32_t inst_per_block; /* instances per thread block of the one-warp BR-0 kernel (1..8); <= 0 -> 4 */
     int32_t pred_mode;      /* H > 0 only.  0: c_hat from the classifier output term_probs (Eqs. 3-5 and the
                                refresh rules); 1: c_hat = min(r_i(k), H) from the known lifetimes, the
                                perfect-lookahead reference of Section 5.1 "Our methods" (needs term_mode 3;
