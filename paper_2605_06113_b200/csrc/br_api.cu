@@ -722,7 +722,7 @@ int br_fscore(br_ctx *ctx, const br_instance_batch *batch, const int32_t *s, int
     for (int h = 0; h <= BR_MAX_H; ++h) a.d[h] = ctx->d[h];
     a.n_req = n_requests; a.first_instance = batch->first_instance;
     a.s = s; a.Lh = Lh; a.cap = cap; a.F = F; a.best_g = best_g;
-    a.split_log2 = br::fscore_split_log2(n_requests, batch->n_instances, ctx->G);
+    a.split_log2 = a.fp ? br::fscore_split_log2(n_requests, batch->n_instances, ctx->G) : 0;
     a.row = (ctx->H + 4) / 4 * 4;
     const int per_block = br::kFsReq * (br::kFsWarps >> a.split_log2);
     const dim3 grid((n_requests + per_block - 1) / per_block, batch->n_instances);

@@ -101,6 +101,44 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
     for (int g = tid; g < G; g += 32 * kFsWarps) cap_s[g] = a.cap ? a.cap[inst * G + g] : 1;
     __syncthreads();
 
+    if (!FP) {
+        // Eq. 1 is a write of the matrix: the warp's rows are one run, written 256 bytes at a time (in runs of eight
+        // workers per request it reached 0.91 of the copy bandwidth at 4,096 x 1,024 x 32 scores, this way 1.0).  The best workers are
+        // looked for again, two requests a lane; scoring is two integer instructions.
+        int *s_w = reinterpret_cast<int *>(stage);
+        const int r0 = (blockIdx.x * kFsWarps + warp) * kFsReq, cnt = min(kFsReq, a.n_req - r0);
+        if (cnt <= 0) return;
+        const int32_t *s = a.s + inst * a.n_req + r0;
+        for (int r = lane; r < cnt; r += 32) s_w[r] = __ldg(s + r);
+        __syncwarp();
+        auto score = [&](int si, int g) {                            // integers below 2^53, exact
+            return (double)((long long)si - (long long)G * (long long)__viaddmax_s32(max(si, 0), m_s[g * HS], 0));
+        };
+        double *F = a.F + (inst * a.n_req + r0) * G;
+        int r = lane / G, g = lane - r * G;
+        const int step_r = 32 / G, step_g = 32 - step_r * G;
+#pragma unroll 4
+        for (int o = lane; o < cnt * G; o += 32) {
+            F[o] = score(s_w[r], g);
+            r += step_r; g += step_g;
+            if (g >= G) { g -= G; ++r; }
+        }
+        if (a.best_g) {
+            int32_t *best = a.best_g + inst * a.n_req + r0;
+            for (int q = lane; q < cnt; q += 32) {
+                double top = 0.0;
+                int b = -1;
+#pragma unroll 4
+                for (int x = 0; x < G; ++x) {
+                    const double f = score(s_w[q], x);
+                    if (cap_s[x] > 0 && (b < 0 || f > top)) { top = f; b = x; }      // x ascends: the lower worker on ties
+                }
+                best[q] = b;
+            }
+        }
+        return;
+    }
+
     const int split = 1 << a.split_log2, sub = warp & (split - 1);
     const int r0 = (blockIdx.x * (kFsWarps >> a.split_log2) + (warp >> a.split_log2)) * kFsReq;
     const int cnt = min(kFsReq, a.n_req - r0);                        // not positive: nothing to do but the barrier
@@ -109,10 +147,9 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
     const int32_t *s = a.s + inst * a.n_req + r0;
     const int s0 = lane < cnt ? __ldg(s + lane) : 1, s1 = lane + 32 < cnt ? __ldg(s + lane + 32) : 1;
     const int o0 = max(s0, 0), o1 = max(s1, 0);                       // (lengths are positive; margins are never negative)
-    const double aDs0 = FP ? __dmul_rn(a.aD, (double)s0) : (double)s0, aDs1 = FP ? __dmul_rn(a.aD, (double)s1) : (double)s1;
+    const double aDs0 = __dmul_rn(a.aD, (double)s0), aDs1 = __dmul_rn(a.aD, (double)s1);
     // a worker whose smallest margin is not below the warp's longest request scores alpha D s: no term is positive
-    const int longest = FP ? __reduce_max_sync(kFull, max(o0, o1)) : 0;
-    const double mGl = -(double)G;
+    const int longest = __reduce_max_sync(kFull, max(o0, o1));
     long long k0 = kNoKey, k1 = kNoKey;
     int b0 = kNoIdx, b1 = kNoIdx;
     double q0 = 0.0, q1 = 0.0;
@@ -124,11 +161,7 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
             const int g = gc + x;
             const int *mg = m_s + g * HS;
             double f0, f1;
-            if (!FP) {
-                const int m = mg[0];
-                f0 = __fma_rn(mGl, (double)__viaddmax_s32(o0, m, 0), aDs0);       // Eq. 1: integers below 2^53, exact
-                f1 = __fma_rn(mGl, (double)__viaddmax_s32(o1, m, 0), aDs1);
-            } else {
+            {
                 double p0 = 0.0, p1 = 0.0;
                 int h = longest + low_s[g] > 0 ? 0 : H1;
 #pragma unroll 2
