@@ -94,7 +94,8 @@ constexpr int kHostWarps = 4;          // instances resident per SM when their r
 // warps pay off even for small ones, because the requests that end are drawn while warp 0 routes (84 of
 // G = 4, W = 56: 19.9 us with one warp, 15.2 with four).  When the batch puts several instances on an SM they
 // share its registers, which hold 21 warps (16 for long horizons): each takes its share, so that all are
-// resident (777 of G = 21, W = 300, three steps: 234 / 169 / 201 us with two / three / four warps).  Instances
+// resident (777 of G = 21, W = 300, three steps: 234 / 169 / 201 us with two / three / four warps); a second warp is
+// worth a few instances less (2,048 of G = 16, W = 512, H = 8: 102 us with one, 86 with two).  Instances
 // that stream 2,048 slots and more of classifier state are bound by memory while they do; fewer of them at a time
 // with more warps each, so that some stream while others route (1,024 of G = 64, H = 8: 77 us with three warps,
 // 64.5 with four, 63.0 with five, 85 with eight).
@@ -110,7 +111,8 @@ int threads_for(const br_ctx *ctx, int n_instances)
     int per_sm = (n_instances + kSMs - 1) / kSMs;
     const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
     if (per_sm > fit) per_sm = fit;
-    int w = (4 * (br::step_groups(ctx->H) ? 21 : 16) / per_sm + 1) / 4;
+    const int regs = br::step_groups(ctx->H) ? 21 : 16;                     // warps
+    int w = 2 * regs >= 3 * per_sm && regs < 2 * per_sm ? 2 : (4 * regs / per_sm + 1) / 4;
     if (ctx->H > 0 && ctx->p.pred_mode == 0 && A >= 2048 && w < 5) w = 5;
     w = w < 1 ? 1 : (w > most ? most : w);
     return 32 * w;

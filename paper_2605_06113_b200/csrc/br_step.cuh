@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 67 / 181 / 119 now.
+// the lanes' lists at every pop, 68 / 183 / 116 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -439,7 +439,6 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
     const auto fin = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.fin), G * OW);
     const auto endm = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.endm), G * OW);
     const auto endm32 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.endm), 2 * G * OW);
-    const auto endm8 = mk_span(smem + a.lay.endm, 8 * G * OW);
     const auto occ32 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.occ), 2 * G * OW);
     const auto L0_s = mk_span(reinterpret_cast<int *>(smem + a.lay.L0), G);
     const auto cap_s = mk_span(reinterpret_cast<int *>(smem + a.lay.cap), G);
@@ -772,40 +771,37 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
                     sub_load[g] = sub;
                 }
             } else if (a.term_mode >= 2) {
-                const unsigned A8 = (unsigned)A >> 3;
+                // quads in order: the rows that a warp reads lie side by side
+                const int A4 = A >> 2, B4 = B >> 2;
 #pragma unroll 1
-                for (unsigned o = t0; o < A8; o += nt) {
-                    const int p = (int)(o / (unsigned)G), g = (int)o - p * G, a0 = g * B + 8 * p;
-                    const unsigned ob = (unsigned)(occ0[g * OW + (p >> 3)] >> (8 * (p & 7))) & 0xFFu;
+                for (int q = t0; q < A4; q += nt) {
+                    const int g = (int)((unsigned)q / (unsigned)B4), slot = 4 * (q - g * B4);
+                    const unsigned ob = (unsigned)(occ0[g * OW + (slot >> 6)] >> (slot & 63)) & 0xFu;
                     unsigned fb = 0u;
                     if (life) {
                         // a request ends with its o_i-th step: act_end == k
-                        const int4 e0 = *vec_at<const int4>(g_end, a0), e1 = *vec_at<const int4>(g_end, a0 + 4);
-                        const int en[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) if (en[j] == k) fb |= 1u << j;
-                    } else {
+                        const int4 e = *vec_at<const int4>(g_end, 4 * q);
+                        fb = (e.x == k ? 1u : 0u) | (e.y == k ? 2u : 0u) | (e.z == k ? 4u : 0u) | (e.w == k ? 8u : 0u);
+                    } else if (ob) {
                         // Bernoulli(term_probs[slot][0]): 24-bit uniform below the probability
-#pragma unroll 1
-                        for (int half = 0; half < 2; ++half) {
-                            if (!((ob >> (4 * half)) & 0xFu)) continue;
-                            const uint4 r = philox_call((uint32_t)k, (uint32_t)((a0 >> 2) + half), kStreamTerm, key0, key1);
-                            const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+                        float p4[4];
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if ((ob >> (4 * half + j)) & 1u) {
-                                    const float q = probs[(size_t)(a0 + 4 * half + j) * H];
-                                    if (__fmul_rn((float)(rr[j] >> 8), 5.9604644775390625e-8f) < q) fb |= 1u << (4 * half + j);
-                                }
-                        }
+                        for (int j = 0; j < 4; ++j) p4[j] = probs[(size_t)(4 * q + j) * H];
+                        const uint4 r = philox_call((uint32_t)k, (uint32_t)q, kStreamTerm, key0, key1);
+                        const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if (__fmul_rn((float)(rr[j] >> 8), 5.9604644775390625e-8f) < p4[j]) fb |= 1u << j;
                     }
                     fb &= ob;
-                    endm8[g * OW * 8 + p] = (unsigned char)fb;
+                    if (fb) {
+                        atomicOr(&endm32[2 * g * OW + (slot >> 5)], fb << (slot & 31));
 #pragma unroll 1
-                    for (; fb; fb &= fb - 1u) {
-                        const int sa = a0 + __ffs(fb) - 1;
-                        atomicAdd(&sub_load[g], (unsigned)(g_base[sa] + k));
-                        g_base[sa] = kEmpty;
+                        for (; fb; fb &= fb - 1u) {
+                            const int sa = 4 * q + __ffs(fb) - 1;
+                            atomicAdd(&sub_load[g], (unsigned)(g_base[sa] + k));
+                            g_base[sa] = kEmpty;
+                        }
                     }
                 }
             }
@@ -868,6 +864,7 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
                 __syncwarp();
             };
             if (FP) {
+                __syncwarp();                          // every lane has read L_g(k) before rows become margins
                 rows(true);
 #pragma unroll
                 for (int c = 0; c < HC; ++c) if (lane + 32 * c < HS) Ms[lane + 32 * c] = 0;
