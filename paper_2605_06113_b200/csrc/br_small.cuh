@@ -116,6 +116,8 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         if (cap < 0 || cap > B) { status0 = BR_ST_BAD_STATE; cap = cap < 0 ? 0 : B; }
         cap = B - cap;
     }
+    // a worker whose occupancy word has fewer free slots than its count says may turn a request away below
+    const bool odd = __any_sync(kFull, lane < G && cap > __popcll(~occ));
     // ---- the queue moves to shared memory once per launch: packed keys and ids ----
 #pragma unroll
     for (int t = 0; t < NT4; ++t) {
@@ -309,7 +311,7 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
                         cap = 0;
                     }
                 }
-                Lg += s;
+                Lg = rare(odd) ? __shfl_sync(kFull, L, g) : Lg + s;     // (a request turned away adds no load)
                 M = max(M, Lg);
                 if (qk >= gw[RM - 1]) gw_valid = false;                 // a cached window entry leaves
                 first_rm = min(first_rm, pos);
