@@ -24,7 +24,7 @@ def _stale(lib: str = LIB) -> bool:
         return True
     t = os.path.getmtime(lib)
     # every file of csrc/ is a dependency: the kernels live in headers included by br_api.cu
-    deps = glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    deps = glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
     deps.append(os.path.join(os.path.dirname(HERE), "include", "br.h"))
     deps.append(os.path.abspath(__file__))
     return any(os.path.getmtime(d) > t for d in deps)

@@ -1,5 +1,6 @@
 // C-ABI entry points of the BalanceRoute routing library (declared in include/br.h).
 // Host side only validates, fills the kernel argument block and launches.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdio.h>
@@ -8,6 +9,7 @@
 #include <atomic>
 #include <new>
 
+#include "br_plan.h"
 #include "br_step.cuh"
 #include "br_small.cuh"
 #include "br_fscore.cuh"
@@ -480,21 +482,38 @@ int plan_host_step(const br_ctx *ctx, const br_instance_batch *batch, br_worker_
     return BR_OK;
 }
 
-// Device address of a host array that the kernels can use in place (page-locked memory, 16-byte aligned),
-// or NULL.  Both ends are looked up: a registration that ends inside the array does not count.
-void *device_alias(const void *host, size_t bytes)
+typedef CUresult (*pointer_attributes_t)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+
+pointer_attributes_t pointer_attributes()
 {
-    cudaPointerAttributes first, last;
-    if (!bytes || misaligned(host, 16)) return nullptr;
-    if (cudaPointerGetAttributes(&first, host) != cudaSuccess ||
-        cudaPointerGetAttributes(&last, (const char *)host + bytes - 1) != cudaSuccess) {
+    static const pointer_attributes_t fn = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &found) != cudaSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (pointer_attributes_t)f;
+    }();
+    return fn;
+}
+
+// the page-locked range around a host address; the runtime does not tell its extent, the driver does
+bool locked_range(uintptr_t host, br::LockedRange *r)
+{
+    cudaPointerAttributes attr;
+    if (cudaPointerGetAttributes(&attr, (const void *)host) != cudaSuccess) {
         cudaGetLastError();
-        return nullptr;
+        return false;
     }
-    if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
-        (char *)last.devicePointer - (char *)first.devicePointer != (ptrdiff_t)(bytes - 1) || misaligned(first.devicePointer, 16))
-        return nullptr;
-    return first.devicePointer;
+    if (attr.type != cudaMemoryTypeHost || !attr.devicePointer || !pointer_attributes()) return false;
+    r->dev = (uintptr_t)attr.devicePointer;
+    CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    CUdeviceptr start = 0; size_t size = 0;
+    void *to[2] = {&start, &size};
+    if (pointer_attributes()(2, what, to, (CUdeviceptr)r->dev) != CUDA_SUCCESS) return false;
+    r->start = (uintptr_t)start; r->size = size;
+    return true;
 }
 
 }  // namespace
@@ -524,9 +543,9 @@ int br_step_host(br_ctx *ctx, const br_instance_batch *batch, br_worker_state *h
     bool in_place = true;
     size_t total = 0;
     for (int i = 0; i < kStageBlks; ++i) {
-        void *alias = whole || blks[i].sparse ? device_alias(blks[i].host, blks[i].bytes) : nullptr;
-        direct[i] = alias != nullptr;
-        if (direct[i]) *blks[i].dev = alias;
+        const uintptr_t alias = whole || blks[i].sparse ? br::device_alias((uintptr_t)blks[i].host, blks[i].bytes, locked_range) : 0;
+        direct[i] = alias != 0;
+        if (direct[i]) *blks[i].dev = (void *)alias;
         else if (blks[i].bytes) { in_place = false; total += (blks[i].bytes + 255) & ~(size_t)255; }
     }
     if (total > ctx->stage_bytes) {

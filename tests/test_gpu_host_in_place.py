@@ -32,9 +32,10 @@ def test_in_place_matches_device_step(name, n_inst, kw, pinned):
     st_d, out_d = r.device_state(), r.outputs(n_inst)
     st_h = {k: host(k, v) for k, v in st_d.items()}
     out_h = {k: host(k, v) for k, v in out_d.items()}
+    moved = []
     for k in range(3):
         probs = torch.from_numpy(np.ascontiguousarray(wlm.term_probs_np(wl, k))) if cfg.H > 0 and cfg.pred_mode == 0 else None
-        r.step_host(st_h, out_h, None if probs is None else host("probs", probs))
+        moved.append(sum(r.step_host(st_h, out_h, None if probs is None else host("probs", probs))))
         r.step(st_d, out_d, None if probs is None else probs.cuda())
         torch.cuda.synchronize()
         for a, b in ((out_h, out_d), (st_h, st_d)):
@@ -42,4 +43,7 @@ def test_in_place_matches_device_step(name, n_inst, kw, pinned):
                 if cfg.pred_mode == 1 and key in ("act_chat0", "act_kref"):
                     continue                      # not part of a snapshot with known lifetimes: the host step leaves them alone
                 assert torch.equal(a[key], b[key].cpu()), (k, key)
+    # act_id of page-locked snapshots stays where it is: it is not among the bytes that move
+    every = 2 * sum(v.nbytes for v in st_h.values()) + sum(v.nbytes for v in out_h.values())
+    assert pinned != "all" or moved[0] < every - st_h["act_id"].nbytes + (0 if probs is None else probs.nbytes)
     r.close()
