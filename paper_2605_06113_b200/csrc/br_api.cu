@@ -168,6 +168,14 @@ cudaError_t launch_overlapped(step_kernel_t kern, int blocks, int threads, size_
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
+// Opts a kernel in to dynamic shared memory beyond the default 48 KB.  Always to the device's maximum: the limit is
+// the kernel's, shared by all contexts and threads of the process, and one that is set to what this launch needs
+// would be too low for a launch of another thread in between.
+cudaError_t opt_in_shared(step_kernel_t kern)
+{
+    return cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, br::kMaxShared);
+}
+
 int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *ws,
                 const br_waiting_queue *wq, const float *term_probs, int32_t *assign_out,
                 const br_load_out *out, cudaStream_t stream, bool overlap = true, bool host_rows = false)
@@ -198,8 +206,8 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
         if (host_rows && (b->n_instances > kHostWarps * kSMs)) {
             // rows in host memory: with few instances resident at a time, some read their snapshot while others
             // write theirs, and the bus is used in both directions
-            const size_t one = (size_t)227 * 1024 / (kHostWarps / wpb > 0 ? kHostWarps / wpb : 1) - 1024;
-            cudaError_t eo = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one);
+            const size_t one = (size_t)br::kMaxShared / (kHostWarps / wpb > 0 ? kHostWarps / wpb : 1) - 1024;
+            cudaError_t eo = opt_in_shared(kern);
             if (eo != cudaSuccess) return cuda_fail(eo, "cudaFuncSetAttribute(shared memory)");
             smem = one;
         }
@@ -215,8 +223,8 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
     while (a.seg_log2 < 5 && (ctx->G << (a.seg_log2 + 1)) <= threads && (2 << a.seg_log2) <= ctx->H + 1) ++a.seg_log2;
     const int smem = a.lay.total;
     if (smem > 48 * 1024) {
-        // beyond the default limit: opt the kernel in (br_create has checked the device maximum)
-        cudaError_t eo = cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // (br_create has checked the device maximum)
+        cudaError_t eo = opt_in_shared(kern);
         if (eo != cudaSuccess) return cuda_fail(eo, "cudaFuncSetAttribute(shared memory)");
     }
     cudaError_t e = launch_overlapped(kern, b->n_instances, threads, (size_t)smem, stream, a, overlap);
@@ -367,7 +375,7 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
     a.big_window = p.R_max > br::kRegWin ? 1 : 0;
     if (a.big_window && !ctx->two_probe_ok) { delete ctx; return BR_EINVAL; }
     a.lay = br::step_layout(G, H, p.B, p.W, a.occ_words, p.term_mode == 3, a.big_window != 0, H > 0 && p.pred_mode == 0);
-    if (a.lay.total > 227 * 1024) { delete ctx; return BR_EINVAL; }    // one instance must fit a thread block's shared memory
+    if (a.lay.total > br::kMaxShared) { delete ctx; return BR_EINVAL; }    // one instance must fit a thread block's shared memory
     // br_small_kernel: Eq. 1, one worker per lane, one occupancy word, at most 512 waiting requests,
     // arrivals served by one Philox call, and negative queue keys scoring below every waiting request
     ctx->small_ok = p.score_mode == 0 && G <= 32 && p.B <= 64 && p.W <= 512 && p.term_mode <= 1 && p.R_max <= br::kRegWin &&

@@ -5,6 +5,8 @@
 
 namespace br {
 
+constexpr int kMaxShared = 227 * 1024;     // dynamic shared memory of a thread block, at most
+
 // A page-locked allocation or registration around an address, in the device's address space.
 struct LockedRange {
     uintptr_t dev;         // device address of the address asked for
