@@ -233,6 +233,8 @@ class Router:
             if self._raw_stream is not None and self.device.index is not None:
                 return self._raw_stream(self.device.index)        # without building a stream object
             return self.torch.cuda.current_stream(self.device).cuda_stream
+        if isinstance(stream, C.c_void_p):
+            return stream.value
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
     # ---- the calls of include/br.h -------------------------------------------
@@ -308,7 +310,7 @@ class Router:
         return up.value, down.value
 
     def fscore(self, s, Lh, F, cap=None, best_g=None, N=None, first=0, stream=None):
-        n, n_req = s.shape
+        n, n_req = s.shape[0], s.shape[1]             # (trailing dimensions of one are fine)
         b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
         rc = lib().br_fscore(self._h, b, _addr(s), n_req, _addr(Lh), _addr(cap), _addr(F), _addr(best_g))
         if rc != BR_OK:
@@ -316,7 +318,7 @@ class Router:
 
 
     def bypass_dispatch(self, s, virtual_load, inflight, inflight_cap, worker_out, N=None, first=0, stream=None):
-        n, n_req = s.shape
+        n, n_req = s.shape[0], s.shape[1]             # (trailing dimensions of one are fine)
         b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
         rc = lib().br_bypass_dispatch(self._h, b, _addr(s), n_req, _addr(virtual_load), _addr(inflight),
                                       _addr(inflight_cap), _addr(worker_out))

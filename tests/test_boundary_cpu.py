@@ -101,3 +101,22 @@ def test_step_rejects_null_and_misaligned_pointers_without_touching_the_gpu():
     b.n_instances = 1
     assert L.br_step(h, C.byref(b), C.byref(ws), C.byref(wq), None, fake, C.byref(lo)) == BR_EINVAL
     L.br_destroy(h)
+
+
+def test_binding_takes_every_form_of_stream_and_of_prompt_lengths():
+    # batches of no instances: marshalled and validated, nothing launched
+    import torch
+    from paper_2605_06113_b200 import workload as wlm
+    cfg = wlm.get_config("c3", init_active=2, init_queue=2)
+    wl = wlm.make_workload(cfg, n_instances=1)
+    r = binding.Router(wl, device="cpu")
+    st, out = r.device_state(), r.outputs(1, device="cpu")
+    s = torch.zeros((1, 8, 1), dtype=torch.int32)
+    L = torch.zeros((1, cfg.G), dtype=torch.int64)
+    n = torch.zeros((1, cfg.G), dtype=torch.int32)
+    F = torch.zeros((1, 8, cfg.G), dtype=torch.float64)
+    for stream in (0, C.c_void_p(0), C.c_void_p(16)):
+        r.step(st, out, N=0, stream=stream)
+        r.fscore(s, L, F, N=0, stream=stream)
+        r.bypass_dispatch(s, L, n, n, torch.zeros((1, 8), dtype=torch.int32), N=0, stream=stream)
+    r.close()
