@@ -429,8 +429,7 @@ namespace {
 
 // One block of the staging area of the host-buffer entry points: a [N][row] array that goes up
 // before the kernel (in), comes down after it (out), or both.
-// sparse: a step reads and writes only the slots that change, a few per instance.
-struct StageBlk { size_t bytes; void **dev; void *host; bool in, out, sparse; };
+struct StageBlk { size_t bytes; void **dev; void *host; bool in, out; br::HostUse use; };
 constexpr int kStageBlks = 23;
 
 struct StagePlan {
@@ -464,8 +463,8 @@ int plan_host_step(const br_ctx *ctx, const br_instance_batch *batch, br_worker_
         {N * G * 8, (void **)&pl->dws.load, hws->load, true, true},
         {N * G * 4, (void **)&pl->dws.nact, hws->nact, true, true},
         {N * G * OW * 8, (void **)&pl->dws.occ, hws->occ, true, true},
-        {N * A * 4, (void **)&pl->dws.act_base, hws->act_base, true, true, H == 0 && !life},
-        {hws->act_id ? N * A * 4 : 0, (void **)&pl->dws.act_id, hws->act_id, true, true, true},
+        {N * A * 4, (void **)&pl->dws.act_base, hws->act_base, true, true, H == 0 && !life ? br::kHostSparse : br::kHostRows},
+        {hws->act_id ? N * A * 4 : 0, (void **)&pl->dws.act_id, hws->act_id, true, true, br::kHostSparse},
         {pred ? N * A * 4 : 0, (void **)&pl->dws.act_chat0, hws->act_chat0, true, true},
         {pred ? N * A : 0, (void **)&pl->dws.act_kref, hws->act_kref, true, true},
         {life ? N * A * 4 : 0, (void **)&pl->dws.act_end, hws->act_end, true, true},
@@ -482,7 +481,7 @@ int plan_host_step(const br_ctx *ctx, const br_instance_batch *batch, br_worker_
         {N * 3 * 8, (void **)&pl->dout.trace, hout->trace, false, true},
         {hout->status ? N * 4 : 0, (void **)&pl->dout.status, hout->status, false, true},
         {hout->counters ? N * 16 : 0, (void **)&pl->dout.counters, hout->counters, false, true},
-        {hout->fscore ? N * W * G * 8 : 0, (void **)&pl->dout.fscore, hout->fscore, false, true},
+        {hout->fscore ? N * W * G * 8 : 0, (void **)&pl->dout.fscore, hout->fscore, false, true, br::kHostScores},
         {hout->phase_cycles ? N * 32 : 0, (void **)&pl->dout.phase_cycles, hout->phase_cycles, false, true},
     };
     pl->total = 0;
@@ -540,18 +539,12 @@ int br_step_host(br_ctx *ctx, const br_instance_batch *batch, br_worker_state *h
     Blk (&blks)[kStageBlks] = pl.blk;
     br_worker_state &dws = pl.dws; br_waiting_queue &dwq = pl.dwq; br_load_out &dout = pl.dout;
     float *&d_probs = pl.d_probs; int32_t *&d_assign = pl.d_assign;
-    // Page-locked arrays are used in place where that moves less or saves copies: BR-0 reads and writes every
-    // row once, at the rate of the copy engines (50 GB/s measured either way), and of the sparse arrays only
-    // the slots that change (3 ns each against 150 ns for the 8 KB of an instance).  4,096 instances of G = 32,
-    // W = 256: 2.4 ms with every array copied both ways, 0.84 with only the sparse ones in place, 0.48 with
-    // all.  BR-H in large batches reads its snapshot and its classifier rows in smaller pieces than the bus
-    // likes and copies them; small batches save the copies' call time (16 instances: 147 us -> 47).
-    const bool whole = (ctx->H == 0 && ctx->p.term_mode <= 1) || N < 64;
     bool direct[kStageBlks];
     bool in_place = true;
     size_t total = 0;
     for (int i = 0; i < kStageBlks; ++i) {
-        const uintptr_t alias = whole || blks[i].sparse ? br::device_alias((uintptr_t)blks[i].host, blks[i].bytes, locked_range) : 0;
+        const bool may = br::host_in_place(blks[i].use, ctx->H, ctx->p.term_mode, batch->n_instances);
+        const uintptr_t alias = may ? br::device_alias((uintptr_t)blks[i].host, blks[i].bytes, locked_range) : 0;
         direct[i] = alias != 0;
         if (direct[i]) *blks[i].dev = (void *)alias;
         else if (blks[i].bytes) { in_place = false; total += (blks[i].bytes + 255) & ~(size_t)255; }
@@ -571,8 +564,8 @@ int br_step_host(br_ctx *ctx, const br_instance_batch *batch, br_worker_state *h
         off += (b.bytes + 255) & ~(size_t)255;
     }
     for (int i = 0; i < kStageBlks; ++i) {                  // (of a sparse array in place only a few slots move)
-        if (blks[i].in && !(direct[i] && blks[i].sparse)) up += (int64_t)blks[i].bytes;
-        if (blks[i].out && !(direct[i] && blks[i].sparse)) down += (int64_t)blks[i].bytes;
+        if (blks[i].in && !(direct[i] && blks[i].use == br::kHostSparse)) up += (int64_t)blks[i].bytes;
+        if (blks[i].out && !(direct[i] && blks[i].use == br::kHostSparse)) down += (int64_t)blks[i].bytes;
     }
     br_instance_batch db = *batch; db.n_steps = 1;
     rc = check_step_args(ctx, &db, &dws, &dwq, d_probs, d_assign, &dout);

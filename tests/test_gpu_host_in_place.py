@@ -1,5 +1,7 @@
 """br_step_host on page-locked buffers, which the kernels use in place, on pageable ones, which are copied, and on a
 mixture: state and outputs equal those of br_step on device buffers."""
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -46,4 +48,44 @@ def test_in_place_matches_device_step(name, n_inst, kw, pinned):
     # act_id of page-locked snapshots stays where it is: it is not among the bytes that move
     every = 2 * sum(v.nbytes for v in st_h.values()) + sum(v.nbytes for v in out_h.values())
     assert pinned != "all" or moved[0] < every - st_h["act_id"].nbytes + (0 if probs is None else probs.nbytes)
+    r.close()
+
+
+def _host_step_us(cfg, wl, place, fscore):
+    """Shortest host-buffer step on buffers that `place` makes from pageable ones."""
+    r = Router(wl, device="cuda:0")
+    n = wl.state["step"].shape[0]
+    st = {k: place(v.cpu()) for k, v in r.device_state().items()}
+    out = {k: place(v) for k, v in r.outputs(n, device="cpu", fscore=fscore).items()}
+    probs = place(torch.full((n, cfg.G, cfg.B, cfg.H), 0.02)) if cfg.H else None
+    best = 1e30
+    for _ in range(9):
+        t0 = time.perf_counter()
+        r.step_host(st, out, probs)
+        best = min(best, time.perf_counter() - t0)
+    r.close()
+    return 1e6 * best
+
+
+def test_score_matrix_is_not_slower_page_locked():
+    # written an element at a time (in place it took 2.4 times as long as from pageable memory)
+    cfg = wlm.get_config("c3")
+    wl = wlm.make_workload(cfg, n_instances=512)
+    assert _host_step_us(cfg, wl, torch.Tensor.pin_memory, True) < _host_step_us(cfg, wl, lambda t: t.clone(), True)
+
+
+@pytest.mark.parametrize("name,n_inst", [("c3", 3), ("c3", 520), ("c2", 3)])
+def test_score_matrix_to_page_locked_memory(name, n_inst):
+    cfg = wlm.get_config(name)
+    wl = wlm.make_workload(cfg, n_instances=n_inst)
+    r = Router(wl, device="cuda:0")
+    st_d, out_d = r.device_state(), r.outputs(n_inst, fscore=True)
+    st_h = {k: v.cpu().pin_memory() for k, v in st_d.items()}
+    out_h = {k: v.cpu().pin_memory() for k, v in out_d.items()}
+    probs = torch.from_numpy(np.ascontiguousarray(wlm.term_probs_np(wl, 0))) if cfg.H else None
+    r.step_host(st_h, out_h, None if probs is None else probs.pin_memory())
+    r.step(st_d, out_d, None if probs is None else probs.cuda())
+    for a, b in ((out_h, out_d), (st_h, st_d)):
+        for key in a:
+            assert torch.equal(a[key], b[key].cpu()), key
     r.close()

@@ -21,6 +21,10 @@ extern "C" uintptr_t alias(uintptr_t host, size_t bytes, int n, const uintptr_t 
         return false;
     });
 }
+extern "C" int in_place(int use, int H, int term_mode, long long n)
+{
+    return br::host_in_place((br::HostUse)use, H, term_mode, n);
+}
 """
 
 
@@ -57,3 +61,16 @@ def test_arrays_are_used_in_place_only_where_every_byte_is_page_locked(plan):
     assert _alias(plan, base + P, 6 * P, [(base, 2 * P, 64), (base + 2 * P, 6 * P, 64)]) == base + P + 64
     assert _alias(plan, base + P, 6 * P, [(base, 2 * P, 0), (base + 2 * P, 6 * P, P)]) == 0
     assert _alias(plan, base, 16, [(base, P, 8)]) == 0                            # the device address is not aligned
+
+
+def test_which_page_locked_arrays_are_used_in_place(plan):
+    rows, sparse, scores = 0, 1, 2
+
+    def in_place(use, H, term, n):
+        return bool(plan.in_place(use, H, term, C.c_longlong(n)))
+
+    for H, term, n in ((0, 1, 1), (0, 0, 4096), (8, 2, 40), (80, 3, 4096)):
+        assert not in_place(scores, H, term, n)          # an element at a time over the bus
+        assert in_place(sparse, H, term, n)
+    assert in_place(rows, 0, 1, 4096) and in_place(rows, 8, 1, 63) and in_place(rows, 80, 3, 63)
+    assert not in_place(rows, 8, 1, 64) and not in_place(rows, 0, 3, 64)
