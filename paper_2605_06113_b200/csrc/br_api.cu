@@ -543,7 +543,7 @@ int br_step_host(br_ctx *ctx, const br_instance_batch *batch, br_worker_state *h
     bool in_place = true;
     size_t total = 0;
     for (int i = 0; i < kStageBlks; ++i) {
-        const bool may = br::host_in_place(blks[i].use, ctx->H, ctx->p.term_mode, batch->n_instances);
+        const bool may = br::host_in_place(blks[i].use, ctx->H, ctx->p.term_mode, batch->n_instances, (long long)ctx->G * ctx->p.B);
         const uintptr_t alias = may ? br::device_alias((uintptr_t)blks[i].host, blks[i].bytes, locked_range) : 0;
         direct[i] = alias != 0;
         if (direct[i]) *blks[i].dev = (void *)alias;

@@ -42,12 +42,15 @@ enum HostUse { kHostRows, kHostSparse, kHostScores };
 // against 150 ns for the 8 KB of an instance).  4,096 instances of G = 32, W = 256: 2.4 ms with every array copied
 // both ways, 0.84 with only the sparse ones in place, 0.48 with all.  BR-H in large batches reads its snapshot
 // and its classifier rows in smaller pieces than the bus likes and copies them; small batches save the
-// copies' call time (16 instances: 147 us -> 47).  Scores go out eight bytes at a time: 1,024 instances of G = 32, W = 256: 19.4 ms in place, 2.0 copied.
-inline bool host_in_place(HostUse use, int H, int term_mode, long long n_instances)
+// copies' call time (16 instances: 147 us -> 47).  Terminations drawn from the classifier's output read every row in
+// pieces, which costs more than those calls beyond about 100,000 slots (G = 64, H = 8, B = 64, us in place / copied:
+// 224 / 276 at 16 instances, 456 / 380 at 40, 656 / 487 at 63; H = 16, B = 256: 294 / 382 at 4, 750 / 632 at 16).
+// Scores go out eight bytes at a time: 1,024 instances of G = 32, W = 256: 19.4 ms in place, 2.0 copied.
+inline bool host_in_place(HostUse use, int H, int term_mode, long long n_instances, long long slots_per_instance)
 {
     if (use == kHostScores) return false;
     if (use == kHostSparse || (H == 0 && term_mode <= 1)) return true;
-    return n_instances < 64;
+    return n_instances < 64 && (term_mode != 2 || n_instances * slots_per_instance <= 100000);
 }
 
 }  // namespace br

@@ -21,9 +21,9 @@ extern "C" uintptr_t alias(uintptr_t host, size_t bytes, int n, const uintptr_t 
         return false;
     });
 }
-extern "C" int in_place(int use, int H, int term_mode, long long n)
+extern "C" int in_place(int use, int H, int term_mode, long long n, long long slots)
 {
-    return br::host_in_place((br::HostUse)use, H, term_mode, n);
+    return br::host_in_place((br::HostUse)use, H, term_mode, n, slots);
 }
 """
 
@@ -66,11 +66,13 @@ def test_arrays_are_used_in_place_only_where_every_byte_is_page_locked(plan):
 def test_which_page_locked_arrays_are_used_in_place(plan):
     rows, sparse, scores = 0, 1, 2
 
-    def in_place(use, H, term, n):
-        return bool(plan.in_place(use, H, term, C.c_longlong(n)))
+    def in_place(use, H, term, n, slots):
+        return bool(plan.in_place(use, H, term, C.c_longlong(n), C.c_longlong(slots)))
 
-    for H, term, n in ((0, 1, 1), (0, 0, 4096), (8, 2, 40), (80, 3, 4096)):
-        assert not in_place(scores, H, term, n)          # an element at a time over the bus
-        assert in_place(sparse, H, term, n)
-    assert in_place(rows, 0, 1, 4096) and in_place(rows, 8, 1, 63) and in_place(rows, 80, 3, 63)
-    assert not in_place(rows, 8, 1, 64) and not in_place(rows, 0, 3, 64)
+    for H, term, n, slots in ((0, 1, 1, 2048), (0, 0, 4096, 2048), (8, 2, 40, 4096), (80, 3, 4096, 512)):
+        assert not in_place(scores, H, term, n, slots)          # an element at a time over the bus
+        assert in_place(sparse, H, term, n, slots)
+    assert in_place(rows, 0, 1, 4096, 4096) and in_place(rows, 8, 1, 63, 16384) and in_place(rows, 80, 3, 63, 16384)
+    assert not in_place(rows, 8, 1, 64, 64) and not in_place(rows, 0, 3, 64, 64)
+    # terminations drawn from every classifier row
+    assert in_place(rows, 8, 2, 24, 4096) and not in_place(rows, 8, 2, 25, 4096) and not in_place(rows, 16, 2, 63, 16384)
