@@ -744,9 +744,9 @@ int br_fscore(br_ctx *ctx, const br_instance_batch *batch, const int32_t *s, int
     for (int h = 0; h <= BR_MAX_H; ++h) a.d[h] = ctx->d[h];
     a.n_req = n_requests; a.first_instance = batch->first_instance;
     a.s = s; a.Lh = Lh; a.cap = cap; a.F = F; a.best_g = best_g;
-    a.split_log2 = a.fp ? br::fscore_split_log2(n_requests, batch->n_instances, ctx->G) : 0;
+    a.split_log2 = br::fscore_split_log2(a.fp, n_requests, batch->n_instances, ctx->G);
     a.row = (ctx->H + 4) / 4 * 4;
-    const int per_block = br::kFsReq * (br::kFsWarps >> a.split_log2);
+    const int per_block = (br::kFsReq * br::kFsWarps) >> a.split_log2;
     const dim3 grid((n_requests + per_block - 1) / per_block, batch->n_instances);
     const int smem = br::fscore_smem(ctx->G, a.row);                      // at most 42 KB
     void (*kern)(const br::FscoreArgs) = a.fp ? br::br_fscore_kernel<true> : br::br_fscore_kernel<false>;

@@ -16,7 +16,7 @@ struct FscoreArgs {
     double aD, beta;
     double d[BR_MAX_H + 1];
     int32_t n_req, first_instance;
-    int32_t split_log2;    // log2 of the warps that share 64 requests, each with a stretch of workers
+    int32_t split_log2;    // log2 of the warps that share 64 requests, each with a stretch of workers (Eq. 1: of requests)
     int32_t row;           // row stride of the margins in shared memory
     const int32_t *s;      // [N][n_req]
     const int64_t *Lh;     // [N][G][H+1]
@@ -42,12 +42,15 @@ __device__ __forceinline__ long long fscore_key(const FscoreArgs &a, int delta, 
     return key_of_double(__dsub_rn(__dmul_rn(a.aD, dl), __dmul_rn(a.beta, pen)));
 }
 
-// Warps that share 64 requests: one where there are warps enough, up to four where short calls would
-// leave the schedulers with fewer than four each.
-inline int fscore_split_log2(int n_req, int n_instances, int G)
+// Warps that share 64 requests: one where there are warps enough, up to four (Eq. 1: eight) where short calls would
+// leave the schedulers with fewer than four each.  Eq. 2 splits the workers, Eq. 1, whose warps write whole
+// runs of the matrix, the requests (16 x 100 x 64 scores: 10.9 us with one thread per element of a
+// block's rows, 14.5 with 64 requests per warp, 8.3 with eight).
+inline int fscore_split_log2(bool fp, int n_req, int n_instances, int G)
 {
     int l = 0;
-    while (l < 2 && (kFsCols << l) < G && ((long long)n_instances * ((n_req + kFsReq - 1) / kFsReq) << l) < 4ll * 4 * 148) ++l;
+    while (l < (fp ? 2 : 3) && (!fp || (kFsCols << l) < G) &&
+           ((long long)n_instances * ((n_req + kFsReq - 1) / kFsReq) << l) < 4ll * 4 * 148) ++l;
     return l;
 }
 // margin rows [g][h], (d_h, -2^52 d_h) pairs, one staging area per warp
@@ -106,7 +109,8 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
         // workers per request it reached 0.91 of the copy bandwidth at 4,096 x 1,024 x 32 scores, this way 1.0).  The best workers are
         // looked for again, two requests a lane; scoring is two integer instructions.
         int *s_w = reinterpret_cast<int *>(stage);
-        const int r0 = (blockIdx.x * kFsWarps + warp) * kFsReq, cnt = min(kFsReq, a.n_req - r0);
+        const int per_warp = kFsReq >> a.split_log2;
+        const int r0 = (blockIdx.x * kFsWarps + warp) * per_warp, cnt = min(per_warp, a.n_req - r0);
         if (cnt <= 0) return;
         const int32_t *s = a.s + inst * a.n_req + r0;
         for (int r = lane; r < cnt; r += 32) s_w[r] = __ldg(s + r);

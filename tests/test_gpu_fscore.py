@@ -78,6 +78,38 @@ def test_fscore_edges(G, H, n_req):
     r.close()
 
 
+@pytest.mark.parametrize("G", [1, 2, 7, 9, 31, 33, 64])
+@pytest.mark.parametrize("N,n_req", [(1, 4), (3, 60), (3, 64), (2, 260), (40, 1100)])
+@pytest.mark.parametrize("with_cap", [False, True])
+def test_fscore_edges_in_integers(G, N, n_req, with_cap):
+    # Eq. 1: the walk over (request, worker) at every remainder of 32 by G, warps with 64 requests and with fewer, and the
+    # best worker among all and among those with room
+    cfg = wlm.get_config("c3", G=G, init_active=2, init_queue=0)
+    assert cfg.score_mode == 0
+    r = Router(wlm.make_workload(cfg, n_instances=1), device="cuda:0")
+    rng = np.random.default_rng(G + 7 * n_req)
+    Lh = rng.integers(1000, 9000, (N, G, 1)).astype(np.int64)
+    if N > 1:
+        Lh[1] += np.int64(1) << 40
+    m = Lh.max(axis=1, keepdims=True) - Lh
+    s = np.clip(m[:, rng.integers(0, G, n_req), 0] + rng.integers(-1, 2, (N, n_req)), 1, 200000).astype(np.int32)
+    cap = rng.integers(0, 2, (N, G)).astype(np.int32)
+    cap[0] = 0
+    st, Lt, ct = (torch.from_numpy(x).cuda() for x in (s, Lh, cap))
+    F = torch.zeros((N, n_req, G), dtype=torch.float64, device="cuda")
+    best = torch.full((N, n_req), -7, dtype=torch.int32, device="cuda")
+    r.fscore(st, Lt, F, cap=ct if with_cap else None, best_g=best)
+    ref = np.array([[[oracle.f_br0(G, int(x), int(y)) for y in m[n, :, 0]] for x in s[n]] for n in range(min(N, 3))], dtype=np.float64)
+    over = np.maximum(s[:, :, None].astype(np.int64) - m[:, None, :, 0], 0)
+    every = (s[:, :, None].astype(np.int64) - G * over).astype(np.float64)
+    assert np.array_equal(ref, every[:3])
+    assert np.array_equal(F.cpu().numpy(), every)
+    room = cap > 0 if with_cap else np.ones((N, G), dtype=bool)
+    masked = np.where(room[:, None, :], every, -np.inf)
+    assert np.array_equal(best.cpu().numpy(), np.where(room.any(axis=1)[:, None], masked.argmax(axis=2), -1))
+    r.close()
+
+
 @pytest.mark.parametrize("G,score_mode", [(32, 0), (64, 0), (5, 0), (16, 1)])
 def test_pool_bypass_dispatch(G, score_mode):
     """br_bypass_dispatch against the checker: workers, virtual loads and inflight counts."""
