@@ -80,27 +80,41 @@ __global__ void __launch_bounds__(32 * kFsWarps) br_fscore_kernel(const FscoreAr
         for (int g = tid; g < G; g += 32 * kFsWarps) low_s[g] = (int)0x80000000;
         __syncthreads();
     }
-    // margins: one warp per offset, lanes over workers
-    for (int h = warp; h < H1; h += kFsWarps) {
-        const int64_t *row = a.Lh + inst * G * (a.H + 1) + h;
+    // margins: one warp per four offsets, lanes over workers; the loads of the four are asked for together (one offset
+    // at a time, the trips to memory of a long horizon came one after the other: 16 x 100 requests, G = 1,
+    // H = 80: 8.6 us with whole rows staged at once, 12.4, 8.3 this way)
+    for (int h0 = 4 * warp; h0 < H1; h0 += 4 * kFsWarps) {
+        const int64_t *row = a.Lh + inst * G * (a.H + 1) + h0;
         const long long none = (long long)0x8000000000000000ull;
-        const long long L0 = lane < G ? row[(size_t)lane * (a.H + 1)] : none;
-        const long long L1 = lane + 32 < G ? row[(size_t)(lane + 32) * (a.H + 1)] : none;
-        long long M = L0 > L1 ? L0 : L1;
-        for (int o = 16; o > 0; o >>= 1) {
-            const long long v = __shfl_xor_sync(kFull, M, o);
-            M = v > M ? v : M;
-        }
+        long long L[2][4];
 #pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            const int g = lane + 32 * w;
-            if (g >= G) continue;
-            const int v = -(int)min(M - (w ? L1 : L0), 0x7FFFFFFFll);
-            m_s[g * HS + h] = v;
-            if (FP) atomicMax(&low_s[g], v);
-        }
-        if (lane == 0) d_s[h] = make_double2(a.d[h], __dmul_rn(a.d[h], -4503599627370496.0));
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const int g = lane + 32 * w;
+                L[w][j] = g < G && h0 + j < H1 ? row[(size_t)g * (a.H + 1) + j] : none;
+            }
+        long long M[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) M[j] = L[0][j] > L[1][j] ? L[0][j] : L[1][j];
+        for (int o = 1; o < 32 && o < G; o <<= 1)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const long long v = __shfl_xor_sync(kFull, M[j], o);
+                M[j] = v > M[j] ? v : M[j];
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const int g = lane + 32 * w;
+                if (g >= G || h0 + j >= H1) continue;
+                const int v = -(int)min(M[j] - L[w][j], 0x7FFFFFFFll);
+                m_s[g * HS + h0 + j] = v;
+                if (FP) atomicMax(&low_s[g], v);
+            }
     }
+    for (int h = tid; h < H1; h += 32 * kFsWarps) d_s[h] = make_double2(a.d[h], __dmul_rn(a.d[h], -4503599627370496.0));
     for (int g = tid; g < G; g += 32 * kFsWarps) cap_s[g] = a.cap ? a.cap[inst * G + g] : 1;
     __syncthreads();
 

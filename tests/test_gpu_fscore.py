@@ -110,6 +110,29 @@ def test_fscore_edges_in_integers(G, N, n_req, with_cap):
     r.close()
 
 
+@pytest.mark.parametrize("G", [1, 2, 3, 17, 32, 33])
+@pytest.mark.parametrize("H", [31, 78, 80])
+def test_fscore_long_horizons_on_small_fleets(G, H):
+    # margins taken four offsets at a time, of which the last warp's may be fewer; equality
+    cfg = wlm.get_config("h80", G=G, H=H, init_active=2, init_queue=0)
+    r = Router(wlm.make_workload(cfg, n_instances=1), device="cuda:0")
+    rng = np.random.default_rng(G + H)
+    N, n_req = 2, 12
+    Lh = rng.integers(1000, 9000, (N, G, H + 1)).astype(np.int64)
+    s = rng.integers(1, 9000, (N, n_req)).astype(np.int32)
+    st, Lt = torch.from_numpy(s).cuda(), torch.from_numpy(Lh).cuda()
+    F = torch.zeros((N, n_req, G), dtype=torch.float64, device="cuda")
+    best = torch.full((N, n_req), -7, dtype=torch.int32, device="cuda")
+    r.fscore(st, Lt, F, best_g=best)
+    Fh, bh = F.cpu().numpy(), best.cpu().numpy()
+    for n in range(N):
+        M = Lh[n].max(axis=0)
+        for i in range(n_req):
+            ref = np.array([oracle.f_brh(H, cfg.alpha, cfg.beta, cfg.gamma, int(s[n, i]), M - Lh[n, g]) for g in range(G)])
+            assert np.array_equal(Fh[n, i], ref) and bh[n, i] == int(np.argmax(ref)), (n, i)
+    r.close()
+
+
 @pytest.mark.parametrize("G,score_mode", [(32, 0), (64, 0), (5, 0), (16, 1)])
 def test_pool_bypass_dispatch(G, score_mode):
     """br_bypass_dispatch against the checker: workers, virtual loads and inflight counts."""
