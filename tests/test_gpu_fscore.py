@@ -189,6 +189,35 @@ def test_pool_bypass_edges(G, n_req, lo, hi):
     r.close()
 
 
+@pytest.mark.parametrize("G", [31, 33, 64])
+@pytest.mark.parametrize("n_req", [1, 45, 64])
+def test_pool_bypass_scores_that_tie(G, n_req):
+    # Eq. 2 scores with one and two workers per lane: equal virtual loads, among them those of workers g and g + 32, are
+    # told apart by the lower index; the margins are re-based whenever the largest load grows.  Equality
+    cfg = wlm.get_config("c3", G=G, init_active=8, init_queue=0, score_mode=1, alpha=1.0, beta=7.5, gamma=1.0)
+    r = Router(wlm.make_workload(cfg, n_instances=1), device="cuda:0")
+    rng = np.random.default_rng(G + n_req)
+    N = 6
+    s = rng.integers(1, 30000, (N, n_req)).astype(np.int32)
+    s[0] = 700
+    L = (rng.integers(0, 4, (N, G)) * 9000).astype(np.int64)               # many equal loads
+    L[1] = 5000
+    L[2, 32:] = L[2, :G - 32] if G > 32 else L[2, 32:]
+    L[3] += np.int64(1) << 40
+    infl = rng.integers(0, 3, (N, G)).astype(np.int32)
+    cap = rng.integers(1, 4, (N, G)).astype(np.int32)
+    cap[4, :G // 2] = 0
+    st, Lt, it, ct = (torch.from_numpy(x.copy()).cuda() for x in (s, L, infl, cap))
+    out = torch.full((N, n_req), -7, dtype=torch.int32, device="cuda")
+    r.bypass_dispatch(st, Lt, it, ct, out)
+    for n in range(N):
+        want, Lw, nw = oracle.bypass(G, s[n], L[n], infl[n], cap[n], score_mode=1, alpha=cfg.alpha, beta=cfg.beta)
+        assert np.array_equal(out[n].cpu().numpy(), want), n
+        assert np.array_equal(Lt[n].cpu().numpy(), Lw) and np.array_equal(it[n].cpu().numpy(), nw), n
+    r.close()
+
+
+
 def test_empirical_survival_estimator():
     """br_survival_chat against the checker's counting definition (same fp64 operations: equality)."""
     cfg = wlm.get_config("c4")                              # H = 8
