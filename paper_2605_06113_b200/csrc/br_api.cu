@@ -374,7 +374,7 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
     // two-probe rule
     a.big_window = p.R_max > br::kRegWin ? 1 : 0;
     if (a.big_window && !ctx->two_probe_ok) { delete ctx; return BR_EINVAL; }
-    a.lay = br::step_layout(G, H, p.B, p.W, a.occ_words, p.term_mode == 3, a.big_window != 0, H > 0 && p.pred_mode == 0);
+    a.lay = br::step_layout(p.score_mode == 1, G, H, p.B, p.W, a.occ_words, p.term_mode == 3, a.big_window != 0, H > 0 && p.pred_mode == 0);
     if (a.lay.total > br::kMaxShared) { delete ctx; return BR_EINVAL; }    // one instance must fit a thread block's shared memory
     // br_small_kernel: Eq. 1, one worker per lane, one occupancy word, at most 512 waiting requests,
     // arrivals served by one Philox call, and negative queue keys scoring below every waiting request

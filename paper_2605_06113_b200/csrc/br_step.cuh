@@ -85,7 +85,7 @@ __host__ __device__ constexpr int step_row_stride(int H)
     return 4 * ((step_groups(H) ? step_groups(H) : (H + 4) / 4) | 1);
 }
 
-inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool lifetimes, bool big_window, bool classifier)
+inline StepLayout step_layout(bool fp, int G, int H, int B, int W, int occ_words, bool lifetimes, bool big_window, bool classifier)
 {
     StepLayout l;
     const int Wp = (W + 127) / 128 * 128, HS = step_row_stride(H), words = 8 * G * occ_words;
@@ -94,11 +94,11 @@ inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool li
     l.q_key = take(4 * Wp);
     l.q_id = take(4 * Wp);
     l.q_o = take(lifetimes ? 4 * Wp : 0);
-    l.Lh = take(4 * (G * HS + 4));              // PREDICT: load sums per (worker, floor(c_hat)); L_g(k+h); margins m_{g,h}
+    l.Lh = take(fp ? 4 * (G * HS + 4) : 0);     // (Eq. 2, as the next four) PREDICT: load sums per (worker, floor(c_hat)); L_g(k+h); margins m_{g,h}
     l.Ch = take(H > 0 ? 4 * G * HS : 0);        // PREDICT: request counts
-    l.dn = take(16 * (HS + 4));                 // (d_h, -2^52 d_h)
-    l.iw = take(4 * (HS + 4));                  // d_h in fixed point
-    l.Ms = take(4 * HS);                        // envelope M_h; then its growth by an admission
+    l.dn = take(fp ? 16 * (HS + 4) : 0);        // (d_h, -2^52 d_h)
+    l.iw = take(fp ? 4 * (HS + 4) : 0);         // d_h in fixed point
+    l.Ms = take(fp ? 4 * HS : 0);               // envelope M_h; then its growth by an admission
     l.occ = take(words);                        // occupied slots
     l.occ0 = take(words);                       // ... at the start of the step
     l.fin = take(words);                        // constant hazard: slots whose draw says "ends"
@@ -109,7 +109,7 @@ inline StepLayout step_layout(int G, int H, int B, int W, int occ_words, bool li
     l.scal = take(4 * 32);
     l.bw = take(big_window ? 8 * (1 << 8) + 4 * 32 : 0);
     const int most = W < G * B ? W : G * B;     // admissions of a step
-    l.due = take(classifier && G * B > 4 * most ? 2 * G * B : 8 * most);   // requests whose c_hat is refreshed; then the admissions
+    l.due = take(classifier && G * B > 2 * most ? 2 * G * B : 4 * most);   // requests whose c_hat is refreshed; then the admissions
     l.total = n;
     return l;
 }
@@ -428,11 +428,11 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
     const auto q_key = mk_span(reinterpret_cast<int *>(smem + a.lay.q_key), a.Wp);
     const auto q_id = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.q_id), a.Wp);
     const auto q_o = mk_span(reinterpret_cast<int *>(smem + a.lay.q_o), life ? a.Wp : 0);
-    const auto Lh = mk_span(reinterpret_cast<int *>(smem + a.lay.Lh), G * HS + 4);
+    const auto Lh = mk_span(reinterpret_cast<int *>(smem + a.lay.Lh), FP ? G * HS + 4 : 0);
     const auto Ch = mk_span(reinterpret_cast<int *>(smem + a.lay.Ch), H > 0 ? G * HS : 0);
     const auto dn_s = mk_span(reinterpret_cast<double *>(smem + a.lay.dn), FP ? 2 * (HS + 4) : 0);
     const auto iw_s = mk_span(reinterpret_cast<int *>(smem + a.lay.iw), FP ? HS + 4 : 0);
-    const auto Ms = mk_span(reinterpret_cast<int *>(smem + a.lay.Ms), HS);
+    const auto Ms = mk_span(reinterpret_cast<int *>(smem + a.lay.Ms), FP ? HS : 0);
     const auto occ = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ), G * OW);
     const auto occ0 = mk_span(reinterpret_cast<unsigned long long *>(smem + a.lay.occ0), G * OW);
     const auto occ032 = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.occ0), 2 * G * OW);
@@ -448,9 +448,11 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
     const auto bw_off = mk_span(reinterpret_cast<int *>(smem + a.lay.bw + (8 << kBigWinLow)), a.big_window ? 16 : 0);
     const auto bw_win = mk_span(reinterpret_cast<int *>(smem + a.lay.bw + (8 << kBigWinLow) + 64), a.big_window ? 16 : 0);
     const auto due_list = mk_span(reinterpret_cast<unsigned short *>(smem + a.lay.due), classifier ? A : 0);
-    // admissions of the step in order: (key, worker << 16 | free slots of the worker before it); shares the
-    // memory of the due list, which is not needed once the projection stands
-    const auto adm = mk_span(reinterpret_cast<int2 *>(smem + a.lay.due), min(W, A));
+    // admissions of the step in order: queue position << 15 | worker << 9 | free slots of the worker before it; shares the
+    // memory of the due list, which is not needed once the projection stands.  The key of an admitted request stays in
+    // the queue, its sign bit set, until slots are given out (8 bytes an admission, the key among them, left room for
+    // 19 instances of BR-0 at G = 64, W = 512 on an SM instead of 22)
+    const auto adm = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.due), min(W, A));
     // scal: [0] queue length after routing, [1] admitted, [2] Stage-1 iterations, [3] Stage-2 pops,
     //       [4] status bits of the step, [5] status bits of the prologue, [6] lowest admitted position,
     //       [8] requests on the due list, [16..31] kept entries per warp (two sets of eight, compaction)
@@ -1211,8 +1213,8 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
                     }
                     const int at = __popc(chosen & ((1u << lane) - 1u)), pos = (int)(posmask - ((unsigned)key & posmask));
                     if ((chosen >> lane) & 1u) {
-                        adm[n_w - n_left + at] = make_int2(key, (g << 16) | (mc - at));
-                        q_key[pos] = kQBeyond;
+                        adm[n_w - n_left + at] = ((unsigned)pos << 15) | ((unsigned)g << 9) | (unsigned)(mc - at);
+                        q_key[pos] = key | (int)0x80000000u;
                         first_rm = min(first_rm, pos);
                     }
                 }
@@ -1306,9 +1308,9 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
         const int n_new = scal[0], n_adm = n_w - n_new;
 #pragma unroll 1
         for (int e = tid; e < n_adm; e += NT) {
-            const int2 r = adm[e];
-            const int g = r.y >> 16, s = r.x >> WL, pos = (int)(posmask - ((unsigned)r.x & posmask));
-            int rank = cap_s[g] - (r.y & 0xFFFF), slot = B;
+            const unsigned r = adm[e];
+            const int g = (int)(r >> 9) & 63, pos = (int)(r >> 15), s = (q_key[pos] & 0x7FFFFFFF) >> WL;
+            int rank = cap_s[g] - (int)(r & 511u), slot = B;
 #pragma unroll 1
             for (int x = 0; x < 2 * OW; ++x) {
                 unsigned fr = ~occ032[2 * g * OW + x];
@@ -1323,6 +1325,7 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
             }
             if (slot >= B) {                                      // free-slot count and occupancy word disagree: gone, no slot
                 atomicOr(&scal[4], BR_ST_BAD_STATE);
+                q_key[pos] = kQBeyond;
                 continue;
             }
             const int sa = g * B + slot;

@@ -48,3 +48,14 @@ def test_one_lane_holds_the_whole_window(H, R_max, threads, monkeypatch):
     cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
                          term_mode=1, S_greedy=1 << 20, score_mode=-1, delta_T=-1)
     run_parity(cfg, 2, 8, threads=threads, check_every=1)
+
+
+@pytest.mark.parametrize("H", [0, 2])
+def test_admissions_at_the_largest_positions_workers_and_counts(H):
+    # the entry of an admission packs the queue position (4,096), the worker (64) and its free slots (256)
+    cfg = wlm.get_config("c2", G=64, B=256, W=4096, H=H, R_max=5, init_active=230, init_queue=4096, hazard=0.02, term_mode=1,
+                         score_mode=-1, S_greedy=600, delta_T=-1, arrival=("const", 30.0))
+    run_parity(cfg, 1, 4, check_every=1)
+    cfg = wlm.get_config("c2", G=64, B=256, W=4096, H=H, R_max=5, init_active=0, init_queue=4096, hazard=0.02, term_mode=1,
+                         score_mode=-1, S_greedy=10, delta_T=-1, arrival=("const", 30.0))
+    run_parity(cfg, 1, 2, check_every=1)
