@@ -116,8 +116,6 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         if (cap < 0 || cap > B) { status0 = BR_ST_BAD_STATE; cap = cap < 0 ? 0 : B; }
         cap = B - cap;
     }
-    // a worker whose occupancy word has fewer free slots than its count says may turn a request away below
-    const bool odd = __any_sync(kFull, lane < G && cap > __popcll(~occ));
     // ---- the queue moves to shared memory once per launch: packed keys and ids ----
 #pragma unroll
     for (int t = 0; t < NT4; ++t) {
@@ -195,7 +193,10 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
         __syncwarp();
 
         // ================= ROUTE (Algorithm 1) =================
-        int S_tot = (int)__reduce_add_sync(kFull, (unsigned)(cap > 0 ? cap : 0));
+        // (odd: a worker's occupancy word has fewer free slots than its count says, and may turn a request away)
+        int S_tot = (int)__reduce_add_sync(kFull, (unsigned)(cap > 0 ? cap : 0) + (cap > __popcll(~occ) ? 0x10000u : 0u));
+        const bool odd = S_tot > 0xFFFF;
+        S_tot &= 0xFFFF;
         int M = __reduce_max_sync(kFull, L);
         int n_left = n_w, admitted = 0, s1_iters = 0, s2_pops = 0, status = status0;
         int first_rm = W;                     // lowest queue position admitted so far
@@ -211,6 +212,7 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
             // worker: most free slots, then smallest L_g (= largest safe margin), then lowest g
             const int mc = __reduce_max_sync(kFull, cap);
             if (mc <= 0) break;
+            if (rare(odd)) M = __reduce_max_sync(kFull, L);             // a request turned away adds no load
             const unsigned ml = __reduce_min_sync(kFull, cap == mc ? (unsigned)L : 0xFFFFFFFFu);
             const int g = (int)__reduce_min_sync(kFull, cap == mc && (unsigned)L == ml ? (unsigned)lane : 32u);
             int Lg = (int)ml;
@@ -311,7 +313,7 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
                         cap = 0;
                     }
                 }
-                Lg = rare(odd) ? __shfl_sync(kFull, L, g) : Lg + s;     // (a request turned away adds no load)
+                Lg += s;
                 M = max(M, Lg);
                 if (qk >= gw[RM - 1]) gw_valid = false;                 // a cached window entry leaves
                 first_rm = min(first_rm, pos);
@@ -319,6 +321,8 @@ __global__ void __maxnreg__(NT4 <= 2 ? 72 : 128) br_small_kernel(const StepArgs 
                 __syncwarp();
             }
         }
+
+        if (rare(odd)) M = __reduce_max_sync(kFull, L);
 
         // ================= RECORD (Section 3.1) =================
         {
