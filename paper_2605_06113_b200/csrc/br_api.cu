@@ -70,22 +70,37 @@ inline bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintp
 
 typedef void (*step_kernel_t)(const StepArgs);
 
-template <bool FP, int NC>
+template <bool FP, int NC, bool EARLY>
 step_kernel_t pick_kernel_gw(int G)
 {
-    return G <= 32 ? br::br_step_kernel<FP, 1, NC> : br::br_step_kernel<FP, 2, NC>;
+    return G <= 32 ? br::br_step_kernel<FP, 1, NC, EARLY> : br::br_step_kernel<FP, 2, NC, EARLY>;
+}
+
+template <int NC>
+step_kernel_t pick_kernel_early(int G, bool early)
+{
+    return early ? pick_kernel_gw<true, NC, true>(G) : pick_kernel_gw<true, NC, false>(G);
 }
 
 // Eq. 1 or Eq. 2; one or two workers per router lane; horizon offsets unrolled in groups of four or not at all
-step_kernel_t pick_kernel(bool fp, int H, int G)
+step_kernel_t pick_kernel(bool fp, int H, int G, bool early)
 {
-    if (!fp) return pick_kernel_gw<false, 2>(G);
+    if (!fp) return early ? pick_kernel_gw<false, 2, true>(G) : pick_kernel_gw<false, 2, false>(G);
     switch (br::step_groups(H)) {
-    case 2: return pick_kernel_gw<true, 2>(G);
-    case 3: return pick_kernel_gw<true, 3>(G);
-    case 5: return pick_kernel_gw<true, 5>(G);
-    default: return pick_kernel_gw<true, 0>(G);
+    case 2: return pick_kernel_early<2>(G, early);
+    case 3: return pick_kernel_early<3>(G, early);
+    case 5: return pick_kernel_early<5>(G, early);
+    default: return pick_kernel_gw<true, 0, false>(G);
     }
+}
+
+// Whether a single warp settles the requests that end ahead of the router (constant hazard): with many instances
+// resident it saves two trips to memory of each, which the router's chain would wait for: us per call of one step,
+// 3,040 instances: G = 40, H = 0, W = 256: 26.9 -> 22.3, G = 64, W = 512: 45.6 -> 29.8, G = 48, H = 4: 165 -> 157.
+// Instances of few slots and long horizons gain nothing.
+bool step_early(const br_ctx *ctx)
+{
+    return ctx->p.term_mode == 1 && (ctx->p.score_mode == 0 || (br::step_groups(ctx->H) && ctx->G * ctx->p.B >= 512));
 }
 
 constexpr int kSMs = 148;
@@ -216,8 +231,8 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
         if (e != cudaSuccess) return cuda_fail(e, "br_step launch");
         return BR_OK;
     }
-    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G);
     const int threads = threads_for(ctx, b->n_instances);
+    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, threads == 32 && step_early(ctx));
     // lanes per worker that turn its buckets into projected loads
     a.seg_log2 = 0;
     while (a.seg_log2 < 5 && (ctx->G << (a.seg_log2 + 1)) <= threads && (2 << a.seg_log2) <= ctx->H + 1) ++a.seg_log2;

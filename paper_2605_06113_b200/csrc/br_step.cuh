@@ -408,11 +408,13 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
 // Registers: the router's chain is the longest path, and it is shorter with more of them than with more
 // warps resident (G = 64, H = 8, one instance: 22.0 us at 72 registers, 19.4 at 96; 777 instances of G = 21,
 // H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128).
-template <bool FP, int GW, int NC>
+// EARLY: a single warp under the constant hazard (32 threads, term_mode 1), with the requests that end settled ahead of
+// the router.
+template <bool FP, int GW, int NC, bool EARLY>
 __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_constant__ StepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int NT = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = NT >> 5;
+    const int NT = EARLY ? 32 : blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = EARLY ? 0 : tid >> 5, nwarps = NT >> 5;
     stream_order_gate();
     const int G = a.G, H = FP ? a.H : 0, B = a.B, W = a.W, A = G * B, OW = a.occ_words, WL = a.wl;
     const int H1 = H + 1, HS = NC > 0 ? 4 * (NC | 1) : a.HS;
@@ -547,6 +549,27 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
             u_arr = __shfl_sync(kFull, r.x, 31);
             const uint32_t last = __shfl_sync(kFull, r.w, 30);
             s_new = t_len[(cnt ? last : word_of(r, tid & 3)) >> a.len_shift];
+        }
+        // A single warp settles, while these loads are on their way, which of the running requests end at this step, and asks
+        // for the first of every worker's: the values are used after routing.
+        int pend[GW], pslot[GW];
+#pragma unroll
+        for (int w = 0; w < GW; ++w) { pend[w] = 0; pslot[w] = -1; }
+        if (EARLY) {
+#pragma unroll
+            for (int w = 0; w < GW; ++w) {
+                const int g = lane + 32 * w;
+                if (g < G) {
+                    draw_ending(t_term, B, OW, (uint32_t)k, (uint32_t)g, key0, key1, fin + (size_t)g * OW);
+#pragma unroll 1
+                    for (int x = 0; x < OW; ++x) {
+                        const unsigned long long e = occ0[g * OW + x] & fin[g * OW + x];
+                        endm[g * OW + x] = e;
+                        if (e && pslot[w] < 0) pslot[w] = 64 * x + __ffsll((long long)e) - 1;
+                    }
+                    if (pslot[w] >= 0) pend[w] = ld_now(&g_base[g * B + pslot[w]]);
+                }
+            }
         }
         if (timing) t_phase[1] = (unsigned)clock64();
 
@@ -752,7 +775,7 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
         if (timing) t_phase[2] = (unsigned)clock64();
 
         // ---- requests running before this step that end at it: by warps 1.. while warp 0 routes ----
-        if ((warp > 0 || nwarps == 1) && a.pred_mode != 1) {
+        if ((warp > 0 || nwarps == 1) && a.pred_mode != 1 && !EARLY) {
             const int t0 = nwarps == 1 ? tid : tid - 32, nt = nwarps == 1 ? NT : NT - 32;
             if (a.term_mode == 1) {
 #pragma unroll 1
@@ -1302,6 +1325,29 @@ __global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_const
             }
         }
         __syncthreads();                                          // admissions visible
+        if (EARLY) {
+#pragma unroll
+            for (int w = 0; w < GW; ++w) {
+                const int g = lane + 32 * w;
+                if (pslot[w] >= 0) {
+                    unsigned sub = (unsigned)(pend[w] + k);
+                    g_base[g * B + pslot[w]] = kEmpty;
+#pragma unroll 1
+                    for (int x = pslot[w] >> 6; x < OW; ++x) {            // rare: more than one
+                        unsigned long long e = endm[g * OW + x];
+                        if (x == pslot[w] >> 6) e &= ~(1ull << (pslot[w] & 63));
+#pragma unroll 1
+                        for (; e; e &= e - 1ull) {
+                            const int sa = g * B + 64 * x + __ffsll((long long)e) - 1;
+                            sub += (unsigned)(g_base[sa] + k);
+                            g_base[sa] = kEmpty;
+                        }
+                    }
+                    sub_load[g] = sub;
+                }
+            }
+            __syncwarp();
+        }
 
         // ============ sticky admissions, one thread each ============
         // a worker's requests take its free slots in ascending order, in the order of their admission

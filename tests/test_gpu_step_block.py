@@ -59,3 +59,12 @@ def test_admissions_at_the_largest_positions_workers_and_counts(H):
     cfg = wlm.get_config("c2", G=64, B=256, W=4096, H=H, R_max=5, init_active=0, init_queue=4096, hazard=0.02, term_mode=1,
                          score_mode=-1, S_greedy=10, delta_T=-1, arrival=("const", 30.0))
     run_parity(cfg, 1, 2, check_every=1)
+
+
+@pytest.mark.parametrize("hazard", [0.0, 0.01, 0.4, 1.0])
+@pytest.mark.parametrize("G,B,W,H", [(33, 24, 128, 0), (5, 200, 64, 0), (16, 64, 128, 4), (64, 8, 64, 18), (3, 256, 64, 9), (40, 16, 64, 40)])
+def test_single_warp_settles_endings_ahead_of_the_router(G, B, W, H, hazard):
+    # none, one and several requests of a worker end at a step, in every word of its occupancy, admitted ones among them
+    cfg = wlm.get_config("c2", G=G, B=B, W=W, H=H, init_active=B - B // 8, init_queue=W - 1, hazard=hazard, term_mode=1,
+                         score_mode=-1, S_greedy=-1, delta_T=-1, arrival=("const", 9.0))
+    run_parity(cfg, 2, 8, threads=32, launch_steps=2, check_every=1)
