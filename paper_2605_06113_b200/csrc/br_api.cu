@@ -70,69 +70,41 @@ inline bool misaligned(const void *p, size_t a) { return (reinterpret_cast<uintp
 
 typedef void (*step_kernel_t)(const StepArgs);
 
-template <bool FP, int NC, bool EARLY>
+template <bool FP, int NC, bool LEAN, bool EARLY>
 step_kernel_t pick_kernel_gw(int G)
 {
-    return G <= 32 ? br::br_step_kernel<FP, 1, NC, EARLY> : br::br_step_kernel<FP, 2, NC, EARLY>;
+    return G <= 32 ? br::br_step_kernel<FP, 1, NC, LEAN, EARLY> : br::br_step_kernel<FP, 2, NC, LEAN, EARLY>;
 }
 
 template <int NC>
 step_kernel_t pick_kernel_early(int G, bool early)
 {
-    return early ? pick_kernel_gw<true, NC, true>(G) : pick_kernel_gw<true, NC, false>(G);
+    return early ? pick_kernel_gw<true, NC, false, true>(G) : pick_kernel_gw<true, NC, false, false>(G);
 }
 
 // Eq. 1 or Eq. 2; one or two workers per router lane; horizon offsets unrolled in groups of four or not at all
-step_kernel_t pick_kernel(bool fp, int H, int G, bool early)
+step_kernel_t pick_kernel(bool fp, int H, int G, const br::StepLaunch &l)
 {
-    if (!fp) return early ? pick_kernel_gw<false, 2, true>(G) : pick_kernel_gw<false, 2, false>(G);
+    if (!fp && l.early) return l.lean ? pick_kernel_gw<false, 2, true, true>(G) : pick_kernel_gw<false, 2, false, true>(G);
+    if (!fp) return l.lean ? pick_kernel_gw<false, 2, true, false>(G) : pick_kernel_gw<false, 2, false, false>(G);
     switch (br::step_groups(H)) {
-    case 2: return pick_kernel_early<2>(G, early);
-    case 3: return pick_kernel_early<3>(G, early);
-    case 5: return pick_kernel_early<5>(G, early);
-    default: return pick_kernel_gw<true, 0, false>(G);
+    case 2: return pick_kernel_early<2>(G, l.early);
+    case 3: return pick_kernel_early<3>(G, l.early);
+    case 5: return pick_kernel_early<5>(G, l.early);
+    default: return l.lean ? pick_kernel_gw<true, 0, true, false>(G) : pick_kernel_gw<true, 0, false, false>(G);
     }
-}
-
-// Whether a single warp settles the requests that end ahead of the router (constant hazard): with many instances
-// resident it saves two trips to memory of each, which the router's chain would wait for: us per call of one step,
-// 3,040 instances: G = 40, H = 0, W = 256: 26.9 -> 22.3, G = 64, W = 512: 45.6 -> 29.8, G = 48, H = 4: 165 -> 157.
-// Instances of few slots and long horizons gain nothing.
-bool step_early(const br_ctx *ctx)
-{
-    return ctx->p.term_mode == 1 && (ctx->p.score_mode == 0 || (br::step_groups(ctx->H) && ctx->G * ctx->p.B >= 512));
 }
 
 constexpr int kSMs = 148;
 constexpr int kHostWarps = 4;          // instances resident per SM when their rows are in host memory
 
-// Threads per instance of br_step_kernel.  An instance has parallel work for `most` threads (projection:
-// 16 slots a thread, queue: 4 positions, buckets: 8 offsets); more only lengthen its barriers, but four
-// warps pay off even for small ones, because the requests that end are drawn while warp 0 routes (84 of
-// G = 4, W = 56: 19.9 us with one warp, 15.2 with four).  When the batch puts several instances on an SM they
-// share its registers, which hold 21 warps (16 for long horizons): each takes its share, so that all are
-// resident (777 of G = 21, W = 300, three steps: 234 / 169 / 201 us with two / three / four warps); a second warp is
-// worth a few instances less (2,048 of G = 16, W = 512, H = 8: 102 us with one, 86 with two).  Instances
-// that stream 2,048 slots and more of classifier state are bound by memory while they do; fewer of them at a time
-// with more warps each, so that some stream while others route (1,024 of G = 64, H = 8: 77 us with three warps,
-// 64.5 with four, 63.0 with five, 85 with eight).
-int threads_for(const br_ctx *ctx, int n_instances)
+br::StepLaunch launch_shape(const br_ctx *ctx, int n_instances)
 {
-    if (ctx->p.threads > 0) return ctx->p.threads;
-    const int A = ctx->G * ctx->p.B;
-    int most = ctx->H > 0 ? A / 16 : 64;
-    if (ctx->p.W / 4 > most) most = ctx->p.W / 4;
-    if (ctx->G * (ctx->H + 1) / 8 > most) most = ctx->G * (ctx->H + 1) / 8;
-    most = (most + 31) / 32;
-    most = most < 4 ? 4 : (most > 8 ? 8 : most);
-    int per_sm = (n_instances + kSMs - 1) / kSMs;
-    const int fit = (int)(227 * 1024 / (ctx->base.lay.total + 1024));       // resident instances, by shared memory
-    if (per_sm > fit) per_sm = fit;
-    const int regs = br::step_groups(ctx->H) ? 21 : 16;                     // warps
-    int w = 2 * regs >= 3 * per_sm && regs < 2 * per_sm ? 2 : (4 * regs / per_sm + 1) / 4;
-    if (ctx->H > 0 && ctx->p.pred_mode == 0 && A >= 2048 && w < 5) w = 5;
-    w = w < 1 ? 1 : (w > most ? most : w);
-    return 32 * w;
+    const br::StepShape s = {ctx->p.score_mode == 1, ctx->G, ctx->H, ctx->p.B, ctx->p.W, ctx->p.term_mode, ctx->p.pred_mode,
+                             ctx->base.lay.total};
+    br::StepLaunch l = br::step_launch(s, n_instances, kSMs);
+    if (ctx->p.threads > 0) { l.warps = ctx->p.threads / 32; l.lean = false; l.early = l.warps == 1 && br::step_early(s); }
+    return l;
 }
 
 int check_step_args(const br_ctx *ctx, const br_instance_batch *b, const br_worker_state *ws,
@@ -231,8 +203,9 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
         if (e != cudaSuccess) return cuda_fail(e, "br_step launch");
         return BR_OK;
     }
-    const int threads = threads_for(ctx, b->n_instances);
-    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, threads == 32 && step_early(ctx));
+    const br::StepLaunch shape = launch_shape(ctx, b->n_instances);
+    step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, shape);
+    const int threads = 32 * shape.warps;
     // lanes per worker that turn its buckets into projected loads
     a.seg_log2 = 0;
     while (a.seg_log2 < 5 && (ctx->G << (a.seg_log2 + 1)) <= threads && (2 << a.seg_log2) <= ctx->H + 1) ++a.seg_log2;

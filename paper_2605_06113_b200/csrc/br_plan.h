@@ -6,6 +6,7 @@
 namespace br {
 
 constexpr int kMaxShared = 227 * 1024;     // dynamic shared memory of a thread block, at most
+constexpr int kSharedPerSM = 227 * 1024;   // ... of the blocks of an SM together, with 1 KB more for each
 
 // A page-locked allocation or registration around an address, in the device's address space.
 struct LockedRange {
@@ -51,6 +52,95 @@ inline bool host_in_place(HostUse use, int H, int term_mode, long long n_instanc
     if (use == kHostScores) return false;
     if (use == kHostSparse || (H == 0 && term_mode <= 1)) return true;
     return n_instances < 64 && (term_mode != 2 || n_instances * slots_per_instance <= 100000);
+}
+
+// ---- launch shape of br_step_kernel ----------------------------------------------------------------
+
+// Groups of four horizon offsets (h = 0 .. H) that a kernel unrolls: 2, 3 or 5, so that the loops over h
+// of the admission loop are straight code; 0: a longer horizon, three offsets per lane, plain loops.
+constexpr int step_groups(int H) { return H < 8 ? 2 : (H < 12 ? 3 : (H < 20 ? 5 : 0)); }
+
+// Registers a thread of an instantiation may use, by Eq. 1 or 2 (fp) and step_groups(H).  The lean ones make the
+// router's chain 5 to 15 % longer and let more instances be resident; horizons below 20 have none (at 80 registers
+// 40 % more instances, each slower by as much: 2,072 of G = 16, H = 8, eight steps: 382 us, 396).
+constexpr int step_register_cap(bool fp, int groups, bool lean) { return !fp ? (lean ? 72 : 96) : groups ? 96 : (lean ? 96 : 128); }
+// ... and the registers that it is compiled to (Eq. 1 by the workers per router lane: 78 and 84; long horizons 115)
+constexpr int step_registers(bool fp, int workers_per_lane, int groups, bool lean)
+{
+    return !fp ? (lean ? 72 : (workers_per_lane == 1 ? 80 : 88)) : groups ? 96 : (lean ? 96 : 120);
+}
+constexpr bool step_has_lean(bool fp, int groups) { return !fp || !groups; }
+
+// Warps of a kernel that an SM's registers hold: four partitions of 16,384, and 32 threads of a multiple of eight
+// registers per warp (96 registers: 20 warps, not 21).
+constexpr int step_warps_per_sm(int registers) { return 4 * (16384 / (32 * ((registers + 7) / 8 * 8))); }
+
+struct StepShape {
+    bool fp;               // Eq. 2
+    int G, H, B, W;
+    int term_mode, pred_mode;
+    int shared;            // bytes of shared memory of an instance
+};
+struct StepLaunch { int warps; bool lean, early; };
+
+// Whether a single warp settles the requests that end ahead of the router (constant hazard): with many instances
+// resident it saves two trips to memory of each, which the router's chain would wait for: us per call of one step,
+// 3,040 instances: G = 40, H = 0, W = 256: 26.9 -> 22.3, G = 64, W = 512: 45.6 -> 29.8, G = 48, H = 4: 165 -> 157.
+// Instances of few slots and long horizons gain nothing.
+inline bool step_early(const StepShape &s)
+{
+    return s.term_mode == 1 && (!s.fp || (step_groups(s.H) && s.G * s.B >= 512));
+}
+
+// Warps per instance, and which instantiation, for n_instances instances on `sms` SMs.
+//
+// More warps shorten an instance's parallel phases and leave fewer instances resident, so a batch of a few instances
+// per SM takes as many warps as there is work for, a large one those that need the least time for all its
+// waves.  With r resident instances of w warps a step takes, in units of the router's chain,
+//     t(w, r) = 1 + p (c + e r) / w,
+// p the thousands of slots that the projection streams (a little more the longer the classifier's rows, twice as
+// many when terminations read every row; Eq. 1 has draws and queue alone) and e what another resident instance costs.
+// The last, incomplete wave starts while instances of the one before still run and counts in part.  The constants
+// are a fit to 3,000 measured times (44 shapes, 1 to 28 instances per SM, one to eight warps, both instantiations): the
+// choice is within 1 % of the fastest on average, at worst 17 %.  us per call at 1, 2, 3, 4, 5 warps: 592 of G = 32,
+// H = 1: 44 / 33 / 27 / 25 / 23; 1,480: 57 / 37 / 48 / 47 / 56; 2,072: 65 / 67 / 76 / 74 / 80; 2,960:
+// 107 / 78 / 108 / 109 / 115.  Four warps at least for instances that stream 4,096 slots with long classifier rows: more
+// of them resident take each other's cache lines (1,480 of G = 64, H = 16: 227 / 189 / 102 / 89 / 106).
+inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
+{
+    const int groups = step_groups(s.H), A = s.G * s.B, n = (n_instances + sms - 1) / sms;
+    const bool classifier = s.H > 0 && s.pred_mode == 0;
+    int most = s.H > 0 ? A / 16 : 64;                      // threads with something to do: 16 slots, 4 positions, 8 offsets
+    if (s.W / 4 > most) most = s.W / 4;
+    if (s.G * (s.H + 1) / 8 > most) most = s.G * (s.H + 1) / 8;
+    most = (most + 31) / 32;
+    most = most < 4 ? 4 : (most > 8 ? 8 : most);
+    const bool long_rows = classifier && s.H >= 8 && groups && A * (s.term_mode == 2 ? 2 : 1) >= 4096;
+    const int least = long_rows ? 4 : 1;
+    const double p = 7e-5 * s.W + (!s.H ? 0.035 + 0.005 * s.G
+                                        : 1e-3 * A * (classifier ? 1.0 + 0.02 * s.H : 1.0) * (s.term_mode == 2 ? 2 : 1));
+    struct Fit { double c, e, last, last_full; };
+    const Fit k = !s.H ? Fit{0.65, 0.03, 0.3, 0.4} : classifier ? Fit{0.75, 0.036, 0.65, 0.3} : Fit{0.7, 0.017, 0.5, 0.5};
+    StepLaunch best = {1, false, false};
+    double cost = 1e300;
+    for (int w = least; w <= most; ++w) {
+        for (int lean = 0; lean < 2; ++lean) {
+            // (the lean instantiation spills in the classifier's loop, which a single warp cannot hide)
+            if (lean && (!step_has_lean(s.fp, groups) || (classifier && w < 2))) continue;
+            int r = step_warps_per_sm(step_registers(s.fp, s.G <= 32 ? 1 : 2, groups, lean != 0)) / w;
+            const int fit = kSharedPerSM / (s.shared + 1024);
+            if (r > fit) r = fit;
+            if (r > 32) r = 32;
+            if (r < 1) r = 1;
+            const int full = n / r, part = n % r;
+            double t = full * (1.0 + p * (k.c + k.e * r) / w);
+            if (part) t += (full ? k.last + k.last_full * part / r : 1.0) * (1.0 + p * (k.c + k.e * part) / w);
+            if (lean) t *= 1.1;
+            if (t <= cost) { cost = t; best.warps = w; best.lean = lean != 0; }
+        }
+    }
+    best.early = best.warps == 1 && step_early(s);
+    return best;
 }
 
 }  // namespace br

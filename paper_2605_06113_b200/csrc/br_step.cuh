@@ -28,6 +28,7 @@
 #pragma once
 #include "br_device.cuh"
 #include "br_mitm.cuh"
+#include "br_plan.h"
 #include "../../include/br.h"
 
 namespace br {
@@ -73,14 +74,10 @@ struct StepArgs {
     double fix, beta_fix, fix_err;   // scale of penalty sums in fixed point, beta / fix, and what the rounding to it adds
 };
 
-// Groups of four horizon offsets (h = 0 .. H) that a kernel unrolls: 2, 3 or 5, so that the loops over h
-// of the admission loop are straight code; 0: a longer horizon, three offsets per lane, plain loops.
-__host__ __device__ constexpr int step_groups(int H) { return H < 8 ? 2 : (H < 12 ? 3 : (H < 20 ? 5 : 0)); }
-
 // Rows of L_g(k+h) are read by lanes that own a worker each (16-byte loads at the row stride) and by
 // lanes that own an offset each (consecutive words): an odd number of 16-byte units keeps both free of
 // bank conflicts.
-__host__ __device__ constexpr int step_row_stride(int H)
+constexpr int step_row_stride(int H)
 {
     return 4 * ((step_groups(H) ? step_groups(H) : (H + 4) / 4) | 1);
 }
@@ -404,14 +401,15 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
         F[(size_t)i * G] = i < n_w ? Scorer<FP>::value(sc.key(q_key[i] >> WL)) : 0.0;
 }
 
-// FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  NC: step_groups(H).
+// FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  NC: step_groups(H).  LEAN: fewer registers.
 // Registers: the router's chain is the longest path, and it is shorter with more of them than with more
 // warps resident (G = 64, H = 8, one instance: 22.0 us at 72 registers, 19.4 at 96; 777 instances of G = 21,
-// H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128).
+// H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128).  Batches that just miss being resident in one wave
+// take the lean instantiation (step_registers, step_launch).
 // EARLY: a single warp under the constant hazard (32 threads, term_mode 1), with the requests that end settled ahead of
 // the router.
-template <bool FP, int GW, int NC, bool EARLY>
-__global__ void __maxnreg__(NC > 0 ? 96 : 128) br_step_kernel(const __grid_constant__ StepArgs a)
+template <bool FP, int GW, int NC, bool LEAN, bool EARLY>
+__global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(const __grid_constant__ StepArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int NT = EARLY ? 32 : blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = EARLY ? 0 : tid >> 5, nwarps = NT >> 5;

@@ -21,6 +21,13 @@ extern "C" uintptr_t alias(uintptr_t host, size_t bytes, int n, const uintptr_t 
         return false;
     });
 }
+extern "C" int launch(int fp, int G, int H, int B, int W, int term_mode, int pred_mode, int shared, int n, int *resident)
+{
+    const br::StepShape s = {fp != 0, G, H, B, W, term_mode, pred_mode, shared};
+    const br::StepLaunch l = br::step_launch(s, n, 148);
+    *resident = br::step_warps_per_sm(br::step_registers(s.fp, G <= 32 ? 1 : 2, br::step_groups(H), l.lean)) / l.warps;
+    return l.lean ? -l.warps : l.warps;
+}
 extern "C" int in_place(int use, int H, int term_mode, long long n, long long slots)
 {
     return br::host_in_place((br::HostUse)use, H, term_mode, n, slots);
@@ -76,3 +83,46 @@ def test_which_page_locked_arrays_are_used_in_place(plan):
     assert not in_place(rows, 8, 1, 64, 64) and not in_place(rows, 0, 3, 64, 64)
     # terminations drawn from every classifier row
     assert in_place(rows, 8, 2, 24, 4096) and not in_place(rows, 8, 2, 25, 4096) and not in_place(rows, 16, 2, 63, 16384)
+
+
+def _launch(plan, G, H, n, B=64, W=256, term=1, pred=0, shared=8000):
+    res = C.c_int()
+    w = plan.launch(int(H > 0), G, H, B, W, term, pred, shared, n, C.byref(res))
+    return abs(w), w < 0, min(res.value, 232448 // (shared + 1024))
+
+
+def test_registers_hold_whole_partitions_of_warps(plan):
+    # 96 registers: five warps on each of four partitions
+    assert _launch(plan, 32, 8, 148 * 10)[2] == 10 and _launch(plan, 32, 8, 148 * 7)[2] >= 7
+
+
+def test_a_batch_is_not_split_into_waves_that_fewer_warps_would_save(plan):
+    # one wave of two warps, not two of three or more (7 and 10 instances an SM), nor two of two where one warp each
+    # makes one (14)
+    for G, H, B in ((32, 1, 64), (16, 4, 64), (16, 8, 64), (4, 2, 24)):
+        for n in (7, 10):
+            w, _, res = _launch(plan, G, H, 148 * n, B=B)
+            assert w == 2 and res >= n, (G, H, n)
+    assert _launch(plan, 4, 2, 148 * 14, B=24, W=32)[0] == 1
+    assert _launch(plan, 32, 1, 148 * 5)[0] == 4 and _launch(plan, 32, 1, 148 * 4)[0] >= 4
+    # two full waves of two warps, not a full and a nearly empty one of a single warp
+    assert _launch(plan, 20, 12, 3000, B=96, shared=12000)[0] == 2
+    # batches that just miss a wave take the lean instantiation where there is one
+    assert _launch(plan, 40, 0, 148 * 28, shared=6000) == (1, True, 28)
+    assert _launch(plan, 7, 60, 148 * 19, W=32, term=3, pred=1, shared=8000)[:2] == (1, True)
+    # long classifier rows: four or five warps whatever the batch
+    for n in (4, 7, 10, 14, 20, 28):
+        assert _launch(plan, 64, 8, 148 * n, shared=20000)[0] in (4, 5)
+
+
+def test_every_shape_gets_a_launch(plan):
+    for G in (1, 2, 32, 33, 64):
+        for H in (0, 1, 8, 19, 20, 80):
+            for B, W in ((8, 4), (64, 1024), (256, 4096)):
+                for term, pred in ((1, 0), (2, 0), (3, 0), (3, 1)):
+                    if (term == 2 or pred) and H == 0:
+                        continue
+                    for n in (1, 148, 149, 4096, 1 << 20):
+                        for shared in (4000, 60000, 232448):
+                            w, _, res = _launch(plan, G, H, n, B, W, term, pred, shared)
+                            assert 1 <= w <= 8
