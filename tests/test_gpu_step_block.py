@@ -68,3 +68,11 @@ def test_single_warp_settles_endings_ahead_of_the_router(G, B, W, H, hazard):
     cfg = wlm.get_config("c2", G=G, B=B, W=W, H=H, init_active=B - B // 8, init_queue=W - 1, hazard=hazard, term_mode=1,
                          score_mode=-1, S_greedy=-1, delta_T=-1, arrival=("const", 9.0))
     run_parity(cfg, 2, 8, threads=32, launch_steps=2, check_every=1)
+
+
+@pytest.mark.parametrize("G,H", [(5, 0), (33, 0), (33, 3), (16, 8), (40, 11), (7, 12), (33, 19), (3, 20), (34, 33)])
+def test_score_matrix_of_every_horizon_group(G, H):
+    # every number of offset groups and both numbers of workers per lane; the scores are compared for equality
+    cfg = wlm.get_config("c2", G=G, B=16, W=132, H=H, init_active=14, init_queue=120, hazard=0.05, term_mode=1, score_mode=-1,
+                         S_greedy=-1, delta_T=-1, arrival=("const", 4.0))
+    run_parity(cfg, 2, 4, check_every=1, fscore=True)
