@@ -1209,8 +1209,9 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     }
                     if (ordered) {
                         const int thr = peak >= (1 << (31 - WL)) ? 0x7FFFFFFF : ((peak << WL) | (int)posmask);
-                        // entries that are gone or beyond the queue have negative keys: as unsigned distances they
-                        // lie beyond every waiting one
+                        // entries that are gone or beyond the queue have negative keys: as unsigned distances they lie
+                        // beyond every waiting one on the side that is searched.  A waiting one on the other side
+                        // lies beyond them, and is what comes out where there is no other
                         unsigned below = 0xFFFFFFFFu, above = 0xFFFFFFFFu;
 #pragma unroll 2
                         for (int t = 0; t < n_groups; ++t) {
@@ -1224,7 +1225,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                         }
                         below = __reduce_min_sync(kFull, below);
                         above = __reduce_min_sync(kFull, above);
-                        const int ka = max((int)((unsigned)thr - below), 0);
+                        const int kl = (int)((unsigned)thr - below), ka = kl > 0 && kl <= thr ? kl : 0;
                         const int kx = (int)(above + (unsigned)thr + 1u);
                         const int kb = kx > thr ? (int)((unsigned)kx ^ posmask) : 0;
                         qk = ka | kb;

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2605_06113_b200 import workload as wlm
-from helpers import run_parity
+from helpers import EMPTY, run_parity
 
 pytestmark = pytest.mark.gpu
 
@@ -48,6 +48,30 @@ def test_one_lane_holds_the_whole_window(H, R_max, threads, monkeypatch):
     cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
                          term_mode=1, S_greedy=1 << 20, score_mode=-1, delta_T=-1)
     run_parity(cfg, 2, 8, threads=threads, check_every=1)
+
+
+@pytest.mark.parametrize("H", [0, 8, 40])
+@pytest.mark.parametrize("W,n", [(128, 128), (256, 256), (260, 256), (128, 127)])
+def test_every_request_beyond_the_peak(H, W, n, monkeypatch):
+    # the queue fills whole groups of 128 positions, so no empty one ends the search for the largest request at or
+    # below the peak of the score, and every request is above it (equal margins: the first admission's peak is zero)
+    make = wlm.make_workload
+
+    def patched(*args, **kwargs):
+        wl = make(*args, **kwargs)
+        st = wl.state
+        run = st["act_base"] != EMPTY
+        st["act_base"][...] = np.where(run, 500, EMPTY)
+        st["load"][...] = 500 * run.sum(-1)
+        st["wq_s"][:, :n] = 3000 + (np.arange(n) * 37) % 500
+        return wl
+
+    monkeypatch.setattr(wlm, "make_workload", patched)
+    for S_greedy in (0, 1 << 20):
+        cfg = wlm.get_config("c2", G=9, B=16, W=W, H=H, R_max=4, init_active=14, init_queue=n, hazard=0.05, term_mode=1,
+                             S_greedy=S_greedy, score_mode=-1, delta_T=-1, arrival=("const", 0.0))
+        for threads in (32, 128):
+            run_parity(cfg, 2, 5, threads=threads, check_every=1)
 
 
 @pytest.mark.parametrize("H", [0, 2])
