@@ -29,25 +29,26 @@ def test_tile_edges(G, B, W, H, kw):
 
 @pytest.mark.parametrize("threads", [32, 96, 256])
 @pytest.mark.parametrize("H,R_max", [(0, 5), (4, 5), (40, 4)])
-def test_one_lane_holds_the_whole_window(H, R_max, threads, monkeypatch):
-    # the largest requests sit at positions of one router lane (4 consecutive of each 128): its list of four
-    # keys runs dry inside a window of five, and again after admissions
+@pytest.mark.parametrize("positions", [
+    [5 + 32 * i for i in range(10)],                      # one router lane's (it reads every 32nd): its list of four runs dry
+                                                          # while the window of five is built
+    [37, 69, 101, 133] + [65 + 6 * i for i in range(6)],  # its list is used up by the window and runs dry after an admission
+])
+def test_one_lane_holds_the_whole_window(H, R_max, threads, positions, monkeypatch):
     make = wlm.make_workload
 
     def patched(*args, **kwargs):
         wl = make(*args, **kwargs)
         q = wl.state["wq_s"]
-        for i, pos in enumerate([0, 1, 2, 3, 128, 129, 130, 131, 256, 257]):
+        for i, pos in enumerate(positions):
             q[:, pos] = 90000 - 7 * i
         return wl
 
     monkeypatch.setattr(wlm, "make_workload", patched)
-    cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
-                         term_mode=1, S_greedy=0, score_mode=-1, delta_T=-1)
-    run_parity(cfg, 2, 8, threads=threads, check_every=1)
-    cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
-                         term_mode=1, S_greedy=1 << 20, score_mode=-1, delta_T=-1)
-    run_parity(cfg, 2, 8, threads=threads, check_every=1)
+    for S_greedy in (0, 1 << 20):
+        cfg = wlm.get_config("c2", G=33, B=16, W=384, H=H, R_max=R_max, init_active=15, init_queue=380, hazard=0.05,
+                             term_mode=1, S_greedy=S_greedy, score_mode=-1, delta_T=-1)
+        run_parity(cfg, 2, 8, threads=threads, check_every=1)
 
 
 @pytest.mark.parametrize("H", [0, 8, 40])
