@@ -206,9 +206,7 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
     const br::StepLaunch shape = launch_shape(ctx, b->n_instances);
     step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, shape);
     const int threads = 32 * shape.warps;
-    // lanes per worker that turn its buckets into projected loads
-    a.seg_log2 = 0;
-    while (a.seg_log2 < 5 && (ctx->G << (a.seg_log2 + 1)) <= threads && (2 << a.seg_log2) <= ctx->H + 1) ++a.seg_log2;
+    a.seg_log2 = br::step_seg_log2(ctx->G, ctx->H, threads);
     const int smem = a.lay.total;
     if (smem > 48 * 1024) {
         // (br_create has checked the device maximum)

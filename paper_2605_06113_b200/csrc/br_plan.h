@@ -92,20 +92,31 @@ inline bool step_early(const StepShape &s)
     return s.term_mode == 1 && (!s.fp || (step_groups(s.H) && s.G * s.B >= 512));
 }
 
+// log2 of the lanes per worker that turn its prediction buckets into L_g(k+h), of `threads`
+inline int step_seg_log2(int G, int H, int threads)
+{
+    int q = 0;
+    while (q < 5 && (G << (q + 1)) <= threads && (2 << q) <= H + 1) ++q;
+    return q;
+}
+
 // Warps per instance, and which instantiation, for n_instances instances on `sms` SMs.
 //
 // More warps shorten an instance's parallel phases and leave fewer instances resident, so a batch of a few instances
 // per SM takes as many warps as there is work for, a large one those that need the least time for all its
 // waves.  With r resident instances of w warps a step takes, in units of the router's chain,
-//     t(w, r) = 1 + p (c + e r) / w,
-// p the thousands of slots that the projection streams (a little more the longer the classifier's rows, twice as
-// many when terminations read every row; Eq. 1 has draws and queue alone) and e what another resident instance costs.
-// The last, incomplete wave starts while instances of the one before still run and counts in part.  The constants
-// are a fit to 3,000 measured times (44 shapes, 1 to 28 instances per SM, one to eight warps, both instantiations): the
-// choice is within 1 % of the fastest on average, at worst 17 %.  us per call at 1, 2, 3, 4, 5 warps: 592 of G = 32,
-// H = 1: 44 / 33 / 27 / 25 / 23; 1,480: 57 / 37 / 48 / 47 / 56; 2,072: 65 / 67 / 76 / 74 / 80; 2,960:
-// 107 / 78 / 108 / 109 / 115.  Four warps at least for instances that stream 4,096 slots with long classifier rows: more
-// of them resident take each other's cache lines (1,480 of G = 64, H = 16: 227 / 189 / 102 / 89 / 106).
+//     t(w, r) = 1 + 0.015 u(w) + p (c + e r) / w,
+// u the offsets that a lane sums one after the other for L_g(k+h), each of which raises one word with the other
+// workers (41 workers and 60 offsets: 60 each with two warps, 30 with three; 1,738 instances, H = 59, eleven steps: 510
+// and 400 us, 367 in one wave), p the thousands of slots that the projection streams (a little more the longer the
+// classifier's rows, a fifth more where they are not whole vectors, twice as many when terminations read every
+// row; Eq. 1 has draws and queue alone) and e what another resident instance costs.  The last, incomplete wave starts
+// while instances of the one before still run and counts in part.  The constants are a fit to 3,000 measured times
+// (50 shapes, 1 to 28 instances per SM, one to eight warps, both instantiations): the choice is within 1 % of the
+// fastest on average, at worst 17 %.  us per call at 1, 2, 3, 4, 5 warps: 592 of G = 32, H = 1: 44 / 33 / 27 / 25 / 23;
+// 1,480: 57 / 37 / 48 / 47 / 56; 2,072: 65 / 67 / 76 / 74 / 80; 2,960: 107 / 78 / 108 / 109 / 115.  Four warps
+// at least for instances that stream 4,096 slots with long classifier rows: more of them resident take each
+// other's cache lines (1,480 of G = 64, H = 16: 227 / 189 / 102 / 89 / 106).
 inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
 {
     const int groups = step_groups(s.H), A = s.G * s.B, n = (n_instances + sms - 1) / sms;
@@ -117,13 +128,21 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
     most = most < 4 ? 4 : (most > 8 ? 8 : most);
     const bool long_rows = classifier && s.H >= 8 && groups && A * (s.term_mode == 2 ? 2 : 1) >= 4096;
     const int least = long_rows ? 4 : 1;
-    const double p = 7e-5 * s.W + (!s.H ? 0.035 + 0.005 * s.G
-                                        : 1e-3 * A * (classifier ? 1.0 + 0.02 * s.H : 1.0) * (s.term_mode == 2 ? 2 : 1));
+    double p = 1e-3 * A;
+    if (!s.H) p = 0.035 + 0.006 * s.G + 7e-5 * s.W;
+    else if (classifier) p = p * (1.0 + 0.02 * s.H) * ((s.H & 3) && s.H > 2 ? 1.2 : 1.0) * (s.term_mode == 2 ? 2 : 1) + 7e-5 * s.W;
+    else p += 2e-4 * s.W;
     struct Fit { double c, e, last, last_full; };
-    const Fit k = !s.H ? Fit{0.65, 0.03, 0.3, 0.4} : classifier ? Fit{0.75, 0.036, 0.65, 0.3} : Fit{0.7, 0.017, 0.5, 0.5};
+    const Fit k = !s.H ? Fit{0.65, 0.03, 0.3, 0.4} : classifier ? Fit{0.75, 0.036, 0.65, 0.3} : Fit{0.7, 0.013, 0.5, 0.5};
     StepLaunch best = {1, false, false};
     double cost = 1e300;
     for (int w = least; w <= most; ++w) {
+        double base = 1.0;
+        if (s.H > 0) {
+            const int q = step_seg_log2(s.G, s.H, 32 * w);
+            const int u = (((s.G << q) + 32 * w - 1) / (32 * w)) * ((s.H + (1 << q)) >> q);
+            base += 0.015 * u * (s.G < 32 ? s.G : 32) / 32.0;
+        }
         for (int lean = 0; lean < 2; ++lean) {
             // (the lean instantiation spills in the classifier's loop, which a single warp cannot hide)
             if (lean && (!step_has_lean(s.fp, groups) || (classifier && w < 2))) continue;
@@ -133,8 +152,8 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
             if (r > 32) r = 32;
             if (r < 1) r = 1;
             const int full = n / r, part = n % r;
-            double t = full * (1.0 + p * (k.c + k.e * r) / w);
-            if (part) t += (full ? k.last + k.last_full * part / r : 1.0) * (1.0 + p * (k.c + k.e * part) / w);
+            double t = full * (base + p * (k.c + k.e * r) / w);
+            if (part) t += (full ? k.last + k.last_full * part / r : 1.0) * (base + p * (k.c + k.e * part) / w);
             if (lean) t *= 1.1;
             if (t <= cost) { cost = t; best.warps = w; best.lean = lean != 0; }
         }

@@ -110,6 +110,8 @@ def test_a_batch_is_not_split_into_waves_that_fewer_warps_would_save(plan):
     # batches that just miss a wave take the lean instantiation where there is one
     assert _launch(plan, 40, 0, 148 * 28, shared=6000) == (1, True, 28)
     assert _launch(plan, 7, 60, 148 * 19, W=32, term=3, pred=1, shared=8000)[:2] == (1, True)
+    # three warps split the offsets of 41 workers, two do not
+    assert _launch(plan, 41, 59, 1738, B=24, W=84, term=3, pred=1, shared=27000)[:2] == (3, True)
     # long classifier rows: four or five warps whatever the batch
     for n in (4, 7, 10, 14, 20, 28):
         assert _launch(plan, 64, 8, 148 * n, shared=20000)[0] in (4, 5)
