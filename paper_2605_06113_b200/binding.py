@@ -310,7 +310,7 @@ class Router:
         return up.value, down.value
 
     def fscore(self, s, Lh, F, cap=None, best_g=None, N=None, first=0, stream=None):
-        n, n_req = s.shape[0], s.shape[1]             # (trailing dimensions of one are fine)
+        n, n_req = s.shape[:2]                         # (trailing dimensions of one are fine)
         b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
         rc = lib().br_fscore(self._h, b, _addr(s), n_req, _addr(Lh), _addr(cap), _addr(F), _addr(best_g))
         if rc != BR_OK:
@@ -318,7 +318,7 @@ class Router:
 
 
     def bypass_dispatch(self, s, virtual_load, inflight, inflight_cap, worker_out, N=None, first=0, stream=None):
-        n, n_req = s.shape[0], s.shape[1]             # (trailing dimensions of one are fine)
+        n, n_req = s.shape[:2]                         # (trailing dimensions of one are fine)
         b = _pack_batch(n - first if N is None else N, first, 1, self._stream(stream) or 0)
         rc = lib().br_bypass_dispatch(self._h, b, _addr(s), n_req, _addr(virtual_load), _addr(inflight),
                                       _addr(inflight_cap), _addr(worker_out))
