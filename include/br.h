@@ -192,7 +192,8 @@ int br_graph_step(br_ctx *ctx);
  * kernel in place where that is the faster way; the others go through device staging owned by ctx
  * (grown on demand with cudaMalloc), in batches of 512 instances or more in chunks of instances on three
  * internal streams (created on first use), so that uploads, kernels and downloads of different chunks
- * overlap.  Until the call returns the host arrays must not be touched.
+ * overlap.  Until the call returns the host arrays must not be touched; a call that fails with BR_ECUDA may leave
+ * arrays that are used in place, and after a failed copy back the others too, partly stepped.
  * h2d_bytes / d2h_bytes, if not NULL, receive the bytes of the arrays moved in each direction; arrays
  * used in place of which only the slots that change are touched (act_id, act_base with H = 0) do not count.
  * batch.n_steps must be 1 and batch.first_instance 0.
