@@ -207,6 +207,7 @@ int launch_step(br_ctx *ctx, const br_instance_batch *b, const br_worker_state *
     step_kernel_t kern = pick_kernel(ctx->p.score_mode == 1, ctx->H, ctx->G, shape);
     const int threads = 32 * shape.warps;
     a.seg_log2 = br::step_seg_log2(ctx->G, ctx->H, threads);
+    a.quads = (ctx->G * ctx->p.B / 4 + threads - 1) / threads;
     const int smem = a.lay.total;
     if (smem > 48 * 1024) {
         // (br_create has checked the device maximum)
@@ -290,6 +291,7 @@ int br_create(int32_t G, int32_t H, const br_params *params, br_ctx **out)
     StepArgs &a = ctx->base;
     a.G = G; a.H = H; a.B = p.B; a.W = p.W; a.R_max = p.R_max; a.S_greedy = p.S_greedy;
     a.occ_words = (p.B + 63) / 64;
+    a.b4_magic = br::quad_magic(p.B);
     a.wl = wl;
     a.Wp = (p.W + 127) / 128 * 128; a.HS = br::step_row_stride(H);
     a.delta_T = p.delta_T; a.gate = p.gate; a.c_floor = p.c_floor;

@@ -92,6 +92,10 @@ inline bool step_early(const StepShape &s)
     return s.term_mode == 1 && (!s.fp || (step_groups(s.H) && s.G * s.B >= 512));
 }
 
+// ceil(2^32 / (B / 4)): the worker of slot quad q < 2^14 is the upper half of q times this (B / 4 <= 64, so the error
+// stays below q * 64 < 2^32)
+inline uint32_t quad_magic(int B) { return (uint32_t)(((1ull << 32) + B / 4 - 1) / (B / 4)); }
+
 // log2 of the lanes per worker that turn its prediction buckets into L_g(k+h), of `threads`
 inline int step_seg_log2(int G, int H, int threads)
 {

@@ -45,6 +45,8 @@ struct StepArgs {
     int32_t HS;                 // row stride of L_g(k+h) in shared memory (>= H + 1)
     int32_t lpw_log2;           // log2 of the lanes that share a worker's row (fleets of up to 16 workers, long horizons)
     int32_t seg_log2;           // lanes per worker that turn its prediction buckets into L_g(k+h)
+    int32_t quads;              // slot quads that a thread takes in PREDICT (NT * quads covers A / 4)
+    uint32_t b4_magic;          // ceil(2^32 / (B / 4)): the worker of quad q is the upper half of q * b4_magic
     int32_t delta_T;
     float gate, c_floor;
     int32_t term_mode;
@@ -218,49 +220,115 @@ __device__ __forceinline__ long long ld_now8(const void *p)
 
 // Loads of classifier output.  A row is read once, by one thread, at a scattered address; left to
 // itself the L2 fetches 128 bytes around a missing sector, of which a refresh uses 32 on average,
-// so the loads ask for the smallest fetch the instruction set offers (64 bytes).
+// so the loads ask for the smallest fetch the instruction set offers (64 bytes).  Nor do they allocate in L1: where
+// shared memory leaves it little, the lines that wait for rows limit how many are in flight (1,024 instances of two
+// warps, a quarter of 4,096 rows each: 22.7 us, 15.9 this way; 28 KB of L1).
 __device__ __forceinline__ float4 ld_row4(const float *p)
 {
     float4 v;
-    asm volatile("ld.global.nc.L2::64B.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 // a whole row of eight probabilities (32-byte aligned) as one 256-bit load
 __device__ __forceinline__ void ld_row8(const float *p, float *o)
 {
     unsigned r[8];
-    asm volatile("ld.global.nc.L2::64B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "l"(p));
 #pragma unroll
     for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(r[i]);
 }
 
-// Sum and smallest element of the H probabilities of a classifier row.  The order of the fp32 sum is
-// free: it only feeds a bound with slack.
-__device__ __forceinline__ void row_sum(const float *q, int H, bool rows32, float &sum, float &low)
+// R classifier rows of H < HT probabilities, zero beyond, asked for together in the widest pieces that every row
+// allows (width: 8, 4, 2 or 1 probabilities).
+template <int HT, int R>
+__device__ __forceinline__ void load_rows(const float *const (&row)[R], int H, int width, float (&v)[R][HT])
 {
-    float s = 0.0f, mn = 0.0f;
-    if (rows32) {
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int h = 0; h < HT; ++h) v[r][h] = 0.0f;
+    if (width == 8) {
+#pragma unroll
+        for (int h = 0; h + 8 <= HT; h += 8)
+            if (h < H)
+#pragma unroll
+                for (int r = 0; r < R; ++r) ld_row8(row[r] + h, &v[r][h]);
+    } else if (width == 4) {
+#pragma unroll
+        for (int h = 0; h < HT; h += 4)
+            if (h < H)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float4 x = ld_row4(row[r] + h);
+                    v[r][h] = x.x; v[r][h + 1] = x.y; v[r][h + 2] = x.z; v[r][h + 3] = x.w;
+                }
+    } else if (width == 2) {
+#pragma unroll
+        for (int h = 0; h < HT; h += 2)
+            if (h < H)
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float2 x = __ldg(reinterpret_cast<const float2 *>(row[r] + h));
+                    v[r][h] = x.x; v[r][h + 1] = x.y;
+                }
+    } else {
+#pragma unroll
+        for (int h = 0; h < HT; ++h)
+            if (h < H)
+#pragma unroll
+                for (int r = 0; r < R; ++r) v[r][h] = __ldg(row[r] + h);
+    }
+}
+
+// Sum of the absolute probabilities of a row of a long horizon.  The order of the fp32 sum is free: it only feeds a
+// bound with slack.
+__device__ __forceinline__ float row_sum(const float *q, int H, int width)
+{
+    float s = 0.0f;
+    if (width == 8) {
         for (int h = 0; h < H; h += 8) {
             float v[8];
             ld_row8(q + h, v);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { s += v[j]; mn = fminf(mn, v[j]); }
+            for (int j = 0; j < 8; ++j) s += fabsf(v[j]);
         }
-    } else if ((H & 3) == 0) {
+    } else if (width == 4) {
 #pragma unroll 2
         for (int h = 0; h < H; h += 4) {
             const float4 v = ld_row4(q + h);
-            s += (v.x + v.y) + (v.z + v.w);
-            mn = fminf(fminf(fminf(mn, v.x), fminf(v.y, v.z)), v.w);
+            s += (fabsf(v.x) + fabsf(v.y)) + (fabsf(v.z) + fabsf(v.w));
         }
     } else {
 #pragma unroll 4
-        for (int h = 0; h < H; ++h) { const float v = __ldg(q + h); s += v; mn = fminf(mn, v); }
+        for (int h = 0; h < H; ++h) s += fabsf(__ldg(q + h));
     }
-    sum = s; low = mn;
+    return s;
 }
 
+// a[i] += x in shared memory, or a[i] = x, where `on`: predicated, not branched around.  (A branch that lanes leave and
+// join again costs about 50 cycles, and a warp's four slots of PREDICT had twelve: 1,350 cycles for 128 slots
+// whose data had arrived, 950 this way.)
+template <typename S>
+__device__ __forceinline__ void add_if(bool on, S a, int i, unsigned x)
+{
+#ifdef BR_BOUNDS
+    if (on) atomicAdd(reinterpret_cast<unsigned *>(&a[i]), x);
+#else
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p red.shared.add.u32 [%0], %1; }"
+                 :: "r"((unsigned)__cvta_generic_to_shared(a + i)), "r"(x), "r"((unsigned)on));
+#endif
+}
+template <typename S>
+__device__ __forceinline__ void put16_if(bool on, S a, int i, unsigned x)
+{
+#ifdef BR_BOUNDS
+    if (on) a[i] = (unsigned short)x;
+#else
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u16 [%0], %1; }"
+                 :: "r"((unsigned)__cvta_generic_to_shared(a + i)), "h"((unsigned short)x), "r"((unsigned)on));
+#endif
+}
 constexpr int kRegWin = 5;       // Stage-2 windows of up to five requests are scored one subset per lane
 constexpr int kBigWinLow = 8;    // larger windows (up to BR_MAX_RMAX = 16): subsets of the low eight entries are sorted
 // marks a condition as the exception, so that its block leaves the straight path of the admission loop
@@ -440,7 +508,6 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int NT = EARLY ? 32 : blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = EARLY ? 0 : tid >> 5, nwarps = NT >> 5;
-    stream_order_gate();
     const int G = a.G, H = FP ? a.H : 0, B = a.B, W = a.W, A = G * B, OW = a.occ_words, WL = a.wl;
     const int H1 = H + 1, HS = NC > 0 ? 4 * (NC | 1) : a.HS;
     constexpr int HC = NC > 0 ? 1 : 3;                // horizon offsets per lane
@@ -482,7 +549,21 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
     const auto adm = mk_span(reinterpret_cast<unsigned *>(smem + a.lay.due), min(W, A));
     // scal: [0] queue length after routing, [1] admitted, [2] Stage-1 iterations, [3] Stage-2 pops,
     //       [4] status bits of the step, [5] status bits of the prologue, [6] lowest admitted position,
-    //       [8] requests on the due list, [16..31] kept entries per warp (two sets of eight, compaction)
+    //       [16..31] kept entries per warp (two sets of eight, compaction)
+
+    // what comes from the arguments alone is set up while the kernel before this one drains
+    if (tid < 32) scal[tid] = 0;
+    if (FP) {
+#pragma unroll 1
+        for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
+#pragma unroll 1
+        for (int h = tid; h < HS + 4; h += NT) {
+            dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1];
+            iw_s[h] = a.iw[h];
+            if (h < HS) Ms[h] = h < H1 ? 0 : 0x7FFFFFFF;
+        }
+    }
+    stream_order_gate();
 
     // ---- per-instance global rows ----
     const auto g_base = mk_span(a.ws.act_base + (size_t)inst * A, A);
@@ -497,54 +578,59 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
     const auto t_out = mk_span(a.out_tab, a.out_tab ? (1ll << (32 - a.out_shift)) : 0);
     const auto t_term = mk_span(a.term_cdf, B);
 
-    const unsigned long long seed = a.ws.seed[inst];
+    // ---- snapshot to shared memory: everything is asked for before the first answer is used ----
+    // (one array after another, each loop waiting for its loads: 3,500 cycles for one instance of G = 64, W = 1,024;
+    // 2,600 this way)
+    const unsigned long long seed = (unsigned long long)ld_now8(a.ws.seed + inst);
+    int k = ld_now(a.ws.step + inst);
+    uint32_t next_id = (uint32_t)ld_now(a.ws.next_id + inst);
+    int n_w = ld_now(a.wq.n + inst);
+    unsigned long long occ_1 = 0ull;
+    int nact_1 = 0, load_1 = 0;
+    if (tid < G * OW) occ_1 = (unsigned long long)ld_now8(a.ws.occ + (size_t)inst * G * OW + tid);
+    if (tid < G) {
+        nact_1 = ld_now(a.ws.nact + (size_t)inst * G + tid);
+        load_1 = (int)ld_now8(a.ws.load + (size_t)inst * G + tid);
+    }
+    int4 s_1 = make_int4(0, 0, 0, 0), id_1 = s_1, o_1 = s_1;
+    if (4 * tid < W) {
+        s_1 = ld_now4(vec_at<const int4>(g_qs, 4 * tid));
+        id_1 = ld_now4(vec_at<const int4>(g_qid, 4 * tid));
+        if (life) o_1 = ld_now4(vec_at<const int4>(g_qo, 4 * tid));
+    }
     const uint32_t key0 = (uint32_t)seed, key1 = (uint32_t)(seed >> 32);
-    int k = a.ws.step[inst];
-    uint32_t next_id = a.ws.next_id[inst];
-    int n_w = a.wq.n[inst];
     int bad = 0;
     if (n_w < 0 || n_w > W) { bad = BR_ST_BAD_STATE; n_w = n_w < 0 ? 0 : W; }
-
-    // ---- snapshot to shared memory ----
-    if (tid < 32) scal[tid] = 0;
-#pragma unroll 1
-    for (int p0 = 4 * tid; p0 < a.Wp; p0 += 4 * NT) {
-        int4 v = make_int4(0, 0, 0, 0), o = make_int4(0, 0, 0, 0); uint4 u = make_uint4(0u, 0u, 0u, 0u);
-        if (p0 < W) {
-            v = *vec_at<const int4>(g_qs, p0);
-            u = *vec_at<const uint4>(g_qid, p0);
-            if (life) o = *vec_at<const int4>(g_qo, p0);
-        }
-        int4 kk;
-        kk.x = p0 + 0 < n_w ? (v.x << WL) | (int)(posmask - (unsigned)(p0 + 0)) : kQBeyond;
-        kk.y = p0 + 1 < n_w ? (v.y << WL) | (int)(posmask - (unsigned)(p0 + 1)) : kQBeyond;
-        kk.z = p0 + 2 < n_w ? (v.z << WL) | (int)(posmask - (unsigned)(p0 + 2)) : kQBeyond;
-        kk.w = p0 + 3 < n_w ? (v.w << WL) | (int)(posmask - (unsigned)(p0 + 3)) : kQBeyond;
-        *vec_at<int4>(q_key, p0) = kk;
-        *vec_at<uint4>(q_id, p0) = u;
-        if (life) *vec_at<int4>(q_o, p0) = o;
-    }
 #pragma unroll 1
     for (int i = tid; i < G * OW; i += NT) {
-        const unsigned long long o = reinterpret_cast<const unsigned long long *>(a.ws.occ)[(size_t)inst * G * OW + i];
+        const unsigned long long o = i == tid ? occ_1 : reinterpret_cast<const unsigned long long *>(a.ws.occ)[(size_t)inst * G * OW + i];
         occ[i] = o; occ0[i] = o; endm[i] = 0ull;
     }
 #pragma unroll 1
     for (int g = tid; g < G; g += NT) {
-        int na = a.ws.nact[(size_t)inst * G + g];
+        int na = g == tid ? nact_1 : a.ws.nact[(size_t)inst * G + g];
+        const int l = g == tid ? load_1 : (int)a.ws.load[(size_t)inst * G + g];
         if (na < 0 || na > B) { bad = BR_ST_BAD_STATE; na = na < 0 ? 0 : B; }
         cap_s[g] = B - na;
-        L0_s[g] = (int)a.ws.load[(size_t)inst * G + g];
+        L0_s[g] = l;
         sub_load[g] = 0u;
     }
-    if (FP) {
 #pragma unroll 1
-        for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
-#pragma unroll 1
-        for (int h = tid; h < HS + 4; h += NT) {
-            dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1];
-            iw_s[h] = a.iw[h];
-            if (h < HS) Ms[h] = h < H1 ? 0 : 0x7FFFFFFF;
+    for (int p0 = 4 * tid; p0 < a.Wp; p0 += 4 * NT) {
+        int4 kk;
+        kk.x = p0 + 0 < n_w ? (s_1.x << WL) | (int)(posmask - (unsigned)(p0 + 0)) : kQBeyond;
+        kk.y = p0 + 1 < n_w ? (s_1.y << WL) | (int)(posmask - (unsigned)(p0 + 1)) : kQBeyond;
+        kk.z = p0 + 2 < n_w ? (s_1.z << WL) | (int)(posmask - (unsigned)(p0 + 2)) : kQBeyond;
+        kk.w = p0 + 3 < n_w ? (s_1.w << WL) | (int)(posmask - (unsigned)(p0 + 3)) : kQBeyond;
+        *vec_at<int4>(q_key, p0) = kk;
+        *vec_at<int4>(q_id, p0) = id_1;
+        if (life) *vec_at<int4>(q_o, p0) = o_1;
+        const int p1 = p0 + 4 * NT;                       // the next piece
+        s_1 = id_1 = o_1 = make_int4(0, 0, 0, 0);
+        if (p1 < W) {
+            s_1 = ld_now4(vec_at<const int4>(g_qs, p1));
+            id_1 = ld_now4(vec_at<const int4>(g_qid, p1));
+            if (life) o_1 = ld_now4(vec_at<const int4>(g_qo, p1));
         }
     }
     __syncthreads();
@@ -600,19 +686,21 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
 
         // ============ PREDICT (H > 0): c_hat maintenance + horizon projection ============
         // Every running request adds (cur, 1) to the bucket (worker, floor(c_hat)); the buckets become
-        // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  Consecutive threads take
-        // consecutive slot quads: the loads have to be coalesced.  (Eight slots of one worker per thread and
-        // consecutive workers in consecutive threads keep the atomics of a warp on different rows but touch
-        // 32 lines with every load: 82 us a step against 77 at G = 64, H = 8, 1,024 instances.)  The next quad is
-        // requested before this one is worked on.
+        // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  A thread takes `quads` slot quads, the next one
+        // requested before this one is worked on.  The 32 lanes of a warp read eight pieces of 64 bytes, 4 * quads quads
+        // apart: consecutive quads in consecutive lanes are one worker's, whose few buckets serialise the atomics, and
+        // eight slots of one worker per thread touch 32 lines with every load.
+        const int q_first = ((warp << 5) + (lane & ~3)) * a.quads + (lane & 3);
+        int n_due = 0;                                    // requests on this warp's part of the due list
+        const auto due_w = due_list + (size_t)(classifier ? 128 * warp * a.quads : 0);
         if (FP && H > 0) {
-            const int A4 = A >> 2, B4 = B >> 2;
+            const int A4 = A >> 2, q_end = q_first + 4 * a.quads;
             const bool look = a.pred_mode == 1;
             int4 b4, x4 = make_int4(0, 0, 0, 0);                              // act_base; act_end or chat0
             unsigned kr = 0u;                                                 // refresh stamps
             auto fetch = [&](int q) {
                 b4 = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
-                if (q < A4) {
+                if (q < A4 && q < q_end) {
                     b4 = *vec_at<const int4>(g_base, 4 * q);
                     if (look) {
                         x4 = *vec_at<const int4>(g_end, 4 * q);
@@ -622,70 +710,167 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     }
                 }
             };
-            fetch(tid);
+            fetch(q_first);
+            const unsigned k_4 = (unsigned)(k & 255) * 0x01010101u, lt = (1u << lane) - 1u;
+            const float Hf = (float)H, dTf = (float)a.delta_T, two23 = 8388608.0f;
 #pragma unroll 1
-            for (int q0 = 0; q0 < A4; q0 += NT) {
-                const int q = q0 + tid, g = (int)((unsigned)q / (unsigned)B4);
+            for (int it4 = 0; it4 < 4 * a.quads; it4 += 4) {
+                const int q = q_first + it4;
+                const int g = (int)__umulhi((unsigned)q, a.b4_magic);
                 const int bs[4] = {b4.x, b4.y, b4.z, b4.w}, xs[4] = {x4.x, x4.y, x4.z, x4.w};
                 const unsigned k4 = kr;
-                fetch(q + NT);
+                fetch(q + 4);
                 if (look) {
                     // perfect lookahead: c_hat = min(r_i(k), H) with r_i(k) = act_end - k + 1 steps still to run.
                     // A request whose last step this is (act_end == k) is settled right here.
                     unsigned fb = 0u;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        if (bs[j] != kEmpty) {
-                            const int nh = min(max(xs[j] - k + 1, 0), H);
-                            const unsigned cur = (unsigned)(bs[j] + k);
-                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur);
-                            atomicAdd(&Ch[g * HS + nh], 1);
-                            if (xs[j] == k) { fb |= 1u << j; atomicAdd(&sub_load[g], cur); g_base[4 * q + j] = kEmpty; }
-                        }
+                        const bool live = bs[j] != kEmpty;
+                        const int at = g * HS + min(max(xs[j] - k + 1, 0), H);
+                        add_if(live, Lh, at, (unsigned)(bs[j] + k));
+                        add_if(live, Ch, at, 1u);
+                        fb |= live && xs[j] == k ? 1u << j : 0u;
                     }
-                    const int slot = 4 * (q - g * B4);
-                    if (fb) atomicOr(&endm32[2 * g * OW + (slot >> 5)], fb << (slot & 31));
+                    if (fb) {
+                        const int slot = 4 * q - g * B;
+                        atomicOr(&endm32[2 * g * OW + (slot >> 5)], fb << (slot & 31));
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            if ((fb >> j) & 1u) { atomicAdd(&sub_load[g], (unsigned)(bs[j] + k)); g_base[4 * q + j] = kEmpty; }
+                    }
                 } else {
                     // requests that are not due only age; the ones due for a refresh take c_hat = H (gate closed:
-                    // the conservative anchor) and go on a list, whose rows are read below
-                    unsigned dm[4], kn = k4;
-                    int cs[4], n_due = 0;
-                    bool due[4];
+                    // the conservative anchor) and go on the warp's list, whose rows are read below.  Ages are bytes, taken
+                    // from k four at a time; a byte t and floor(c) become a float and an integer through the
+                    // mantissa of 2^23 + x (conversions have a quarter of the rate).
+                    const unsigned t4 = ((k_4 | 0x80808080u) - (k4 & 0x7F7F7F7Fu)) ^ ((k_4 ^ ~k4) & 0x80808080u);
+                    bool live[4], due[4];
+                    int at[4], n = 0, to[4];
+                    unsigned dues = 0u;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int t = (k - (int)((k4 >> (8 * j)) & 0xFFu)) & 255;
-                        const float c = __int_as_float(xs[j]) - (float)t;
-                        const bool live = bs[j] != kEmpty;
-                        due[j] = live && (t >= a.delta_T || c < a.c_floor);
-                        dm[j] = __ballot_sync(kFull, due[j]);
-                        n_due += __popc(dm[j]);
-                        cs[j] = due[j] ? __float_as_int((float)H) : xs[j];
-                        int nh = H;
-                        if (due[j]) kn = (kn & ~(0xFFu << (8 * j))) | ((unsigned)(k & 255) << (8 * j));
-                        else nh = min(max((int)floorf(c), 0), H);
-                        if (live) {
-                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), (unsigned)(bs[j] + k));
-                            atomicAdd(&Ch[g * HS + nh], 1);
-                        }
+                        const float t = __int_as_float((int)__byte_perm(t4, 0x4B000000u, 0x7540u + j)) - two23;
+                        const float c = __int_as_float(xs[j]) - t;
+                        live[j] = bs[j] != kEmpty;
+                        due[j] = live[j] & ((t >= dTf) | (c < a.c_floor));
+                        const float ch = due[j] ? Hf : fminf(fmaxf(c, 0.0f), Hf);
+                        at[j] = g * HS + __float_as_int(__fadd_rd(ch, two23)) - 0x4B000000;
+                        to[j] = n;                                            // place among the thread's
+                        n += due[j] ? 1 : 0;
+                        dues |= due[j] ? 0xFFu << (8 * j) : 0u;
                     }
-                    if (n_due) {                                              // uniform over the warp
-                        int at = 0;
-                        if (lane == 0) at = atomicAdd(&scal[8], n_due);
-                        at = __shfl_sync(kFull, at, 0);
-                        const unsigned lt = (1u << lane) - 1u;
+                    // places among the warp's: the counts of the lanes below, bit by bit
+                    const unsigned n1 = __ballot_sync(kFull, n & 1), n2 = __ballot_sync(kFull, n & 2), n4 = __ballot_sync(kFull, n & 4);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            if (due[j]) due_list[at + __popc(dm[j] & lt)] = (unsigned short)(4 * q + j);
-                            at += __popc(dm[j]);
+                    for (int j = 0; j < 4; ++j) {
+                        add_if(live[j], Lh, at[j], (unsigned)(bs[j] + k));
+                        add_if(live[j], Ch, at[j], 1u);
+                    }
+                    const int first = n_due + __popc(n1 & lt) + 2 * __popc(n2 & lt) + 4 * __popc(n4 & lt);
+                    n_due += __popc(n1) + 2 * __popc(n2) + 4 * __popc(n4);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) put16_if(due[j], due_w, first + to[j], (unsigned)(4 * q + j));
+                    if (dues) {
+                        const int anchor = __float_as_int(Hf);
+                        *vec_at<int4>(g_chat0, 4 * q) = make_int4(due[0] ? anchor : xs[0], due[1] ? anchor : xs[1], due[2] ? anchor : xs[2], due[3] ? anchor : xs[3]);
+                        *vec_at<unsigned>(g_kref, 4 * q) = (k4 & ~dues) | (k_4 & dues);
+                    }
+                }
+            }
+            if (classifier) {
+                // The classifier row of every request on the warp's list.  p_fin = 1 - prod (1 - q_h) <= sum |q_h| while that
+                // sum is below one: when the fp32 sum is clearly below the gate the fp64 product cannot reach it and is
+                // not evaluated.
+                __syncwarp();
+                const float *rows = reinterpret_cast<const float *>(raw_of(probs));
+                const int width = (H & 7) == 0 && (reinterpret_cast<size_t>(rows) & 31) == 0 ? 8 : (H & 3) == 0 ? 4 : (H & 1) == 0 ? 2 : 1;
+                const float closed = fminf(a.gate, 1.0f);
+                constexpr int R = NC == 2 ? 4 : NC == 3 ? 3 : 2;                  // rows in flight per thread
+#pragma unroll 1
+                for (int e1 = 0; e1 < n_due; e1 += 32 * R) {
+                    const int e0 = e1 + lane;
+                    int sa[R];
+                    const float *row[R];
+                    bool open[R];
+                    double c[R], surv[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        sa[r] = due_w[e0 + 32 * r < n_due ? e0 + 32 * r : e1];
+                        row[r] = rows + (size_t)sa[r] * H;
+                        c[r] = 0.0; surv[r] = 1.0;
+                    }
+                    bool any = false;
+                    if (NC > 0) {
+                        float v[R][NC > 0 ? 4 * NC : 1];
+                        load_rows(row, H, width, v);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            float sum = 0.0f;
+#pragma unroll
+                            for (int h = 0; h < HT; ++h) sum += fabsf(v[r][h]);
+                            open[r] = e0 + 32 * r < n_due && !(sum * 1.0001f < closed);
+                            any = any || open[r];
                         }
-                        if (due[0] || due[1] || due[2] || due[3]) {
-                            *vec_at<int4>(g_chat0, 4 * q) = make_int4(cs[0], cs[1], cs[2], cs[3]);
-                            *vec_at<unsigned>(g_kref, 4 * q) = kn;
+                        if (any) {
+                            // E[min(r, H)] = sum_h prod_{j<h} (1 - q_j)
+#pragma unroll
+                            for (int h = 0; h < HT; ++h)
+                                if (h < H)
+#pragma unroll
+                                    for (int r = 0; r < R; ++r) {
+                                        c[r] = __dadd_rn(c[r], surv[r]);
+                                        surv[r] = __dmul_rn(surv[r], __dsub_rn(1.0, (double)v[r][h]));
+                                    }
+                        }
+                    } else {
+                        float sum[R];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) sum[r] = row_sum(row[r], H, width);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            open[r] = e0 + 32 * r < n_due && !(sum[r] * 1.0001f < closed);
+                            any = any || open[r];
+                        }
+                        if (any)
+#pragma unroll 1
+                            for (int h = 0; h < H; ++h)
+#pragma unroll
+                                for (int r = 0; r < R; ++r) {
+                                    c[r] = __dadd_rn(c[r], surv[r]);
+                                    surv[r] = __dmul_rn(surv[r], __dsub_rn(1.0, (double)__ldg(row[r] + h)));
+                                }
+                    }
+                    if (any) {
+                        unsigned cur[R];
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            open[r] = open[r] && __dsub_rn(1.0, surv[r]) >= (double)a.gate;
+                            cur[r] = open[r] ? (unsigned)(g_base[sa[r]] + k) : 0u;
+                        }
+#pragma unroll
+                        for (int r = 0; r < R; ++r) {
+                            if (!open[r]) continue;
+                            double cc = c[r] < (double)a.c_floor ? (double)a.c_floor : c[r];      // clipped to [floor, H]
+                            cc = cc > (double)H ? (double)H : cc;
+                            const float cf = (float)cc;
+                            g_chat0[sa[r]] = cf;
+                            const int nh = min(max((int)floorf(cf), 0), H);
+                            if (nh != H) {                                      // from the anchor's bucket to its own
+                                const int g = (int)__umulhi((unsigned)sa[r] >> 2, a.b4_magic);
+                                atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + H]), 0u - cur[r]);
+                                atomicAdd(&Ch[g * HS + H], -1);
+                                atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur[r]);
+                                atomicAdd(&Ch[g * HS + nh], 1);
+                            }
                         }
                     }
                 }
             }
         }
+        // (This barrier is for the compiler: where it cannot tell that a warp is whole after loops of divergent length, it
+        // guards every warp maximum of the admission loop, and a pop takes a fifth longer.)
+        if (FP && H > 0) __syncthreads();
         // arrivals join the queue
         int n_arr = 0;
         if (a.arr_cdf) {
@@ -720,54 +905,9 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
         next_id += (uint32_t)n_arr;
 
         if (FP) {
-            __syncthreads();                              // buckets and due list complete
-            if (classifier) {
-                // the classifier row of every request on the list, two in flight per thread.
-                // p_fin = 1 - prod (1 - q_h) <= sum q_h for probabilities: when the fp32 sum is clearly below
-                // the gate the fp64 product cannot reach it and is not evaluated.
-                const int n_due = scal[8];
-                const bool rows32 = (H & 7) == 0 && (reinterpret_cast<size_t>(raw_of(probs)) & 31) == 0;
-                const float *rows = reinterpret_cast<const float *>(raw_of(probs));
-#pragma unroll 1
-                for (int e0 = tid; e0 < n_due; e0 += 2 * NT) {
-                    const int e1 = e0 + NT;
-                    const int sa0 = due_list[e0], sa1 = e1 < n_due ? due_list[e1] : sa0;
-                    float sum[2], low[2];
-                    row_sum(rows + (size_t)sa0 * H, H, rows32, sum[0], low[0]);
-                    row_sum(rows + (size_t)sa1 * H, H, rows32, sum[1], low[1]);
-#pragma unroll 1
-                    for (int e = 0; e < 2; ++e) {
-                        const float sm = e ? sum[1] : sum[0], lo = e ? low[1] : low[0];
-                        if ((lo >= 0.0f && sm * 1.0001f < a.gate) || (e && e1 >= n_due)) continue;
-                        const int sa = e ? sa1 : sa0;
-                        // gate open: E[min(r, H)] = sum_h prod_{j<h} (1 - q_j)
-                        double surv = 1.0, c = 0.0;
-#pragma unroll 1
-                        for (int h = 0; h < H; ++h) {
-                            c = __dadd_rn(c, surv);
-                            surv = __dmul_rn(surv, __dsub_rn(1.0, (double)__ldg(rows + (size_t)sa * H + h)));
-                        }
-                        if (!(__dsub_rn(1.0, surv) >= (double)a.gate)) continue;
-                        if (c < (double)a.c_floor) c = (double)a.c_floor;   // clipped to [floor, H]
-                        if (c > (double)H) c = (double)H;
-                        const float cf = (float)c;
-                        g_chat0[sa] = cf;
-                        int nh = (int)floorf(cf);
-                        nh = nh < 0 ? 0 : (nh > H ? H : nh);
-                        if (nh != H) {                                      // from the anchor's bucket to its own
-                            const int g = sa / B;
-                            const unsigned cur = (unsigned)(g_base[sa] + k);
-                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + H]), 0u - cur);
-                            atomicAdd(&Ch[g * HS + H], -1);
-                            atomicAdd(reinterpret_cast<unsigned *>(&Lh[g * HS + nh]), cur);
-                            atomicAdd(&Ch[g * HS + nh], 1);
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-            // buckets -> L_g(k+h): 2^seg_log2 lanes per worker, each with a stretch of offsets
-            if (H > 0) {
+            __syncthreads();                              // buckets complete
+            // buckets -> L_g(k+h), long horizons: 2^seg_log2 lanes per worker, each with a stretch of offsets
+            if (NC == 0) {
                 const int SEG = 1 << a.seg_log2, SL = (H1 + SEG - 1) >> a.seg_log2;
 #pragma unroll 1
                 for (int i0 = warp << 5; i0 < (G << a.seg_log2); i0 += NT) {
@@ -791,12 +931,11 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                         atomicMax(&Ms[h], x);                               // envelope M_h
                     }
                 }
-            } else {
-#pragma unroll 1
-                for (int g = tid; g < G; g += NT) { Lh[g * HS] = L0_s[g]; atomicMax(&Ms[0], L0_s[g]); }
+                __syncthreads();
             }
+        } else {
+            __syncthreads();
         }
-        __syncthreads();
         if (timing) t_phase[2] = (unsigned)clock64();
 
         // ---- requests running before this step that end at it: by warps 1.. while warp 0 routes ----
@@ -868,7 +1007,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
             for (int w = 0; w < GW; ++w) {
                 const int g = lane + 32 * w;
                 cap[w] = g < G ? cap_s[g] : -1;
-                L0[w] = g < G ? (FP ? Lh[g * HS] : L0_s[g]) : 0;
+                L0[w] = g < G ? (NC == 0 ? Lh[g * HS] : L0_s[g]) : 0;
                 mm[w] = 0;
             }
             // rows of all workers: Ms - row (FIRST: loads become margins) or Ms + row (the envelope grew by Ms), and
@@ -913,7 +1052,59 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                 }
                 __syncwarp();
             };
-            if (FP) {
+            if (FP && NC > 0) {
+                // buckets -> L_g(k+h) by suffix sums in registers, envelope M_h by warp maxima, margins to shared memory
+                // (with a phase of all warps for the sums, and the envelope by shared-memory maxima, 2,300 to 3,200 cycles
+                // a step in batches, 2,000 to 2,300 this way)
+                int l[GW][HT > 0 ? HT : 1];
+#pragma unroll
+                for (int w = 0; w < GW; ++w) {
+                    const int g = lane + 32 * w;
+#pragma unroll
+                    for (int h = 0; h < HT; ++h) l[w][h] = 0;
+                    if (g < G) {
+                        if (H > 0) {
+                            int cn[HT > 0 ? HT : 1];
+#pragma unroll
+                            for (int h = 0; h < HT; h += 4) {
+                                const int4 t = *vec_at<const int4>(Lh, g * HS + h), c = *vec_at<const int4>(Ch, g * HS + h);
+                                l[w][h] = t.x; l[w][h + 1] = t.y; l[w][h + 2] = t.z; l[w][h + 3] = t.w;
+                                cn[h] = c.x; cn[h + 1] = c.y; cn[h + 2] = c.z; cn[h + 3] = c.w;
+                            }
+#pragma unroll
+                            for (int h = HT - 2; h >= 0; --h) { l[w][h] += l[w][h + 1]; cn[h] += cn[h + 1]; }
+#pragma unroll
+                            for (int h = 0; h < HT; ++h) l[w][h] += h * cn[h];
+                            L0[w] = l[w][0];
+                        } else {
+                            l[w][0] = L0[w];
+                        }
+                        mm[w] = 0x7FFFFFFF;
+                    }
+                }
+#pragma unroll
+                for (int h = 0; h < HT; ++h) {
+                    int e = l[0][h];
+#pragma unroll
+                    for (int w = 1; w < GW; ++w) e = max(e, l[w][h]);
+                    e = __reduce_max_sync(kFull, e);                    // (lanes without a worker hold zero)
+#pragma unroll
+                    for (int w = 0; w < GW; ++w) {
+                        l[w][h] = h < H1 ? e - l[w][h] : 0x7FFFFFFF;
+                        mm[w] = min(mm[w], l[w][h]);
+                    }
+                }
+#pragma unroll
+                for (int w = 0; w < GW; ++w) {
+                    const int g = lane + 32 * w;
+                    if (g < G) {
+#pragma unroll
+                        for (int h = 0; h < HT; h += 4) *vec_at<int4>(Lh, g * HS + h) = make_int4(l[w][h], l[w][h + 1], l[w][h + 2], l[w][h + 3]);
+                    }
+                }
+                __syncwarp();
+                if (lane < HS) Ms[lane] = 0;
+            } else if (FP) {
                 __syncwarp();                          // every lane has read L_g(k) before rows become margins
                 rows(true);
 #pragma unroll
@@ -1546,7 +1737,6 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                 c[0] = (uint32_t)n_drop; c[1] = (uint32_t)scal[1]; c[2] = (uint32_t)scal[2]; c[3] = (uint32_t)scal[3];
             }
             if (a.out.status) a.out.status[orow] = scal[4] | scal[5];
-            scal[8] = 0;
             if (timing) {
                 t_phase[6] = (unsigned)clock64();
                 uint32_t *pc = a.out.phase_cycles + orow * 8;
