@@ -134,11 +134,12 @@ int check_step_args(const br_ctx *ctx, const br_instance_batch *b, const br_work
 }
 
 // Launch with programmatic stream serialisation: the blocks of this launch may become resident
-// while the previous kernel of the stream is still draining.  Both step kernels open with
+// while the previous kernel of the stream is still draining.  The kernels open with
 // griddepcontrol.wait, which returns only when every earlier kernel of the stream has completed
 // and its writes are visible, so only launch latency and block scheduling overlap.
-cudaError_t launch_overlapped(step_kernel_t kern, int blocks, int threads, size_t smem, cudaStream_t stream,
-                              const StepArgs &a, bool overlap)
+template <typename Args>
+cudaError_t launch_overlapped(void (*kern)(const Args), dim3 blocks, int threads, size_t smem, cudaStream_t stream,
+                              const Args &a, bool overlap)
 {
     if (!overlap) {                      // plain launch (stream capture)
         kern<<<blocks, threads, smem, stream>>>(a);
@@ -146,7 +147,7 @@ cudaError_t launch_overlapped(step_kernel_t kern, int blocks, int threads, size_
     }
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3((unsigned)threads);
+    cfg.gridDim = blocks; cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -738,6 +739,8 @@ int br_fscore(br_ctx *ctx, const br_instance_batch *batch, const int32_t *s, int
     const dim3 grid((n_requests + per_block - 1) / per_block, batch->n_instances);
     const int smem = br::fscore_smem(ctx->G, a.row);                      // at most 42 KB
     void (*kern)(const br::FscoreArgs) = a.fp ? br::br_fscore_kernel<true> : br::br_fscore_kernel<false>;
+    // (a plain launch: blocks of the next call that become resident early spread unevenly, 200 x 1,024 x 64 scores at
+    // H = 8 33 us, 40 with overlapping launches)
     kern<<<grid, 32 * br::kFsWarps, smem, (cudaStream_t)batch->stream>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "br_fscore launch");
@@ -791,8 +794,8 @@ int br_bypass_dispatch(br_ctx *ctx, const br_instance_batch *batch, const int32_
     a.s = s; a.vload = virtual_load; a.inflight = inflight; a.cap = inflight_cap; a.g_out = worker_out;
     void (*kern)(const br::BypassArgs) = a.f.fp ? (ctx->G <= 32 ? br::br_bypass_kernel<true, 1> : br::br_bypass_kernel<true, 2>)
                                                 : (ctx->G <= 32 ? br::br_bypass_kernel<false, 1> : br::br_bypass_kernel<false, 2>);
-    kern<<<batch->n_instances, 32, 0, (cudaStream_t)batch->stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_overlapped(kern, dim3((unsigned)batch->n_instances), 32, 0, (cudaStream_t)batch->stream, a, true);
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "br_bypass_dispatch launch");
     return BR_OK;
 }

@@ -32,10 +32,14 @@ struct BypassArgs {
 // a time, and the next length is fetched while the warp maximum is on its way.
 // 256 instances x 200 requests at G = 32: 74 us with the envelope and a 64-bit score reduced over the warp
 // for every request, 19 us with 64-bit margins, 12 this way.
+// The launch overlaps the kernel ahead (launch_overlapped): a pass of two copies and the dispatch, 256 x 200, G = 32: 17.5 us,
+// 16.5; 4,096 x 33, G = 64: 18.5, 17.0; 20,000 x 32: 33.1, 31.1.  Closing workers by a count kept off the chain gained
+// 0.4 us more on the first and lost 1.7 on the second.
 // FP: Eq. 2 scores; GW: workers per lane.
 template <bool FP, int GW>
 __global__ void __launch_bounds__(32) br_bypass_kernel(const BypassArgs a)
 {
+    stream_order_gate();
     const int lane = threadIdx.x;
     const size_t inst = (size_t)a.first_instance + blockIdx.x;
     const int G = a.f.G;
