@@ -555,7 +555,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
     if (tid < 32) scal[tid] = 0;
     if (FP) {
 #pragma unroll 1
-        for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
+        for (int i = 4 * tid; i < G * HS; i += 4 * NT) { *vec_at<int4>(Lh, i) = make_int4(0, 0, 0, 0); if (H > 0) *vec_at<int4>(Ch, i) = make_int4(0, 0, 0, 0); }
 #pragma unroll 1
         for (int h = tid; h < HS + 4; h += NT) {
             dn_s[2 * h] = a.dn[2 * h]; dn_s[2 * h + 1] = a.dn[2 * h + 1];
@@ -928,10 +928,27 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                         Ti += Lh[g * HS + h]; Ci += Ch[g * HS + h];
                         const int x = Ti + h * Ci;
                         Lh[g * HS + h] = x;
-                        atomicMax(&Ms[h], x);                               // envelope M_h
+                        if (G > 16) atomicMax(&Ms[h], x);                   // envelope M_h
                     }
                 }
                 __syncthreads();
+                if (G <= 16) {
+                    // few workers: a thread per offset takes the envelope over them and leaves margins behind
+                    // (XXXX)
+#pragma unroll 1
+                    for (int h = tid; h < HS; h += NT) {
+                        int e = 0;
+#pragma unroll 4
+                        for (int g = 0; g < G; ++g) {
+                            const int x = Lh[g * HS + h];
+                            e = max(e, x);
+                            if (h == 0) L0_s[g] = x;
+                        }
+#pragma unroll 4
+                        for (int g = 0; g < G; ++g) Lh[g * HS + h] = h < H1 ? e - Lh[g * HS + h] : 0x7FFFFFFF;
+                    }
+                    __syncthreads();
+                }
             }
         } else {
             __syncthreads();
@@ -1007,7 +1024,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
             for (int w = 0; w < GW; ++w) {
                 const int g = lane + 32 * w;
                 cap[w] = g < G ? cap_s[g] : -1;
-                L0[w] = g < G ? (NC == 0 ? Lh[g * HS] : L0_s[g]) : 0;
+                L0[w] = g < G ? (NC == 0 && G > 16 ? Lh[g * HS] : L0_s[g]) : 0;
                 mm[w] = 0;
             }
             // rows of all workers: Ms - row (FIRST: loads become margins) or Ms + row (the envelope grew by Ms), and
@@ -1020,11 +1037,12 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     if (g < G) {
 #pragma unroll 2
                         for (int h = 4 * (lane & ((1 << q) - 1)); h < H1; h += 4 << q) {
-                            const int4 e = *vec_at<const int4>(Ms, h);
                             int4 l = *vec_at<const int4>(Lh, g * HS + h);
-                            if (first) { l.x = -l.x; l.y = -l.y; l.z = -l.z; l.w = -l.w; }
-                            l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
-                            *vec_at<int4>(Lh, g * HS + h) = l;
+                            if (!first) {                                   // (these rows are margins already)
+                                const int4 e = *vec_at<const int4>(Ms, h);
+                                l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
+                                *vec_at<int4>(Lh, g * HS + h) = l;
+                            }
                             x = min(min(x, l.x), min(min(l.y, l.z), l.w));
                         }
                     }
@@ -1727,7 +1745,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
         }
         if (FP && it + 1 < a.n_steps) {
 #pragma unroll 1
-            for (int i = tid; i < G * HS; i += NT) { Lh[i] = 0; if (H > 0) Ch[i] = 0; }
+            for (int i = 4 * tid; i < G * HS; i += 4 * NT) { *vec_at<int4>(Lh, i) = make_int4(0, 0, 0, 0); if (H > 0) *vec_at<int4>(Ch, i) = make_int4(0, 0, 0, 0); }
 #pragma unroll 1
             for (int h = tid; h < HS; h += NT) Ms[h] = h < H1 ? 0 : 0x7FFFFFFF;
         }
