@@ -51,20 +51,37 @@ def test_in_place_matches_device_step(name, n_inst, kw, pinned):
     r.close()
 
 
-def _host_step_us(cfg, wl, place, fscore):
-    """Shortest host-buffer step on buffers that `place` makes from pageable ones."""
-    r = Router(wl, device="cuda:0")
-    n = wl.state["step"].shape[0]
-    st = {k: place(v.cpu()) for k, v in r.device_state().items()}
-    out = {k: place(v) for k, v in r.outputs(n, device="cpu", fscore=fscore).items()}
-    probs = place(torch.full((n, cfg.G, cfg.B, cfg.H), 0.02)) if cfg.H else None
-    best = 1e30
-    for _ in range(9):
+class _HostStep:
+    """Host-buffer steps on buffers that `place` makes from pageable ones."""
+
+    def __init__(self, cfg, wl, place, fscore):
+        n = wl.state["step"].shape[0]
+        self.r, self.best = Router(wl, device="cuda:0"), 1e30
+        self.st = {k: place(v.cpu()) for k, v in self.r.device_state().items()}
+        self.out = {k: place(v) for k, v in self.r.outputs(n, device="cpu", fscore=fscore).items()}
+        self.probs = place(torch.full((n, cfg.G, cfg.B, cfg.H), 0.02)) if cfg.H else None
+
+    def step(self):
         t0 = time.perf_counter()
-        r.step_host(st, out, probs)
-        best = min(best, time.perf_counter() - t0)
-    r.close()
-    return 1e6 * best
+        self.r.step_host(self.st, self.out, self.probs)
+        self.best = min(self.best, time.perf_counter() - t0)
+
+
+def _faster(cfg, wl, place, other, factor, fscore):
+    """Whether the shortest step with `place` takes less than `factor` times the shortest with `other`.  The bus has other
+    users, and for seconds at a time every step takes up to twice as long, so the two are timed in turn, and over
+    more rounds while the answer is no: a difference that is there stays in the shortest of them."""
+    a, b = _HostStep(cfg, wl, place, fscore), _HostStep(cfg, wl, other, fscore)
+    for _ in range(8):
+        for _ in range(12):
+            a.step()
+            b.step()
+        if a.best < factor * b.best:
+            break
+        time.sleep(0.2)
+    a.r.close()
+    b.r.close()
+    return a.best < factor * b.best
 
 
 def _page_locked_off_16(t):
@@ -78,7 +95,7 @@ def test_score_matrix_is_not_slower_page_locked():
     # written an element at a time (in place it took 2.4 times as long as from pageable memory)
     cfg = wlm.get_config("c3")
     wl = wlm.make_workload(cfg, n_instances=512)
-    assert _host_step_us(cfg, wl, torch.Tensor.pin_memory, True) < _host_step_us(cfg, wl, lambda t: t.clone(), True)
+    assert _faster(cfg, wl, torch.Tensor.pin_memory, lambda t: t.clone(), 1.0, True)
 
 
 def test_terminations_from_classifier_rows_are_not_slower_in_place():
@@ -86,7 +103,7 @@ def test_terminations_from_classifier_rows_are_not_slower_in_place():
     # are copied now, and a fifth is left for the bus's other users
     cfg = wlm.get_config("c4", term_mode=2, burst_every=0, init_active=60)
     wl = wlm.make_workload(cfg, n_instances=63)
-    assert _host_step_us(cfg, wl, torch.Tensor.pin_memory, False) < 1.2 * _host_step_us(cfg, wl, _page_locked_off_16, False)
+    assert _faster(cfg, wl, torch.Tensor.pin_memory, _page_locked_off_16, 1.2, False)
 
 
 @pytest.mark.parametrize("name,n_inst", [("c3", 3), ("c3", 520), ("c2", 3)])
