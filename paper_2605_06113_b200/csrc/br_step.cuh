@@ -906,7 +906,9 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
 
         if (FP) {
             __syncthreads();                              // buckets complete
-            // buckets -> L_g(k+h), long horizons: 2^seg_log2 lanes per worker, each with a stretch of offsets
+            // buckets -> L_g(k+h), long horizons: 2^seg_log2 lanes per worker, each with a stretch of offsets.  (The envelope
+            // by a thread per offset over the workers, behind one more barrier, instead of shared-memory maxima: H = 80, four
+            // steps, 1,036 of G = 8, W = 512: 71.8 us, 66.1 this way; 2,072 of G = 16: 167.6, 157.8; one cluster of G = 8 11.4, 11.2)
             if (NC == 0) {
                 const int SEG = 1 << a.seg_log2, SL = (H1 + SEG - 1) >> a.seg_log2;
 #pragma unroll 1
@@ -928,27 +930,10 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                         Ti += Lh[g * HS + h]; Ci += Ch[g * HS + h];
                         const int x = Ti + h * Ci;
                         Lh[g * HS + h] = x;
-                        if (G > 16) atomicMax(&Ms[h], x);                   // envelope M_h
+                        atomicMax(&Ms[h], x);                               // envelope M_h
                     }
                 }
                 __syncthreads();
-                if (G <= 16) {
-                    // few workers: a thread per offset takes the envelope over them and leaves margins behind
-                    // (XXXX)
-#pragma unroll 1
-                    for (int h = tid; h < HS; h += NT) {
-                        int e = 0;
-#pragma unroll 4
-                        for (int g = 0; g < G; ++g) {
-                            const int x = Lh[g * HS + h];
-                            e = max(e, x);
-                            if (h == 0) L0_s[g] = x;
-                        }
-#pragma unroll 4
-                        for (int g = 0; g < G; ++g) Lh[g * HS + h] = h < H1 ? e - Lh[g * HS + h] : 0x7FFFFFFF;
-                    }
-                    __syncthreads();
-                }
             }
         } else {
             __syncthreads();
@@ -1024,7 +1009,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
             for (int w = 0; w < GW; ++w) {
                 const int g = lane + 32 * w;
                 cap[w] = g < G ? cap_s[g] : -1;
-                L0[w] = g < G ? (NC == 0 && G > 16 ? Lh[g * HS] : L0_s[g]) : 0;
+                L0[w] = g < G ? (NC == 0 ? Lh[g * HS] : L0_s[g]) : 0;
                 mm[w] = 0;
             }
             // rows of all workers: Ms - row (FIRST: loads become margins) or Ms + row (the envelope grew by Ms), and
@@ -1037,12 +1022,11 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     if (g < G) {
 #pragma unroll 2
                         for (int h = 4 * (lane & ((1 << q) - 1)); h < H1; h += 4 << q) {
+                            const int4 e = *vec_at<const int4>(Ms, h);
                             int4 l = *vec_at<const int4>(Lh, g * HS + h);
-                            if (!first) {                                   // (these rows are margins already)
-                                const int4 e = *vec_at<const int4>(Ms, h);
-                                l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
-                                *vec_at<int4>(Lh, g * HS + h) = l;
-                            }
+                            if (first) { l.x = -l.x; l.y = -l.y; l.z = -l.z; l.w = -l.w; }
+                            l.x += e.x; l.y += e.y; l.z += e.z; l.w += e.w;
+                            *vec_at<int4>(Lh, g * HS + h) = l;
                             x = min(min(x, l.x), min(min(l.y, l.z), l.w));
                         }
                     }
@@ -1743,6 +1727,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
             L0_s[g] = L0_s[g] - (int)sub_load[g] + na;
             sub_load[g] = 0u;
         }
+        // (16 bytes a store: 592 of G = 32, H = 8, four steps, 75.8 us with four, 74.0 this way; 2,072: 211.6, 208.0)
         if (FP && it + 1 < a.n_steps) {
 #pragma unroll 1
             for (int i = 4 * tid; i < G * HS; i += 4 * NT) { *vec_at<int4>(Lh, i) = make_int4(0, 0, 0, 0); if (H > 0) *vec_at<int4>(Ch, i) = make_int4(0, 0, 0, 0); }
