@@ -308,6 +308,13 @@ int br_survival_chat(br_ctx *ctx, void *stream, const int32_t *hist_sorted, cons
 int br_debug_bounds_hits(void);
 int br_debug_bounds_selftest(int32_t *four_ints);
 
+/*
+ * Registers a thread of the block-per-instance step kernel for these sizes uses (lean: the instantiation with fewer
+ * registers, early: the one for a single warp under the constant hazard; where there is none, the common one), and in
+ * *planned what the choice of a launch shape counts with.  BR_EINVAL for sizes outside the compiled limits.
+ */
+int br_debug_step_registers(int32_t score_mode, int32_t G, int32_t H, int32_t lean, int32_t early, int32_t *planned);
+
 /* Frees the context, its staging buffers and graph.  NULL is accepted. */
 int br_destroy(br_ctx *ctx);
 

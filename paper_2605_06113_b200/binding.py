@@ -56,7 +56,7 @@ class BrLoadOut(C.Structure):
 
 
 EXPORTS = ["br_create", "br_step", "br_graph_capture", "br_graph_step", "br_step_host",
-           "br_step_host_static", "br_debug_bounds_hits", "br_debug_bounds_selftest",
+           "br_step_host_static", "br_debug_bounds_hits", "br_debug_bounds_selftest", "br_debug_step_registers",
            "br_fscore", "br_best_subset", "br_bypass_dispatch", "br_survival_chat", "br_destroy", "br_strerror", "br_version"]
 
 _lib = None
@@ -94,6 +94,7 @@ def lib():
                                        C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p]
         L.br_debug_bounds_hits.argtypes = []
         L.br_debug_bounds_selftest.argtypes = [C.c_void_p]
+        L.br_debug_step_registers.argtypes = [C.c_int32] * 5 + [C.POINTER(C.c_int32)]
         L.br_destroy.argtypes = [C.c_void_p]
         L.br_strerror.restype = C.c_char_p
         L.br_strerror.argtypes = [C.c_int]

@@ -864,6 +864,20 @@ int br_debug_bounds_selftest(int32_t *four_ints)
 #endif
 }
 
+int br_debug_step_registers(int32_t score_mode, int32_t G, int32_t H, int32_t lean, int32_t early, int32_t *planned)
+{
+    if (score_mode < 0 || score_mode > 1 || G < 1 || G > BR_MAX_G || H < 0 || H > BR_MAX_H || (score_mode == 0 && H != 0) || !planned)
+        return BR_EINVAL;
+    const bool fp = score_mode == 1;
+    const int groups = br::step_groups(H);
+    br::StepLaunch l;
+    l.warps = 1; l.lean = lean != 0 && br::step_has_lean(fp, groups); l.early = early != 0 && groups != 0;
+    cudaFuncAttributes f;
+    BR_CUDA(cudaFuncGetAttributes(&f, (const void *)pick_kernel(fp, H, G, l)));
+    *planned = br::step_registers(fp, G <= 32 ? 1 : 2, groups, l.lean, l.early);
+    return f.numRegs;
+}
+
 int br_destroy(br_ctx *ctx)
 {
     if (!ctx) return BR_OK;

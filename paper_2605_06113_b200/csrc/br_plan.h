@@ -64,10 +64,12 @@ constexpr int step_groups(int H) { return H < 8 ? 2 : (H < 12 ? 3 : (H < 20 ? 5 
 // router's chain 5 to 15 % longer and let more instances be resident; horizons below 20 have none (at 80 registers
 // 40 % more instances, each slower by as much: 2,072 of G = 16, H = 8, eight steps: 382 us, 396).
 constexpr int step_register_cap(bool fp, int groups, bool lean) { return !fp ? (lean ? 72 : 96) : groups ? 96 : (lean ? 96 : 128); }
-// ... and the registers that it is compiled to (Eq. 1 by the workers per router lane: 78 and 84; long horizons 115)
-constexpr int step_registers(bool fp, int workers_per_lane, int groups, bool lean)
+// ... and the registers that it is compiled to, in the multiples of eight that an SM gives out (br_debug_step_registers
+// compares them with the kernels).  Eq. 1: 75 and 79 for one worker per router lane, 80 for two, 87 where a single warp
+// settles endings early; long horizons 111 and 114.
+constexpr int step_registers(bool fp, int workers_per_lane, int groups, bool lean, bool early = false)
 {
-    return !fp ? (lean ? 72 : (workers_per_lane == 1 ? 80 : 88)) : groups ? 96 : (lean ? 96 : 120);
+    return !fp ? (lean ? 72 : (workers_per_lane == 2 && early ? 88 : 80)) : groups ? 96 : (lean ? 96 : (workers_per_lane == 1 ? 112 : 120));
 }
 constexpr bool step_has_lean(bool fp, int groups) { return !fp || !groups; }
 
@@ -150,7 +152,7 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
         for (int lean = 0; lean < 2; ++lean) {
             // (the lean instantiation spills in the classifier's loop, which a single warp cannot hide)
             if (lean && (!step_has_lean(s.fp, groups) || (classifier && w < 2))) continue;
-            int r = step_warps_per_sm(step_registers(s.fp, s.G <= 32 ? 1 : 2, groups, lean != 0)) / w;
+            int r = step_warps_per_sm(step_registers(s.fp, s.G <= 32 ? 1 : 2, groups, lean != 0, w == 1 && step_early(s))) / w;
             const int fit = kSharedPerSM / (s.shared + 1024);
             if (r > fit) r = fit;
             if (r > 32) r = 32;

@@ -503,6 +503,10 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
 // take the lean instantiation (step_registers, step_launch).
 // EARLY: a single warp under the constant hazard (32 threads, term_mode 1), with the requests that end settled ahead of
 // the router.
+// (It has no output lengths to carry: with the loads of a queue that might carry them, Eq. 1 on up to 32 workers took 88
+// registers instead of 75, 20 warps to an SM instead of 24.  G = 16, B = 96, W = 256, 3,256 instances: 21.5 us, 17.2 this
+// way.  18 to 20 an SM, which either holds, gain 2 % in the kernel and lose 3 to 4 back to back, 2,960: 16.3, 16.9: the
+// next launch's first blocks find room on some SMs only.)
 template <bool FP, int GW, int NC, bool LEAN, bool EARLY>
 __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(const __grid_constant__ StepArgs a)
 {
@@ -514,7 +518,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
     constexpr int HT = 4 * NC;                        // offsets of the unrolled loops
     const unsigned posmask = (1u << WL) - 1u;
     const int inst = a.first_instance + blockIdx.x;
-    const bool life = a.term_mode == 3;               // requests carry their output lengths
+    const bool life = !EARLY && a.term_mode == 3;     // requests carry their output lengths
     const bool classifier = FP && H > 0 && a.pred_mode == 0;
     const unsigned t_entry = (unsigned)clock64();
 
