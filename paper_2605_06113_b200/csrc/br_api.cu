@@ -794,7 +794,11 @@ int br_bypass_dispatch(br_ctx *ctx, const br_instance_batch *batch, const int32_
     a.s = s; a.vload = virtual_load; a.inflight = inflight; a.cap = inflight_cap; a.g_out = worker_out;
     void (*kern)(const br::BypassArgs) = a.f.fp ? (ctx->G <= 32 ? br::br_bypass_kernel<true, 1> : br::br_bypass_kernel<true, 2>)
                                                 : (ctx->G <= 32 ? br::br_bypass_kernel<false, 1> : br::br_bypass_kernel<false, 2>);
-    cudaError_t e = launch_overlapped(kern, dim3((unsigned)batch->n_instances), 32, 0, (cudaStream_t)batch->stream, a, true);
+    // (a plain launch while the caller captures the stream, as in br_graph_capture)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    BR_CUDA(cudaStreamIsCapturing((cudaStream_t)batch->stream, &capturing));
+    cudaError_t e = launch_overlapped(kern, dim3((unsigned)batch->n_instances), 32, 0, (cudaStream_t)batch->stream, a,
+                                      capturing == cudaStreamCaptureStatusNone);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "br_bypass_dispatch launch");
     return BR_OK;

@@ -65,11 +65,13 @@ __global__ void __launch_bounds__(32) br_bypass_kernel(const BypassArgs a)
     for (int w = 0; w < GW; ++w) m[w] = M - L[w];
     const int32_t *s = a.s + inst * a.n_req;
     int32_t *out = a.g_out + inst * a.n_req;
-    int next = lane < a.n_req ? __ldg(s + lane) : 0;
+    // (plain loads: with an overlapping launch the kernel ahead may write the lengths while this one is resident, which
+    // read-only loads do not allow)
+    int next = lane < a.n_req ? s[lane] : 0;
 #pragma unroll 1
     for (int i0 = 0; i0 < a.n_req; i0 += 32) {
         const int mine = next, cnt = min(32, a.n_req - i0);
-        if (i0 + 32 + lane < a.n_req) next = __ldg(s + i0 + 32 + lane);
+        if (i0 + 32 + lane < a.n_req) next = s[i0 + 32 + lane];
         int answer = -1;
         bool packed = !FP && (unsigned)mine < (1u << 25);
 #pragma unroll
