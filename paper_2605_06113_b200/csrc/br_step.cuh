@@ -222,18 +222,19 @@ __device__ __forceinline__ long long ld_now8(const void *p)
 // itself the L2 fetches 128 bytes around a missing sector, of which a refresh uses 32 on average,
 // so the loads ask for the smallest fetch the instruction set offers (64 bytes).  Nor do they allocate in L1: where
 // shared memory leaves it little, the lines that wait for rows limit how many are in flight (1,024 instances of two
-// warps, a quarter of 4,096 rows each: 22.7 us, 15.9 this way; 28 KB of L1).
+// warps, a quarter of 4,096 rows each: 22.7 us, 15.9 this way; 28 KB of L1).  They are coherent loads: the
+// launch overlaps the kernel ahead, which may be the one that writes the rows.
 __device__ __forceinline__ float4 ld_row4(const float *p)
 {
     float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.L2::64B.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
 // a whole row of eight probabilities (32-byte aligned) as one 256-bit load
 __device__ __forceinline__ void ld_row8(const float *p, float *o)
 {
     unsigned r[8];
-    asm volatile("ld.global.nc.L1::no_allocate.L2::64B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+    asm volatile("ld.global.L1::no_allocate.L2::64B.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "l"(p));
 #pragma unroll
     for (int i = 0; i < 8; ++i) o[i] = __uint_as_float(r[i]);
@@ -269,7 +270,7 @@ __device__ __forceinline__ void load_rows(const float *const (&row)[R], int H, i
             if (h < H)
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
-                    const float2 x = __ldg(reinterpret_cast<const float2 *>(row[r] + h));
+                    const float2 x = *reinterpret_cast<const float2 *>(row[r] + h);
                     v[r][h] = x.x; v[r][h + 1] = x.y;
                 }
     } else {
@@ -277,7 +278,7 @@ __device__ __forceinline__ void load_rows(const float *const (&row)[R], int H, i
         for (int h = 0; h < HT; ++h)
             if (h < H)
 #pragma unroll
-                for (int r = 0; r < R; ++r) v[r][h] = __ldg(row[r] + h);
+                for (int r = 0; r < R; ++r) v[r][h] = row[r][h];
     }
 }
 
@@ -301,7 +302,7 @@ __device__ __forceinline__ float row_sum(const float *q, int H, int width)
         }
     } else {
 #pragma unroll 4
-        for (int h = 0; h < H; ++h) s += fabsf(__ldg(q + h));
+        for (int h = 0; h < H; ++h) s += fabsf(q[h]);
     }
     return s;
 }
@@ -827,7 +828,7 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
 #pragma unroll
                                 for (int r = 0; r < R; ++r) {
                                     c[r] = __dadd_rn(c[r], surv[r]);
-                                    surv[r] = __dmul_rn(surv[r], __dsub_rn(1.0, (double)__ldg(row[r] + h)));
+                                    surv[r] = __dmul_rn(surv[r], __dsub_rn(1.0, (double)row[r][h]));
                                 }
                     }
                     if (any) {
