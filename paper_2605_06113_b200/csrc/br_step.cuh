@@ -669,20 +669,34 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
         // ============ PREDICT (H > 0): c_hat maintenance + horizon projection ============
         // Every running request adds (cur, 1) to the bucket (worker, floor(c_hat)); the buckets become
         // L_g(k+h) = sum_{j >= h} T_j + h * sum_{j >= h} C_j by suffix sums.  A thread takes `quads` slot quads, the next one
-        // requested before this one is worked on.  The 32 lanes of a warp read eight pieces of 64 bytes, 4 * quads quads
-        // apart: consecutive quads in consecutive lanes are one worker's, whose few buckets serialise the atomics, and
-        // eight slots of one worker per thread touch 32 lines with every load.
-        const int q_first = ((warp << 5) + (lane & ~3)) * a.quads + (lane & 3);
+        // requested before this one is worked on.  The 32 lanes of a warp read eight pieces of 64 bytes a worker apart, or a
+        // little more (the pieces of a run of eight workers one after another): consecutive quads in consecutive lanes are
+        // one worker's, whose few buckets serialise the atomics; rows of workers several apart share banks; and
+        // eight slots of one worker per thread touch 32 lines with every load.  (Look-ahead, 1,184 instances of G = 64, B = 64,
+        // three steps, H = 2 / 25: 77 / 106 us with consecutive quads, 77 / 112 with pieces 4 * quads quads, here four
+        // workers, apart, 63 / 99 this way.)
         int n_due = 0;                                    // requests on this warp's part of the due list
         const auto due_w = due_list + (size_t)(classifier ? 128 * warp * a.quads : 0);
         if (FP && H > 0) {
-            const int A4 = A >> 2, q_end = q_first + 4 * a.quads;
+            const int A4 = A >> 2, span = (B + 15) >> 4;
+            int left = a.quads, run = min(span, left), in_run = run;
+            int q = (warp << 5) * left + (lane & ~3) * run + (lane & 3);
+            auto next = [&]() {
+                --left;
+                q += 4;
+                if (--in_run == 0) {
+                    // the other lanes' pieces of the run, then this lane's first of the next
+                    q += 28 * run - (lane & ~3) * run;
+                    in_run = run = min(span, left);
+                    q += (lane & ~3) * run;
+                }
+            };
             const bool look = a.pred_mode == 1;
             int4 b4, x4 = make_int4(0, 0, 0, 0);                              // act_base; act_end or chat0
             unsigned kr = 0u;                                                 // refresh stamps
-            auto fetch = [&](int q) {
+            auto fetch = [&]() {
                 b4 = make_int4(kEmpty, kEmpty, kEmpty, kEmpty);
-                if (q < A4 && q < q_end) {
+                if (q < A4 && left > 0) {
                     b4 = *vec_at<const int4>(g_base, 4 * q);
                     if (look) {
                         x4 = *vec_at<const int4>(g_end, 4 * q);
@@ -692,19 +706,20 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     }
                 }
             };
-            fetch(q_first);
+            fetch();
             // (Adds and stores that are predicated in inline assembly instead of branched around: the compiler must not move
             // accesses across them, and its own atomics are faster, a count of one above all.  592 of G = 48, B = 96, H = 6,
             // 97 % of the slots in one bucket: 11,600 cycles a step that way, 10,400 this; 425 shapes 1.2 % on average)
             const unsigned k_4 = (unsigned)(k & 255) * 0x01010101u, lt = (1u << lane) - 1u;
             const float Hf = (float)H, dTf = (float)a.delta_T, two23 = 8388608.0f;
 #pragma unroll 1
-            for (int it4 = 0; it4 < 4 * a.quads; it4 += 4) {
-                const int q = q_first + it4;
-                const int g = (int)__umulhi((unsigned)q, a.b4_magic);
+            while (left > 0) {
+                const int q_now = q;
+                const int g = (int)__umulhi((unsigned)q_now, a.b4_magic);
                 const int bs[4] = {b4.x, b4.y, b4.z, b4.w}, xs[4] = {x4.x, x4.y, x4.z, x4.w};
                 const unsigned k4 = kr;
-                fetch(q + 4);
+                next();
+                fetch();
                 if (look) {
                     // perfect lookahead: c_hat = min(r_i(k), H) with r_i(k) = act_end - k + 1 steps still to run.
                     // A request whose last step this is (act_end == k) is settled right here.
@@ -720,11 +735,11 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                         fb |= live && xs[j] == k ? 1u << j : 0u;
                     }
                     if (fb) {
-                        const int slot = 4 * q - g * B;
+                        const int slot = 4 * q_now - g * B;
                         atomicOr(&endm32[2 * g * OW + (slot >> 5)], fb << (slot & 31));
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            if ((fb >> j) & 1u) { atomicAdd(&sub_load[g], (unsigned)(bs[j] + k)); g_base[4 * q + j] = kEmpty; }
+                            if ((fb >> j) & 1u) { atomicAdd(&sub_load[g], (unsigned)(bs[j] + k)); g_base[4 * q_now + j] = kEmpty; }
                     }
                 } else {
                     // requests that are not due only age; the ones due for a refresh take c_hat = H (gate closed:
@@ -760,11 +775,11 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                     n_due += __popc(n1) + 2 * __popc(n2) + 4 * __popc(n4);
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (due[j]) due_w[first + to[j]] = (unsigned short)(4 * q + j);
+                        if (due[j]) due_w[first + to[j]] = (unsigned short)(4 * q_now + j);
                     if (dues) {
                         const int anchor = __float_as_int(Hf);
-                        *vec_at<int4>(g_chat0, 4 * q) = make_int4(due[0] ? anchor : xs[0], due[1] ? anchor : xs[1], due[2] ? anchor : xs[2], due[3] ? anchor : xs[3]);
-                        *vec_at<unsigned>(g_kref, 4 * q) = (k4 & ~dues) | (k_4 & dues);
+                        *vec_at<int4>(g_chat0, 4 * q_now) = make_int4(due[0] ? anchor : xs[0], due[1] ? anchor : xs[1], due[2] ? anchor : xs[2], due[3] ? anchor : xs[3]);
+                        *vec_at<unsigned>(g_kref, 4 * q_now) = (k4 & ~dues) | (k_4 & dues);
                     }
                 }
             }
