@@ -76,10 +76,10 @@ step_kernel_t pick_kernel_gw(int G)
     return G <= 32 ? br::br_step_kernel<FP, 1, NC, LEAN, EARLY> : br::br_step_kernel<FP, 2, NC, LEAN, EARLY>;
 }
 
-template <int NC>
+template <int NC, bool LEAN>
 step_kernel_t pick_kernel_early(int G, bool early)
 {
-    return early ? pick_kernel_gw<true, NC, false, true>(G) : pick_kernel_gw<true, NC, false, false>(G);
+    return early ? pick_kernel_gw<true, NC, LEAN, true>(G) : pick_kernel_gw<true, NC, LEAN, false>(G);
 }
 
 // Eq. 1 or Eq. 2; one or two workers per router lane; horizon offsets unrolled in groups of four or not at all
@@ -88,9 +88,9 @@ step_kernel_t pick_kernel(bool fp, int H, int G, const br::StepLaunch &l)
     if (!fp && l.early) return l.lean ? pick_kernel_gw<false, 2, true, true>(G) : pick_kernel_gw<false, 2, false, true>(G);
     if (!fp) return l.lean ? pick_kernel_gw<false, 2, true, false>(G) : pick_kernel_gw<false, 2, false, false>(G);
     switch (br::step_groups(H)) {
-    case 2: return pick_kernel_early<2>(G, l.early);
-    case 3: return pick_kernel_early<3>(G, l.early);
-    case 5: return pick_kernel_early<5>(G, l.early);
+    case 2: return pick_kernel_early<2, false>(G, l.early);
+    case 3: return pick_kernel_early<3, false>(G, l.early);
+    case 5: return l.lean ? pick_kernel_early<5, true>(G, l.early) : pick_kernel_early<5, false>(G, l.early);
     default: return l.lean ? pick_kernel_gw<true, 0, true, false>(G) : pick_kernel_gw<true, 0, false, false>(G);
     }
 }

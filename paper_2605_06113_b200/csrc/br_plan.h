@@ -61,17 +61,23 @@ inline bool host_in_place(HostUse use, int H, int term_mode, long long n_instanc
 constexpr int step_groups(int H) { return H < 8 ? 2 : (H < 12 ? 3 : (H < 20 ? 5 : 0)); }
 
 // Registers a thread of an instantiation may use, by Eq. 1 or 2 (fp) and step_groups(H).  The lean ones make the
-// router's chain 5 to 15 % longer and let more instances be resident; horizons below 20 have none (at 80 registers
-// 40 % more instances, each slower by as much: 2,072 of G = 16, H = 8, eight steps: 382 us, 396).
-constexpr int step_register_cap(bool fp, int groups, bool lean) { return !fp ? (lean ? 72 : 96) : groups ? 96 : (lean ? 96 : 128); }
+// router's chain 5 to 15 % longer and let more instances be resident; horizons below 12 have none (at 80 registers
+// 40 % more instances, each slower by as much: 2,072 of G = 16, H = 8, eight steps: 382 us, 396).  H = 12 to 19 at 96
+// registers keeps values of the admission loop in memory: 1,184 of G = 8, H = 16, look-ahead, three steps 51.4 us, 46.9 at
+// 112; of G = 48, B = 24, H = 12, classifier, 100.6, 80.9.  An SM holds 16 such warps, 20 of the lean ones: 2,960 of G = 8, H = 12
+// 39.3 us, 29.6.
+constexpr int step_register_cap(bool fp, int groups, bool lean)
+{
+    return !fp ? (lean ? 72 : 96) : groups == 5 ? (lean ? 96 : 112) : groups ? 96 : (lean ? 96 : 128);
+}
 // ... and the registers that it is compiled to, in the multiples of eight that an SM gives out (br_debug_step_registers
 // compares them with the kernels).  Eq. 1: 75 and 79 for one worker per router lane, 80 for two, 87 where a single warp
 // settles endings early; long horizons 111 and 114.
 constexpr int step_registers(bool fp, int workers_per_lane, int groups, bool lean, bool early = false)
 {
-    return !fp ? (lean ? 72 : (workers_per_lane == 2 && early ? 88 : 80)) : groups ? 96 : (lean ? 96 : (workers_per_lane == 1 ? 112 : 120));
+    return !fp ? (lean ? 72 : (workers_per_lane == 2 && early ? 88 : 80)) : groups == 5 ? (lean ? 96 : 112) : groups ? 96 : (lean ? 96 : (workers_per_lane == 1 ? 112 : 120));
 }
-constexpr bool step_has_lean(bool fp, int groups) { return !fp || !groups; }
+constexpr bool step_has_lean(bool fp, int groups) { return !fp || !groups || groups == 5; }
 
 // Warps of a kernel that an SM's registers hold: four partitions of 16,384, and 32 threads of a multiple of eight
 // registers per warp (96 registers: 20 warps, not 21).
@@ -150,8 +156,8 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
             base += 0.015 * u * (s.G < 32 ? s.G : 32) / 32.0;
         }
         for (int lean = 0; lean < 2; ++lean) {
-            // (the lean instantiation spills in the classifier's loop, which a single warp cannot hide)
-            if (lean && (!step_has_lean(s.fp, groups) || (classifier && w < 2))) continue;
+            // (the lean instantiation of H >= 20 spills in the classifier's loop, which a single warp cannot hide)
+            if (lean && (!step_has_lean(s.fp, groups) || (classifier && !groups && w < 2))) continue;
             int r = step_warps_per_sm(step_registers(s.fp, s.G <= 32 ? 1 : 2, groups, lean != 0, w == 1 && step_early(s))) / w;
             const int fit = kSharedPerSM / (s.shared + 1024);
             if (r > fit) r = fit;
