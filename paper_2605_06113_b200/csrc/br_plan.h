@@ -117,18 +117,26 @@ inline int step_seg_log2(int G, int H, int threads)
 // More warps shorten an instance's parallel phases and leave fewer instances resident, so a batch of a few instances
 // per SM takes as many warps as there is work for, a large one those that need the least time for all its
 // waves.  With r resident instances of w warps a step takes, in units of the router's chain,
-//     t(w, r) = 1 + 0.015 u(w) + p (c + e r) / w,
-// u the offsets that a lane sums one after the other for L_g(k+h), each of which raises one word with the other
-// workers (41 workers and 60 offsets: 60 each with two warps, 30 with three; 1,738 instances, H = 59, eleven steps: 510
-// and 400 us, 367 in one wave), p the thousands of slots that the projection streams (a little more the longer the
-// classifier's rows, a fifth more where they are not whole vectors, twice as many when terminations read every
-// row; Eq. 1 has draws and queue alone) and e what another resident instance costs.  The last, incomplete wave starts
-// while instances of the one before still run and counts in part.  The constants are a fit to 3,000 measured times
-// (50 shapes, 1 to 28 instances per SM, one to eight warps, both instantiations): the choice is within 1 % of the
-// fastest on average, at worst 17 %.  us per call at 1, 2, 3, 4, 5 warps: 592 of G = 32, H = 1: 44 / 33 / 27 / 25 / 23;
-// 1,480: 57 / 37 / 48 / 47 / 56; 2,072: 65 / 67 / 76 / 74 / 80; 2,960: 107 / 78 / 108 / 109 / 115.  Four warps
-// at least for instances that stream 4,096 slots with long classifier rows: more of them resident take each
-// other's cache lines (1,480 of G = 64, H = 16: 227 / 189 / 102 / 89 / 106).
+//     t(w, r) = 1 + 0.05 u(w) + p (c + e r) / w,
+// u (H >= 20 alone; below, the router sums in registers) the offsets that a lane sums one after the other for L_g(k+h),
+// each of which raises one word with the other workers (41 workers and 60 offsets: 60 each with two warps, 30 with three;
+// 2,051 instances, H = 59, three steps: 162 and 131 us), p the thousands of slots that the projection streams (look-ahead,
+// which reads no rows, half of it; more the longer the classifier's rows, above all where terminations read every
+// row, two fifths more under the constant hazard where they are not whole vectors; Eq. 1 has draws and queue alone) and e what another
+// resident instance costs.  The last, incomplete wave starts while instances of the one before still run and counts in part.
+// The constants of Eq. 2 are a fit to 40,000 measured times (3,976 batches of 160 shapes, 20 to 4,500 instances, one to eight
+// warps, both instantiations; full fleets, and fleets after some hundred steps), by terminations.  The choice is on average
+// within 1.2 % of the fastest with look-ahead (at worst 13), 2.8 % under the constant hazard, 3.4 % where terminations read
+// every row (5 in 100 more than 20 % off).  Neighbouring counts differ by up to a factor of two where rows fall out of the
+// cache, which the estimate does not know: 1,455 of G = 29, B = 128, H = 34, three steps: 534 us at two warps, 348 at three.
+// us per call at 1, 2, 3, 4, 5 warps: 1,036 of G = 64, W = 1,024, H = 8: 62 / 63 / 65 / 56 / 57; 1,332: 104 / 88 / 71 / 64 / 76;
+// 2,960 of G = 15, W = 40, H = 19: 49 (41 lean) / 61 / 70 / 77 / 91; 1,036 of G = 24, B = 40, H = 12, terminations from rows: 79 /
+// 55 / 67 / 67 / 84.  Four warps at least for instances that stream 4,096 slots with rows of 8 to 19, or half as many when
+// terminations read every row: more of them resident take each other's cache lines (2,960 of G = 32, H = 11, terminations
+// from rows: 428 / 255 / 203 / 193).
+// Eq. 1 keeps its own older constants: within 2 % of the fastest on average over its usual shapes, 6 % over 364 batches of
+// large fleets and queues, where routers of two- and four-warp blocks meet on the same partitions (1,006 of G = 54, B = 96,
+// W = 888, four steps, 78 / 90 / 66 / 88 us at 1, 2, 3, 4 warps).
 inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
 {
     const int groups = step_groups(s.H), A = s.G * s.B, n = (n_instances + sms - 1) / sms;
@@ -138,22 +146,25 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
     if (s.G * (s.H + 1) / 8 > most) most = s.G * (s.H + 1) / 8;
     most = (most + 31) / 32;
     most = most < 4 ? 4 : (most > 8 ? 8 : most);
-    const bool long_rows = classifier && s.H >= 8 && groups && A * (s.term_mode == 2 ? 2 : 1) >= 4096;
+    const bool every_row = classifier && s.term_mode == 2, ragged = (s.H & 3) && s.H > 2;
+    const bool long_rows = classifier && s.H >= 8 && groups && A * (every_row ? 2 : 1) >= 4096;
     const int least = long_rows ? 4 : 1;
     double p = 1e-3 * A;
     if (!s.H) p = 0.035 + 0.006 * s.G + 7e-5 * s.W;
-    else if (classifier) p = p * (1.0 + 0.02 * s.H) * ((s.H & 3) && s.H > 2 ? 1.2 : 1.0) * (s.term_mode == 2 ? 2 : 1) + 7e-5 * s.W;
-    else p += 2e-4 * s.W;
+    else if (every_row) p = p * (1.0 + 0.054 * s.H) + 7e-5 * s.W;
+    else if (classifier) p = p * (1.0 + 0.025 * s.H) * (ragged ? 1.4 : 1.0) + 7e-5 * s.W;
+    else p = 0.5 * p + 2e-4 * s.W;
     struct Fit { double c, e, last, last_full; };
-    const Fit k = !s.H ? Fit{0.65, 0.03, 0.3, 0.4} : classifier ? Fit{0.75, 0.036, 0.65, 0.3} : Fit{0.7, 0.013, 0.5, 0.5};
+    const Fit k = !s.H ? Fit{0.65, 0.03, 0.3, 0.4} : every_row ? Fit{0.34, 0.09, 0.47, 0.71}
+                              : classifier ? Fit{0.65, 0.04, 0.45, 0.65} : Fit{0.39, 0.002, 0.27, 0.8};
     StepLaunch best = {1, false, false};
     double cost = 1e300;
     for (int w = least; w <= most; ++w) {
         double base = 1.0;
-        if (s.H > 0) {
+        if (s.H > 0 && !groups) {
             const int q = step_seg_log2(s.G, s.H, 32 * w);
             const int u = (((s.G << q) + 32 * w - 1) / (32 * w)) * ((s.H + (1 << q)) >> q);
-            base += 0.015 * u * (s.G < 32 ? s.G : 32) / 32.0;
+            base += 0.05 * u * (s.G < 32 ? s.G : 32) / 32.0;
         }
         for (int lean = 0; lean < 2; ++lean) {
             // (the lean instantiation of H >= 20 spills in the classifier's loop, which a single warp cannot hide)
@@ -166,7 +177,7 @@ inline StepLaunch step_launch(const StepShape &s, int n_instances, int sms)
             const int full = n / r, part = n % r;
             double t = full * (base + p * (k.c + k.e * r) / w);
             if (part) t += (full ? k.last + k.last_full * part / r : 1.0) * (base + p * (k.c + k.e * part) / w);
-            if (lean) t *= 1.1;
+            if (lean) t *= s.H ? 1.16 : 1.1;
             if (t <= cost) { cost = t; best.warps = w; best.lean = lean != 0; }
         }
     }
