@@ -38,6 +38,8 @@ struct StepLayout {
     int32_t q_key, q_id, q_o, Lh, Ch, dn, iw, Ms, occ, occ0, fin, endm, L0, cap, sub, scal, bw, due, total;
 };
 
+// (`quads` and `b4_magic` fill gaps between pointers: with every array behind them eight bytes further on, br_small_kernel
+// took 1 % longer over 16 steps, 4,096 instances of G = 32: 172.8 us, 171.7 this way.)
 struct StepArgs {
     int32_t G, H, B, W, R_max, S_greedy, occ_words;
     int32_t wl;                 // log2 of the queue-position field of a packed key
@@ -45,17 +47,17 @@ struct StepArgs {
     int32_t HS;                 // row stride of L_g(k+h) in shared memory (>= H + 1)
     int32_t lpw_log2;           // log2 of the lanes that share a worker's row (fleets of up to 16 workers, long horizons)
     int32_t seg_log2;           // lanes per worker that turn its prediction buckets into L_g(k+h)
-    int32_t quads;              // slot quads that a thread takes in PREDICT (NT * quads covers A / 4)
-    uint32_t b4_magic;          // ceil(2^32 / (B / 4)): the worker of quad q is the upper half of q * b4_magic
     int32_t delta_T;
     float gate, c_floor;
     int32_t term_mode;
     int32_t pred_mode;          // 1: c_hat = min(remaining steps, H) from act_end (term_mode 3)
     const int32_t *out_tab;     // output lengths of arrivals (term_mode 3)
     int32_t out_shift;
+    int32_t quads;              // slot quads that a thread takes in PREDICT (NT * quads covers A / 4)
     const uint32_t *term_cdf;   // [B] gap thresholds of the constant hazard
     const uint32_t *arr_cdf;
     int32_t arr_len, arr_period, arr_inst_stride;
+    uint32_t b4_magic;          // ceil(2^32 / (B / 4)): the worker of quad q is the upper half of q * b4_magic
     const int32_t *len_tab;
     int32_t len_shift;
     int32_t burst_every, burst_size;
