@@ -144,7 +144,9 @@ typedef struct {
                                      first admission (0 beyond the queue length); NULL in timed runs */
     uint32_t *phase_cycles; /* [N][8] optional: SM clock cycles this step spent in ARRIVE, PREDICT,
                                      Stage 1, Stage 2, RECORD + queue compaction, ADVANCE (the split the
-                                     paper reports for its dispatcher: preparation / Stage 1 / Stage 2),
+                                     paper reports for its dispatcher: preparation / Stage 1 / Stage 2;
+                                     for H < 20 the sums that turn the projection into L_g(k+h) are the
+                                     router's and count as Stage 1, for longer horizons as PREDICT),
                                      then the launch's state-load prologue and its total from kernel
                                      entry to the state write-back; may be NULL */
 } br_load_out;

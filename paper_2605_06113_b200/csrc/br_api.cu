@@ -134,9 +134,9 @@ int check_step_args(const br_ctx *ctx, const br_instance_batch *b, const br_work
 }
 
 // Launch with programmatic stream serialisation: the blocks of this launch may become resident
-// while the previous kernel of the stream is still draining.  The kernels open with
-// griddepcontrol.wait, which returns only when every earlier kernel of the stream has completed
-// and its writes are visible, so only launch latency and block scheduling overlap.
+// while the previous kernel of the stream is still draining.  Ahead of their first access to global memory the kernels
+// wait (griddepcontrol.wait) until every earlier kernel of the stream has completed and its writes are visible, so only
+// launch latency, block scheduling and what is set up from the arguments overlap.
 template <typename Args>
 cudaError_t launch_overlapped(void (*kern)(const Args), dim3 blocks, int threads, size_t smem, cudaStream_t stream,
                               const Args &a, bool overlap)

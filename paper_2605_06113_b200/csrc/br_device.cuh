@@ -63,8 +63,8 @@ __device__ __forceinline__ V *vec_at(T *p, long long i)
 template <typename T> __device__ __forceinline__ T *raw_of(T *p) { return p; }
 #endif
 
-// First statements of a step kernel: let the next kernel of the stream start becoming resident,
-// then wait until every earlier kernel of the stream has completed and flushed its writes
+// Ahead of a step or dispatch kernel's first access to global memory: let the next kernel of the stream start becoming
+// resident, then wait until every earlier kernel of the stream has completed and flushed its writes
 // (both are no-ops for a launch without programmatic stream serialisation).
 __device__ __forceinline__ void stream_order_gate()
 {

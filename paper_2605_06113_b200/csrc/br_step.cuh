@@ -19,7 +19,7 @@
 // W = 1,024, H = 8, 1,024 instances / G = 21, W = 300, H = 6, 777 instances, 3 steps / G = 8, W = 512, H = 80,
 // 1,024 instances, 8 steps: 110 / 672 / 503 with a copy of every part per stage and all loops over h
 // unrolled, 77 / 313 / 166 with one loop, loads and envelope in shared memory and the window merged from
-// the lanes' lists at every pop, 68 / 183 / 116 now.
+// the lanes' lists at every pop, 59 / 175 / 105 now.
 //
 // Loads are advanced incrementally: L_g(k+1) = L_g(k) - sum of the loads of the requests
 // that end at k + number of survivors, so ADVANCE touches only the occupancy bit masks,
@@ -479,8 +479,8 @@ __device__ __noinline__ void score_column(const Scorer<FP> sc, double *F, span_t
 // FP: Eq. 2 scores (else Eq. 1).  GW: workers per router lane.  NC: step_groups(H).  LEAN: fewer registers.
 // Registers: the router's chain is the longest path, and it is shorter with more of them than with more
 // warps resident (G = 64, H = 8, one instance: 22.0 us at 72 registers, 19.4 at 96; 777 instances of G = 21,
-// H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128).  Batches that just miss being resident in one wave
-// take the lean instantiation (step_registers, step_launch).
+// H = 6: 194 and 181; G = 8, H = 80: 127 at 96, 119 at 128; H = 12 to 19: step_register_cap).  Batches that just miss being
+// resident in one wave take the lean instantiation where there is one (step_registers, step_launch).
 // EARLY: a single warp under the constant hazard (32 threads, term_mode 1), with the requests that end settled ahead of
 // the router.
 // (It has no output lengths to carry: with the loads of a queue that might carry them, Eq. 1 on up to 32 workers took 88
@@ -793,7 +793,10 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                 const float *rows = reinterpret_cast<const float *>(raw_of(probs));
                 const int width = (H & 7) == 0 && (reinterpret_cast<size_t>(rows) & 31) == 0 ? 8 : (H & 3) == 0 ? 4 : (H & 1) == 0 ? 2 : 1;
                 const float closed = fminf(a.gate, 1.0f);
-                constexpr int R = NC == 2 ? 4 : NC == 3 ? 3 : 2;                  // rows in flight per thread
+                // rows in flight per thread: as many as registers hold beside their probabilities (H = 8 to 11, two instead of
+                // three: one cluster of G = 32 with terminations from rows 24.9 us, 26.7; batches level.  H = 12 to 19, one
+                // instead of two: 2,072 of G = 32, H = 16 131 us, 137)
+                constexpr int R = NC == 2 ? 4 : NC == 3 ? 3 : 2;
 #pragma unroll 1
                 for (int e1 = 0; e1 < n_due; e1 += 32 * R) {
                     const int e0 = e1 + lane;
@@ -1019,8 +1022,8 @@ __global__ void __maxnreg__(step_register_cap(FP, NC, LEAN)) br_step_kernel(cons
                 L0[w] = g < G ? (NC == 0 ? Lh[g * HS] : L0_s[g]) : 0;
                 mm[w] = 0;
             }
-            // rows of all workers: Ms - row (FIRST: loads become margins) or Ms + row (the envelope grew by Ms), and
-            // their minima
+            // rows of all workers: Ms - row (FIRST, long horizons: loads become margins) or Ms + row (the envelope grew by
+            // Ms), and their minima
             auto rows = [&](const bool first) {
                 if (NC == 0 && G <= 16) {
                     // long rows, few workers: 32 / G lanes share a row

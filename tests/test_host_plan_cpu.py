@@ -28,6 +28,7 @@ extern "C" int launch(int fp, int G, int H, int B, int W, int term_mode, int pre
     *resident = br::step_warps_per_sm(br::step_registers(s.fp, G <= 32 ? 1 : 2, br::step_groups(H), l.lean)) / l.warps;
     return l.lean ? -l.warps : l.warps;
 }
+extern "C" uint32_t magic(int B) { return br::quad_magic(B); }
 extern "C" int in_place(int use, int H, int term_mode, long long n, long long slots)
 {
     return br::host_in_place((br::HostUse)use, H, term_mode, n, slots);
@@ -128,3 +129,11 @@ def test_every_shape_gets_a_launch(plan):
                         for shared in (4000, 60000, 232448):
                             w, _, res = _launch(plan, G, H, n, B, W, term, pred, shared)
                             assert 1 <= w <= 8
+
+
+def test_the_worker_of_a_slot_quad(plan):
+    plan.magic.restype = C.c_uint32
+    for B in range(8, 257, 8):
+        m = plan.magic(B)
+        for q in range(64 * B // 4):                       # every quad of the largest fleet
+            assert (q * m) >> 32 == q // (B // 4), (B, q)
