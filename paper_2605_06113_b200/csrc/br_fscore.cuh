@@ -60,8 +60,9 @@ inline int fscore_smem(int G, int row) { return 4 * G * row + 16 * row + kFsWarp
 // worker so far stays in registers, and eight scores of each request at a time go through shared memory so that
 // they are written in runs.  A term of Eq. 2 is RN(d_h * over), over = max(s - m_h, 0) an integer:
 // X = 2^52 + over needs no conversion, and fma(X, d_h, -2^52 d_h) rounds d_h * over once, so a term is two
-// fp64 instructions and one integer one.  Eq. 2 is bound by instruction issue (and, next, by the
-// fp64 pipe, which takes two cycles for an instruction), Eq. 1 by the writes.  200 x 1,024 x 64 scores at
+// fp64 instructions and one integer one.  Eq. 2 is bound by instruction latency with five
+// warps a scheduler (issue 0.59 of its peak, the fp64 pipe 0.13 busy; a warp waits for shared memory and for the instruction
+// before in equal parts) and by uneven blocks (an SM is busy for 50,400 cycles on average, 57,400 at most), Eq. 1 by the writes.  200 x 1,024 x 64 scores at
 // H = 8 with best workers: 224 us with five fp64 operations a term, blocks of 1,024 requests and the best
 // worker found by scoring everything again; 57 with the terms above for every pair, 31 with the workers whose
 // smallest margin no request of the warp exceeds left at alpha D s.
