@@ -124,11 +124,11 @@ inline int step_seg_log2(int G, int H, int threads)
 // which reads no rows, half of it; more the longer the classifier's rows, above all where terminations read every
 // row, two fifths more under the constant hazard where they are not whole vectors; Eq. 1 has draws and queue alone) and e what another
 // resident instance costs.  The last, incomplete wave starts while instances of the one before still run and counts in part.
-// The constants of Eq. 2 are a fit to 40,000 measured times (3,976 batches of 160 shapes, 20 to 4,500 instances, one to eight
+// The constants of Eq. 2 are a fit to 37,000 measured times (3,364 batches of 226 shapes, 20 to 4,500 instances, one to eight
 // warps, both instantiations; full fleets, and fleets after some hundred steps), by terminations.  The choice is on average
-// within 1.2 % of the fastest with look-ahead (at worst 13), 2.8 % under the constant hazard, 3.4 % where terminations read
-// every row (5 in 100 more than 20 % off).  Neighbouring counts differ by up to a factor of two where rows fall out of the
-// cache, which the estimate does not know: 1,455 of G = 29, B = 128, H = 34, three steps: 534 us at two warps, 348 at three.
+// within 1.2 % of the fastest with look-ahead (at worst 13), 2.7 % under the constant hazard (5 in 100 more than 11), 3.3 %
+// where terminations read every row (5 in 100 more than 20).  Neighbouring counts differ by up to a factor of two where rows
+// fall out of the cache, which the estimate does not know: 1,455 of G = 29, B = 128, H = 34, three steps: 534 us at two warps, 348 at three.
 // us per call at 1, 2, 3, 4, 5 warps: 1,036 of G = 64, W = 1,024, H = 8: 62 / 63 / 65 / 56 / 57; 1,332: 104 / 88 / 71 / 64 / 76;
 // 2,960 of G = 15, W = 40, H = 19: 49 (41 lean) / 61 / 70 / 77 / 91; 1,036 of G = 24, B = 40, H = 12, terminations from rows: 79 /
 // 55 / 67 / 67 / 84.  Four warps at least for instances that stream 4,096 slots with rows of 8 to 19, or half as many when

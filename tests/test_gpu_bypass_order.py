@@ -1,5 +1,5 @@
 """br_bypass_dispatch may become resident while the kernel ahead of it still runs: what that kernel writes is what it reads, in
-eager streams and in captured graphs.  Whole numbers against the checker: the tolerance is equality."""
+eager streams and in captured graphs.  Whole numbers against the oracle: the tolerance is equality."""
 import numpy as np
 import pytest
 import torch
